@@ -199,8 +199,8 @@ struct SmallBlockArgs {
   int64_t scale_ld = 0;
 };
 cudaError_t small_block_launch(const SmallBlockArgs& a, cudaStream_t stream);
-// The same computation for r <= 256 in fp32 from fp32 partials, entirely in the shared memory of a
-// cluster of eight CTAs (no scratch).  small_block_launch uses it whenever it applies.
+// The same computation for r <= 256 in fp32 from fp32 partials, or r <= 192 in fp64 from fp64 partials, entirely in the
+// shared memory of a cluster of up to eight CTAs (no scratch).  small_block_launch uses it whenever it applies.
 bool small_block_cluster_supported(const SmallBlockArgs& a);
 cudaError_t small_block_cluster_launch(const SmallBlockArgs& a, cudaStream_t stream);
 

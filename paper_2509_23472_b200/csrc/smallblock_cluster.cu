@@ -1,28 +1,38 @@
-// Small-block factorisation for r <= 256, fp32: Cholesky factor of an r x r Gram matrix and the inverse
-// of that factor (the serial part of the orthonormalisation, the QR step of Algorithm 1 done through Gram
-// matrices), as one thread-block-cluster kernel whose working set never leaves shared memory.
+// Small-block factorisation: Cholesky factor of an r x r Gram matrix and the inverse of that factor (the serial part of
+// the orthonormalisation, the QR step of Algorithm 1 done through Gram matrices), as one thread-block-cluster kernel
+// whose working set never leaves shared memory.  fp32 up to r = 256, fp64 up to r = 192.
 //
-// The matrix is cut into 32 x 32 blocks.  Eight CTAs form a cluster:
-//   * CTA 0 is the pivot chain.  For block column k two warps factor the diagonal block in registers
-//     (one the columns 0..15, one the columns 16..31) while eight more invert the factor alongside; the
-//     CTA then forms L(k+1,k) = A(k+1,k) D_k^{-T} and applies it to the next diagonal block itself, so the
-//     chain waits for nothing but the two blocks it needs next.  One more warp only sends.
-//   * CTAs 1..7 own all blocks (dealt out column by column).  Half of their warps do the factorisation:
-//     for column k each forms its L(i,k), then updates its trailing blocks, A(i,j) -= L(i,k) L(j,k)^T; the
-//     two blocks the chain needs next, (k+2,k+1) and (k+2,k+2), are updated first and sent to CTA 0.
-//     The other half computes the inverse X = L^{-1} by block columns, right-looking: block row k becomes
-//     final at step k, X(k,j) = -D_k^{-1} T(k,j), is written out and added into the sums of the later rows,
-//     T(i,j) += L(i,k) X(k,j).  It stands back while the first half is on the chain's critical path.
-//   * Every finished block (D_k^{-1}, L(i,k)) is copied into the same slot of every worker's shared memory
-//     with bulk distributed-shared-memory copies (cp.async.bulk shared::cta -> shared::cluster) that count
-//     bytes on an mbarrier of the receiving CTA, so each worker ends up with a full copy of L without a
-//     global-memory round trip, a fence or a remote arrive.  (16-byte st.async stores were tried first:
-//     one barrier update per 16 bytes made the sends the bottleneck.)
-//   * 32 x 32 block products run on CUDA cores with 4 x 4 (or 2 x 2) outputs per thread; they are bound by
-//     shared-memory bandwidth (a 16-byte load costs about four cycles of the pipe), hence the tiling.
-// Every wait is bounded (a wall-clock limit for barriers, an iteration limit for flag words); on expiry the
-// CTA records LORACT_DEV_WAIT_EXPIRED, stops waiting and runs to its end (results are then invalid but
-// every access stays in bounds).
+// What bounds it is the chain of r pivots: nothing else is large (11 MFLOP at r = 256).  So the matrix is cut into
+// 32 x 32 blocks, block ROW i and block COLUMN i of the inverse belong to CTA i of the cluster, and everything flows
+// forward along the chain in groups of four columns -- no block ever makes a round trip:
+//   * pivot warp: factors the diagonal block, four columns at a time.  Every lane holds the 4 x 4 pivot block of a group
+//     and factors it for itself (one reciprocal square root, one product, one FMA per pivot on the chain), lane = matrix
+//     row otherwise.  Published columns are read back once by the warp itself to bring the next 4 x 4 block up to date.
+//   * follow-up warps (four, eight columns each): take every published group off the rest of the diagonal block and hand
+//     the pivot warp its columns one group ahead.  Between diagonal blocks they do the same for the block that the chain
+//     needs next: A(i, k+1) -= L(i, k) L(k+1, k)^T group by group while L(i, k) is being solved.
+//   * solver warps (four, eight rows each): L(i, k) = A(i, k) L(k, k)^-T by forward substitution while block k is being
+//     factored, and later the block column of the inverse, whose transpose solves the same system.  No inverse of a
+//     diagonal block is formed.
+//   * bulk warps (eight, two to a block): the updates nobody waits for, and the output.
+//   * the sender copies finished groups and blocks to the CTAs that need them (bulk distributed-shared-memory copies).
+// A block is stored as eight groups of [32 rows][4 columns]: a group is one contiguous copy, a lane's row and a
+// broadcast row are one 16-byte load each, without bank conflicts.  Loops over groups are rolled.  The hand-offs of the
+// pivot warp are named barriers (31 cycles against 110 for an mbarrier), all others are mbarriers that complete once.
+//
+// Shared-memory rates that fixed the shapes (measured on B200, cycles of the SM's pipe per warp instruction): a 16-byte
+// load takes two cycles when each quarter of the warp reads one address, four otherwise; a store and a load of it behind
+// a warp barrier take 30 cycles, a bulk copy to another CTA 280 (512 bytes) to 480 (4.6 KB) or 730 with seven receivers.
+//
+// Measured (one Gram matrix, back to back, against a form with one chain CTA, workers that sent blocks back to it and an
+// inverse of every diagonal block): fp32 r = 32 / 64 / 128 / 256: 7.1 / 8.5 / 13.8 / 28.8 us (7.4 / 11.8 / 20.0 / 40.4).
+// fp64, against a kernel that kept the matrix in global memory: r = 64 / 96 / 192: 13.0 / 17.7 / 33.7 us (75.8 / 120.9 /
+// 282).  Cycles per group of four columns: 398 in the pivot warp alone, about 475 with its companions at work; the step
+// from one diagonal block to the next adds about 1000.
+//
+// Every wait on another CTA is bounded by a wall-clock limit; on expiry the CTA records LORACT_DEV_WAIT_EXPIRED, stops
+// waiting and runs to its end (results are then invalid but every access stays in bounds).  The named barriers need no
+// limit: both sides run through the same fixed sequence whatever the data and whether or not a wait has expired.
 #include <atomic>
 
 #include "common.cuh"
@@ -32,21 +42,29 @@ namespace loract {
 namespace {
 
 constexpr int kB = 32;                   // block edge
-constexpr int kLd = 36;                  // padded row stride of a block slot (floats): rows 16-byte aligned
-constexpr int kSlot = kB * kLd;          // floats per slot
-constexpr int kSlotTx = kSlot * 4;        // bytes one sent block (padding included) adds to a barrier's transaction count
-constexpr int kMaxBlk = 8;               // r <= 256
-constexpr int kCl = 8;                   // CTAs per cluster
-constexpr int kWorkers = kCl - 1;
-constexpr int kCThreads = 512;
-constexpr int kGroup = 256;              // threads of a warp group (8 warps, 4 block rows each)
-constexpr int kMaxTri = kMaxBlk * (kMaxBlk + 1) / 2;
-constexpr int kXSlots = kMaxBlk;         // inverse blocks of the block columns one CTA owns
+constexpr int kMaxBlk = 8;               // block rows, and CTAs of the cluster
+constexpr int kWarps = 18;
+constexpr int kCThreads = kWarps * 32;
+constexpr int kPan = 8;                  // groups of four columns in a block
+constexpr int kMaxOff = kMaxBlk * (kMaxBlk - 1) / 2;
 constexpr uint64_t kClusterWaitNs = 50000000ull;  // 50 ms
+// Warp -> role (plus the index inside the role).  The scheduler a warp shares is its number mod 4: the pivot warp's
+// companions are the sender and three bulk warps, which are idle while it works.
+enum Role : int { R_PIVOT = 0, R_FOLLOW = 1, R_SOLVE = 5, R_BULK = 9, R_SEND = 17 };
+constexpr int kBulkWarps = 8;
+__constant__ unsigned char kRoleOf[kWarps] = {R_PIVOT, R_FOLLOW + 0, R_FOLLOW + 1, R_FOLLOW + 2, R_SEND, R_SOLVE + 0,
+                                              R_FOLLOW + 3, R_SOLVE + 2, R_BULK + 0, R_SOLVE + 3, R_SOLVE + 1, R_BULK + 6,
+                                              R_BULK + 1, R_BULK + 3, R_BULK + 5, R_BULK + 7, R_BULK + 2, R_BULK + 4};
+
+constexpr int kGrp = kB * 4;             // elements of a group of four columns
+constexpr int kBlk = kB * kB;            // elements of a block
+template <typename T> struct Cfg;
+template <> struct Cfg<float> { static constexpr int kMaxR = 256; };
+template <> struct Cfg<double> { static constexpr int kMaxR = 192; };
 
 struct SCParams {
   int r;
-  const float* partials;
+  const void* partials;    // T
   int n_partials;
   int64_t partial_stride;
   float shift_rel;
@@ -62,30 +80,18 @@ struct SCParams {
   __nv_bfloat16* linv_lo;
   uint32_t* dev_status;
   int64_t in_ld, out_ld;   // row strides of the partial matrices and of the outputs
-  const float* scale_diag; // optional: another matrix whose diagonal sets the scale of shift and floor
+  const float* scale_diag; // optional: another matrix whose diagonal sets the scale of shift and floor (fp32)
   int scale_n;
   int64_t scale_ld;
 };
 
-__device__ __forceinline__ int tri(int i, int j) { return i * (i + 1) / 2 + j; }
-
-// Worker (1..7) that owns block (i, j), i >= j: blocks are dealt out in column-major order, so the blocks
-// of one column sit on different CTAs.
-__device__ __forceinline__ int owner_of(int i, int j, int nblk) {
-  const int n = j * nblk - j * (j - 1) / 2 + (i - j);
-  return 1 + n % kWorkers;
-}
+__device__ __forceinline__ int off_slot(int i, int k) { return i * (i - 1) / 2 + k; }   // block (i, k), i > k
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ uint32_t map_to_cta(uint32_t local_addr, int rank) {
   uint32_t r;
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(local_addr), "r"(rank));
   return r;
-}
-__device__ __forceinline__ void st_cluster_v4(uint32_t addr, float4 v) {
-  asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(v.x), "f"(v.y), "f"(v.z),
-               "f"(v.w)
-               : "memory");
 }
 __device__ __forceinline__ void bar_init(uint64_t* bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(bar)), "r"(count));
@@ -97,11 +103,16 @@ __device__ __forceinline__ void bar_expect(uint64_t* bar, uint32_t bytes) {
 __device__ __forceinline__ void bar_arrive_local(uint64_t* bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(bar)) : "memory");
 }
+// All lanes have written; one arrival announces it.
+__device__ __forceinline__ void warp_arrive(uint64_t* bar, int lane) {
+  __syncwarp();
+  if (lane == 0) bar_arrive_local(bar);
+}
 __device__ __forceinline__ bool bar_try(uint64_t* bar) {
   uint32_t ok;
   asm volatile(
       "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], 0;\n\t"
+      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], 0;\n\t"
       "selp.b32 %0, 1, 0, p;\n\t}"
       : "=r"(ok)
       : "r"(smem_addr(bar))
@@ -113,16 +124,13 @@ __device__ __forceinline__ uint64_t timer_ns() {
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
   return t;
 }
-// Every barrier of this kernel completes exactly once (phase 0).  Called by ONE thread of a warp group;
-// the others block on the named barrier that follows, so that waiting costs no issue slots.  Returns
-// false once the CTA has given up.
+// Every barrier of this kernel completes exactly once (phase 0).  Called by all lanes of a warp.  Returns false once
+// the CTA has given up.
 __device__ __forceinline__ bool bar_wait(uint64_t* bar, volatile int* gave_up, uint64_t limit_ns = kClusterWaitNs) {
   if (bar_try(bar)) return true;
-  if (*gave_up) return false;
   uint64_t t0 = 0;
   for (uint32_t spin = 1;; ++spin) {
     if (bar_try(bar)) return true;
-    __nanosleep(20);
     if ((spin & 255u) == 0u) {
       if (*gave_up) return false;
       const uint64_t now = timer_ns();
@@ -131,63 +139,19 @@ __device__ __forceinline__ bool bar_wait(uint64_t* bar, volatile int* gave_up, u
     }
   }
 }
-__device__ __forceinline__ void group_sync(int id) {
-  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(kGroup) : "memory");
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+// Named barriers between the pivot warp and the follow-up warps, each used once: group g of the diagonal block has been
+// handed over (64 threads), group g has been published (the pivot warp and every follow-up warp that needs it).
+__device__ __forceinline__ void named_sync(int id, int threads) {
+  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
 }
-__device__ __forceinline__ void chain_sync() { asm volatile("bar.sync 3, 352;" ::: "memory"); }   // warps 0..10 of CTA 0
-__device__ __forceinline__ void cluster_sync_all() {
-  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+__device__ __forceinline__ void named_arrive(int id, int threads) {
+  asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(threads) : "memory");
 }
-
-// 32 x 32 block product C += A B^T on (32 / TM) * (32 / TN) threads, thread t of them holding the TM x TN
-// outputs C[TM tm + i][tn + NT j], NT = 32 / TN, tm = t / NT, tn = t % NT.  Both operands are read along
-// the contraction index with 16-byte loads: TM + TN loads feed 4 TM TN FMAs, which is what keeps the
-// shared-memory pipe (the limit of these products) below the FMA pipe.  The eight lanes of a quarter
-// warp read one row of A (a broadcast) and eight different rows of B, whose stride of 36 words spreads
-// them over all banks.
-template <int TM, int TN>
-__device__ __forceinline__ void tile_mac(float (&acc)[TM][TN], const float* __restrict__ A,
-                                         const float* __restrict__ Bm, int tm, int tn) {
-  constexpr int NT = kB / TN;
-#pragma unroll
-  for (int q4 = 0; q4 < kB / 4; ++q4) {
-    float4 a[TM], b[TN];
-#pragma unroll
-    for (int i = 0; i < TM; ++i) a[i] = *reinterpret_cast<const float4*>(A + (TM * tm + i) * kLd + 4 * q4);
-#pragma unroll
-    for (int j = 0; j < TN; ++j) b[j] = *reinterpret_cast<const float4*>(Bm + (tn + NT * j) * kLd + 4 * q4);
-#pragma unroll
-    for (int i = 0; i < TM; ++i)
-#pragma unroll
-      for (int j = 0; j < TN; ++j) {
-        acc[i][j] = fmaf(a[i].x, b[j].x, acc[i][j]);
-        acc[i][j] = fmaf(a[i].y, b[j].y, acc[i][j]);
-        acc[i][j] = fmaf(a[i].z, b[j].z, acc[i][j]);
-        acc[i][j] = fmaf(a[i].w, b[j].w, acc[i][j]);
-      }
-  }
-}
-template <int TM, int TN>
-__device__ __forceinline__ void tile_zero(float (&acc)[TM][TN]) {
-#pragma unroll
-  for (int i = 0; i < TM; ++i)
-#pragma unroll
-    for (int j = 0; j < TN; ++j) acc[i][j] = 0.f;
-}
-// dst[TM tm + i][tn + NT j] = alpha * acc[i][j] + beta * dst[...]
-template <int TM, int TN>
-__device__ __forceinline__ void tile_store(float* dst, const float (&acc)[TM][TN], int tm, int tn, float alpha,
-                                           bool add) {
-  constexpr int NT = kB / TN;
-#pragma unroll
-  for (int i = 0; i < TM; ++i)
-#pragma unroll
-    for (int j = 0; j < TN; ++j) {
-      float* d = dst + (TM * tm + i) * kLd + tn + NT * j;
-      *d = add ? fmaf(alpha, acc[i][j], *d) : alpha * acc[i][j];
-    }
-}
+__device__ __forceinline__ int id_staged(int g) { return 1 + g; }
+__device__ __forceinline__ int id_published(int g) { return 9 + g; }                 // g < 6: nobody needs the last two
+__device__ __forceinline__ int readers_of(int g) { return 32 * (4 - (g >> 1)); }     // pivot warp + follow-up warps
 
 // Bulk copy of `bytes` (a multiple of 16, both addresses 16-byte aligned) from this CTA's shared memory
 // into a peer's; on arrival `bytes` is taken off the transaction count of the peer's barrier `bar`.
@@ -200,254 +164,247 @@ __device__ __forceinline__ void bulk_to_peer(uint32_t dst_cluster_addr, uint32_t
 }
 __device__ __forceinline__ void fence_async_proxy() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
-// One warp has just written rows [row0, row0 + n_rows) of the block in `slot_local` (plain stores, every
-// lane has executed fence_async_proxy).  Lanes first_dst .. last_dst (except `skip`) each copy those rows
-// into the same slot of the CTA with their number, counting the bytes on that CTA's barrier `bar_local`.
-__device__ __forceinline__ void send_rows(const float* slot_local, int row0, int n_rows, const uint64_t* bar_local,
-                                          int first_dst, int last_dst, int skip, int lane) {
-  __syncwarp();
-  if (lane >= first_dst && lane <= last_dst && lane != skip) {
-    const uint32_t src = smem_addr(slot_local + row0 * kLd);
-    bulk_to_peer(map_to_cta(src, lane), src, (uint32_t)(n_rows * kLd * 4),
-                 map_to_cta(smem_addr(bar_local), lane));
-  }
+// ------------------------------------------------------------------ four consecutive elements
+template <typename T> struct V4 { T v[4]; };
+__device__ __forceinline__ V4<float> ld4(const float* p) {
+  const float4 q = *reinterpret_cast<const float4*>(p);
+  return {{q.x, q.y, q.z, q.w}};
+}
+__device__ __forceinline__ V4<double> ld4(const double* p) {
+  const double2 a = *reinterpret_cast<const double2*>(p), b = *reinterpret_cast<const double2*>(p + 2);
+  return {{a.x, a.y, b.x, b.y}};
+}
+__device__ __forceinline__ void st4(float* p, const V4<float>& x) {
+  *reinterpret_cast<float4*>(p) = make_float4(x.v[0], x.v[1], x.v[2], x.v[3]);
+}
+__device__ __forceinline__ void st4(double* p, const V4<double>& x) {
+  *reinterpret_cast<double2*>(p) = make_double2(x.v[0], x.v[1]);
+  *reinterpret_cast<double2*>(p + 2) = make_double2(x.v[2], x.v[3]);
+}
+// acc - a . b over four elements
+template <typename T>
+__device__ __forceinline__ T sub4(T acc, const V4<T>& a, const V4<T>& b) {
+#pragma unroll
+  for (int u = 0; u < 4; ++u) acc = fma(-a.v[u], b.v[u], acc);
+  return acc;
 }
 
-// The 32 x 32 diagonal block is handled by ten warps that run side by side: two factor it (one the
-// columns 0..15, one the columns 16..31), eight invert the factor, four columns each.  Straight-line
-// code like this runs at the rate instructions can be fetched, so the work per column is spread thin;
-// what remains per column is the latency of the pivot (broadcast, reciprocal square root, one FMA).
-//
-// As soon as column k of L is known it is published twice, both arrays starting out as kUnset so that a
-// consumer needs no flag and no fence -- it waits for its word to change:
-//   lcol[k][i] = L[i][k] (i > k), 1 / L[k][k] (i = k), 0 (i < k)             for the other factor warp
-//   mcol[k][i] = L[i][k] / L[k][k] (i > k), 1 / L[k][k] (i = k), 0 (i < k)   for the inverting warps
-constexpr uint32_t kUnset = 0xFFFFFFFFu;   // a NaN pattern arithmetic does not produce
-constexpr int kLcolLd = kLd;              // rows of `lcol` are read back as float4
-constexpr int kHalf = kB / 2;
-constexpr int kInvWarps = 8;
-constexpr int kInvCols = kB / kInvWarps;  // columns of the inverse one of those warps holds
-
-// One MUFU instruction (2 ulp); the argument is a clamped, positive, normal pivot.
-__device__ __forceinline__ float fast_rsqrt(float x) {
+// Reciprocal square root of a pivot (positive and normal where the result is used).  fp32: one MUFU instruction (2 ulp).
+// fp64: the hardware's starting value (about 20 bits) and two Newton steps y <- y + y (1 - x y^2) / 2.
+__device__ __forceinline__ float pivot_rsqrt(float x) {
   float y;
   asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
-__device__ __forceinline__ float not_unset(float v) { return __float_as_uint(v) == kUnset ? 0.f : v; }
-
-// Bounded wait for one word of lcol / mcol.
-__device__ __forceinline__ float wait_word(const float* addr, volatile int* gave_up) {
-  const volatile uint32_t* src = reinterpret_cast<const volatile uint32_t*>(addr);
-  uint32_t bits = *src;
-  for (uint32_t spin = 0; bits == kUnset; ++spin) {
-    if (spin > (1u << 20) || *gave_up) { *gave_up = 1; bits = 0u; break; }
-    __nanosleep(32);   // a warp that spins would take issue slots from the factoring warp next to it
-    bits = *src;
-  }
-  return __uint_as_float(bits);
+__device__ __forceinline__ double pivot_rsqrt(double x) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+#pragma unroll
+  for (int s = 0; s < 2; ++s) y = fma(0.5 * y, fma(-x * y, y, 1.0), y);
+  return y;
 }
 
-// One pivot column of the right-looking Cholesky inside a warp that holds the columns [c0, c0 + 16) of
-// every row (lane = row) as float2 pairs `a2`: takes the pivot's reciprocal square root `rinv`, forms and
-// publishes the column, updates the later columns of this warp with 16-byte broadcast loads and packed
-// FMAs, and starts the next pivot early.  K is the column inside the warp's range (compile time).
-template <int K>
-__device__ __forceinline__ void pivot_column(float2 (&a2)[kHalf / 2], float& diag, float& rinv, bool& bad,
-                                             bool& clamped, int c0, float* lcol, float* mcol, float pivot_floor,
-                                             int lane) {
-  const int k = c0 + K;
-  const float ak = (K & 1) ? a2[K >> 1].y : a2[K >> 1].x;
-  // a pivot that is not safely positive was replaced by the floor; its column is dropped (entries below
-  // such a pivot are rounding noise; dividing them by the tiny pivot would overflow later columns)
-  const float lik = (lane > k && !bad) ? ak * rinv : 0.f;   // L[lane][k]
-  lcol[k * kLcolLd + lane] = not_unset((lane == k) ? rinv : lik);
-  mcol[k * kLcolLd + lane] = not_unset((lane == k) ? rinv : lik * rinv);
-  diag = fmaf(-lik, lik, diag);
-  if (K + 1 < kHalf) {
-    // the next column first, through a shuffle (shorter than the round trip through shared memory), and
-    // the next pivot straight away: its square root is in flight while the rest of this column's
-    // updates are issued
-    const float l1 = __shfl_sync(0xffffffffu, lik, k + 1);
-    if ((K + 1) & 1) a2[(K + 1) >> 1].y = fmaf(-lik, l1, a2[(K + 1) >> 1].y);
-    else a2[(K + 1) >> 1].x = fmaf(-lik, l1, a2[(K + 1) >> 1].x);
-    float an = __shfl_sync(0xffffffffu, diag, k + 1);
-    bad = !(an > pivot_floor);
-    if (bad) { an = pivot_floor; clamped = true; }
-    rinv = fast_rsqrt(an);
-    __syncwarp();
-    const float2 nl = make_float2(-lik, -lik);
-    const float4* col = reinterpret_cast<const float4*>(lcol + k * kLcolLd + c0);
-    // columns K + 2 ..: 16-byte broadcast loads of the published column, packed FMAs.  In the quad that
-    // holds column K + 1 the entries up to it are masked out (K + 1 is done, earlier ones are not read).
-    constexpr int q1 = (K + 2) >> 2;
-#pragma unroll
-    for (int q = q1; q < kHalf / 4; ++q) {
-      float4 l2 = col[q];
-      if (4 * q + 0 < K + 2) l2.x = 0.f;
-      if (4 * q + 1 < K + 2) l2.y = 0.f;
-      if (4 * q + 2 < K + 2) l2.z = 0.f;
-      if (4 * q + 3 < K + 2) l2.w = 0.f;
-      a2[2 * q] = __ffma2_rn(nl, make_float2(l2.x, l2.y), a2[2 * q]);
-      a2[2 * q + 1] = __ffma2_rn(nl, make_float2(l2.z, l2.w), a2[2 * q + 1]);
-    }
-  }
-}
+// One published group of four columns of a diagonal block's factor: L[0..31][4], then the four reciprocals of the
+// diagonal with zero where a pivot was clamped (what a column of L is scaled with: entries below such a pivot are
+// rounding noise and are dropped), then the four reciprocals themselves (for the inverse).
+constexpr int kPanElems = kGrp + 8;
 
-template <int K>
-__device__ __forceinline__ void pivot_columns_from(float2 (&a2)[kHalf / 2], float& diag, float& rinv, bool& bad,
-                                                   bool& clamped, int c0, float* lcol, float* mcol,
-                                                   float pivot_floor, int lane) {
-  if constexpr (K < kHalf) {
-    pivot_column<K>(a2, diag, rinv, bad, clamped, c0, lcol, mcol, pivot_floor, lane);
-    pivot_columns_from<K + 1>(a2, diag, rinv, bad, clamped, c0, lcol, mcol, pivot_floor, lane);
-  }
-}
-
-// Factor warp `half` (0: columns 0..15, 1: columns 16..31) of the diagonal block in `slot`.  The second
-// warp first follows the columns the first one publishes, taking them off its own columns, then carries
-// on with the pivots 16..31.  Returns true if a pivot was clamped.
-__device__ __forceinline__ bool factor_diag_half(const float* slot, float* lcol, float* mcol, float pivot_floor,
-                                                 volatile int* gave_up, int half, int lane) {
-  const int c0 = half * kHalf;
-  float2 a2[kHalf / 2];   // row `lane`, columns (c0 + 2p, c0 + 2p + 1), below the diagonal only
-  float diag = slot[lane * kLd + lane];   // used by the lanes whose diagonal lies in this warp's columns
-  if (half == 0) {
-#pragma unroll
-    for (int pp = 0; pp < kHalf / 2; ++pp)
-      a2[pp] = make_float2(2 * pp < lane ? slot[lane * kLd + 2 * pp] : 0.f,
-                           2 * pp + 1 < lane ? slot[lane * kLd + 2 * pp + 1] : 0.f);
-  } else {
-    // The following warp.  Rows 0..15 have nothing below the diagonal in the columns 16..31, so their lanes
-    // would idle: instead lane i and lane i - 16 share row i while the columns of the first warp are taken
-    // off (lane i its columns 16..23, lane i - 16 the columns 24..31), which halves the instructions per
-    // followed column -- this warp ran a thousand cycles behind the one it follows -- and the upper lanes
-    // collect the whole row with eight shuffles before their own pivots start.  Two columns are taken per
-    // round trip: the updates commute (both use final values of L) and their loads overlap.
-    const int row = lane | kHalf;
-    const int cb = kHalf + ((lane < kHalf) ? kHalf / 2 : 0);   // first of this lane's eight columns
-    float2 f[kHalf / 4];
-#pragma unroll
-    for (int pp = 0; pp < kHalf / 4; ++pp)
-      f[pp] = make_float2(cb + 2 * pp < row ? slot[row * kLd + cb + 2 * pp] : 0.f,
-                          cb + 2 * pp + 1 < row ? slot[row * kLd + cb + 2 * pp + 1] : 0.f);
-#pragma unroll
-    for (int k = 0; k < kHalf; k += 2) {
-      const float l0 = wait_word(lcol + k * kLcolLd + row, gave_up);         // L[row][k]
-      const float l1 = wait_word(lcol + (k + 1) * kLcolLd + row, gave_up);   // L[row][k + 1]
-      __syncwarp();
-      const float2 n0 = make_float2(-l0, -l0), n1 = make_float2(-l1, -l1);
-      const float4* c0p = reinterpret_cast<const float4*>(lcol + k * kLcolLd + cb);
-      const float4* c1p = reinterpret_cast<const float4*>(lcol + (k + 1) * kLcolLd + cb);
-      const float4 la0 = c0p[0], la1 = c0p[1], lb0 = c1p[0], lb1 = c1p[1];
-      if (lane >= kHalf) diag = fmaf(-l1, l1, fmaf(-l0, l0, diag));
-      f[0] = __ffma2_rn(n0, make_float2(la0.x, la0.y), f[0]);
-      f[1] = __ffma2_rn(n0, make_float2(la0.z, la0.w), f[1]);
-      f[2] = __ffma2_rn(n0, make_float2(la1.x, la1.y), f[2]);
-      f[3] = __ffma2_rn(n0, make_float2(la1.z, la1.w), f[3]);
-      f[0] = __ffma2_rn(n1, make_float2(lb0.x, lb0.y), f[0]);
-      f[1] = __ffma2_rn(n1, make_float2(lb0.z, lb0.w), f[1]);
-      f[2] = __ffma2_rn(n1, make_float2(lb1.x, lb1.y), f[2]);
-      f[3] = __ffma2_rn(n1, make_float2(lb1.z, lb1.w), f[3]);
-    }
-#pragma unroll
-    for (int pp = 0; pp < kHalf / 4; ++pp) {
-      // columns 24..31 of row `lane` come up from lane - 16 (the source lane wraps for the lower lanes,
-      // whose registers are cleared right after)
-      const float tx = __shfl_sync(0xffffffffu, f[pp].x, (lane + kHalf) & 31);
-      const float ty = __shfl_sync(0xffffffffu, f[pp].y, (lane + kHalf) & 31);
-      a2[pp] = (lane >= kHalf) ? f[pp] : make_float2(0.f, 0.f);
-      a2[kHalf / 4 + pp] = (lane >= kHalf) ? make_float2(tx, ty) : make_float2(0.f, 0.f);
-    }
-  }
+// ------------------------------------------------------------------ the pivots (one warp, lane = row of the block)
+// `staged`: the diagonal block, whose group g has every earlier group but g - 1 taken off when id_staged(g) completes.
+// Rows of a group above its own diagonal carry values nobody reads.  Returns true if a pivot was clamped.
+template <typename T>
+__device__ __forceinline__ bool factor_diagonal(const T* staged, T* panels, uint64_t* bars, T floor_, int lane) {
   bool clamped = false;
-  float akk = __shfl_sync(0xffffffffu, diag, c0);
-  bool bad = !(akk > pivot_floor);
-  if (bad) { akk = pivot_floor; clamped = true; }
-  float rinv = fast_rsqrt(akk);
-  pivot_columns_from<0>(a2, diag, rinv, bad, clamped, c0, lcol, mcol, pivot_floor, lane);
+  const T rfloor = pivot_rsqrt(floor_);
+  V4<T> x = {{(T)0, (T)0, (T)0, (T)0}};
+  V4<T> b[4] = {x, x, x, x};
+  T* pan = panels;
+#pragma unroll 1
+  for (int p = 0; p < kPan; ++p) {
+    named_sync(id_staged(p), 64);
+    V4<T> a = ld4(staged + lane * 4);
+    V4<T> g[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) g[i] = ld4(staged + (4 * p + i) * 4);
+    if (p > 0) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) b[i] = ld4(pan - kPanElems + (4 * p + i) * 4);
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+#pragma unroll
+      for (int i = j; i < 4; ++i) g[i].v[j] = sub4(g[i].v[j], b[i], b[j]);
+      a.v[j] = sub4(a.v[j], x, b[j]);
+    }
+    V4<T> rz, rd;
+    auto pivot = [&](int c, T d) {
+      const bool bad = !(d > floor_);
+      clamped |= bad;
+      const T y = pivot_rsqrt(d);
+      rz.v[c] = bad ? (T)0 : y;
+      rd.v[c] = bad ? rfloor : y;
+    };
+    // column 0
+    pivot(0, g[0].v[0]);
+    const T l10 = g[1].v[0] * rz.v[0], l20 = g[2].v[0] * rz.v[0], l30 = g[3].v[0] * rz.v[0];
+    x.v[0] = a.v[0] * rz.v[0];
+    const T d1 = fma(-l10, l10, g[1].v[1]);
+    const T s21 = fma(-l20, l10, g[2].v[1]), s31 = fma(-l30, l10, g[3].v[1]), t1 = fma(-x.v[0], l10, a.v[1]);
+    const T d2 = fma(-l20, l20, g[2].v[2]), s32 = fma(-l30, l20, g[3].v[2]), t2 = fma(-x.v[0], l20, a.v[2]);
+    const T d3 = fma(-l30, l30, g[3].v[3]), t3 = fma(-x.v[0], l30, a.v[3]);
+    // column 1
+    pivot(1, d1);
+    const T l21 = s21 * rz.v[1], l31 = s31 * rz.v[1];
+    x.v[1] = t1 * rz.v[1];
+    const T e2 = fma(-l21, l21, d2), u32 = fma(-l31, l21, s32), v2 = fma(-x.v[1], l21, t2);
+    const T e3 = fma(-l31, l31, d3), v3 = fma(-x.v[1], l31, t3);
+    // column 2
+    pivot(2, e2);
+    const T l32 = u32 * rz.v[2];
+    x.v[2] = v2 * rz.v[2];
+    const T f3 = fma(-l32, l32, e3), w3 = fma(-x.v[2], l32, v3);
+    // column 3
+    pivot(3, f3);
+    x.v[3] = w3 * rz.v[3];
+    st4(pan + lane * 4, x);
+    if (lane == 0) st4(pan + kGrp, rz);
+    if (lane == 1) st4(pan + kGrp + 4, rd);
+    __syncwarp();
+    if (p < kPan - 2) named_arrive(id_published(p), readers_of(p));
+    if (lane == 0) bar_arrive_local(bars + p);
+    staged += kGrp;
+    pan += kPanElems;
+  }
   return clamped;
 }
 
-// Inverting warp `part` (lane i holds row i of X = L^{-1}, columns 4 part .. 4 part + 3): takes the scaled
-// columns of L as they appear in `mcol` and works right-looking: once column k is known, row k of X is
-// final up to its scale 1 / L[k][k], and every later row takes L[i][k] / L[k][k] times the unscaled row k
-// (four shuffles from lane k) off -- no serial dot products.  Columns k < 4 part cannot touch this warp's
-// columns and are skipped.  Writes its columns of X (lower triangular, zeros above) into `slot`.
-__device__ __forceinline__ void invert_diag_part(float* slot, const float* mcol, volatile int* gave_up, int part,
-                                                 int lane) {
-  const int j0 = part * kInvCols;
-  float2 x01 = make_float2(j0 == lane ? 1.f : 0.f, j0 + 1 == lane ? 1.f : 0.f);
-  float2 x23 = make_float2(j0 + 2 == lane ? 1.f : 0.f, j0 + 3 == lane ? 1.f : 0.f);
-  float my_rinv = 1.f;
-  // Four columns per round: the words of all four are fetched together (and waited for only if one is still
-  // unset), then the four updates run back to back with nothing in them but the broadcast of row k and two
-  // packed FMAs.  One column per round cost about 180 cycles, a chain of load, compare, branch, select,
-  // shuffle and FMA latencies, which is more than the factoring warps need per pivot: the warp with all 32
-  // columns to go through finished 1400 cycles after the last pivot and held up the whole block step.
-  // The count of columns, 32 - 4 part, is a multiple of four.  A rolled loop: small enough to be served from
-  // the innermost instruction cache.
+// ------------------------------------------------------------------ forward substitution (four warps, eight rows each)
+// Solves x L^T = t in place (blk: t, then x) for the triangular factor L of a diagonal block that is being published.
+// A lane holds one row's columns of the groups cg and cg + 4 (cg = lane / 8): the lanes of the current group form x, the
+// others get it by shuffle and take the group off their columns.  `inverse`: scale with the plain reciprocals.
+template <typename T, int H>
+__device__ __forceinline__ void solve_half(V4<T> (&acc)[2], T* blk, const T* panels, uint64_t* pan_bars, uint64_t* sol_bars,
+                                           bool inverse, int row, int lane, volatile int* gave_up) {
+  const int cg = lane >> 3;
 #pragma unroll 1
-  for (int k = j0; k < kB; k += 4) {
-    uint32_t bits[4];
+  for (int q = 0; q < 4; ++q) {
+    const int p = 4 * H + q;
+    const T* pan = panels + p * kPanElems;
+    const T* low = pan + 16 * p;                           // row 4 p
+    bar_wait(pan_bars + p, gave_up);
+    const V4<T> rr = ld4(pan + kGrp + (inverse ? 4 : 0));
+    const V4<T> r1 = ld4(low + 4), r2 = ld4(low + 8), r3 = ld4(low + 12);
+    const V4<T>& t = acc[H];
+    V4<T> x;
+    x.v[0] = t.v[0] * rr.v[0];
+    x.v[1] = fma(-x.v[0], r1.v[0], t.v[1]) * rr.v[1];
+    x.v[2] = fma(-x.v[1], r2.v[1], fma(-x.v[0], r2.v[0], t.v[2])) * rr.v[2];
+    x.v[3] = fma(-x.v[2], r3.v[2], fma(-x.v[1], r3.v[1], fma(-x.v[0], r3.v[0], t.v[3]))) * rr.v[3];
+    if (cg == q) st4(blk + p * kGrp + row * 4, x);
+    warp_arrive(sol_bars + p, lane);
 #pragma unroll
-    for (int q = 0; q < 4; ++q)
-      bits[q] = *reinterpret_cast<const volatile uint32_t*>(mcol + (k + q) * kLcolLd + lane);
-    float w[4];
+    for (int u = 0; u < 4; ++u) x.v[u] = __shfl_sync(0xffffffffu, x.v[u], (q << 3) | (lane & 7));
 #pragma unroll
-    for (int q = 0; q < 4; ++q)
-      w[q] = (bits[q] != kUnset) ? __uint_as_float(bits[q]) : wait_word(mcol + (k + q) * kLcolLd + lane, gave_up);
-    __syncwarp();
+    for (int h = H; h < 2; ++h)
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int kk = k + q;
-      my_rinv = (lane == kk) ? w[q] : my_rinv;
-      const float m = (lane > kk) ? w[q] : 0.f;
-      const float2 nm = make_float2(-m, -m);
-      const float2 r01 = make_float2(__shfl_sync(0xffffffffu, x01.x, kk), __shfl_sync(0xffffffffu, x01.y, kk));
-      const float2 r23 = make_float2(__shfl_sync(0xffffffffu, x23.x, kk), __shfl_sync(0xffffffffu, x23.y, kk));
-      x01 = __ffma2_rn(nm, r01, x01);
-      x23 = __ffma2_rn(nm, r23, x23);
-    }
+      for (int j = 0; j < 4; ++j) acc[h].v[j] = sub4(acc[h].v[j], x, ld4(pan + (4 * (cg + 4 * h) + j) * 4));
   }
-  *reinterpret_cast<float4*>(slot + lane * kLd + j0) =
-      make_float4(x01.x * my_rinv, x01.y * my_rinv, x23.x * my_rinv, x23.y * my_rinv);
-  fence_async_proxy();   // the block is sent on with a bulk copy
-  __syncwarp();
 }
 
-__global__ void __launch_bounds__(kCThreads, 1) small_block_cluster_kernel(SCParams p) {
-  extern __shared__ __align__(16) unsigned char sc_smem[];
-  // all barriers complete once; the same layout in every CTA, so a local address maps to any peer
-  __shared__ __align__(8) uint64_t dinv_bar[kMaxBlk];    // workers: D_k^{-1} has arrived
-  __shared__ __align__(8) uint64_t panel_bar[kMaxBlk];   // workers: every L(i,k), i > k, has arrived
-  __shared__ __align__(8) uint64_t chain_bar[kMaxBlk];   // CTA 0: blocks (j, j-1) and (j, j) have arrived
-  // workers: L(k+1, k) and L(k+2, k) have arrived -- all that the two blocks CTA 0 waits for next need, so
-  // their update does not wait for the whole panel (every worker's blocks, copied to every other worker)
-  __shared__ __align__(8) uint64_t urgent_bar[kMaxBlk];
-  __shared__ float s_red[kCThreads / 32];
-  __shared__ float s_shift, s_floor;
-  __shared__ int s_gave_up;
-  __shared__ volatile int s_urgent;                       // workers: the factorisation half is on the chain's critical path
-  __shared__ volatile int s_chain_step;                   // CTA 0: what the sender warps may send
-  __shared__ int s_clamped;
-  __shared__ float s_est[kCl];       // CTA 0: the workers' shares of the estimate; workers: per-warp sums
-  // blocks (i, j) owned by this CTA, in column-major order
-  __shared__ unsigned char s_mine_i[kMaxTri], s_mine_j[kMaxTri];
-  __shared__ int s_n_mine;
+// ------------------------------------------------------------------ block updates
+// acc (this lane's row, columns 8 w .. 8 w + 7) -= (row of group A) . (rows of group B)
+template <typename T>
+__device__ __forceinline__ void take_off_group(V4<T> (&acc)[2], const T* A, const T* Bg, int w, int lane) {
+  const V4<T> a = ld4(A + lane * 4);
+#pragma unroll
+  for (int h = 0; h < 2; ++h)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[h].v[j] = sub4(acc[h].v[j], a, ld4(Bg + (8 * w + 4 * h + j) * 4));
+}
+// C (or zero) -= A B^T for rows 16 half .. 16 half + 15 of a block, 4 x 4 outputs per lane: rows tm + 4 i (one address per
+// quarter warp), columns tn + 8 j (32 consecutive rows of B).
+template <typename T>
+__device__ __forceinline__ void take_off_half(T* C, const T* A, const T* Bm, bool from_zero, int half, int lane) {
+  const int row0 = 16 * half + (lane >> 3), col0 = lane & 7;
+  T acc[4][4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[i][j] = (T)0;
+#pragma unroll 2
+  for (int q = 0; q < kPan; ++q) {
+    V4<T> b[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) b[j] = ld4(Bm + q * kGrp + (col0 + 8 * j) * 4);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const V4<T> a = ld4(A + q * kGrp + (row0 + 4 * i) * 4);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) acc[i][j] = sub4(acc[i][j], a, b[j]);
+    }
+  }
+#pragma unroll
+  for (int j = 0; j < 4; ++j)
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int col = col0 + 8 * j;
+      T* c = C + (col >> 2) * kGrp + (row0 + 4 * i) * 4 + (col & 3);
+      *c = from_zero ? acc[i][j] : *c + acc[i][j];
+    }
+}
 
-  float* slots = reinterpret_cast<float*>(sc_smem);        // kMaxTri slots: the matrix, then L / D^{-1}
-  float* xt = slots + kMaxTri * kSlot;                      // kXSlots slots: transposed inverse blocks
-  float* lcol = xt + kXSlots * kSlot;                       // columns of the diagonal block's factor
-  float* mcol = lcol + kB * kLcolLd;                        // the same, scaled by the pivot
+__device__ __forceinline__ void load_quad(const float* src, V4<float>& s) {
+  const float4 v = __ldg(reinterpret_cast<const float4*>(src));
+  s.v[0] += v.x; s.v[1] += v.y; s.v[2] += v.z; s.v[3] += v.w;
+}
+__device__ __forceinline__ void load_quad(const double* src, V4<double>& s) {
+  const double2 a = __ldg(reinterpret_cast<const double2*>(src)), b = __ldg(reinterpret_cast<const double2*>(src) + 1);
+  s.v[0] += a.x; s.v[1] += a.y; s.v[2] += b.x; s.v[3] += b.y;
+}
+
+// Shared memory of every CTA (the same layout in all of them, so a local address maps to any peer), in elements of T:
+// off-diagonal blocks (own row: A, then L; other rows: L as it arrives), the blocks of the own column of the inverse
+// (transposed), and the published diagonal blocks.  The own diagonal block borrows a slot of the inverse that is not in
+// use yet (the last one, first written after the block has been factored) or never used by this CTA.
+__host__ __device__ constexpr int x_slots(int nblk) { return nblk < 3 ? 3 : nblk; }
+template <typename T>
+__host__ __device__ constexpr size_t smem_elems(int nblk) {
+  return (size_t)kBlk * (nblk * (nblk - 1) / 2 + x_slots(nblk)) + (size_t)nblk * kPan * kPanElems;
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kCThreads, 1) small_block_cluster_kernel(SCParams p) {
+  constexpr uint32_t kBlkBytes = (uint32_t)(kBlk * sizeof(T)), kGrpBytes = (uint32_t)(kGrp * sizeof(T));
+  constexpr uint32_t kPanBytes = (uint32_t)(kPanElems * sizeof(T));
+  extern __shared__ __align__(16) unsigned char sc_smem[];
+  __shared__ __align__(8) uint64_t pan_bar[kMaxBlk][kPan];   // group g of diagonal block k is here
+  __shared__ __align__(8) uint64_t next_bar[kMaxBlk][kPan];  // group g of L(k + 1, k), another CTA's, is here
+  __shared__ __align__(8) uint64_t off_bar[kMaxOff];         // L(i, k), i >= k + 2, another CTA's, is here
+  __shared__ __align__(8) uint64_t sol_bar[kMaxBlk][kPan];   // group g of L(own, k), k < own, or X(k, own) is solved
+  __shared__ __align__(8) uint64_t rdy_bar[kMaxBlk];         // the block to solve at step k has every update
+  __shared__ __align__(8) uint64_t bulk_bar[kMaxBlk];        // block j has every update but that of step j - 1
+  __shared__ T s_red[kWarps];
+  __shared__ T s_shift, s_floor;
+  __shared__ int s_gave_up;
+  __shared__ float s_est[kBulkWarps * kMaxBlk];   // CTA 0: the shares of the estimate
 
   uint32_t rank;
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
-  const int cta = (int)rank;
+  const int me = (int)rank;              // block row and block column of the inverse of this CTA
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int r = p.r;
   const int nblk = (r + kB - 1) / kB;
-  const int ntri = nblk * (nblk + 1) / 2;
+  const int noff = nblk * (nblk - 1) / 2;
+  const bool active = me < nblk;
+  T* off = reinterpret_cast<T*>(sc_smem);
+  T* xt = off + (size_t)noff * kBlk;                     // block (k, own) of the inverse at slot k
+  T* pans = xt + (size_t)x_slots(nblk) * kBlk;
+  T* own = xt + (size_t)(me + 2 <= nblk - 1 ? nblk - 1 : (me >= 1 ? 0 : 2)) * kBlk;
+  auto slot = [&](int i, int k) { return off + (size_t)off_slot(i, k) * kBlk; };
+  auto panel = [&](int k) { return pans + (size_t)k * kPan * kPanElems; };
+  // the block this CTA solves at step k, and where an update of block j (row: j < me, diagonal: j = me) goes
+  auto solved = [&](int k) { return k < me ? slot(me, k) : xt + (size_t)k * kBlk; };
+  auto target = [&](int j) { return j == me ? own : solved(j); };
 
   // A gated launch that is not needed leaves before any set-up: the same word in every CTA of the cluster, written at
   // least two kernels back in the stream (this grid only starts once its predecessor has passed its own
@@ -455,88 +412,62 @@ __global__ void __launch_bounds__(kCThreads, 1) small_block_cluster_kernel(SCPar
   // must imply the completion of every earlier one.
   if (p.gate != nullptr && *(const volatile uint32_t*)p.gate == 0u) { pdl_wait(); pdl_launch_dependents(); return; }
 
-  // ---- set-up, spread over threads: barriers (with the byte counts they will receive, known up front),
-  // this CTA's block list, the sentinel words of the diagonal-block column buffer
-  if (tid < kMaxBlk) {
-    const int k = tid;
-    bar_init(&dinv_bar[k], 1);
-    bar_init(&panel_bar[k], 2);   // the byte count (below) and the CTA's own blocks of the column
-    bar_init(&chain_bar[k], 1);
-    bar_init(&urgent_bar[k], 2);  // the byte count, and this CTA's own L(k+2, k) (at once if it owns none)
+  // ---- set-up: barriers, with the byte counts they will receive
+  if (tid < kMaxBlk * kPan) {
+    const int k = tid / kPan, q = tid % kPan;
+    bar_init(&pan_bar[k][q], 1);
+    bar_init(&next_bar[k][q], 1);
+    bar_init(&sol_bar[k][q], 4);
+    if (q == 0) { bar_init(&rdy_bar[k], 4); bar_init(&bulk_bar[k], 2); }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    if (k < nblk) {
-      if (cta != 0) {
-        bar_expect(&dinv_bar[k], kSlotTx);
-        if (k + 1 < nblk) {
-          int from_peers = 0;   // rows k + 3 and below; L(k+1, k) (from CTA 0) and L(k+2, k) count on urgent_bar
-          for (int bi = k + 3; bi < nblk; ++bi) from_peers += owner_of(bi, k, nblk) != cta ? 1 : 0;
-          bar_expect(&panel_bar[k], (uint32_t)from_peers * kSlotTx);
-          const bool own_k2 = k + 2 < nblk && owner_of(k + 2, k, nblk) == cta;
-          const bool peer_k2 = k + 2 < nblk && !own_k2;
-          bar_expect(&urgent_bar[k], (peer_k2 ? 2u : 1u) * kSlotTx);
-          if (!own_k2) bar_arrive_local(&urgent_bar[k]);
-        }
-      } else if (k >= 2) {
-        bar_expect(&chain_bar[k], 2 * kSlotTx);
-      }
-    }
-  } else if (tid == 32) {
+    if (active && k < nblk && k != me) bar_expect(&pan_bar[k][q], kPanBytes);
+    if (active && k + 1 < nblk && k + 1 != me) bar_expect(&next_bar[k][q], kGrpBytes);
+  } else if (tid >= 64 && tid < 64 + kMaxOff) {
+    const int b = tid - 64;
+    int i = 1;
+    while (off_slot(i + 1, 0) <= b) ++i;
+    const int k = b - off_slot(i, 0);
+    bar_init(&off_bar[b], 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    if (active && i < nblk && i != me && i >= k + 2 && (me <= k || me > i)) bar_expect(&off_bar[b], kBlkBytes);
+  } else if (tid == 64 + kMaxOff) {
     s_gave_up = 0;
-    s_clamped = 0;
-    s_chain_step = 0;
-    s_urgent = 0;
-    int n = 0;
-    for (int bj = 0; bj < nblk; ++bj)
-      for (int bi = bj; bi < nblk; ++bi)
-        if (owner_of(bi, bj, nblk) == cta) { s_mine_i[n] = (unsigned char)bi; s_mine_j[n] = (unsigned char)bj; ++n; }
-    s_n_mine = n;
   }
-  for (int e = tid; e < 2 * kB * kLcolLd; e += kCThreads) reinterpret_cast<uint32_t*>(lcol)[e] = kUnset;
+  __syncthreads();
+  cluster_arrive();                       // waited for below: nobody sends before every CTA's barriers exist
   // everything above overlaps the tail of the previous kernel; global memory only from here on
   pdl_wait();
   pdl_launch_dependents();
-  // The same word in every CTA, read before anything crosses between them: the whole cluster leaves together.
-  if (p.gate != nullptr && *(const volatile uint32_t*)p.gate == 0u) return;
 
-  // ---- load.  Block t is summed over the partials by CTA t mod 8 and written into the slot of the CTA
-  // that works on it first (CTA 0 for block rows 0 and 1, the owner otherwise).  All global loads of a
-  // thread are issued before the first use; the trace of W (same order of additions in every CTA) gives
-  // the diagonal shift and the pivot floor.
+  // ---- load: this CTA's block row, summed over the partials; the trace of W (same order of additions in every CTA)
+  // gives the diagonal shift and the pivot floor.  All loads of a thread are issued before the first use.
   {
-    float t = 0.f;
+    const T* parts = (const T*)p.partials;
+    T t = (T)0;
     const int n_scale = p.scale_diag ? p.scale_n : r;
     if (p.scale_diag) {
-      for (int i = tid; i < n_scale; i += kCThreads) t += __ldg(p.scale_diag + (int64_t)i * (p.scale_ld + 1));
+      for (int i = tid; i < n_scale; i += kCThreads) t += (T)__ldg(p.scale_diag + (int64_t)i * (p.scale_ld + 1));
     } else {
       for (int i = tid; i < r; i += kCThreads) {
-        float d = 0.f;
+        T d = (T)0;
         for (int q = 0; q < p.n_partials; ++q)
-          d += __ldg(p.partials + (int64_t)q * p.partial_stride + (int64_t)i * p.in_ld + i);
+          d += __ldg(parts + (int64_t)q * p.partial_stride + (int64_t)i * p.in_ld + i);
         t += d;
       }
     }
-    constexpr int kMaxMine = (kMaxTri + kCl - 1) / kCl;          // blocks one CTA loads
-    constexpr int kPerThread = kMaxMine * (kB * kB / 4) / kCThreads + 1;
-    float4 acc[kPerThread];
-    const int n_load = (ntri - cta + kCl - 1) / kCl;              // blocks cta, cta + 8, ...
+    constexpr int kQuads = kB * kB / 4;
+    constexpr int kPerThread = ((Cfg<T>::kMaxR / kB) * kQuads + kCThreads - 1) / kCThreads;
+    V4<T> acc[kPerThread];
+    const int n_quads = active ? (me + 1) * kQuads : 0;
 #pragma unroll
     for (int u = 0; u < kPerThread; ++u) {
-      acc[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+      acc[u] = {{(T)0, (T)0, (T)0, (T)0}};
       const int e = tid + u * kCThreads;
-      const int lb = e >> 8;                                      // 256 quads per block
-      if (lb >= n_load) continue;
-      const int blk = cta + lb * kCl;
-      int bi = 0;
-      while (tri(bi + 1, 0) <= blk) ++bi;
-      const int bj = blk - tri(bi, 0);
-      const int a = (e & 255) >> 3, q4 = e & 7;
-      const int row = bi * kB + a, col = bj * kB + 4 * q4;
+      if (e >= n_quads) continue;
+      const int row = me * kB + ((e & (kQuads - 1)) >> 3), col = (e / kQuads) * kB + 4 * (e & 7);
       if (row < r && col < r) {
-        const float* src = p.partials + (int64_t)row * p.in_ld + col;
-        for (int q = 0; q < p.n_partials; ++q) {
-          const float4 v = __ldg(reinterpret_cast<const float4*>(src + (int64_t)q * p.partial_stride));
-          acc[u].x += v.x; acc[u].y += v.y; acc[u].z += v.z; acc[u].w += v.w;
-        }
+        const T* src = parts + (int64_t)row * p.in_ld + col;
+        for (int q = 0; q < p.n_partials; ++q) load_quad(src + (int64_t)q * p.partial_stride, acc[u]);
       }
     }
 #pragma unroll
@@ -544,312 +475,215 @@ __global__ void __launch_bounds__(kCThreads, 1) small_block_cluster_kernel(SCPar
     if (lane == 0) s_red[warp] = t;
     __syncthreads();
     if (tid == 0) {
-      float tr = 0.f;
-      for (int q = 0; q < kCThreads / 32; ++q) tr += s_red[q];
-      float mean_diag = tr / (float)n_scale;
-      if (!(mean_diag == mean_diag) || mean_diag > 3.0e38f || mean_diag < 0.f) {
-        if (p.dev_status && cta == 0) atomicOr(p.dev_status, LORACT_DEV_NONFINITE);
-        mean_diag = 1.f;
+      T tr = (T)0;
+      for (int q = 0; q < kWarps; ++q) tr += s_red[q];
+      T mean_diag = tr / (T)n_scale;
+      if (!(mean_diag == mean_diag) || mean_diag > (T)3.0e38 || mean_diag < (T)0) {
+        if (p.dev_status && me == 0) atomicOr(p.dev_status, LORACT_DEV_NONFINITE);
+        mean_diag = (T)1;
       }
-      if (mean_diag == 0.f) mean_diag = 1.f;
-      s_shift = p.shift_rel * mean_diag;
-      s_floor = mean_diag * 1e-7f;
+      if (mean_diag == (T)0) mean_diag = (T)1;
+      s_shift = (T)p.shift_rel * mean_diag;
+      s_floor = mean_diag * (sizeof(T) == 8 ? (T)1e-15 : (T)1e-7);
     }
     __syncthreads();
-    const float shift = s_shift;
+    const T shift = s_shift;
 #pragma unroll
     for (int u = 0; u < kPerThread; ++u) {
       const int e = tid + u * kCThreads;
-      const int lb = e >> 8;
-      if (lb >= n_load) continue;
-      const int blk = cta + lb * kCl;
-      int bi = 0;
-      while (tri(bi + 1, 0) <= blk) ++bi;
-      const int bj = blk - tri(bi, 0);
-      const int a = (e & 255) >> 3, q4 = e & 7;
-      float4 sv = acc[u];
-      if (bi == bj) {
+      if (e >= n_quads) continue;
+      const int bj = e / kQuads, a = (e & (kQuads - 1)) >> 3, q4 = e & 7;
+      T* dst = target(bj) + q4 * kGrp + a * 4;
+      if (bj == me) {
         const int dcol = a - 4 * q4;  // position of the diagonal element inside this quad, if any
-        const bool in_range = (bi * kB + a) < r;            // padding rows of a ragged last block: identity
-        const float mul = in_range ? p.shift_diag_rel : 0.f, add = in_range ? shift : 1.f;
-        if (dcol == 0) sv.x += sv.x * mul + add; else if (dcol == 1) sv.y += sv.y * mul + add;
-        else if (dcol == 2) sv.z += sv.z * mul + add; else if (dcol == 3) sv.w += sv.w * mul + add;
+        const bool in_range = (me * kB + a) < r;            // padding rows of a ragged last block: identity
+        const T mul = in_range ? (T)p.shift_diag_rel : (T)0, add = in_range ? shift : (T)1;
+#pragma unroll
+        for (int h = 0; h < 4; ++h)
+          if (dcol == h) acc[u].v[h] += acc[u].v[h] * mul + add;
       }
-      const int dst_cta = bi <= 1 ? 0 : owner_of(bi, bj, nblk);
-      const uint32_t dst = map_to_cta(smem_addr(slots + blk * kSlot), dst_cta);
-      st_cluster_v4(dst + (uint32_t)((a * kLd + 4 * q4) * 4), sv);
+      st4(dst, acc[u]);
     }
   }
-  cluster_sync_all();
+  __syncthreads();
+  cluster_wait();
 
-  if (cta == 0) {
-    // =========================================================== pivot chain
-    // Phase A: warps 0, 1 factor the diagonal block, warps 2..9 invert it alongside, a thread of warp 10
-    // waits for the two blocks of the next step.  Phase B (warps 0..7): L(k+1, k).  Phase C (warps 0..7):
-    // the next diagonal block.  Warp 11 only sends: D_k^{-1} after phase A, L(k+1, k) after phase B; it
-    // follows a step counter in shared memory and never holds the others up.
-    constexpr int kChainWarps = 11;   // warps that take part in the phase barriers
-    if (warp < kChainWarps) {
-      for (int k = 0; k < nblk; ++k) {
-        float* dslot = slots + tri(k, k) * kSlot;
-        if (warp < 2) {
-          if (factor_diag_half(dslot, lcol, mcol, s_floor, &s_gave_up, warp, lane) && lane == 0) s_clamped = 1;
-        } else if (warp < 2 + kInvWarps) {
-          invert_diag_part(dslot, mcol, &s_gave_up, warp - 2, lane);
-        } else if (lane == 0 && k + 1 < nblk && k >= 1) {
-          bar_wait(&chain_bar[k + 1], &s_gave_up);   // blocks (k+1, k) and (k+1, k+1)
-        }
-        chain_sync();
-        if (tid == 0) { __threadfence_block(); s_chain_step = 2 * k + 1; }
-        if (k + 1 >= nblk) break;
-        // L(k+1, k) = A(k+1, k) D_k^{-T}, in place (a warp reads only the rows it writes)
-        float* sub = slots + tri(k + 1, k) * kSlot;
-        if (warp < 8) {
-          float acc[2][2];
-          tile_zero(acc);
-          tile_mac<2, 2>(acc, sub, dslot, tid >> 4, tid & 15);
-          group_sync(1);   // in place: everyone has read the block
-          tile_store<2, 2>(sub, acc, tid >> 4, tid & 15, 1.f, false);
-          fence_async_proxy();   // the block is sent on with a bulk copy
-        }
-        chain_sync();
-        if (tid == 0) { __threadfence_block(); s_chain_step = 2 * k + 2; }
-        if (warp < 8) {
-          // next diagonal block: A(k+1, k+1) -= L(k+1, k) L(k+1, k)^T
-          float acc2[2][2];
-          tile_zero(acc2);
-          tile_mac<2, 2>(acc2, sub, sub, tid >> 4, tid & 15);
-          tile_store<2, 2>(slots + tri(k + 1, k + 1) * kSlot, acc2, tid >> 4, tid & 15, -1.f, true);
-        } else {
-          for (int e = tid - 8 * 32; e < 2 * kB * kLcolLd; e += (kChainWarps - 8) * 32)
-            reinterpret_cast<uint32_t*>(lcol)[e] = kUnset;
-        }
-        chain_sync();
+  volatile int* gave_up = &s_gave_up;
+  const T floor_ = s_floor;
+  const int role = kRoleOf[warp];
+  const bool peer = lane < nblk && lane != me;
+  // Lane c copies something this CTA has finished to CTA c, if `to_me` says so.  Whoever wrote it arrived on a barrier
+  // this warp has waited for (or is this warp); the proxy fence makes those stores visible to the copy.
+  auto send = [&](const T* what, uint32_t bytes, uint64_t* bar, bool to_me) {
+    fence_async_proxy();
+    __syncwarp();
+    if (to_me) {
+      const uint32_t src = smem_addr(what);
+      bulk_to_peer(map_to_cta(src, lane), src, bytes, map_to_cta(smem_addr(bar), lane));
+    }
+  };
+  if (!active) {
+    // a CTA without a block row (the cluster size is a power of two)
+  } else if (role == R_PIVOT) {
+    const bool clamped = factor_diagonal<T>(own, panel(me), pan_bar[me], floor_, lane);
+    send(panel(me) + (kPan - 1) * kPanElems, kPanBytes, &pan_bar[me][kPan - 1], peer);
+    if (clamped && lane == 0 && p.dev_status) atomicOr(p.dev_status, LORACT_DEV_PIVOT_CLAMPED);
+  } else if (role < R_SOLVE) {
+    // ---- follow-up warps: lane = row, columns 8 w .. 8 w + 7
+    const int w = role - R_FOLLOW;
+    for (int k = -1; k + 1 < nblk; ++k) {
+      // step k: the block that step k + 1 works on takes L(own, k) or X(k, own) off, group by group
+      const int j = k + 1;
+      T* tgt = target(j);
+      const bool fresh = j > me && k == me;                 // the first update of an inverse block
+      if (j == 0 && me != 0) continue;                      // (the first block of a row needs no update)
+      if (k >= 0 && (j <= me ? k >= 1 : k > me)) bar_wait(&bulk_bar[j], gave_up);
+      V4<T> acc[2];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        acc[h] = {{(T)0, (T)0, (T)0, (T)0}};
+        if (!fresh) acc[h] = ld4(tgt + (2 * w + h) * kGrp + lane * 4);
       }
-      if (tid == 0 && s_clamped && p.dev_status) atomicOr(p.dev_status, LORACT_DEV_PIVOT_CLAMPED);
-    } else if (warp == kChainWarps) {
-      // the sender: lane c copies each finished block to CTA c
-      for (int step = 1; step <= 2 * nblk - 1; ++step) {
-        // step 2k + 1: D_k^{-1} is ready;  step 2k + 2: L(k+1, k) is ready
-        if (lane == 0) {
-          uint64_t t0 = 0;
-          for (uint32_t spin = 1; s_chain_step < step; ++spin) {
-            __nanosleep(20);
-            if ((spin & 255u) == 0u) {
-              if (*(volatile int*)&s_gave_up) break;
-              const uint64_t now = timer_ns();
-              if (t0 == 0) t0 = now;
-              else if (now - t0 > kClusterWaitNs) { s_gave_up = 1; break; }
-            }
-          }
-          __threadfence_block();
+      if (k >= 0) {
+        const T* A = solved(k);
+        const T* Bm = j == me ? A : slot(j, k);
+#pragma unroll 1
+        for (int q = 0; q < kPan; ++q) {
+          bar_wait(&sol_bar[k][q], gave_up);
+          if (j != me) bar_wait(&next_bar[k][q], gave_up);
+          take_off_group<T>(acc, A + q * kGrp, Bm + q * kGrp, w, lane);
         }
-        __syncwarp();
-        const int k = (step - 1) >> 1;
-        const bool is_dinv = (step & 1) != 0;
-        const float* blk = slots + (is_dinv ? tri(k, k) : tri(k + 1, k)) * kSlot;
-        if (lane >= 1 && lane < kCl) {
-          const uint32_t src = smem_addr(blk);
-          bulk_to_peer(map_to_cta(src, lane), src, kSlotTx,
-                       map_to_cta(smem_addr(is_dinv ? &dinv_bar[k] : &urgent_bar[k]), lane));
+      }
+      if (j != me) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) st4(tgt + (2 * w + h) * kGrp + lane * 4, acc[h]);
+        warp_arrive(&rdy_bar[j], lane);
+        continue;
+      }
+      // the diagonal block itself: groups 2 w and 2 w + 1 go to the pivot warp, each when every group but the one before
+      // it has been taken off
+      if (w == 0) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) { st4(own + h * kGrp + lane * 4, acc[h]); named_arrive(id_staged(h), 64); }
+      }
+      const T* pan = panel(me);
+#pragma unroll 1
+      for (int g = 0; g < 2 * w; ++g) {
+        named_sync(id_published(g), readers_of(g));
+        take_off_group<T>(acc, pan, pan, w, lane);
+        pan += kPanElems;
+        if (g + 2 >= 2 * w) {
+          const int h = g + 2 - 2 * w;
+          st4(own + (g + 2) * kGrp + lane * 4, h ? acc[1] : acc[0]);
+          named_arrive(id_staged(g + 2), 64);
         }
       }
     }
-  } else if (warp < 8) {
-    // =========================================================== workers, factorisation half
-    // Four pairs of warps; a pair does one 32 x 32 block product at a time (4 x 4 outputs per thread), the
-    // blocks of a phase are dealt out to the pairs in turn.  Warp h of a pair holds rows 16 h .. 16 h + 15.
-    const int pair = warp >> 1;
-    const int tp = tid & 63, tm = tp >> 3, tn = tp & 7;   // 4 x 4 outputs per thread on a pair of warps
-    const int t2m = tid >> 4, t2n = tid & 15;             // 2 x 2 outputs per thread on all eight warps
-    const int n_mine = s_n_mine;
+  } else if (role < R_BULK) {
+    // ---- solver warps: eight rows each
+    const int row = 8 * (role - R_SOLVE) + (lane & 7), cg = lane >> 3;
     for (int k = 0; k < nblk; ++k) {
-      if (tid == 0) {
-        bar_wait(&dinv_bar[k], &s_gave_up);
-        s_urgent = 1;   // the other half of the CTA stands back until the chain has what it waits for
+      T* blk = solved(k);
+      V4<T> acc[2];
+      if (k != me) {
+        if (k > 0) bar_wait(&rdy_bar[k], gave_up);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) acc[h] = ld4(blk + (cg + 4 * h) * kGrp + row * 4);
+      } else {
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) acc[h].v[j] = 4 * (cg + 4 * h) + j == row ? (T)1 : (T)0;
       }
-      group_sync(1);
-      const float* dk = slots + tri(k, k) * kSlot;
-      // L(i, k) = A(i, k) D_k^{-T} for the block of column k this CTA owns (CTA 0 does block k + 1): on the
-      // critical path, so all eight warps share the one product; in place
-      for (int q = 0; q < n_mine; ++q) {
-        const int bi = s_mine_i[q], bj = s_mine_j[q];
-        if (bj != k || bi < k + 2) continue;
-        float* blk = slots + tri(bi, k) * kSlot;
-        float acc[2][2];
-        tile_zero(acc);
-        tile_mac<2, 2>(acc, blk, dk, t2m, t2n);
-        group_sync(1);   // everyone has read the block
-        tile_store<2, 2>(blk, acc, t2m, t2n, 1.f, false);
-        fence_async_proxy();
-        send_rows(blk, warp * 4, 4, bi == k + 2 ? &urgent_bar[k] : &panel_bar[k], 1, kCl - 1, cta, lane);
+      solve_half<T, 0>(acc, blk, panel(k), pan_bar[k], sol_bar[k], k >= me, row, lane, gave_up);
+      solve_half<T, 1>(acc, blk, panel(k), pan_bar[k], sol_bar[k], k >= me, row, lane, gave_up);
+    }
+  } else if (role < R_SEND) {
+    // ---- bulk warps: the updates of step k to blocks beyond k + 1 (block j always by the same pair of warps), and the
+    // output
+    const int m = role - R_BULK;
+    const int col = me * kB + lane;
+    float wdiag = 0.f, est = 0.f;
+    if (p.gate_out && col < r) {
+      // for the estimate: the diagonal entry of this lane's column, as factored
+      const T* parts = (const T*)p.partials;
+      T d = (T)0;
+      for (int q = 0; q < p.n_partials; ++q)
+        d += __ldg(parts + (int64_t)q * p.partial_stride + (int64_t)col * p.in_ld + col);
+      wdiag = (float)(d + d * (T)p.shift_diag_rel + s_shift);
+    }
+    // zeros above the diagonal block
+    for (int row = m; row < me * kB; row += kBulkWarps) {
+      if (col >= r) continue;
+      const int64_t o = (int64_t)row * p.out_ld + col;
+      if (p.linv_f32) p.linv_f32[o] = 0.f;
+      if (p.linv_hi) p.linv_hi[o] = __float2bfloat16(0.f);
+      if (p.linv_lo) p.linv_lo[o] = __float2bfloat16(0.f);
+    }
+    for (int k = 0; k < nblk; ++k) {
+      const T* blk = solved(k);
+      bar_wait(&sol_bar[k][kPan - 1], gave_up);
+      const int j_end = k < me ? me + 1 : nblk;
+      for (int j = k + 2; j < j_end; ++j) {
+        if ((j & 3) != (m >> 1)) continue;
+        if (j != me) bar_wait(&off_bar[off_slot(j, k)], gave_up);
+        take_off_half<T>(target(j), blk, j == me ? blk : slot(j, k), k == me, m & 1, lane);
+        if (j == k + 2) warp_arrive(&bulk_bar[j], lane);
       }
-      // this CTA's own blocks of column k are in place: the second arrival on its own barriers
-      group_sync(1);
-      if (tid == 0 && k + 1 < nblk) {
-        bar_arrive_local(&panel_bar[k]);
-        if (k + 2 < nblk && owner_of(k + 2, k, nblk) == cta) bar_arrive_local(&urgent_bar[k]);
+      if (k < me) continue;
+      // rows 32 k + 4 m .. + 3 of the result: element (32 k + 4 m + u, col) = X[group m][lane][u]
+      const V4<T> v4 = ld4(blk + m * kGrp + lane * 4);
+      const int row = k * kB + 4 * m;
+#pragma unroll
+      for (int a = 0; a < 4; ++a) {
+        if (row + a >= r || col >= r) continue;
+        const float v = (float)v4.v[a];
+        est = fmaf(v * v, wdiag, est);
+        const int64_t o = (int64_t)(row + a) * p.out_ld + col;
+        if (p.linv_f32) p.linv_f32[o] = v;
+        if (p.linv_hi) {
+          const __nv_bfloat16 hi = __float2bfloat16(v);
+          p.linv_hi[o] = hi;
+          if (p.linv_lo) p.linv_lo[o] = __float2bfloat16(v - __bfloat162float(hi));
+        }
       }
-      if (k + 1 >= nblk) { if (tid == 0) s_urgent = 0; break; }
-      if (tid == 0) bar_wait(&urgent_bar[k], &s_gave_up);
-      group_sync(1);
-      // trailing update with column k.  A diagonal block (j, j) takes columns k <= j - 2 here (CTA 0
-      // applies column j - 1 itself), every other block (i, j) columns k <= j - 1.  First the two blocks
-      // CTA 0 needs next, each on all eight warps, sent on as soon as they are done ...
-      for (int q = 0; q < n_mine; ++q) {
-        const int bi = s_mine_i[q], bj = s_mine_j[q];
-        if (bi != k + 2 || (bj != k + 1 && bj != k + 2)) continue;
-        float acc[2][2];
-        tile_zero(acc);
-        tile_mac<2, 2>(acc, slots + tri(bi, k) * kSlot, slots + tri(bj, k) * kSlot, t2m, t2n);
-        float* blk = slots + tri(bi, bj) * kSlot;
-        tile_store<2, 2>(blk, acc, t2m, t2n, -1.f, true);
-        fence_async_proxy();
-        send_rows(blk, warp * 4, 4, &chain_bar[k + 2], 0, 0, -1, lane);
-      }
-      if (tid == 0) { s_urgent = 0; bar_wait(&panel_bar[k], &s_gave_up); }
-      group_sync(1);
-      // ... then the rest, one block per pair of warps at a time
-      int turn = 0;
-      for (int q = 0; q < n_mine; ++q) {
-        const int bi = s_mine_i[q], bj = s_mine_j[q];
-        if (bi < 2) continue;
-        const bool active = (bi == bj) ? (k <= bj - 2) : (k <= bj - 1);
-        if (!active) continue;
-        if ((bi == k + 2) && (bj == k + 1 || bj == k + 2)) continue;
-        if ((turn++ & 3) != pair) continue;
-        float acc[4][4];
-        tile_zero(acc);
-        tile_mac<4, 4>(acc, slots + tri(bi, k) * kSlot, slots + tri(bj, k) * kSlot, tm, tn);
-        tile_store<4, 4>(slots + tri(bi, bj) * kSlot, acc, tm, tn, -1.f, true);
-      }
+    }
+    if (p.gate_out) {
+      // this warp's share of the estimate, summed in a fixed order and handed to CTA 0
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) est += __shfl_xor_sync(0xffffffffu, est, o);
+      if (lane == 0)
+        asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(map_to_cta(smem_addr(&s_est[kBulkWarps * me + m]), 0)), "f"(est)
+                     : "memory");
     }
   } else {
-    // =========================================================== workers, inverse half (warps 8..15)
-    // Right-looking by block rows, in transposed storage Xt(i,j)[b][a] = X(i,j)[a][b]: at step k block row
-    // k of the inverse becomes final, X(k,j) = -D_k^{-1} T(k,j) (X(k,k) = D_k^{-1}), is written out, and is
-    // added into the sums of all later rows, T(i,j) += L(i,k) X(k,j).  Finishing a block is one product on
-    // all eight warps (2 x 2 outputs per thread); the products into the later rows are dealt out to four
-    // pairs of warps (4 x 4 outputs per thread).
-    const int gt = tid - kGroup;
-    const int pair = (warp - 8) >> 1;
-    const int tp = gt & 63, tm = tp >> 3, tn = tp & 7;
-    const int t2m = gt >> 4, t2n = gt & 15;
-    // block columns of the inverse this CTA computes: j0 = cta - 1, and 7 as well on the last worker
-    const int j0 = cta - 1;
-    const int n_cols = (j0 < nblk ? 1 : 0) + ((cta == kWorkers && kWorkers < nblk) ? 1 : 0);
-    // for the estimate: the diagonal entries (as factored) of the one or two columns this thread writes
-    float wdiag[2] = {0.f, 0.f};
-    float est_acc = 0.f;
-    if (p.gate_out) {
-      for (int cidx = 0; cidx < n_cols; ++cidx) {
-        const int col = (j0 + cidx) * kB + (gt & 31);
-        if (col < r) {
-          float dsum = 0.f;
-          for (int q = 0; q < p.n_partials; ++q)
-            dsum += __ldg(p.partials + (int64_t)q * p.partial_stride + (int64_t)col * p.in_ld + col);
-          wdiag[cidx] = dsum + dsum * p.shift_diag_rel + s_shift;
-        }
+    // ---- the sender
+    for (int k = 0; k + 1 < me; ++k) {
+      bar_wait(&sol_bar[k][kPan - 1], gave_up);
+      send(slot(me, k), kBlkBytes, &off_bar[off_slot(me, k)], peer && (lane <= k || lane > me));
+    }
+    if (me > 0) {
+#pragma unroll 1
+      for (int q = 0; q < kPan; ++q) {
+        bar_wait(&sol_bar[me - 1][q], gave_up);
+        send(slot(me, me - 1) + q * kGrp, kGrpBytes, &next_bar[me - 1][q], peer);
       }
     }
-    // zeros above the diagonal blocks
-    for (int cidx = 0; cidx < n_cols; ++cidx) {
-      const int j = j0 + cidx;
-      const int ncol = min(kB, r - j * kB);
-      for (int e = gt; e < j * kB * kB; e += kGroup) {
-        const int row = e >> 5, b = e & 31;
-        if (b >= ncol) continue;
-        const int64_t off = (int64_t)row * p.out_ld + j * kB + b;
-        if (p.linv_f32) p.linv_f32[off] = 0.f;
-        if (p.linv_hi) p.linv_hi[off] = __float2bfloat16(0.f);
-        if (p.linv_lo) p.linv_lo[off] = __float2bfloat16(0.f);
-      }
-    }
-    for (int k = 0; k < nblk; ++k) {
-      if (gt == 0) bar_wait(&dinv_bar[k], &s_gave_up);
-      group_sync(2);
-      const float* dk = slots + tri(k, k) * kSlot;
-      for (int cidx = 0; cidx < n_cols; ++cidx) {
-        const int j = j0 + cidx;
-        if (j > k) continue;
-        float* dst = xt + ((cidx == 0 ? 0 : (nblk - j0)) + (k - j)) * kSlot;
-        if (j == k) {
-          for (int e = gt; e < kB * kB; e += kGroup) {
-            const int b = e >> 5, a = e & 31;
-            dst[b * kLd + a] = dk[a * kLd + b];
-          }
-        } else {
-          // Xt(k,j)[b][a] = -sum_q Tt(k,j)[b][q] D_k^{-1}[a][q], in place
-          float acc[2][2];
-          tile_zero(acc);
-          tile_mac<2, 2>(acc, dst, dk, t2m, t2n);
-          group_sync(2);   // everyone has read the sums
-          tile_store<2, 2>(dst, acc, t2m, t2n, -1.f, false);
-        }
-      }
-      group_sync(2);
-      // block row k of the result: Linv[k*32 + a][j*32 + b] = Xt(k,j)[b][a]
-      for (int cidx = 0; cidx < n_cols; ++cidx) {
-        const int j = j0 + cidx;
-        if (j > k) continue;
-        const float* src = xt + ((cidx == 0 ? 0 : (nblk - j0)) + (k - j)) * kSlot;
-        const int ncol = min(kB, r - j * kB);
-        for (int e = gt; e < kB * kB; e += kGroup) {
-          const int a = e >> 5, b = e & 31;
-          const int row = k * kB + a;
-          if (row >= r || b >= ncol) continue;
-          const float v = src[b * kLd + a];
-          est_acc = fmaf(v * v, wdiag[cidx], est_acc);
-          const int64_t off = (int64_t)row * p.out_ld + j * kB + b;
-          if (p.linv_f32) p.linv_f32[off] = v;
-          if (p.linv_hi) {
-            const __nv_bfloat16 hi = __float2bfloat16(v);
-            p.linv_hi[off] = hi;
-            if (p.linv_lo) p.linv_lo[off] = __float2bfloat16(v - __bfloat162float(hi));
-          }
-        }
-      }
-      if (k + 1 >= nblk) break;
-      if (gt == 0) { bar_wait(&urgent_bar[k], &s_gave_up); bar_wait(&panel_bar[k], &s_gave_up); }
-      group_sync(2);
-      // Tt(i,j)[b][a] (+)= sum_q Xt(k,j)[b][q] L(i,k)[a][q] for the rows below
-      int turn = 0;
-      for (int cidx = 0; cidx < n_cols; ++cidx) {
-        const int j = j0 + cidx;
-        if (j > k) continue;
-        float* xcol = xt + (cidx == 0 ? 0 : (nblk - j0)) * kSlot;   // block (i, j) at xcol + (i - j) slots
-        const float* xk = xcol + (k - j) * kSlot;
-        for (int i = k + 1; i < nblk; ++i) {
-          if ((turn++ & 3) != pair) continue;
-          for (int spin = 0; s_urgent && spin < 256; ++spin) __nanosleep(64);   // a hint, not a lock
-          float acc[4][4];
-          tile_zero(acc);
-          tile_mac<4, 4>(acc, xk, slots + tri(i, k) * kSlot, tm, tn);
-          tile_store<4, 4>(xcol + (i - j) * kSlot, acc, tm, tn, 1.f, j != k);
-        }
-      }
-    }
-    if (p.gate_out) {
-      // this CTA's share of the estimate, summed in a fixed order and handed to CTA 0
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) est_acc += __shfl_xor_sync(0xffffffffu, est_acc, o);
-      if (lane == 0) s_est[warp - 8] = est_acc;
-      group_sync(2);
-      if (gt == 0) {
-        float t = 0.f;
-        for (int q = 0; q < 8; ++q) t += s_est[q];
-        asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(map_to_cta(smem_addr(&s_est[cta]), 0)), "f"(t) : "memory");
-      }
+#pragma unroll 1
+    for (int q = 0; q + 1 < kPan; ++q) {   // (the pivot warp sends the last one itself)
+      bar_wait(&pan_bar[me][q], gave_up);
+      send(panel(me) + q * kPanElems, kPanBytes, &pan_bar[me][q], peer);
     }
   }
   __syncthreads();
   if (tid == 0 && s_gave_up && p.dev_status) atomicOr(p.dev_status, LORACT_DEV_WAIT_EXPIRED);
-  // no CTA leaves while another may still write into its shared memory
-  cluster_sync_all();
-  if (p.gate_out && cta == 0 && tid == 0) {
-    // after the cluster barrier: every worker's share has arrived, every status bit of this call is set
+  // no CTA leaves while another may still write into its shared memory or read its own through a copy
+  cluster_arrive();
+  cluster_wait();
+  if (p.gate_out && me == 0 && tid == 0) {
+    // after the cluster barrier: every share has arrived, every status bit of this call is set
     float est = 0.f;
-    for (int c = 1; c < kCl; ++c) est += s_est[c];
+    for (int c = 0; c < kBulkWarps * nblk; ++c) est += s_est[c];
     const uint32_t st = p.dev_status ? atomicOr(p.dev_status, 0u) : 0u;
     const bool again = !(est <= p.gate_threshold) || st != 0u;
     p.gate_out[0] = again ? 1u : 0u;
@@ -872,11 +706,46 @@ __global__ void __cluster_dims__(2, 1, 1) cluster_wait_probe_kernel(uint32_t* de
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     bar_expect(&bar, 16);   // sixteen bytes that never arrive
   }
-  cluster_sync_all();
+  __syncthreads();
+  cluster_arrive();
+  cluster_wait();
   if (rank == 1 && threadIdx.x == 0) bar_wait(&bar, &gave_up, limit_ns);
   __syncthreads();
   if (threadIdx.x == 0 && gave_up && dev_status) atomicOr(dev_status, LORACT_DEV_WAIT_EXPIRED);
-  cluster_sync_all();
+  cluster_arrive();
+  cluster_wait();
+}
+
+template <typename T>
+cudaError_t launch_cluster(const SCParams& p, cudaStream_t stream) {
+  const int nblk = (p.r + kB - 1) / kB;
+  int ctas = 1;                           // cluster sizes are powers of two
+  while (ctas < nblk) ctas *= 2;
+  static std::atomic<bool> configured[64];
+  int dev = 0;
+  LORACT_CUDA_TRY(cudaGetDevice(&dev));
+  if (dev < 0 || dev >= 64 || !configured[dev].load(std::memory_order_acquire)) {
+    LORACT_CUDA_TRY(cudaFuncSetAttribute(small_block_cluster_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)(smem_elems<T>(Cfg<T>::kMaxR / kB) * sizeof(T))));
+    if (dev >= 0 && dev < 64) configured[dev].store(true, std::memory_order_release);
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(ctas, 1, 1);
+  cfg.blockDim = dim3(kCThreads, 1, 1);
+  cfg.dynamicSmemBytes = smem_elems<T>(nblk) * sizeof(T);
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = ctas;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  LORACT_CUDA_TRY(cudaLaunchKernelEx(&cfg, small_block_cluster_kernel<T>, p));
+  count_launch(__func__, stream);
+  return cudaGetLastError();
 }
 
 }  // namespace
@@ -888,14 +757,15 @@ cudaError_t small_block_cluster_wait_probe_launch(uint32_t* dev_status, uint64_t
 }
 
 bool small_block_cluster_supported(const SmallBlockArgs& a) {
-  return !a.use_f64 && a.partial_type == ELEM_F32 && a.r <= kMaxBlk * kB && a.r % 4 == 0 &&
-         a.linv_full == nullptr && (((uintptr_t)a.partials & 15) == 0) && (a.partial_stride % 4 == 0) && (a.in_ld % 4 == 0);
+  if (a.linv_full != nullptr || ((uintptr_t)a.partials & 15) || a.partial_stride % 4 || a.in_ld % 4 || a.r % 4) return false;
+  if (a.use_f64) return a.partial_type == ELEM_F64 && a.r <= Cfg<double>::kMaxR && a.scale_diag == nullptr;
+  return a.partial_type == ELEM_F32 && a.r <= Cfg<float>::kMaxR;
 }
 
 cudaError_t small_block_cluster_launch(const SmallBlockArgs& a, cudaStream_t stream) {
   SCParams p;
   p.r = a.r;
-  p.partials = (const float*)a.partials;
+  p.partials = a.partials;
   p.in_ld = a.in_ld ? a.in_ld : a.r;
   p.out_ld = a.out_ld ? a.out_ld : a.r;
   p.n_partials = a.n_partials;
@@ -912,32 +782,7 @@ cudaError_t small_block_cluster_launch(const SmallBlockArgs& a, cudaStream_t str
   p.scale_diag = a.scale_diag;
   p.scale_n = a.scale_n;
   p.scale_ld = a.scale_ld;
-  const size_t smem = (size_t)(kMaxTri + kXSlots) * kSlot * sizeof(float) + (size_t)(2 * kB * kLcolLd) * sizeof(float);
-  static std::atomic<bool> configured[64];
-  int dev = 0;
-  LORACT_CUDA_TRY(cudaGetDevice(&dev));
-  if (dev < 0 || dev >= 64 || !configured[dev].load(std::memory_order_acquire)) {
-    LORACT_CUDA_TRY(cudaFuncSetAttribute(small_block_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem));
-    if (dev >= 0 && dev < 64) configured[dev].store(true, std::memory_order_release);
-  }
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(kCl, 1, 1);
-  cfg.blockDim = dim3(kCThreads, 1, 1);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[2];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = kCl;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[1].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 2;
-  LORACT_CUDA_TRY(cudaLaunchKernelEx(&cfg, small_block_cluster_kernel, p));
-  count_launch();
-  return cudaGetLastError();
+  return a.use_f64 ? launch_cluster<double>(p, stream) : launch_cluster<float>(p, stream);
 }
 
 }  // namespace loract

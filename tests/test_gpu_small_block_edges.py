@@ -1,0 +1,67 @@
+"""GPU tests of the cluster factorisation (Cholesky factor and inverse of an r x r Gram matrix) at the edges of its tiles:
+widths just around a multiple of the 32-wide block and of the four-column group, both arithmetic types, the largest
+width of each, a pivot that has to be clamped in every group of a block.  Reference: numpy in float64."""
+import numpy as np
+import pytest
+import torch
+
+import __graft_entry__ as entry
+from paper_2509_23472_b200 import binding as B
+from tests.test_gpu_small_block import spd
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def dev():
+    entry.build()
+    B.lib()
+    return torch.device("cuda:0")
+
+
+@pytest.mark.parametrize("f64,r,n_partials", [(False, 24, 1), (False, 40, 2), (False, 104, 1), (False, 136, 3),
+                                              (False, 232, 1), (False, 248, 2), (True, 16, 1), (True, 24, 3), (True, 40, 1),
+                                              (True, 64, 2), (True, 96, 8), (True, 136, 1), (True, 160, 4), (True, 184, 1),
+                                              (True, 192, 2), (True, 200, 1)])
+def test_inverse_factor_at_tile_edges(dev, f64, r, n_partials):
+    cond = 1e8 if f64 else 1e3
+    W = spd(r, cond, seed=17 * r + n_partials)
+    P = torch.tensor(np.repeat(W[None] / n_partials, n_partials, axis=0), device=dev,
+                     dtype=torch.float64 if f64 else torch.float32)
+    Ws = P.double().sum(0).cpu().numpy()
+    shift = float(np.float32(1e-10 if f64 else 1e-6))
+    Ws = Ws + shift * np.trace(Ws) / r * np.eye(r)
+    status = torch.zeros(1, dtype=torch.int32, device=dev)
+    for _ in range(2):
+        L32, Lh, Ll = B.debug_small_block(P, use_f64=f64, shift_rel=shift, status=status)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0
+    X = L32.double().cpu().numpy()
+    assert np.abs(np.triu(X, 1)).max() == 0.0
+    Xref = np.linalg.inv(np.linalg.cholesky(Ws))
+    # forward error of the arithmetic, and the rounding of the fp32 result
+    eps = 2.0 ** -53 if f64 else 2.0 ** -24
+    assert np.linalg.norm(X - Xref) <= (50 * r * eps * np.linalg.cond(Ws) + 2.0 ** -24) * np.linalg.norm(Xref)
+    pair = Lh.double().cpu().numpy() + Ll.double().cpu().numpy()
+    assert np.abs(pair - X).max() <= 2.0 ** -15 * np.abs(X).max()
+
+
+@pytest.mark.parametrize("f64", [False, True])
+@pytest.mark.parametrize("at", [0, 3, 4, 17, 31, 32, 50, 95])
+def test_clamped_pivot_drops_its_column_only(dev, f64, at):
+    r = 96
+    W = spd(r, 1e2, seed=at)
+    W[at, :] = 0.0
+    W[:, at] = 0.0                                     # a pivot of exactly zero, coupled to nothing
+    P = torch.tensor(W[None], dtype=torch.float64 if f64 else torch.float32, device=dev)
+    status = torch.zeros(1, dtype=torch.int32, device=dev)
+    L32, _, _ = B.debug_small_block(P, use_f64=f64, shift_rel=0.0, status=status)
+    torch.cuda.synchronize()
+    assert int(status.item()) == B.DEV_PIVOT_CLAMPED
+    X = L32.double().cpu().numpy()
+    assert np.isfinite(X).all()
+    keep = np.delete(np.arange(r), at)
+    Xref = np.linalg.inv(np.linalg.cholesky(W[np.ix_(keep, keep)]))
+    tol = 50 * r * 2.0 ** -24 * 1e2                    # fp32 arithmetic (fp64: the rounding of the result is below it)
+    assert np.linalg.norm(X[np.ix_(keep, keep)] - Xref) <= tol * np.linalg.norm(Xref)
+    assert np.abs(X[at, keep]).max() == 0.0 and np.abs(X[keep, at]).max() == 0.0
