@@ -35,7 +35,8 @@ constexpr uint64_t kWaitLimitNs = 2000000000ull;  // 2 s
 struct alignas(64) TmapPack {
   CUtensorMap a[3];
   CUtensorMap b[3];
-  CUtensorMap c[2];   // outputs (C0, C1) for the staged epilogue: boxes of 128 bytes x 32 rows
+  CUtensorMap c[2];   // outputs (C0, C1) for the staged epilogue: boxes of 128 bytes x 32 rows.  Fused epilogue: the
+                      // output and the matrix it is combined with, both in boxes of 64 bytes x 32 rows
 };
 
 struct TcParams {
@@ -52,18 +53,15 @@ struct TcParams {
   uint32_t b_bytes;   // bytes of one B stage
   uint32_t tmem_cols;
   int accumulate;     // OUT_F32, one split: C += result
-  const void* ep_E;   // OUT_RMS_BWD epilogue operands
-  int64_t ep_ld;
-  const float* ep_row_a;
+  const float* ep_row_a;   // OUT_RMS_BWD
   const float* ep_row_b;
   const void* ep_col;
-  int ep_kind;        // OUT_ACT_BWD: 0 SiLU, 1 GELU
   uint32_t* dev_status;
   int tma_store;      // 1: the epilogue stages 32-row boxes in shared memory and writes them with TMA stores
   int st_m_tiles;     // streaming kernel: 256-row tiles along M
   int st_units;       // streaming kernel: tiles in all (column tile major, then M)
   int st_stages;      // streaming kernel: stages of the A ring (<= kStreamStages)
-  int store_bufs;     // staging boxes per epilogue warp (1 or 2)
+  int store_bufs;     // staging boxes per epilogue warp (1 or 2; fused epilogue 3 or 4)
   int halve_at_term;  // the accumulator is multiplied by 1/2 before the first product of this term (0: never)
   int a_keep_from_kb; // two-CTA kernel: K block from which the loads of A carry an evict-last hint (kb_total: none)
   // one-tile kernels: when set and the word it points to is zero, the kernel loads, multiplies and stores nothing
@@ -192,9 +190,10 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
 
 // f'(a) of the element-wise consumers (OUT_ACT_BWD).  SiLU: s (1 + a (1 - s)), s the logistic function;
 // GELU (exact form): Phi(a) + a phi(a).  The result is multiplied by the upstream gradient and rounded to bf16.
-__device__ __forceinline__ float act_derivative(float a, int kind) {
-  if (kind == 0) {
-    const float s = 1.f / (1.f + __expf(-a));
+template <int kKind>
+__device__ __forceinline__ float act_derivative(float a) {
+  if (kKind == 0) {
+    const float s = __fdividef(1.f, 1.f + __expf(-a));   // 2 ulp; 0 where exp(-a) overflows
     return s * (1.f + a * (1.f - s));
   }
   return 0.5f * (1.f + erff(a * 0.70710678118f)) + a * 0.39894228040f * __expf(-0.5f * a * a);
@@ -263,7 +262,6 @@ __device__ __forceinline__ void tc_store_tile_staged(const TcParams& p, const Tm
                                                      int quad, int half_id, int lane, int m0, int n0,
                                                      int split, StoreStage& st, bool lo_on = true) {
   const int row0 = m0 + quad * 32;
-  const int m = row0 + lane;
   const uint32_t taddr = tmem_base + ((uint32_t)(quad * 32) << 16);
   const int y = split * p.M + row0;
   if (p.out == OUT_F32) {
@@ -281,11 +279,6 @@ __device__ __forceinline__ void tc_store_tile_staged(const TcParams& p, const Tm
     return;
   }
   const bool split_out = p.out == OUT_SPLIT && lo_on;   // lo_on false: only the leading part is wanted
-  const bool rms = p.out == OUT_RMS_BWD;
-  const bool act = p.out == OUT_ACT_BWD;
-  const bool live = m < p.M;                                 // rows past M are clipped by the store
-  float ra = 0.f, rb = 0.f;
-  if (rms && live) { ra = p.ep_row_a[m]; rb = p.ep_row_b[m]; }
   for (int c0 = 64 * half_id; c0 < p.bn && n0 + c0 < p.N; c0 += 128) {
     if (split_out) stage_acquire<2>(st, lane); else stage_acquire<1>(st, lane);
     unsigned char* box_hi = stage_box(st, 0);
@@ -296,67 +289,7 @@ __device__ __forceinline__ void tc_store_tile_staged(const TcParams& p, const Tm
 #pragma unroll
     for (int half = 0; half < 2; ++half) {
       const uint32_t* v = v64 + 32 * half;
-      const int n = n0 + c0 + 32 * half;
-      if (rms) {
-        const bool cols_ok = n + 32 <= p.N;                  // a partial group is clipped anyway; read nothing past N
-        const __nv_bfloat16* e = (const __nv_bfloat16*)p.ep_E + (int64_t)m * p.ep_ld + n;
-        const __nv_bfloat16* col = (const __nv_bfloat16*)p.ep_col + n;
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          uint32_t ow[4] = {0u, 0u, 0u, 0u};
-          if (live && cols_ok) {
-            const uint4 ev = reinterpret_cast<const uint4*>(e)[q];
-            const uint4 cv = __ldg(reinterpret_cast<const uint4*>(col) + q);
-            const uint32_t ew[4] = {ev.x, ev.y, ev.z, ev.w}, cw[4] = {cv.x, cv.y, cv.z, cv.w};
-#pragma unroll
-            for (int h = 0; h < 4; ++h) {
-              const float e0 = __uint_as_float(ew[h] << 16), e1 = __uint_as_float(ew[h] & 0xffff0000u);
-              const float c0f = __uint_as_float(cw[h] << 16), c1f = __uint_as_float(cw[h] & 0xffff0000u);
-              const float a0 = __uint_as_float(v[8 * q + 2 * h]), a1 = __uint_as_float(v[8 * q + 2 * h + 1]);
-              // the quotient is rounded to bf16 below: the fast division (2 ulp in fp32) is exact enough
-              ow[h] = pack_bf16x2(ra * c0f * e0 - __fdividef(rb * a0, c0f), ra * c1f * e1 - __fdividef(rb * a1, c1f));
-            }
-          } else if (live) {
-            for (int h = 0; h < 8; ++h) {
-              const int nn = n + 8 * q + h;
-              if (nn < p.N) {
-                const float c = __bfloat162float(col[8 * q + h]);
-                const float r = ra * c * __bfloat162float(e[8 * q + h]) - rb * __uint_as_float(v[8 * q + h]) / c;
-                const uint32_t bits = (uint32_t)__bfloat16_as_ushort(__float2bfloat16(r));
-                ow[h >> 1] |= (h & 1) ? (bits << 16) : bits;
-              }
-            }
-          }
-          stage_write16(box_hi, lane, 4 * half + q, make_uint4(ow[0], ow[1], ow[2], ow[3]));
-        }
-      } else if (act) {
-        const bool cols_ok = n + 32 <= p.N;
-        const __nv_bfloat16* e = (const __nv_bfloat16*)p.ep_E + (int64_t)m * p.ep_ld + n;
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          uint32_t ow[4] = {0u, 0u, 0u, 0u};
-          if (live && cols_ok) {
-            const uint4 ev = reinterpret_cast<const uint4*>(e)[q];
-            const uint32_t ew[4] = {ev.x, ev.y, ev.z, ev.w};
-#pragma unroll
-            for (int h = 0; h < 4; ++h) {
-              const float e0 = __uint_as_float(ew[h] << 16), e1 = __uint_as_float(ew[h] & 0xffff0000u);
-              const float a0 = __uint_as_float(v[8 * q + 2 * h]), a1 = __uint_as_float(v[8 * q + 2 * h + 1]);
-              ow[h] = pack_bf16x2(e0 * act_derivative(a0, p.ep_kind), e1 * act_derivative(a1, p.ep_kind));
-            }
-          } else if (live) {
-            for (int h = 0; h < 8; ++h) {
-              const int nn = n + 8 * q + h;
-              if (nn < p.N) {
-                const float r = __bfloat162float(e[8 * q + h]) * act_derivative(__uint_as_float(v[8 * q + h]), p.ep_kind);
-                const uint32_t bits = (uint32_t)__bfloat16_as_ushort(__float2bfloat16(r));
-                ow[h >> 1] |= (h & 1) ? (bits << 16) : bits;
-              }
-            }
-          }
-          stage_write16(box_hi, lane, 4 * half + q, make_uint4(ow[0], ow[1], ow[2], ow[3]));
-        }
-      } else if (!split_out) {
+      if (!split_out) {
         // one conversion instruction per pair of columns: this loop runs on a single warp per scheduler, so
         // its length in instructions is its duration
 #pragma unroll
@@ -422,42 +355,6 @@ __device__ __forceinline__ void tc_store_tile(const TcParams& p, const TmapPack&
         } else {
           for (int q = 0; q < valid; ++q) dst[q] = __uint_as_float(v[q]);
         }
-      } else if (p.out == OUT_RMS_BWD) {
-        // grad_X = rstd * (grad_A * gamma - (reconstructed A / gamma) * inner): the tile of the reconstructed
-        // activation exists only in tensor memory and in these registers
-        __nv_bfloat16* dst = (__nv_bfloat16*)p.C0 + (int64_t)m * p.ldc + n;
-        const __nv_bfloat16* e = (const __nv_bfloat16*)p.ep_E + (int64_t)m * p.ep_ld + n;
-        const __nv_bfloat16* col = (const __nv_bfloat16*)p.ep_col + n;
-        const float ra = p.ep_row_a[m], rb = p.ep_row_b[m];
-        if (valid == 32 && ((((uintptr_t)dst) & 15) == 0) && ((((uintptr_t)e) & 15) == 0) &&
-            ((((uintptr_t)col) & 15) == 0)) {
-#pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            const uint4 ev = reinterpret_cast<const uint4*>(e)[q];
-            const uint4 cv = __ldg(reinterpret_cast<const uint4*>(col) + q);
-            const uint32_t ew[4] = {ev.x, ev.y, ev.z, ev.w}, cw[4] = {cv.x, cv.y, cv.z, cv.w};
-            uint32_t ow[4];
-#pragma unroll
-            for (int h = 0; h < 4; ++h) {
-              const float e0 = __uint_as_float(ew[h] << 16), e1 = __uint_as_float(ew[h] & 0xffff0000u);
-              const float c0f = __uint_as_float(cw[h] << 16), c1f = __uint_as_float(cw[h] & 0xffff0000u);
-              const float a0 = __uint_as_float(v[8 * q + 2 * h]), a1 = __uint_as_float(v[8 * q + 2 * h + 1]);
-              ow[h] = pack_bf16x2(ra * c0f * e0 - rb * a0 / c0f, ra * c1f * e1 - rb * a1 / c1f);
-            }
-            reinterpret_cast<uint4*>(dst)[q] = make_uint4(ow[0], ow[1], ow[2], ow[3]);
-          }
-        } else {
-          for (int q = 0; q < valid; ++q) {
-            const float c = __bfloat162float(col[q]);
-            dst[q] = __float2bfloat16(ra * c * __bfloat162float(e[q]) - rb * __uint_as_float(v[q]) / c);
-          }
-        }
-      } else if (p.out == OUT_ACT_BWD) {
-        // grad_X = grad_Z * f'(reconstructed A): the tile of the reconstructed activation exists only here
-        __nv_bfloat16* dst = (__nv_bfloat16*)p.C0 + (int64_t)m * p.ldc + n;
-        const __nv_bfloat16* e = (const __nv_bfloat16*)p.ep_E + (int64_t)m * p.ep_ld + n;
-        for (int q = 0; q < valid; ++q)
-          dst[q] = __float2bfloat16(__bfloat162float(e[q]) * act_derivative(__uint_as_float(v[q]), p.ep_kind));
       } else {
         __nv_bfloat16* dst_hi = (__nv_bfloat16*)p.C0 + (int64_t)m * p.ldc + n;
         __nv_bfloat16* dst_lo = (p.out == OUT_SPLIT && lo_on) ? (__nv_bfloat16*)p.C1 + (int64_t)m * p.ldc + n : nullptr;
@@ -900,6 +797,146 @@ __device__ __forceinline__ bool mbar_wait_cluster_bounded(uint64_t* bar, uint32_
   }
 }
 
+// ---- fused epilogue: the finished tile is combined with another matrix E of the output's shape (read once) and only the
+// result is written.  EP_RMS: row_a col E - row_b / col acc (OUT_RMS_BWD); EP_SILU, EP_GELU: E f'(acc) (OUT_ACT_BWD).
+// A thread owns one accumulator row, so loading E from global memory here would touch 32 lines per instruction with
+// nothing in flight behind it.  Instead E comes in boxes of 32 rows x 32 columns by TMA, requested store_bufs - 1 boxes
+// ahead by each epilogue warp for itself; the result overwrites E in the box and leaves by TMA from there.
+// Measured: SiLU backward of 16384 x 11008 at K = 512: 686 us with direct loads (1.1 TB/s), 296 us with the boxes (2.5 TB/s).
+enum EpKind : int { EP_NONE = 0, EP_RMS = 1, EP_SILU = 2, EP_GELU = 3 };
+constexpr int kFuseMaxBufs = 4;
+constexpr uint32_t kFuseBoxBytes = 2048;                   // 32 rows x 64 bytes
+
+// Boxes of 32 columns that one epilogue warp goes through, in order: unit after unit, every other box of its row group.
+struct FuseCursor {
+  int u, c0;
+  __device__ __forceinline__ void advance(const TcParams& p, int half_id) {
+    c0 += 64;
+    if (c0 >= p.bn) { c0 = 32 * half_id; ++u; }
+  }
+};
+
+template <int kEp>
+__device__ __forceinline__ float fuse_value(float acc, float e, float ra, float rb, float col, float inv_col) {
+  if (kEp == EP_RMS) return ra * col * e - rb * acc * inv_col;
+  if (kEp == EP_SILU) return e * act_derivative<0>(acc);
+  return e * act_derivative<1>(acc);
+}
+
+template <int kEp>
+__device__ __forceinline__ void fused_epilogue(const TcParams& p, const TmapPack& maps, uint32_t tmem_base, int warp,
+                                               int lane, int cta_rank, int u_begin, int u_end, unsigned char* boxes,
+                                               uint64_t* e_full, float* col_inv, uint64_t* acc_full, uint64_t* acc_empty,
+                                               uint64_t* epi_done, volatile int* abort_flag) {
+  const int quad = warp & 3, half_id = (warp - 2) >> 2;
+  const int bufs = p.store_bufs;
+  const __nv_bfloat16* gamma = (const __nv_bfloat16*)p.ep_col;
+  auto row_of = [&](int u) { return ((u % p.st_m_tiles) * 2 + cta_rank) * kBM + quad * 32; };
+  auto col_of = [&](const FuseCursor& k) { return (k.u / p.st_m_tiles) * p.bn + k.c0; };
+  // boxes outside the output are neither loaded nor stored
+  auto live = [&](const FuseCursor& k) { return row_of(k.u) < p.M && col_of(k) < p.N; };
+  FuseCursor ld{u_begin, 32 * half_id};
+  uint32_t n_ld = 0, n_use = 0;              // live boxes requested / used so far
+  uint32_t ld_slot = 0, use_slot = 0, use_phase = 0;
+  auto request = [&]() {                      // the next live box, if any
+    while (ld.u < u_end && !live(ld)) ld.advance(p, half_id);
+    if (ld.u >= u_end) return;
+    if (lane == 0) {
+      mbar_arrive_expect_tx(&e_full[ld_slot], kFuseBoxBytes);
+      tma_load_2d(boxes + ld_slot * kFuseBoxBytes, &maps.c[1], &e_full[ld_slot], col_of(ld), row_of(ld.u));
+    }
+    ++n_ld;
+    if (++ld_slot == (uint32_t)bufs) ld_slot = 0;
+    ld.advance(p, half_id);
+  };
+  for (int b = 0; b + 1 < bufs; ++b) request();
+  int cur_nt = -1;
+  bool ok = true;
+  for (int u = u_begin, ui = 0; u < u_end; ++u, ++ui) {
+    const int j = ui & 1;
+    const int nt = u / p.st_m_tiles;
+    const int row0 = row_of(u), m = row0 + lane;
+    if (kEp == EP_RMS && nt != cur_nt) {
+      // 1 / gamma of this column tile, for all eight warps (which all come through here, even once a wait has expired)
+      asm volatile("bar.sync 1, 256;" ::: "memory");
+      for (int c = (warp - 2) * 32 + lane; c < p.bn; c += 256) {
+        const int n = nt * p.bn + c;
+        col_inv[c] = n < p.N ? 1.f / __bfloat162float(gamma[n]) : 0.f;
+      }
+      asm volatile("bar.sync 1, 256;" ::: "memory");
+      cur_nt = nt;
+    }
+    if (!ok) continue;
+    float ra = 0.f, rb = 0.f;
+    if (kEp == EP_RMS && m < p.M) { ra = p.ep_row_a[m]; rb = p.ep_row_b[m]; }
+    ok = mbar_wait_bounded(&acc_full[j], (uint32_t)((ui >> 1) & 1), abort_flag);
+    ok = __all_sync(0xffffffffu, ok);
+    if (!ok) continue;
+    tc_fence_after();
+    const uint32_t taddr = tmem_base + (uint32_t)(j * p.bn) + ((uint32_t)(quad * 32) << 16);
+    for (FuseCursor k{u, 32 * half_id}; k.u == u && ok; k.advance(p, half_id)) {
+      if (!live(k)) continue;
+      uint32_t v[32];
+      tc_ld32(taddr + (uint32_t)k.c0, v);
+      unsigned char* box = boxes + use_slot * kFuseBoxBytes;
+      ok = mbar_wait_bounded(&e_full[use_slot], use_phase, abort_flag);
+      ok = __all_sync(0xffffffffu, ok);
+      tc_wait_ld();
+      if (!ok) break;
+      const int n = col_of(k);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        // 64-byte swizzle: chunk q of row i is at chunk q ^ ((i >> 1) & 3)
+        uint4* at = reinterpret_cast<uint4*>(box + lane * 64 + ((q ^ ((lane >> 1) & 3)) << 4));
+        const uint4 ev = *at;
+        const uint32_t ew[4] = {ev.x, ev.y, ev.z, ev.w};
+        uint4 gv = make_uint4(0u, 0u, 0u, 0u);             // N is a multiple of 8: a chunk is inside or outside
+        if (kEp == EP_RMS && n + 8 * q < p.N) gv = __ldg(reinterpret_cast<const uint4*>(gamma + n) + q);
+        const uint32_t gw[4] = {gv.x, gv.y, gv.z, gv.w};
+        uint32_t ow[4];
+#pragma unroll
+        for (int h = 0; h < 4; ++h) {
+          float2 ci = make_float2(0.f, 0.f);
+          if (kEp == EP_RMS) ci = *reinterpret_cast<const float2*>(col_inv + k.c0 + 8 * q + 2 * h);
+          ow[h] = pack_bf16x2(fuse_value<kEp>(__uint_as_float(v[8 * q + 2 * h]), __uint_as_float(ew[h] << 16), ra, rb,
+                                              __uint_as_float(gw[h] << 16), ci.x),
+                              fuse_value<kEp>(__uint_as_float(v[8 * q + 2 * h + 1]), __uint_as_float(ew[h] & 0xffff0000u),
+                                              ra, rb, __uint_as_float(gw[h] & 0xffff0000u), ci.y));
+        }
+        *at = make_uint4(ow[0], ow[1], ow[2], ow[3]);
+      }
+      stage_send(&maps.c[0], box, lane, n, row0);
+      ++n_use;
+      if (++use_slot == (uint32_t)bufs) { use_slot = 0; use_phase ^= 1u; }
+      // the next request goes into the box that was sent before this one
+      if (lane == 0) bulk_wait_read<1>();
+      request();
+    }
+    if (!ok) continue;
+    tc_fence_before();
+    __syncwarp();
+    if (lane == 0) {
+      mbar_arrive_local(&epi_done[j]);
+      if (warp == 2) {
+        // one signal per CTA and tile: the first epilogue warp collects the eight and tells the leader
+        if (mbar_wait_bounded(&epi_done[j], (uint32_t)((ui >> 1) & 1), abort_flag)) {
+          if (cta_rank == 0) mbar_arrive_local(&acc_empty[j]);
+          else mbar_arrive_cluster(map_to_rank(smem_u32(&acc_empty[j]), 0u));
+        }
+      }
+    }
+    __syncwarp();
+  }
+  // every box that was requested has landed before the shared memory goes away, and every store is complete
+  for (; n_use < n_ld; ++n_use) {
+    (void)mbar_wait_bounded(&e_full[use_slot], use_phase, abort_flag);
+    if (++use_slot == (uint32_t)bufs) { use_slot = 0; use_phase ^= 1u; }
+  }
+  if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+  __syncwarp();
+}
+
+template <int kEp>
 __global__ void __launch_bounds__(kThreads, 1)
 gemm_tc_stream_kernel(const __grid_constant__ TmapPack maps, const TcParams p) {
   extern __shared__ __align__(1024) unsigned char smem[];
@@ -909,6 +946,8 @@ gemm_tc_stream_kernel(const __grid_constant__ TmapPack maps, const TcParams p) {
   __shared__ __align__(8) uint64_t acc_full[2];
   __shared__ __align__(8) uint64_t acc_empty[2];
   __shared__ __align__(8) uint64_t epi_done[2];
+  __shared__ __align__(8) uint64_t e_full[kEp ? kEpiWarps : 1][kFuseMaxBufs];
+  __shared__ __align__(16) float col_inv[kEp == EP_RMS ? 256 : 1];
   __shared__ uint32_t tmem_slot;
   __shared__ int abort_flag;
 
@@ -934,6 +973,9 @@ gemm_tc_stream_kernel(const __grid_constant__ TmapPack maps, const TcParams p) {
       mbar_init(&acc_empty[j], 2);
       mbar_init(&epi_done[j], kEpiWarps);
     }
+    if (kEp)
+      for (int w = 0; w < kEpiWarps; ++w)
+        for (int b = 0; b < kFuseMaxBufs; ++b) mbar_init(&e_full[kEp ? w : 0][b], 1);
     abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -1029,6 +1071,10 @@ gemm_tc_stream_kernel(const __grid_constant__ TmapPack maps, const TcParams p) {
         if (u + 1 == u_end || (u + 1) / p.st_m_tiles != nt) tc_commit_pair(&b_empty);
       }
     }
+  } else if (kEp) {
+    fused_epilogue<kEp>(p, maps, tmem_base, warp, lane, (int)cta_rank, u_begin, u_end,
+                        ring + (size_t)p.st_stages * kABytes + (uint32_t)(warp - 2) * p.store_bufs * kFuseBoxBytes,
+                        e_full[kEp ? warp - 2 : 0], col_inv, acc_full, acc_empty, epi_done, &abort_flag);
   } else {
     bool ok = true;
     StoreStage st;
@@ -1119,7 +1165,7 @@ std::mutex g_tmap_mutex;
 std::map<TmapKey, CUtensorMap> g_tmap_cache;
 
 // 2-D tensor of bf16 (es = 2) or fp32 (es = 4): `inner` contiguous elements, `outer` rows `ld` elements apart;
-// box inner x outer.
+// box inner x outer, swizzled over its inner extent (128 bytes, or 64).
 cudaError_t get_tmap(const void* ptr, uint64_t inner, uint64_t outer, uint64_t ld, uint32_t box_inner,
                      uint32_t box_outer, CUtensorMap* out, int es = 2) {
   const TmapKey key(ptr, inner, outer, ld, box_inner, box_outer, es);
@@ -1137,7 +1183,7 @@ cudaError_t get_tmap(const void* ptr, uint64_t inner, uint64_t outer, uint64_t l
   CUtensorMap m;
   const CUresult r = fn(&m, es == 4 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(ptr), dims, strides, box,
                         elem, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                        CU_TENSOR_MAP_SWIZZLE_128B,
+                        box_inner * (uint32_t)es == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
                         CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) return cudaErrorInvalidValue;
   {
@@ -1206,6 +1252,7 @@ cudaError_t launch_pair_variant(const TmapPack& maps, const TcParams& p, dim3 gr
 }
 
 // Pairs the streaming kernel is launched with: as many as can be resident at once (one CTA per SM).
+template <int kEp>
 cudaError_t launch_stream(const TmapPack& maps, TcParams p, size_t smem, cudaStream_t stream) {
   static std::atomic<bool> configured[64];   // zero-initialised; set once the attribute is in place on a device
   static std::atomic<int> max_pairs[64];
@@ -1214,8 +1261,8 @@ cudaError_t launch_stream(const TmapPack& maps, TcParams p, size_t smem, cudaStr
   const bool cached = dev >= 0 && dev < 64 && configured[dev].load(std::memory_order_acquire);
   int pairs = cached ? max_pairs[dev].load(std::memory_order_relaxed) : 0;
   if (!cached) {
-    const int smem_max = kStreamSmemMax;
-    LORACT_CUDA_TRY(cudaFuncSetAttribute(gemm_tc_stream_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max));
+    const int smem_max = kStreamSmemMax - (kEp == EP_RMS ? 1024 : 0);   // (1 KB of static tables)
+    LORACT_CUDA_TRY(cudaFuncSetAttribute(gemm_tc_stream_kernel<kEp>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max));
     cudaLaunchConfig_t q = {};
     q.gridDim = dim3(2); q.blockDim = dim3(kThreads); q.dynamicSmemBytes = smem_max;
     cudaLaunchAttribute qa[1];
@@ -1223,7 +1270,7 @@ cudaError_t launch_stream(const TmapPack& maps, TcParams p, size_t smem, cudaStr
     qa[0].val.clusterDim.x = 2; qa[0].val.clusterDim.y = 1; qa[0].val.clusterDim.z = 1;
     q.attrs = qa; q.numAttrs = 1;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, gemm_tc_stream_kernel, &q) != cudaSuccess || n < 1) {
+    if (cudaOccupancyMaxActiveClusters(&n, gemm_tc_stream_kernel<kEp>, &q) != cudaSuccess || n < 1) {
       (void)cudaGetLastError();
       cudaDeviceProp prop;
       LORACT_CUDA_TRY(cudaGetDeviceProperties(&prop, dev));
@@ -1250,7 +1297,7 @@ cudaError_t launch_stream(const TmapPack& maps, TcParams p, size_t smem, cudaStr
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  LORACT_CUDA_TRY(cudaLaunchKernelEx(&cfg, gemm_tc_stream_kernel, maps, p));
+  LORACT_CUDA_TRY(cudaLaunchKernelEx(&cfg, gemm_tc_stream_kernel<kEp>, maps, p));
   count_launch(__func__, stream);
   return cudaGetLastError();
 }
@@ -1271,8 +1318,13 @@ bool gemm_tc_supported(const GemmDesc& g) {
   if (g.a_type != ELEM_BF16 || g.b_type != ELEM_BF16) return false;
   if (!(g.out == OUT_F32 || g.out == OUT_BF16 || g.out == OUT_SPLIT || g.out == OUT_RMS_BWD || g.out == OUT_ACT_BWD))
     return false;
-  if (g.out == OUT_ACT_BWD && (!g.ep_E || g.splits > 1 || g.ep_kind < 0 || g.ep_kind > 1)) return false;
-  if (g.out == OUT_RMS_BWD && (!g.ep_E || !g.ep_row_a || !g.ep_row_b || !g.ep_col || g.splits > 1)) return false;
+  if (g.out == OUT_ACT_BWD || g.out == OUT_RMS_BWD) {
+    // the operand layout, and 16-byte alignment of everything TMA touches
+    if (g.a_mn || !g.b_mn || g.n_terms != 1 || g.splits > 1 || g.K > 8 * kBK || g.gate || g.clear_status) return false;
+    if (!g.ep_E || ((uintptr_t)g.ep_E & 15) || g.ep_ld % 8 || ((uintptr_t)g.C0 & 15) || g.ldc % 8) return false;
+    if (g.out == OUT_ACT_BWD && (g.ep_kind < 0 || g.ep_kind > 1)) return false;
+    if (g.out == OUT_RMS_BWD && (!g.ep_row_a || !g.ep_row_b || !g.ep_col || ((uintptr_t)g.ep_col & 15) || g.N % 8)) return false;
+  }
   if (g.M < 1 || g.N < 1 || g.K < 1 || g.n_terms < 1 || g.n_terms > 3) return false;
   if (g.halve_at_term >= g.n_terms) return false;
   if (g.lda % 8 || g.ldb % 8) return false;
@@ -1342,8 +1394,7 @@ cudaError_t gemm_tc_launch(const GemmDesc& g, uint32_t* dev_status, cudaStream_t
   p.tmem_cols = 32;
   while ((int)p.tmem_cols < p.bn) p.tmem_cols *= 2;
   p.accumulate = g.accumulate ? 1 : 0;
-  p.ep_E = g.ep_E; p.ep_ld = g.ep_ld; p.ep_row_a = g.ep_row_a; p.ep_row_b = g.ep_row_b; p.ep_col = g.ep_col;
-  p.ep_kind = g.ep_kind;
+  p.ep_row_a = g.ep_row_a; p.ep_row_b = g.ep_row_b; p.ep_col = g.ep_col;
   p.dev_status = dev_status;
   p.st_m_tiles = 0; p.st_units = 0; p.tma_store = 0; p.st_stages = kStreamStages; p.store_bufs = kStoreBufs;
   p.halve_at_term = g.halve_at_term > 0 ? g.halve_at_term : 0;
@@ -1370,8 +1421,6 @@ cudaError_t gemm_tc_launch(const GemmDesc& g, uint32_t* dev_status, cudaStream_t
     if (((uintptr_t)g.C0 & 15) || (g.ldc * es) % 16) return false;
     if (g.out == OUT_SPLIT && ((uintptr_t)g.C1 & 15)) return false;
     if (splits > 1 && g.split_stride != (int64_t)g.M * g.ldc) return false;
-    if (g.out == OUT_RMS_BWD && (((uintptr_t)g.ep_E & 15) || ((uintptr_t)g.ep_col & 15) || g.ep_ld % 8)) return false;
-    if (g.out == OUT_ACT_BWD && (((uintptr_t)g.ep_E & 15) || g.ep_ld % 8)) return false;
     return true;
   };
   auto make_out_maps = [&]() -> cudaError_t {
@@ -1382,7 +1431,30 @@ cudaError_t gemm_tc_launch(const GemmDesc& g, uint32_t* dev_status, cudaStream_t
     return cudaSuccess;
   };
 
-  // Short contraction, large output, A K-major, B MN-major, one term (Reconstruct and the pre-norm backward):
+  // The fused epilogues (pre-norm and activation backward) exist in the persistent kernel only, which takes any number
+  // of tiles: 256 columns wide where that gives every SM pair a tile, 128 otherwise.
+  if (g.out == OUT_RMS_BWD || g.out == OUT_ACT_BWD) {
+    TcParams sp = p;
+    sp.st_m_tiles = (g.M + 2 * kBM - 1) / (2 * kBM);
+    sp.bn = (long long)sp.st_m_tiles * ((g.N + 255) / 256) >= 74 ? 256 : 128;
+    sp.b_bytes = (uint32_t)(sp.bn / 2 / 64) * 8192u;
+    sp.tmem_cols = 2u * (uint32_t)sp.bn;
+    const long long units = (long long)sp.st_m_tiles * ((g.N + sp.bn - 1) / sp.bn);
+    if (units >= (1ll << 30)) return cudaErrorNotSupported;
+    sp.st_units = (int)units;
+    // four boxes of E per epilogue warp and a ring of up to six stages, as far as the resident B leaves room: at 512
+    // contraction elements B takes 128 KB, and three stages with three boxes each remain
+    const int room = kStreamSmemMax - 2048 - p.kb_total * (int)sp.b_bytes;
+    sp.store_bufs = (room - kEpiWarps * kFuseMaxBufs * (int)kFuseBoxBytes) / (int)kABytes >= 3 ? kFuseMaxBufs : 3;
+    const int box_bytes = kEpiWarps * sp.store_bufs * (int)kFuseBoxBytes;
+    sp.st_stages = std::min(kStreamStages, (room - box_bytes) / (int)kABytes);
+    LORACT_CUDA_TRY(get_tmap(g.C0, g.N, g.M, g.ldc, 32, 32, &maps.c[0]));
+    LORACT_CUDA_TRY(get_tmap(g.ep_E, g.N, g.M, g.ep_ld, 32, 32, &maps.c[1]));
+    const size_t ssmem = (size_t)sp.kb_total * sp.b_bytes + (size_t)sp.st_stages * kABytes + (size_t)box_bytes + 1024;
+    if (g.out == OUT_RMS_BWD) return launch_stream<EP_RMS>(maps, sp, ssmem, stream);
+    return g.ep_kind == 0 ? launch_stream<EP_SILU>(maps, sp, ssmem, stream) : launch_stream<EP_GELU>(maps, sp, ssmem, stream);
+  }
+  // Short contraction, large output, A K-major, B MN-major, one term (Reconstruct):
   // the persistent kernel with B resident, when there is more than one tile per resident pair.
   if (g_pair_mode == 1 && g.M >= 2 * kBM && !g.a_mn && g.b_mn && g.n_terms == 1 && splits == 1 && p.kb_total <= 8 &&
       g.N >= 256 && g.gate == nullptr && !g.clear_status && g.lo_gate == nullptr) {
@@ -1408,7 +1480,7 @@ cudaError_t gemm_tc_launch(const GemmDesc& g, uint32_t* dev_status, cudaStream_t
       if (sp.tma_store) LORACT_CUDA_TRY(make_out_maps());
       const size_t ssmem = (size_t)sp.kb_total * sp.b_bytes + (size_t)sp.st_stages * kABytes +
                            (size_t)kEpiWarps * sp.store_bufs * kStoreBoxBytes + 1024;
-      return launch_stream(maps, sp, ssmem, stream);
+      return launch_stream<EP_NONE>(maps, sp, ssmem, stream);
     }
   }
   p.tma_store = staged_ok(p.bn) ? 1 : 0;
