@@ -61,7 +61,8 @@ struct TcParams {
   int st_m_tiles;     // streaming kernel: 256-row tiles along M
   int st_units;       // streaming kernel: tiles in all (column tile major, then M)
   int st_stages;      // streaming kernel: stages of the A ring (<= kStreamStages)
-  int store_bufs;     // staging boxes per epilogue warp (1 or 2; fused epilogue 3 or 4)
+  int store_bufs;     // staging boxes per epilogue warp (1 or 2; fused epilogue: 2 or 3)
+  int fuse_parts;     // fused epilogue: warps per quarter of the accumulator's rows
   int halve_at_term;  // the accumulator is multiplied by 1/2 before the first product of this term (0: never)
   int a_keep_from_kb; // two-CTA kernel: K block from which the loads of A carry an evict-last hint (kb_total: none)
   // one-tile kernels: when set and the word it points to is zero, the kernel loads, multiplies and stores nothing
@@ -188,15 +189,40 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
   return *reinterpret_cast<uint32_t*>(&t);
 }
 
-// f'(a) of the element-wise consumers (OUT_ACT_BWD).  SiLU: s (1 + a (1 - s)), s the logistic function;
-// GELU (exact form): Phi(a) + a phi(a).  The result is multiplied by the upstream gradient and rounded to bf16.
+// f'(a) of the element-wise consumers (OUT_ACT_BWD), times the upstream gradient, rounded to bf16 afterwards.  The fused
+// epilogue is bound by the instructions it issues, so both are written out: two special-function instructions each.
+//   SiLU: s (1 + a (1 - s)), s = 1 / (1 + exp(-a)); an exponential that overflows gives s = 0.
+//   GELU (exact form): Phi(a) + a phi(a).  With E = exp(-a^2 / 2), phi(a) = E / sqrt(2 pi) and the upper tail
+//   Q(|a|) = E P(t), t = 1 / (1 + 0.38 |a|), the form of Abramowitz and Stegun 7.1.26; the coefficients of P (degree 6) are
+//   a least-maximum fit of exp(z^2 / 2) Q(z) (absolute error of Q 7e-9, 1.5e-7 when evaluated in fp32; a result is rounded
+//   to 2^-9 of its value).  Phi(a) = Q(-a) for a < 0 and 1 - Q(a) otherwise, so the negative tail has no cancellation.
+__device__ __forceinline__ float exp2_approx(float x) {
+  float y;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ float rcp_approx(float x) {
+  float y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
 template <int kKind>
 __device__ __forceinline__ float act_derivative(float a) {
+  constexpr float kLog2e = 1.4426950408889634f;
   if (kKind == 0) {
-    const float s = __fdividef(1.f, 1.f + __expf(-a));   // 2 ulp; 0 where exp(-a) overflows
-    return s * (1.f + a * (1.f - s));
+    const float s = rcp_approx(1.f + exp2_approx(-kLog2e * a));
+    return fmaf(s, fmaf(-s, a, a), s);
   }
-  return 0.5f * (1.f + erff(a * 0.70710678118f)) + a * 0.39894228040f * __expf(-0.5f * a * a);
+  const float e = exp2_approx(-0.5f * kLog2e * a * a);
+  const float t = rcp_approx(fmaf(0.38f, fabsf(a), 1.f));
+  float q = 0.05599787458777428f;
+  q = fmaf(q, t, -0.28459465503692627f);
+  q = fmaf(q, t, 0.45932143926620483f);
+  q = fmaf(q, t, -0.09984032809734344f);
+  q = fmaf(q, t, 0.2310720831155777f);
+  q = fmaf(q, t, 0.13692614436149597f);
+  q = fmaf(q, t, 0.0011174236424267292f) * e;
+  return fmaf(0.39894228040f * a, e, a < 0.f ? q : 1.f - q);
 }
 
 // ---- staged epilogue.  A thread owns one accumulator row, so a direct store instruction of a warp touches 32
@@ -800,19 +826,24 @@ __device__ __forceinline__ bool mbar_wait_cluster_bounded(uint64_t* bar, uint32_
 // ---- fused epilogue: the finished tile is combined with another matrix E of the output's shape (read once) and only the
 // result is written.  EP_RMS: row_a col E - row_b / col acc (OUT_RMS_BWD); EP_SILU, EP_GELU: E f'(acc) (OUT_ACT_BWD).
 // A thread owns one accumulator row, so loading E from global memory here would touch 32 lines per instruction with
-// nothing in flight behind it.  Instead E comes in boxes of 32 rows x 32 columns by TMA, requested store_bufs - 1 boxes
-// ahead by each epilogue warp for itself; the result overwrites E in the box and leaves by TMA from there.
-// Measured: SiLU backward of 16384 x 11008 at K = 512: 686 us with direct loads (1.1 TB/s), 296 us with the boxes (2.5 TB/s).
+// nothing in flight behind it.  Instead E comes in boxes of 32 rows x 32 columns by TMA, requested store_bufs - 1
+// boxes ahead by each epilogue warp for itself; the result overwrites E in the box and leaves by TMA from there.
+// The epilogue is bound by the instructions it issues and their latency: up to sixteen warps, four per quarter of the
+// accumulator's rows.  Measured, SiLU / GELU backward: 16384 x 11008, K = 512: 686 / 670 us with direct loads, 252 / 376
+// with the boxes and eight warps, 227 / 251 with twelve and the derivatives written out; 16384 x 4096, K = 256: 258 / 251,
+// 96 / 141, 67 / 80 (floor 43).
 enum EpKind : int { EP_NONE = 0, EP_RMS = 1, EP_SILU = 2, EP_GELU = 3 };
-constexpr int kFuseMaxBufs = 4;
+constexpr int kFuseMaxBufs = 3;
+constexpr int kFuseMaxWarps = 16;
 constexpr uint32_t kFuseBoxBytes = 2048;                   // 32 rows x 64 bytes
 
-// Boxes of 32 columns that one epilogue warp goes through, in order: unit after unit, every other box of its row group.
+// Boxes of 32 columns that one epilogue warp goes through: every fuse_parts-th box of its row group, running on from unit to
+// unit (so that a number of warps that does not divide the boxes of a tile is balanced over several tiles).
 struct FuseCursor {
   int u, c0;
-  __device__ __forceinline__ void advance(const TcParams& p, int half_id) {
-    c0 += 64;
-    if (c0 >= p.bn) { c0 = 32 * half_id; ++u; }
+  __device__ __forceinline__ void advance(const TcParams& p) {
+    c0 += 32 * p.fuse_parts;
+    while (c0 >= p.bn) { c0 -= p.bn; ++u; }
   }
 };
 
@@ -828,28 +859,29 @@ __device__ __forceinline__ void fused_epilogue(const TcParams& p, const TmapPack
                                                int lane, int cta_rank, int u_begin, int u_end, unsigned char* boxes,
                                                uint64_t* e_full, float* col_inv, uint64_t* acc_full, uint64_t* acc_empty,
                                                uint64_t* epi_done, volatile int* abort_flag) {
-  const int quad = warp & 3, half_id = (warp - 2) >> 2;
-  const int bufs = p.store_bufs;
+  const int quad = warp & 3, part = (warp - 2) >> 2;
+  const uint32_t bufs = (uint32_t)p.store_bufs;
+  const int threads = 128 * p.fuse_parts;    // of all epilogue warps
   const __nv_bfloat16* gamma = (const __nv_bfloat16*)p.ep_col;
   auto row_of = [&](int u) { return ((u % p.st_m_tiles) * 2 + cta_rank) * kBM + quad * 32; };
   auto col_of = [&](const FuseCursor& k) { return (k.u / p.st_m_tiles) * p.bn + k.c0; };
   // boxes outside the output are neither loaded nor stored
   auto live = [&](const FuseCursor& k) { return row_of(k.u) < p.M && col_of(k) < p.N; };
-  FuseCursor ld{u_begin, 32 * half_id};
+  FuseCursor ld{u_begin, 32 * part}, k = ld;
   uint32_t n_ld = 0, n_use = 0;              // live boxes requested / used so far
   uint32_t ld_slot = 0, use_slot = 0, use_phase = 0;
   auto request = [&]() {                      // the next live box, if any
-    while (ld.u < u_end && !live(ld)) ld.advance(p, half_id);
+    while (ld.u < u_end && !live(ld)) ld.advance(p);
     if (ld.u >= u_end) return;
     if (lane == 0) {
       mbar_arrive_expect_tx(&e_full[ld_slot], kFuseBoxBytes);
       tma_load_2d(boxes + ld_slot * kFuseBoxBytes, &maps.c[1], &e_full[ld_slot], col_of(ld), row_of(ld.u));
     }
     ++n_ld;
-    if (++ld_slot == (uint32_t)bufs) ld_slot = 0;
-    ld.advance(p, half_id);
+    if (++ld_slot == bufs) ld_slot = 0;
+    ld.advance(p);
   };
-  for (int b = 0; b + 1 < bufs; ++b) request();
+  for (uint32_t b = 0; b + 1 < bufs; ++b) request();
   int cur_nt = -1;
   bool ok = true;
   for (int u = u_begin, ui = 0; u < u_end; ++u, ++ui) {
@@ -857,13 +889,13 @@ __device__ __forceinline__ void fused_epilogue(const TcParams& p, const TmapPack
     const int nt = u / p.st_m_tiles;
     const int row0 = row_of(u), m = row0 + lane;
     if (kEp == EP_RMS && nt != cur_nt) {
-      // 1 / gamma of this column tile, for all eight warps (which all come through here, even once a wait has expired)
-      asm volatile("bar.sync 1, 256;" ::: "memory");
-      for (int c = (warp - 2) * 32 + lane; c < p.bn; c += 256) {
+      // 1 / gamma of this column tile, for all epilogue warps (which all come through here, even once a wait has expired)
+      asm volatile("bar.sync 1, %0;" ::"r"(threads) : "memory");
+      for (int c = (warp - 2) * 32 + lane; c < p.bn; c += threads) {
         const int n = nt * p.bn + c;
         col_inv[c] = n < p.N ? 1.f / __bfloat162float(gamma[n]) : 0.f;
       }
-      asm volatile("bar.sync 1, 256;" ::: "memory");
+      asm volatile("bar.sync 1, %0;" ::"r"(threads) : "memory");
       cur_nt = nt;
     }
     if (!ok) continue;
@@ -874,7 +906,7 @@ __device__ __forceinline__ void fused_epilogue(const TcParams& p, const TmapPack
     if (!ok) continue;
     tc_fence_after();
     const uint32_t taddr = tmem_base + (uint32_t)(j * p.bn) + ((uint32_t)(quad * 32) << 16);
-    for (FuseCursor k{u, 32 * half_id}; k.u == u && ok; k.advance(p, half_id)) {
+    for (; k.u == u && ok; k.advance(p)) {
       if (!live(k)) continue;
       uint32_t v[32];
       tc_ld32(taddr + (uint32_t)k.c0, v);
@@ -886,6 +918,12 @@ __device__ __forceinline__ void fused_epilogue(const TcParams& p, const TmapPack
       const int n = col_of(k);
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
+        if (q == 2) {
+          // the next request goes into the box that was sent before this one, which has had half a box's time to be read
+          if (lane == 0) bulk_wait_read<0>();
+          __syncwarp();
+          request();
+        }
         // 64-byte swizzle: chunk q of row i is at chunk q ^ ((i >> 1) & 3)
         uint4* at = reinterpret_cast<uint4*>(box + lane * 64 + ((q ^ ((lane >> 1) & 3)) << 4));
         const uint4 ev = *at;
@@ -907,10 +945,7 @@ __device__ __forceinline__ void fused_epilogue(const TcParams& p, const TmapPack
       }
       stage_send(&maps.c[0], box, lane, n, row0);
       ++n_use;
-      if (++use_slot == (uint32_t)bufs) { use_slot = 0; use_phase ^= 1u; }
-      // the next request goes into the box that was sent before this one
-      if (lane == 0) bulk_wait_read<1>();
-      request();
+      if (++use_slot == bufs) { use_slot = 0; use_phase ^= 1u; }
     }
     if (!ok) continue;
     tc_fence_before();
@@ -918,7 +953,7 @@ __device__ __forceinline__ void fused_epilogue(const TcParams& p, const TmapPack
     if (lane == 0) {
       mbar_arrive_local(&epi_done[j]);
       if (warp == 2) {
-        // one signal per CTA and tile: the first epilogue warp collects the eight and tells the leader
+        // one signal per CTA and tile: the first epilogue warp collects them and tells the leader
         if (mbar_wait_bounded(&epi_done[j], (uint32_t)((ui >> 1) & 1), abort_flag)) {
           if (cta_rank == 0) mbar_arrive_local(&acc_empty[j]);
           else mbar_arrive_cluster(map_to_rank(smem_u32(&acc_empty[j]), 0u));
@@ -930,14 +965,14 @@ __device__ __forceinline__ void fused_epilogue(const TcParams& p, const TmapPack
   // every box that was requested has landed before the shared memory goes away, and every store is complete
   for (; n_use < n_ld; ++n_use) {
     (void)mbar_wait_bounded(&e_full[use_slot], use_phase, abort_flag);
-    if (++use_slot == (uint32_t)bufs) { use_slot = 0; use_phase ^= 1u; }
+    if (++use_slot == bufs) { use_slot = 0; use_phase ^= 1u; }
   }
   if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
   __syncwarp();
 }
 
 template <int kEp>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(kEp ? 64 + 32 * kFuseMaxWarps : kThreads, 1)
 gemm_tc_stream_kernel(const __grid_constant__ TmapPack maps, const TcParams p) {
   extern __shared__ __align__(1024) unsigned char smem[];
   __shared__ __align__(8) uint64_t a_full[kStreamStages];
@@ -946,7 +981,7 @@ gemm_tc_stream_kernel(const __grid_constant__ TmapPack maps, const TcParams p) {
   __shared__ __align__(8) uint64_t acc_full[2];
   __shared__ __align__(8) uint64_t acc_empty[2];
   __shared__ __align__(8) uint64_t epi_done[2];
-  __shared__ __align__(8) uint64_t e_full[kEp ? kEpiWarps : 1][kFuseMaxBufs];
+  __shared__ __align__(8) uint64_t e_full[kEp ? kFuseMaxWarps : 1][kFuseMaxBufs];
   __shared__ __align__(16) float col_inv[kEp == EP_RMS ? 256 : 1];
   __shared__ uint32_t tmem_slot;
   __shared__ int abort_flag;
@@ -971,10 +1006,10 @@ gemm_tc_stream_kernel(const __grid_constant__ TmapPack maps, const TcParams p) {
     for (int j = 0; j < 2; ++j) {
       mbar_init(&acc_full[j], 1);
       mbar_init(&acc_empty[j], 2);
-      mbar_init(&epi_done[j], kEpiWarps);
+      mbar_init(&epi_done[j], kEp ? 4 * p.fuse_parts : kEpiWarps);
     }
     if (kEp)
-      for (int w = 0; w < kEpiWarps; ++w)
+      for (int w = 0; w < kFuseMaxWarps; ++w)
         for (int b = 0; b < kFuseMaxBufs; ++b) mbar_init(&e_full[kEp ? w : 0][b], 1);
     abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -1264,7 +1299,7 @@ cudaError_t launch_stream(const TmapPack& maps, TcParams p, size_t smem, cudaStr
     const int smem_max = kStreamSmemMax - (kEp == EP_RMS ? 1024 : 0);   // (1 KB of static tables)
     LORACT_CUDA_TRY(cudaFuncSetAttribute(gemm_tc_stream_kernel<kEp>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max));
     cudaLaunchConfig_t q = {};
-    q.gridDim = dim3(2); q.blockDim = dim3(kThreads); q.dynamicSmemBytes = smem_max;
+    q.gridDim = dim3(2); q.blockDim = dim3(kEp ? 64 + 32 * kFuseMaxWarps : kThreads); q.dynamicSmemBytes = smem_max;
     cudaLaunchAttribute qa[1];
     qa[0].id = cudaLaunchAttributeClusterDimension;
     qa[0].val.clusterDim.x = 2; qa[0].val.clusterDim.y = 1; qa[0].val.clusterDim.z = 1;
@@ -1285,7 +1320,7 @@ cudaError_t launch_stream(const TmapPack& maps, TcParams p, size_t smem, cudaStr
   if (pairs > p.st_units) pairs = p.st_units;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(2 * pairs);
-  cfg.blockDim = dim3(kThreads);
+  cfg.blockDim = dim3(kEp ? 64 + 128 * p.fuse_parts : kThreads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
   cudaLaunchAttribute attr[2];
@@ -1396,7 +1431,7 @@ cudaError_t gemm_tc_launch(const GemmDesc& g, uint32_t* dev_status, cudaStream_t
   p.accumulate = g.accumulate ? 1 : 0;
   p.ep_row_a = g.ep_row_a; p.ep_row_b = g.ep_row_b; p.ep_col = g.ep_col;
   p.dev_status = dev_status;
-  p.st_m_tiles = 0; p.st_units = 0; p.tma_store = 0; p.st_stages = kStreamStages; p.store_bufs = kStoreBufs;
+  p.st_m_tiles = 0; p.st_units = 0; p.tma_store = 0; p.st_stages = kStreamStages; p.store_bufs = kStoreBufs; p.fuse_parts = 4;
   p.halve_at_term = g.halve_at_term > 0 ? g.halve_at_term : 0;
   p.a_keep_from_kb = g.a_keep_from_k >= 0 ? (int)(g.a_keep_from_k / kBK) : p.kb_total;
   p.gate = g.gate;
@@ -1442,12 +1477,18 @@ cudaError_t gemm_tc_launch(const GemmDesc& g, uint32_t* dev_status, cudaStream_t
     const long long units = (long long)sp.st_m_tiles * ((g.N + sp.bn - 1) / sp.bn);
     if (units >= (1ll << 30)) return cudaErrorNotSupported;
     sp.st_units = (int)units;
-    // four boxes of E per epilogue warp and a ring of up to six stages, as far as the resident B leaves room: at 512
-    // contraction elements B takes 128 KB, and three stages with three boxes each remain
+    // sixteen epilogue warps with three boxes of E each, or two, or twelve warps with two: the first that leaves a ring
+    // of three stages beside the resident B (a ring of two costs a quarter of the rate)
     const int room = kStreamSmemMax - 2048 - p.kb_total * (int)sp.b_bytes;
-    sp.store_bufs = (room - kEpiWarps * kFuseMaxBufs * (int)kFuseBoxBytes) / (int)kABytes >= 3 ? kFuseMaxBufs : 3;
-    const int box_bytes = kEpiWarps * sp.store_bufs * (int)kFuseBoxBytes;
-    sp.st_stages = std::min(kStreamStages, (room - box_bytes) / (int)kABytes);
+    int box_bytes = 0;
+    static const int kChoice[3][2] = {{4, 3}, {4, 2}, {3, 2}};
+    for (const auto& c : kChoice) {
+      sp.fuse_parts = c[0];
+      sp.store_bufs = c[1];
+      box_bytes = 4 * c[0] * c[1] * (int)kFuseBoxBytes;
+      sp.st_stages = std::min(kStreamStages, (room - box_bytes) / (int)kABytes);
+      if (sp.st_stages >= 3) break;
+    }
     LORACT_CUDA_TRY(get_tmap(g.C0, g.N, g.M, g.ldc, 32, 32, &maps.c[0]));
     LORACT_CUDA_TRY(get_tmap(g.ep_E, g.N, g.M, g.ep_ld, 32, 32, &maps.c[1]));
     const size_t ssmem = (size_t)sp.kb_total * sp.b_bytes + (size_t)sp.st_stages * kABytes + (size_t)box_bytes + 1024;
