@@ -448,12 +448,13 @@ __global__ void __launch_bounds__(256) norm_forward_kernel(const T* __restrict__
   }
 }
 
-// The same unit with 16-byte accesses, one warp per row.  A lane takes the chunks lane, lane + 32, ... of the
-// row (8 bf16 or 4 fp32 values each), so every load and store instruction of a warp covers 512 contiguous
-// bytes.  Rows of up to kKeep chunks per lane (d <= 4096 in bf16, 2048 in fp32) stay in registers, packed as
-// loaded: X is read from memory exactly once and the statistics (mean, then the centred second moment, as
-// in the kernel above) are taken from the registers.  Longer rows are read again for each pass.
-constexpr int kNormKeep = 16;
+// The same unit with 16-byte accesses.  A row is shared by kWarps warps of a block: thread t of the row takes the chunks
+// t, t + 32 kWarps, ... (8 bf16 or 4 fp32 values each), so every load and store instruction of a warp covers 512 contiguous
+// bytes, and keeps them in registers, packed as loaded: X is read from memory exactly once and the statistics (mean, then
+// the centred second moment, as in the kernel above) are taken from the registers.  What bounds it is bytes in flight: few
+// chunks per thread keep the registers low and many rows resident.  (Measured with one warp per row and up to sixteen
+// chunks per lane: 16384 x 4096 bf16, LayerNorm 73 us, RMS 58; x 11008: 257 and 187.  Now 60, 49, 155, 124 (floor
+// 41 and 110).)
 
 template <typename T>
 struct NormChunk;
@@ -489,7 +490,7 @@ struct NormChunk<float> {
   }
 };
 
-template <typename T, bool kInRegs>
+template <typename T, int kWarps, int kKeep>
 __global__ void __launch_bounds__(256) norm_forward_vec_kernel(const T* __restrict__ X, int64_t n, int64_t d,
                                                                int64_t ldx, const T* __restrict__ gamma,
                                                                const T* __restrict__ beta, float eps, int kind,
@@ -498,63 +499,68 @@ __global__ void __launch_bounds__(256) norm_forward_vec_kernel(const T* __restri
                                                                float* __restrict__ mean_out) {
   using C = NormChunk<T>;
   constexpr int kV = C::kVals;
-  const int lane = threadIdx.x & 31;
-  const int64_t row = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (row >= n) return;
-  const int n_chunks = (int)(d / kV);
+  __shared__ float s_part[2][8];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int sub = warp % kWarps, t = sub * 32 + lane;        // position inside the row
+  const int64_t row = (int64_t)blockIdx.x * (8 / kWarps) + warp / kWarps;
+  pdl_wait();
+  pdl_launch_dependents();
+  const int n_chunks = row < n ? (int)(d / kV) : 0;          // (a row past the end takes part in the barriers only)
   const uint4* x = reinterpret_cast<const uint4*>(X + row * ldx);
-  const uint4* gm = reinterpret_cast<const uint4*>(gamma);
-  const uint4* bt = reinterpret_cast<const uint4*>(beta);
-  uint4* a = reinterpret_cast<uint4*>(A + row * lda);
-  uint4 keep[kInRegs ? kNormKeep : 1];
-  if (kInRegs) {
+  uint4 keep[kKeep];
 #pragma unroll
-    for (int i = 0; i < kNormKeep; ++i) {
-      const int c = lane + 32 * i;
-      keep[i] = c < n_chunks ? x[c] : make_uint4(0u, 0u, 0u, 0u);
-    }
+  for (int i = 0; i < kKeep; ++i) {
+    const int c = t + 32 * kWarps * i;
+    keep[i] = c < n_chunks ? __ldg(x + c) : make_uint4(0u, 0u, 0u, 0u);
   }
-  auto chunk = [&](int i, int c) -> uint4 { return kInRegs ? keep[i] : x[c]; };
-  const int per_lane = kInRegs ? kNormKeep : (n_chunks + 31) / 32;
+  // sum over the row, in the same order for every thread
+  auto row_sum = [&](float v, float* part) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (kWarps == 1) return v;
+    if (lane == 0) part[warp] = v;
+    __syncthreads();
+    v = 0.f;
+#pragma unroll
+    for (int q = 0; q < kWarps; ++q) v += part[warp - sub + q];
+    return v;
+  };
   float mean = 0.f;
   if (kind == LORACT_NORM_LAYER) {
     float s = 0.f;
 #pragma unroll
-    for (int i = 0; i < per_lane; ++i) {
-      const int c = lane + 32 * i;
-      if (c >= n_chunks) break;
+    for (int i = 0; i < kKeep; ++i) {
       float v[kV];
-      C::unpack(chunk(i, c), v);
+      C::unpack(keep[i], v);
 #pragma unroll
-      for (int q = 0; q < kV; ++q) s += v[q];
+      for (int q = 0; q < kV; ++q) s += v[q];                // (chunks past the row are zeros)
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    mean = s / (float)d;
+    mean = row_sum(s, s_part[0]) / (float)d;
   }
   float ss = 0.f;
 #pragma unroll
-  for (int i = 0; i < per_lane; ++i) {
-    const int c = lane + 32 * i;
-    if (c >= n_chunks) break;
+  for (int i = 0; i < kKeep; ++i) {
+    if (t + 32 * kWarps * i >= n_chunks) continue;
     float v[kV];
-    C::unpack(chunk(i, c), v);
+    C::unpack(keep[i], v);
 #pragma unroll
-    for (int q = 0; q < kV; ++q) { const float t = v[q] - mean; ss += t * t; }
+    for (int q = 0; q < kV; ++q) { const float u = v[q] - mean; ss += u * u; }
   }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
-  const float rstd = rsqrtf(ss / (float)d + eps);
-  if (lane == 0) {
+  const float rstd = rsqrtf(row_sum(ss, s_part[1]) / (float)d + eps);
+  if (row >= n) return;
+  if (t == 0) {
     rstd_out[row] = rstd;
     if (mean_out) mean_out[row] = mean;
   }
+  const uint4* gm = reinterpret_cast<const uint4*>(gamma);
+  const uint4* bt = reinterpret_cast<const uint4*>(beta);
+  uint4* a = reinterpret_cast<uint4*>(A + row * lda);
 #pragma unroll
-  for (int i = 0; i < per_lane; ++i) {
-    const int c = lane + 32 * i;
-    if (c >= n_chunks) break;
+  for (int i = 0; i < kKeep; ++i) {
+    const int c = t + 32 * kWarps * i;
+    if (c >= n_chunks) continue;
     float v[kV], g[kV], b[kV];
-    C::unpack(chunk(i, c), v);
+    C::unpack(keep[i], v);
     C::unpack(__ldg(gm + c), g);
     if (beta) C::unpack(__ldg(bt + c), b);
 #pragma unroll
@@ -564,6 +570,41 @@ __global__ void __launch_bounds__(256) norm_forward_vec_kernel(const T* __restri
     }
     a[c] = C::pack(v);
   }
+}
+
+template <typename T, int kWarps, int kKeep>
+cudaError_t launch_norm_vec(const void* X, int64_t n, int64_t d, int64_t ldx, const void* gamma, const void* beta, float eps,
+                            int kind, void* A, int64_t lda, float* rstd, float* mean, cudaStream_t stream) {
+  const int rows = 8 / kWarps;
+  LORACT_CUDA_TRY(launch_pdl(norm_forward_vec_kernel<T, kWarps, kKeep>, dim3((unsigned)((n + rows - 1) / rows)), dim3(256), 0,
+                             stream, (const T*)X, n, d, ldx, (const T*)gamma, (const T*)beta, eps, kind, (T*)A, lda, rstd,
+                             mean));
+  return cudaGetLastError();
+}
+
+template <typename T>
+cudaError_t launch_norm(const void* X, int64_t n, int64_t d, int64_t ldx, const void* gamma, const void* beta, float eps,
+                        int kind, void* A, int64_t lda, float* rstd, float* mean, cudaStream_t stream) {
+  constexpr int kV = NormChunk<T>::kVals;
+  // 16-byte accesses need every row of X and A, and gamma and beta, on a 16-byte boundary
+  const bool vec = d % kV == 0 && ldx % kV == 0 && lda % kV == 0 && (((uintptr_t)X | (uintptr_t)A |
+                   (uintptr_t)gamma | (uintptr_t)beta) & 15) == 0;
+  const int64_t chunks = d / kV;
+#define LORACT_NORM(W, K) return launch_norm_vec<T, W, K>(X, n, d, ldx, gamma, beta, eps, kind, A, lda, rstd, mean, stream)
+  // at most four chunks per thread up to 1024 chunks (d = 8192 in bf16), eight beyond; longer rows take the plain kernel
+  if (vec) {
+    if (chunks <= 64) LORACT_NORM(1, 2);
+    if (chunks <= 128) LORACT_NORM(1, 4);
+    if (chunks <= 256) LORACT_NORM(2, 4);
+    if (chunks <= 512) LORACT_NORM(4, 4);
+    if (chunks <= 1024) LORACT_NORM(8, 4);
+    if (chunks <= 2048) LORACT_NORM(8, 8);
+  }
+#undef LORACT_NORM
+  const int warps = 8;
+  norm_forward_kernel<T><<<(int)((n + warps - 1) / warps), warps * 32, 0, stream>>>(
+      (const T*)X, n, d, ldx, (const T*)gamma, (const T*)beta, eps, kind, (T*)A, lda, rstd, mean);
+  return cudaGetLastError();
 }
 
 template <typename TA, typename TB>
@@ -831,36 +872,10 @@ cudaError_t rms_backward_rows_launch(const __nv_bfloat16* U, const float* P, con
 cudaError_t norm_forward_launch(const void* X, int64_t n, int64_t d, int64_t ldx, int elem_type,
                                 const void* gamma, const void* beta, float eps, int kind, void* A,
                                 int64_t lda, float* rstd, float* mean, cudaStream_t stream) {
-  const int warps = 8;
-  const int grid = (int)((n + warps - 1) / warps);
-  const int vals = elem_type == ELEM_BF16 ? 8 : 4;
-  // 16-byte accesses need every row of X and A, and gamma and beta, on a 16-byte boundary
-  const bool vec = d % vals == 0 && ldx % vals == 0 && lda % vals == 0 && (((uintptr_t)X | (uintptr_t)A |
-                   (uintptr_t)gamma | (uintptr_t)beta) & 15) == 0;
-  const bool in_regs = d <= (int64_t)vals * 32 * kNormKeep;
-  if (elem_type == ELEM_BF16) {
-    typedef __nv_bfloat16 T;
-    if (vec && in_regs)
-      norm_forward_vec_kernel<T, true><<<grid, warps * 32, 0, stream>>>((const T*)X, n, d, ldx, (const T*)gamma,
-                                                                       (const T*)beta, eps, kind, (T*)A, lda, rstd, mean);
-    else if (vec)
-      norm_forward_vec_kernel<T, false><<<grid, warps * 32, 0, stream>>>((const T*)X, n, d, ldx, (const T*)gamma,
-                                                                        (const T*)beta, eps, kind, (T*)A, lda, rstd, mean);
-    else
-      norm_forward_kernel<T><<<grid, warps * 32, 0, stream>>>((const T*)X, n, d, ldx, (const T*)gamma, (const T*)beta,
-                                                              eps, kind, (T*)A, lda, rstd, mean);
-  } else {
-    typedef float T;
-    if (vec && in_regs)
-      norm_forward_vec_kernel<T, true><<<grid, warps * 32, 0, stream>>>((const T*)X, n, d, ldx, (const T*)gamma,
-                                                                       (const T*)beta, eps, kind, (T*)A, lda, rstd, mean);
-    else if (vec)
-      norm_forward_vec_kernel<T, false><<<grid, warps * 32, 0, stream>>>((const T*)X, n, d, ldx, (const T*)gamma,
-                                                                        (const T*)beta, eps, kind, (T*)A, lda, rstd, mean);
-    else
-      norm_forward_kernel<T><<<grid, warps * 32, 0, stream>>>((const T*)X, n, d, ldx, (const T*)gamma, (const T*)beta,
-                                                              eps, kind, (T*)A, lda, rstd, mean);
-  }
+  const cudaError_t e = elem_type == ELEM_BF16
+      ? launch_norm<__nv_bfloat16>(X, n, d, ldx, gamma, beta, eps, kind, A, lda, rstd, mean, stream)
+      : launch_norm<float>(X, n, d, ldx, gamma, beta, eps, kind, A, lda, rstd, mean, stream);
+  if (e != cudaSuccess) return e;
   count_launch(__func__, stream);
   return cudaGetLastError();
 }
