@@ -109,6 +109,7 @@ struct Plan {
   int l;
   bool bf16;
   int splits_gs, splits_w, splits_v;
+  int splits_y;   // of the sketch over d
 };
 
 inline int simt_splits(int64_t k) {
@@ -126,12 +127,14 @@ Plan make_plan(int64_t n, int64_t d, int l, bool bf16) {
     // added with rounding afterwards) keep that bias below what one orthonormalisation round tolerates.
     p.splits_w = gemm_tc_pick_splits(l, l, (int)n, true, true, 64);
     p.splits_v = gemm_tc_pick_splits(l, (int)d, (int)n, true, true);
+    p.splits_y = gemm_tc_pick_tall_splits((int)n, l, (int)d);
   } else {
     // CUDA-core path: the generic kernel walks K sixteen elements at a time, so a long contraction with few output
     // tiles is split over K (partial sums, added in a fixed order afterwards)
     p.splits_gs = simt_splits(d);
     p.splits_w = simt_splits(n);
     p.splits_v = simt_splits(n);
+    p.splits_y = simt_splits(d);
   }
   return p;
 }
@@ -155,7 +158,9 @@ void carve_basis(Carver& c, const Plan& p, BasisWs* w) {
     w->Yl = (__nv_bfloat16*)c.take(n * l * 2);
     w->Qh = (__nv_bfloat16*)c.take(n * l * 2);
     w->Ql = (__nv_bfloat16*)c.take(n * l * 2);
-    w->v_partials = (float*)c.take((p.splits_v > 1 ? (size_t)p.splits_v : 0) * l * d * 4);
+    // partial sums of V (l x d per split over the tokens) or of the sketch (n x l per split over d)
+    const size_t pv = (p.splits_v > 1 ? (size_t)p.splits_v : 0) * l * d, py = (p.splits_y > 1 ? (size_t)p.splits_y : 0) * n * l;
+    w->v_partials = (float*)c.take((pv > py ? pv : py) * 4);
   } else {
     w->Linv32 = (float*)c.take(l * l * 4);
     w->sb_scratch = c.take((l * l + (l + 31) / 32 * 1024) * sizeof(double));
@@ -263,6 +268,24 @@ cudaError_t precondition_rows(const void* T, int l, int64_t d, bool bf16, void* 
   return run_gemm(g, status, stream);
 }
 
+// The sketch Y = X Omega^T of the bf16 path as a bf16 pair.  With few rows (a context of a few thousand tokens) the tiles
+// of Y do not fill the chip: the product is then split over d and the partial sums are added as the pair is formed.
+cudaError_t sketch(const void* X, int64_t ldx, const Plan& p, const void* Omega, int64_t keep_from, const BasisWs& w,
+                   uint32_t* status, cudaStream_t stream) {
+  GemmDesc g;
+  g.M = (int)p.n; g.N = p.l; g.K = (int)p.d; g.lda = ldx; g.ldb = p.d;
+  g.terms[0] = {X, Omega};
+  g.ldc = p.l;
+  g.a_keep_from_k = keep_from;
+  if (p.splits_y <= 1) {
+    g.out = OUT_SPLIT; g.C0 = w.Yh; g.C1 = w.Yl;
+    return run_gemm(g, status, stream);
+  }
+  g.out = OUT_F32; g.C0 = w.v_partials; g.splits = p.splits_y; g.split_stride = (int64_t)p.n * p.l;
+  LORACT_CUDA_TRY(run_gemm(g, status, stream));
+  return reduce_pair_launch(w.v_partials, p.splits_y, g.split_stride, g.split_stride, w.Yh, w.Yl, stream);
+}
+
 // The sketch and the orthonormalisation of Algorithm 1 for a test matrix Omega (l x d, rows are the test vectors):
 // Y = X Omega^T, then { W = Y^T Y = L L^T ; Y <- Y L^{-T} }, once or (decided on the device, bf16 inputs) twice.
 // U (n x l) receives Q.
@@ -271,25 +294,19 @@ cudaError_t range_basis(const void* X, int64_t ldx, const Plan& p, const void* O
   const int l = p.l;
   const int n = (int)p.n;
   const int el = p.bf16 ? ELEM_BF16 : ELEM_F32;
-  {  // Y = X Omega^T
+  trace_label("pass 1: Y = X Omega^T");
+  if (p.bf16) {
+    // The projection reads X again a few hundred microseconds from now: the last columns this pass streams are
+    // asked to stay in L2 (as many bytes of X as kL2KeepBytes).
+    const double x_bytes = (double)n * (double)p.d * 2.0;
+    const double frac = kL2KeepBytes >= x_bytes ? 1.0 : kL2KeepBytes / x_bytes;
+    LORACT_CUDA_TRY(sketch(X, ldx, p, Omega, (int64_t)((1.0 - frac) * (double)p.d), w, status, stream));
+  } else {
     GemmDesc g;
     g.M = n; g.N = l; g.K = (int)p.d; g.lda = ldx; g.ldb = p.d; g.a_type = g.b_type = el;
     g.terms[0] = {X, Omega};
     g.ldc = l;
-    trace_label("pass 1: Y = X Omega^T");
-    if (p.bf16) {
-      g.out = OUT_SPLIT; g.C0 = w.Yh; g.C1 = w.Yl;
-      // The projection reads X again a few hundred microseconds from now: the last columns this pass streams are
-      // asked to stay in L2 (as many bytes of X as kL2KeepBytes).
-      const double x_bytes = (double)n * (double)p.d * 2.0;
-      if (x_bytes > 0) {
-        const double frac = kL2KeepBytes >= x_bytes ? 1.0 : kL2KeepBytes / x_bytes;
-        g.a_keep_from_k = (int64_t)((1.0 - frac) * (double)p.d);
-      }
-      LORACT_CUDA_TRY(run_gemm(g, status, stream));
-    } else {
-      LORACT_CUDA_TRY(simt_split_f32(g, simt_splits(p.d), w.part32, w.Y32, stream));
-    }
+    LORACT_CUDA_TRY(simt_split_f32(g, p.splits_y, w.part32, w.Y32, stream));
   }
   if (!p.bf16) {
     for (int round = 0; round < 2; ++round) {
@@ -579,6 +596,11 @@ loract_status_t check_joint(const loract_desc_t* desc) {
   return LORACT_OK;
 }
 
+// Workspace of the pre-norm backward with P = grad_A V^T in `splits` partial sums, and two row coefficients.
+size_t prenorm_backward_bytes(int64_t n, int r, int splits) {
+  return 256 + align_up((size_t)splits * n * r * 4) + 2 * align_up((size_t)n * 4);
+}
+
 std::atomic<int> g_last_cuda_error{0};
 loract_status_t from_cuda(cudaError_t e) {
   if (e == cudaSuccess) return LORACT_OK;
@@ -722,12 +744,9 @@ loract_status_t loract_weight_grad(const loract_desc_t* desc, const void* U, con
 
 size_t loract_prenorm_backward_workspace_bytes(const loract_desc_t* desc) {
   if (check_desc(desc) != LORACT_OK) return 0;
-  Carver c(nullptr);
-  c.take(256);
-  c.take((size_t)desc->n_tokens * desc->rank * 4);   // P = grad_A V^T
-  c.take((size_t)desc->n_tokens * 4);                // row_a
-  c.take((size_t)desc->n_tokens * 4);                // row_b
-  return c.off;
+  // P = grad_A V^T in as many partial sums as the shape is split into (a call with less runs on fewer)
+  return prenorm_backward_bytes(desc->n_tokens, desc->rank,
+                                gemm_tc_pick_tall_splits((int)desc->n_tokens, desc->rank, (int)desc->d));
 }
 
 loract_status_t loract_prenorm_backward(const loract_desc_t* desc, const void* U, const void* V, const void* gamma,
@@ -740,11 +759,17 @@ loract_status_t loract_prenorm_backward(const loract_desc_t* desc, const void* U
   if (misaligned(U) || misaligned(V) || misaligned(gamma) || misaligned(grad_A) || misaligned(grad_X) ||
       ((uintptr_t)ws & 255))
     return LORACT_ERR_ALIGNMENT;
-  if (ws_bytes < loract_prenorm_backward_workspace_bytes(desc)) return LORACT_ERR_WORKSPACE_TOO_SMALL;
+  if (ws_bytes < prenorm_backward_bytes(desc->n_tokens, desc->rank, 1)) return LORACT_ERR_WORKSPACE_TOO_SMALL;
   const int n = (int)desc->n_tokens, d = (int)desc->d, r = desc->rank;
+  // P may be formed as partial sums over d (the row coefficients add them): as many as the workspace holds
+  int splits = gemm_tc_pick_tall_splits(n, r, d);
+  const size_t p_bytes = (size_t)n * r * 4;
+  while (splits > 1 && prenorm_backward_bytes(n, r, splits) > ws_bytes) --splits;
+  const int kb = (d + 63) / 64, per = (kb + splits - 1) / splits;
+  splits = (kb + per - 1) / per;   // no empty split
   Carver c(ws);
   uint32_t* status = (uint32_t*)c.take(256);
-  float* P = (float*)c.take((size_t)n * r * 4);
+  float* P = (float*)c.take(p_bytes * splits);
   float* row_a = (float*)c.take((size_t)n * 4);
   float* row_b = (float*)c.take((size_t)n * 4);
   cudaStream_t st = (cudaStream_t)stream;
@@ -755,13 +780,13 @@ loract_status_t loract_prenorm_backward(const loract_desc_t* desc, const void* U
     GemmDesc g;
     g.M = n; g.N = r; g.K = d; g.lda = desc->ldx; g.ldb = d;
     g.terms[0] = {grad_A, V};
-    g.out = OUT_F32; g.C0 = P; g.ldc = r;
+    g.out = OUT_F32; g.C0 = P; g.ldc = r; g.splits = splits; g.split_stride = (int64_t)n * r;
     trace_label("pre-norm backward: P = grad_A V^T");
     e = gemm_tc_supported(g) ? gemm_tc_launch(g, status, st) : cudaErrorNotSupported;
   }
   if (e == cudaSuccess) {
     trace_label("pre-norm backward: row coefficients");
-    e = rms_backward_rows_launch((const __nv_bfloat16*)U, P, rstd, n, r, d, row_a, row_b, st);
+    e = rms_backward_rows_launch((const __nv_bfloat16*)U, P, splits, rstd, n, r, d, row_a, row_b, st);
   }
   if (e == cudaSuccess) {
     // grad_X = rstd * (grad_A * gamma - (A~ / gamma) * inner), A~ tile by tile in tensor memory only
@@ -839,14 +864,8 @@ loract_status_t loract_joint_sketch(const loract_desc_t* desc, const void* X_loc
   const int r = desc->rank, n = (int)desc->n_tokens;
   // the test matrix from the complete sampled rows: the same bits on every shard
   cudaError_t e = precondition_rows(S_sum, r, desc->d, true, w.Omega, w.b, w.status, st);
-  if (e == cudaSuccess) {  // this shard's rows of the sketch, Y = X_local Omega^T
-    GemmDesc g;
-    g.M = n; g.N = r; g.K = (int)desc->d; g.lda = desc->ldx; g.ldb = desc->d;
-    g.terms[0] = {X_local, w.Omega};
-    g.ldc = r; g.out = OUT_SPLIT; g.C0 = w.b.Yh; g.C1 = w.b.Yl;
-    trace_label("joint: pass 1");
-    e = run_gemm(g, w.status, st);
-  }
+  trace_label("joint: pass 1");   // this shard's rows of the sketch, Y = X_local Omega^T
+  if (e == cudaSuccess) e = sketch(X_local, desc->ldx, plan, w.Omega, -1, w.b, w.status, st);
   trace_label("joint: Gram 1 of the shard");
   if (e == cudaSuccess) e = gram_tall_sum(w.b.Yh, w.b.Yl, n, r, w.b, W_partial, w.status, st);
   return from_cuda(e);

@@ -127,6 +127,8 @@ struct GemmDesc {
 bool gemm_tc_supported(const GemmDesc& g);
 cudaError_t gemm_tc_launch(const GemmDesc& g, uint32_t* dev_status, cudaStream_t stream);
 int gemm_tc_pick_splits(int M, int N, int K, bool a_mn, bool b_mn, int max_splits = 32);
+// Splits over K of a product with many rows (M x N, both operands K-major) whose tiles do not fill the chip.
+int gemm_tc_pick_tall_splits(int M, int N, int K);
 void gemm_tc_set_pair_mode(int on);   // test hook: 0 keeps every contraction on the one-CTA kernel
 // Test hooks for the give-up path of the bounded waits: a kernel that waits (with the engine's / the cluster
 // kernel's own wait) on a barrier nothing completes, for at most limit_ns, then sets LORACT_DEV_WAIT_EXPIRED.
@@ -218,6 +220,9 @@ cudaError_t zero3_gated_launch(void* a, size_t a_bytes, void* b, size_t b_bytes,
 cudaError_t reduce_partials_launch(const float* partials, int n_partials, int64_t stride,
                                    int64_t count, float* out_f32, __nv_bfloat16* out_bf16,
                                    cudaStream_t stream, const uint32_t* gate = nullptr);
+// hi + lo = sum_s partials[s] (fixed order) as a bf16 pair; count a multiple of 4, everything 16-byte aligned.
+cudaError_t reduce_pair_launch(const float* partials, int n_partials, int64_t stride, int64_t count, __nv_bfloat16* hi,
+                               __nv_bfloat16* lo, cudaStream_t stream);
 // out (r x r) = S + S^T, S the fixed-order sum of the partials (each r x r, leading dimension r).
 // gate (optional): device word; zero means the launch does nothing.
 cudaError_t reduce_sym_launch(const float* partials, int n_partials, int64_t stride, int r, float* out,
@@ -239,9 +244,10 @@ cudaError_t copy_bf16_gated_launch(const __nv_bfloat16* src, __nv_bfloat16* dst,
 cudaError_t reduce_split3_launch(const float* partials, int n_partials, int64_t stride, int rows, int cols,
                                  int64_t ld_in, int64_t ld_out, __nv_bfloat16* hi, __nv_bfloat16* mid,
                                  __nv_bfloat16* lo, cudaStream_t stream);
-// Section 3.3 backward, row coefficients: inner_i = (1 / d) sum_k U[i][k] P[i][k] (P = grad_A V^T, fp32, n x r),
+// Section 3.3 backward, row coefficients: inner_i = (1 / d) sum_k U[i][k] P[i][k] (P = grad_A V^T, fp32, n x r, the sum of n_partials
+// matrices stored one behind the other),
 // row_a[i] = rstd[i], row_b[i] = rstd[i] * inner_i.  One warp per row.
-cudaError_t rms_backward_rows_launch(const __nv_bfloat16* U, const float* P, const float* rstd, int64_t n, int r,
+cudaError_t rms_backward_rows_launch(const __nv_bfloat16* U, const float* P, int n_partials, const float* rstd, int64_t n, int r,
                                      int64_t d, float* row_a, float* row_b, cudaStream_t stream);
 // Section 3.3 forward: A = Norm(X); per-row rstd (and mean for LayerNorm).  One warp per row.
 cudaError_t norm_forward_launch(const void* X, int64_t n, int64_t d, int64_t ldx, int elem_type,

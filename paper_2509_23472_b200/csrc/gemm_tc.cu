@@ -1412,6 +1412,29 @@ int gemm_tc_pick_splits(int M, int N, int K, bool, bool b_mn, int max_splits) {
   return best < 1 ? 1 : best;
 }
 
+// A product with many rows streams one operand (X) once, and its tiles take about 0.36 us per 64-wide K block whatever
+// their width up to 256 (the issue of the MMAs bounds narrow ones, the loads wide ones).  4096 rows are sixteen pair tiles
+// on 74 SM pairs: split over K the same work uses the idle SMs, at the price of partial sums (written and read through L2
+// at about 3 MB per us) and one more launch.  The split count with the least estimate, if that is at least 10 % below one.
+// (Measured, whole steps: 4096 x 5120, r = 64: 112 -> 90 us with four splits; two passes over 8192 x 5120, r = 128:
+// 269 -> 235 us with two.)
+int gemm_tc_pick_tall_splits(int M, int N, int K) {
+  const int bn = pick_bn(N);
+  const bool pair = M >= 2 * kBM && bn % 32 == 0;
+  const int rows = pair ? 2 * kBM : kBM, slots = pair ? 74 : 148;
+  const long long tiles = (long long)((M + rows - 1) / rows) * ((N + bn - 1) / bn);
+  const int kb = (K + kBK - 1) / kBK;
+  auto cost = [&](int sp) {
+    const double rounds = (double)((tiles * sp + slots - 1) / slots);
+    return rounds * (double)((kb + sp - 1) / sp) * 0.36 + (sp > 1 ? 4.0 + (double)sp * M * N * 4.0 / 3.0e6 : 0.0);
+  };
+  int best = 1;
+  for (int sp = 2; sp <= 8 && kb / sp >= 4; ++sp)
+    if (cost(sp) < cost(best) && cost(sp) < 0.9 * cost(1)) best = sp;
+  const int per = (kb + best - 1) / best;
+  return (kb + per - 1) / per;                             // no empty split
+}
+
 cudaError_t gemm_tc_launch(const GemmDesc& g, uint32_t* dev_status, cudaStream_t stream) {
   if (!gemm_tc_supported(g)) return cudaErrorNotSupported;
   TcParams p;

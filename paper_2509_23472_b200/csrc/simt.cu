@@ -183,6 +183,28 @@ __global__ void __launch_bounds__(256) reduce_partials_vec4_kernel(const float4*
   }
 }
 
+// hi + lo = sum_s partials[s] (fixed order) as a bf16 pair, four elements per thread, all partials of a quad in flight.
+__global__ void __launch_bounds__(256) reduce_pair_kernel(const float4* __restrict__ partials, int n_partials,
+                                                          int64_t stride4, int64_t count4, uint2* __restrict__ hi,
+                                                          uint2* __restrict__ lo) {
+  pdl_wait();
+  pdl_launch_dependents();
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count4;
+       i += (int64_t)gridDim.x * blockDim.x) {
+    float4 s = partials[i];
+#pragma unroll 4
+    for (int q = 1; q < n_partials; ++q) {
+      const float4 a = partials[(int64_t)q * stride4 + i];
+      s.x += a.x; s.y += a.y; s.z += a.z; s.w += a.w;
+    }
+    const __nv_bfloat162 h0 = __floats2bfloat162_rn(s.x, s.y), h1 = __floats2bfloat162_rn(s.z, s.w);
+    const float2 f0 = __bfloat1622float2(h0), f1 = __bfloat1622float2(h1);
+    const __nv_bfloat162 l0 = __floats2bfloat162_rn(s.x - f0.x, s.y - f0.y), l1 = __floats2bfloat162_rn(s.z - f1.x, s.w - f1.y);
+    hi[i] = make_uint2(*reinterpret_cast<const uint32_t*>(&h0), *reinterpret_cast<const uint32_t*>(&h1));
+    lo[i] = make_uint2(*reinterpret_cast<const uint32_t*>(&l0), *reinterpret_cast<const uint32_t*>(&l1));
+  }
+}
+
 // out = S + S^T with S = sum_s partials[s] (fixed order), for r x r matrices: the tall Gram products are formed as
 // D = Yh^T Yh / 2 + Yh^T Yl (two terms), and D + D^T = Yh^T Yh + Yh^T Yl + Yl^T Yh is the three-term Gram matrix,
 // exactly symmetric.  One CTA per pair of 16 x 16 tiles (I, J), (J, I), I >= J: both tiles are summed with
@@ -387,7 +409,7 @@ __global__ void split_block_kernel(const float* __restrict__ src, int rows, int 
 
 // One warp per row: inner = (1 / d) sum_k U[i][k] P[i][k];  row_a = rstd, row_b = rstd * inner.
 __global__ void __launch_bounds__(256) rms_backward_rows_kernel(const __nv_bfloat16* __restrict__ U,
-                                                                const float* __restrict__ P,
+                                                                const float* __restrict__ P, int n_partials,
                                                                 const float* __restrict__ rstd, int64_t n, int r,
                                                                 float inv_d, float* __restrict__ row_a,
                                                                 float* __restrict__ row_b) {
@@ -396,8 +418,21 @@ __global__ void __launch_bounds__(256) rms_backward_rows_kernel(const __nv_bfloa
   const int lane = threadIdx.x & 31;
   const int64_t row = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (row >= n) return;
+  // four columns per lane and step (r is a multiple of 16): an 8-byte load of U, 16-byte loads of the partial sums
+  const uint2* u = reinterpret_cast<const uint2*>(U + row * r);
+  const float4* pr = reinterpret_cast<const float4*>(P + row * r);
+  const int64_t stride = n * r / 4;
   float s = 0.f;
-  for (int k = lane; k < r; k += 32) s += __bfloat162float(U[row * r + k]) * P[row * r + k];
+  for (int k = lane; k < r / 4; k += 32) {
+    const uint2 uv = __ldg(u + k);
+    float4 q = pr[k];
+    for (int i = 1; i < n_partials; ++i) {
+      const float4 t = pr[i * stride + k];
+      q.x += t.x; q.y += t.y; q.z += t.z; q.w += t.w;
+    }
+    s += __uint_as_float(uv.x << 16) * q.x + __uint_as_float(uv.x & 0xffff0000u) * q.y +
+         __uint_as_float(uv.y << 16) * q.z + __uint_as_float(uv.y & 0xffff0000u) * q.w;
+  }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
   if (lane == 0) {
@@ -753,6 +788,18 @@ cudaError_t reduce_partials_launch(const float* partials, int n_partials, int64_
   return cudaGetLastError();
 }
 
+cudaError_t reduce_pair_launch(const float* partials, int n_partials, int64_t stride, int64_t count, __nv_bfloat16* hi,
+                               __nv_bfloat16* lo, cudaStream_t stream) {
+  if (count % 4 || stride % 4 || (((uintptr_t)partials) & 15) || (((uintptr_t)hi | (uintptr_t)lo) & 7)) return cudaErrorInvalidValue;
+  const int64_t count4 = count / 4;
+  int grid = (int)((count4 + 255) / 256);
+  if (grid > 148 * 8) grid = 148 * 8;
+  LORACT_CUDA_TRY(launch_pdl(reduce_pair_kernel, dim3(grid), dim3(256), 0, stream, (const float4*)partials, n_partials,
+                             stride / 4, count4, (uint2*)hi, (uint2*)lo));
+  count_launch(__func__, stream);
+  return cudaGetLastError();
+}
+
 cudaError_t reduce_sym_launch(const float* partials, int n_partials, int64_t stride, int r, float* out,
                               cudaStream_t stream, const uint32_t* gate) {
   const int nt = (r + kSymTile - 1) / kSymTile;
@@ -859,11 +906,11 @@ cudaError_t split_block_launch(const float* src, int rows, int cols, int64_t ld,
   return cudaGetLastError();
 }
 
-cudaError_t rms_backward_rows_launch(const __nv_bfloat16* U, const float* P, const float* rstd, int64_t n, int r,
+cudaError_t rms_backward_rows_launch(const __nv_bfloat16* U, const float* P, int n_partials, const float* rstd, int64_t n, int r,
                                      int64_t d, float* row_a, float* row_b, cudaStream_t stream) {
   const int warps = 8;
   const int grid = (int)((n + warps - 1) / warps);
-  LORACT_CUDA_TRY(launch_pdl(rms_backward_rows_kernel, dim3(grid), dim3(warps * 32), 0, stream, U, P, rstd, n, r,
+  LORACT_CUDA_TRY(launch_pdl(rms_backward_rows_kernel, dim3(grid), dim3(warps * 32), 0, stream, U, P, n_partials, rstd, n, r,
                              1.0f / (float)d, row_a, row_b));
   count_launch(__func__, stream);
   return cudaGetLastError();

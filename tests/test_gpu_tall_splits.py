@@ -1,0 +1,50 @@
+"""GPU tests of the products with many rows that are split over the columns of X when the rows alone do not fill the chip:
+the sketch of Algorithm 1 and the first product of the pre-norm backward, around the sizes where the split count changes."""
+import pytest
+import torch
+
+import __graft_entry__ as entry
+from paper_2509_23472_b200 import binding as B, synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def dev():
+    entry.build()
+    B.lib()
+    return torch.device("cuda:0")
+
+
+@pytest.mark.parametrize("n,d,r", [(64, 2048, 16), (130, 5128, 48), (257, 2056, 16), (1003, 5120, 64), (2500, 8200, 80),
+                                   (4096, 5120, 128), (8192, 2048, 256), (3000, 4096, 336)])
+def test_projection_of_few_rows(dev, n, d, r):
+    sig = torch.exp(-torch.arange(min(2 * r, n), dtype=torch.float64) * 6.0 / r).float()
+    X = synth.low_rank_plus_noise(n, d, min(2 * r, n), sig, 1e-2, n + d, torch.bfloat16, dev)
+    ws = B.alloc_workspace(B.make_desc(X, r), dev)
+    U, V, idx = B.compress(X, r, seed=3, ws=ws)
+    assert B.read_device_status(ws) == 0
+    X64 = X.double()
+    Q = torch.linalg.qr(X64 @ X64[idx.long()].t())[0]
+    want = Q @ (Q.t() @ X64)
+    got = U.double() @ V.double()
+    # two factors rounded to bf16 (sqrt(2) 2^-9 / sqrt(3) of the norm) with the same head-room as the parity tests
+    assert float((got - want).norm() / X64.norm()) <= 2.0 ** -8 + float((X64 - want).norm() / X64.norm()) / 100
+
+
+@pytest.mark.parametrize("n,d,r", [(64, 2048, 16), (1003, 5120, 64), (4096, 4096, 128), (5000, 1000, 32)])
+def test_prenorm_backward_with_a_full_and_a_small_workspace(dev, n, d, r):
+    g = torch.Generator(device=dev)
+    g.manual_seed(n)
+    U = (torch.randn(n, r, generator=g, device=dev) / n ** 0.5).bfloat16()
+    V = torch.randn(r, d, generator=g, device=dev).bfloat16()
+    gA = torch.randn(n, d, generator=g, device=dev).bfloat16()
+    gamma = (1 + 0.1 * torch.randn(d, generator=g, device=dev)).bfloat16()
+    rstd = torch.rand(n, generator=g, device=dev) + 0.5
+    up = lambda v: (v + 255) // 256 * 256
+    small = torch.empty(256 + up(4 * n * r) + 2 * up(4 * n), dtype=torch.uint8, device=dev)   # one partial sum
+    a = B.prenorm_backward(U, V, gamma, rstd, gA)
+    b = B.prenorm_backward(U, V, gamma, rstd, gA, ws=small)
+    assert float((a.double() - b.double()).norm() / b.double().norm()) <= 1e-3   # sums in another order, one rounding
+    with pytest.raises(B.LoractError):
+        B.prenorm_backward(U, V, gamma, rstd, gA, ws=small[:-256])
