@@ -112,8 +112,20 @@ struct Plan {
   int splits_y;   // of the sketch over d
 };
 
-inline int simt_splits(int64_t k) {
-  int64_t s = k / 128;
+// CUDA-core path (32 x 32 tiles, a CTA walks a quarter of K per thread group): splits over K for a product whose partial
+// sums the next kernel adds anyway (Gram matrices), and for one that needs a reduction of its own, which pays only for a
+// long contraction on few tiles.
+inline int64_t simt_tiles(int64_t m, int64_t n) { return ((m + 31) / 32) * ((n + 31) / 32); }
+inline int simt_gram_splits(int64_t l, int64_t k) {
+  int64_t s = (148 + simt_tiles(l, l) - 1) / simt_tiles(l, l);
+  if (s > k / 64) s = k / 64;
+  return s < 1 ? 1 : (s > 8 ? 8 : (int)s);
+}
+constexpr int64_t kSimtCtas = 592;   // four 128-thread CTAs per SM
+inline int simt_splits(int64_t m, int64_t n, int64_t k) {
+  const int64_t tiles = ((m + 63) / 64) * ((n + 63) / 64);
+  int64_t s = (kSimtCtas + tiles - 1) / tiles;
+  if (s > k / 128) s = k / 128;
   return s < 1 ? 1 : (s > 8 ? 8 : (int)s);
 }
 
@@ -129,12 +141,10 @@ Plan make_plan(int64_t n, int64_t d, int l, bool bf16) {
     p.splits_v = gemm_tc_pick_splits(l, (int)d, (int)n, true, true);
     p.splits_y = gemm_tc_pick_tall_splits((int)n, l, (int)d);
   } else {
-    // CUDA-core path: the generic kernel walks K sixteen elements at a time, so a long contraction with few output
-    // tiles is split over K (partial sums, added in a fixed order afterwards)
-    p.splits_gs = simt_splits(d);
-    p.splits_w = simt_splits(n);
-    p.splits_v = simt_splits(n);
-    p.splits_y = simt_splits(d);
+    p.splits_gs = simt_gram_splits(l, d);
+    p.splits_w = simt_gram_splits(l, n);
+    p.splits_v = simt_splits(l, d, n);
+    p.splits_y = simt_splits(n, l, d);
   }
   return p;
 }
@@ -169,7 +179,7 @@ void carve_basis(Carver& c, const Plan& p, BasisWs* w) {
     w->Y32 = (float*)c.take(n * l * 4);
     w->Q32 = (float*)c.take(n * l * 4);
     // partial sums of pass 1 (n x l per split over d) and of pass 2 (l x d per split over the tokens)
-    const size_t p1 = (size_t)simt_splits((int64_t)d) * n * l, p2 = (size_t)p.splits_v * l * d;
+    const size_t p1 = p.splits_y > 1 ? (size_t)p.splits_y * n * l : 0, p2 = p.splits_v > 1 ? (size_t)p.splits_v * l * d : 0;
     w->part32 = (float*)c.take((p1 > p2 ? p1 : p2) * 4);
   }
 }
@@ -191,7 +201,7 @@ cudaError_t gram_rows(const void* S, int l, int64_t d, bool bf16, const BasisWs&
     g.out = OUT_F32; g.C0 = w.gram_partials; g.splits = w.splits_gram_sample;
     g.split_stride = (int64_t)l * l;
   } else {
-    g.out = OUT_F64; g.C0 = w.gram64; g.acc64 = true;
+    g.out = OUT_F64; g.C0 = w.gram64; g.acc64 = true; g.lower_only = true;
     g.splits = w.splits_gram_sample; g.split_stride = (int64_t)l * l;
   }
   return run_gemm(g, status, stream);
@@ -317,7 +327,7 @@ cudaError_t range_basis(const void* X, int64_t ldx, const Plan& p, const void* O
         g.a_type = g.b_type = el;
         g.ldc = l;
         g.terms[0] = {Yc, Yc};
-        g.out = OUT_F64; g.C0 = w.gram64; g.acc64 = true;
+        g.out = OUT_F64; g.C0 = w.gram64; g.acc64 = true; g.lower_only = true;
         g.splits = w.splits_gram; g.split_stride = (int64_t)l * l;
         trace_label(round ? "Gram 2" : "Gram 1");
         LORACT_CUDA_TRY(run_gemm(g, status, stream));
@@ -518,7 +528,7 @@ size_t carve_wgrad(void* ws, const loract_desc_t* desc, int g, WgradWs* out) {
   c.take(256);
   WgradWs w;
   w.splits = desc->dtype == LORACT_BF16 ? gemm_tc_pick_splits(desc->rank, g, (int)desc->n_tokens, true, true)
-                                        : 2 * simt_splits(desc->n_tokens);
+                                        : simt_splits(desc->rank, g, desc->n_tokens);
   w.partials = (float*)c.take((size_t)w.splits * desc->rank * g * 4);
   w.T = (float*)c.take((size_t)desc->rank * g * 4);
   w.g8 = (g + 7) / 8 * 8;
@@ -729,13 +739,16 @@ loract_status_t loract_weight_grad(const loract_desc_t* desc, const void* U, con
     q.out = OUT_F32; q.C0 = dW; q.ldc = g; q.accumulate = accumulate != 0;
     if (e == cudaSuccess && gemm_tc_supported(q)) return from_cuda(gemm_tc_launch(q, status, st));
   }
-  if (e == cudaSuccess)
+  const float* T = w.partials;
+  if (e == cudaSuccess && (w.splits > 1 || el == ELEM_BF16)) {
     e = reduce_partials_launch(w.partials, w.splits, t.split_stride, t.split_stride, w.T, nullptr, st);
+    T = w.T;
+  }
   if (e == cudaSuccess) {
     GemmDesc q;  // dW = V^T T  (d x g)
     q.M = (int)desc->d; q.N = g; q.K = r; q.a_mn = true; q.b_mn = true; q.lda = desc->d; q.ldb = g;
     q.a_type = el; q.b_type = ELEM_F32;
-    q.terms[0] = {V, w.T};
+    q.terms[0] = {V, T};
     q.out = OUT_F32; q.C0 = dW; q.ldc = g; q.accumulate = accumulate != 0;
     e = gemm_simt_launch(q, st);
   }

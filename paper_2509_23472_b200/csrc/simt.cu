@@ -1,5 +1,7 @@
 // CUDA-core kernels: the generic contraction used by the fp32 path and for shapes the tensor-core
 // engine does not take, the fixed-order reduction of split-K partials, and the pre-norm forward.
+#include <algorithm>
+
 #include "common.cuh"
 
 namespace loract {
@@ -27,6 +29,9 @@ struct SimtParams {
   int64_t split_stride;
   int accumulate;
   float alpha;
+  int vec_a, vec_b;   // fp32 tile kernels: the operand is read four elements at a time along its contiguous index
+  int k_per;          // fp32 tile kernels: contraction elements per split
+  int lower_only;     // 32 x 32 tile kernel: tiles above the diagonal are not formed
   int halve_at_term;  // the sum so far is multiplied by 1/2 before this term (0: never)
   const uint32_t* gate;  // 32 x 32 tile kernel: optional device word, zero means the launch does nothing
   // 32 x 32 tile kernel: optional bf16 hi / lo copies of the result, same leading dimension as C0
@@ -271,91 +276,130 @@ __global__ void reduce_split3_kernel(const float* __restrict__ partials, int n_p
   }
 }
 
-// fp32 product for the r x r blocks of the two-level small-block scheme: C = alpha * A B (+ C), all of a few
-// hundred rows and columns.  32 x 32 output tiles, four groups of 64 threads per tile, each group on a quarter of
-// the contraction (4 x 4 outputs per thread, operands read from shared memory along the contraction index with
-// 16-byte loads; the four partial tiles are added in group order), so that a 256 x 256 product spreads over
-// 64 SMs and no thread walks more than a quarter of K; the K loop is double-buffered through registers.  One launch carries up to two independent products
-// (grid.z picks one): the two-level scheme has a pair of them at one point of its chain.
-constexpr int kT32 = 32, kT32Ld = 36;
+// fp32 x fp32 products on CUDA cores: the whole fp32 path, and the r x r blocks of the two-level small-block scheme.
+// C = alpha * A B (+ C), accumulated in fp32, or in fp64 (Gram matrices).  Everything here is small, so what bounds it is
+// latency and the number of SMs at work: 32 x 32 output tiles, four groups of 64 threads per tile, each group on a quarter
+// of the contraction (4 x 4 outputs per thread, operands read from shared memory along the contraction index with 16-byte
+// loads; the four partial tiles are added in group order), the K loop double-buffered through registers.  fp64: operands
+// are converted once, on their way into shared memory.  grid.z: splits over K (partial results), or, with `has_second`, one
+// of two independent products that the two-level scheme has at one point of its chain.
+// (Measured against 64 x 64 tiles with a conversion per use and no dependent launch, whole calls with the same
+// factorisation: 512 x 768, r = 64: 152 -> 100 us; 2000 x 2000, r = 192: 510 -> 324 us.)
+template <typename TAcc> struct Tile32;
+template <> struct Tile32<float> { static constexpr int kKc = 32, kLd = 36, kPartLd = 36; };
+template <> struct Tile32<double> { static constexpr int kKc = 16, kLd = 18, kPartLd = 34; };
+template <typename TAcc> struct Vec16;
+template <> struct Vec16<float> { typedef float4 type; static constexpr int kN = 4; };
+template <> struct Vec16<double> { typedef double2 type; static constexpr int kN = 2; };
+__device__ __forceinline__ float dot16(float4 a, float4 b, float c) {
+  return fmaf(a.w, b.w, fmaf(a.z, b.z, fmaf(a.y, b.y, fmaf(a.x, b.x, c))));
+}
+__device__ __forceinline__ double dot16(double2 a, double2 b, double c) { return fma(a.y, b.y, fma(a.x, b.x, c)); }
 
+constexpr int kT32 = 32;
 constexpr int kT32Groups = 4;   // thread groups of 64 that share one output tile, each on a quarter of the contraction
-__global__ void __launch_bounds__(64 * kT32Groups) gemm_f32_tile32_kernel(SimtParams p0, SimtParams p1) {
+template <typename TAcc>
+__global__ void __launch_bounds__(64 * kT32Groups) gemm_tile32_kernel(SimtParams p0, SimtParams p1, int has_second) {
+  constexpr int kKc = Tile32<TAcc>::kKc, kLd = Tile32<TAcc>::kLd, kPartLd = Tile32<TAcc>::kPartLd;
+  typedef typename Vec16<TAcc>::type V;
+  constexpr int kVn = Vec16<TAcc>::kN;
+  constexpr int kPer = kT32 * kKc / 64;                // elements of either tile a thread stages per K chunk
   // per group: As [m][k] and Bs [n][k]; after the K loop the same memory carries the partial tiles of groups 1..3
-  __shared__ __align__(16) float tiles[kT32Groups][2][kT32 * kT32Ld];
-  const SimtParams& p = blockIdx.z ? p1 : p0;
+  __shared__ __align__(16) TAcc tiles[kT32Groups][2 * kT32 * kLd];
+  const SimtParams& p = has_second && blockIdx.z ? p1 : p0;
+  const int split = has_second ? 0 : (int)blockIdx.z;
   const int grp = threadIdx.x >> 6, tid = threadIdx.x & 63;
-  float* As = tiles[grp][0];
-  float* Bs = tiles[grp][1];
+  TAcc* As = tiles[grp];
+  TAcc* Bs = tiles[grp] + kT32 * kLd;
   const int m0 = blockIdx.y * kT32, n0 = blockIdx.x * kT32;
   pdl_wait();
   pdl_launch_dependents();
   if (p.gate != nullptr && *(const volatile uint32_t*)p.gate == 0u) return;
-  if (m0 >= p.M || n0 >= p.N) return;
+  if (m0 >= p.M || n0 >= p.N || (p.lower_only && n0 > m0)) return;
   const int tm = tid >> 3, tn = tid & 7;               // outputs (4 tm + i, tn + 8 j)
   const float* A = (const float*)p.A[0];
   const float* B = (const float*)p.B[0];
-  // this group's share of the contraction: whole chunks of 32, the same number of chunks in every group
-  const int chunks = ((p.K + kT32 - 1) / kT32 + kT32Groups - 1) / kT32Groups;
-  const int k_begin = grp * chunks * kT32;
-  const int k_end = min(p.K, k_begin + chunks * kT32);
-  float acc[4][4];
+  // this split's share of the contraction, and this group's: whole chunks, the same number of chunks in every group
+  const int k_lo = split * p.k_per, k_hi = min(p.K, k_lo + p.k_per);
+  const int chunks = (max(k_hi - k_lo, 0) + kKc * kT32Groups - 1) / (kKc * kT32Groups);
+  const int k_begin = k_lo + grp * chunks * kKc;
+  const int k_end = min(k_hi, k_begin + chunks * kKc);
+  TAcc acc[4][4];
 #pragma unroll
   for (int i = 0; i < 4; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
-  // each thread stages 16 elements of either tile per K chunk; the faster-varying index follows memory
-  float ra[16], rb[16];
+    for (int j = 0; j < 4; ++j) acc[i][j] = (TAcc)0;
+  // A thread stages kPer elements of either tile, in quads along the operand's contiguous index.  (One element at a time
+  // the address arithmetic and the load instructions took longer than the products.)
+  constexpr int kQuads = kPer / 4;
+  float4 ra[kQuads], rb[kQuads];
+  auto place = [&](int u, bool k_fast, int& mn, int& kk) {
+    const int e = tid + 64 * u;
+    if (k_fast) { kk = 4 * (e % (kKc / 4)); mn = e / (kKc / 4); } else { mn = 4 * (e % (kT32 / 4)); kk = e / (kT32 / 4); }
+  };
+  auto fetch_one = [&](const float* P, int64_t s_mn, int64_t s_k, bool vec, int mn, int k, int mn_end) {
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    const float* src = P + (int64_t)mn * s_mn + (int64_t)k * s_k;
+    if (vec) {                                           // the extent along the quad is a multiple of four
+      if (mn < mn_end && k < k_end) v = __ldg(reinterpret_cast<const float4*>(src));
+    } else if (s_k == 1) {
+      if (mn < mn_end) {
+        if (k < k_end) v.x = src[0];
+        if (k + 1 < k_end) v.y = src[1];
+        if (k + 2 < k_end) v.z = src[2];
+        if (k + 3 < k_end) v.w = src[3];
+      }
+    } else if (k < k_end) {
+      if (mn < mn_end) v.x = src[0];
+      if (mn + 1 < mn_end) v.y = src[1];
+      if (mn + 2 < mn_end) v.z = src[2];
+      if (mn + 3 < mn_end) v.w = src[3];
+    }
+    return v;
+  };
   auto fetch = [&](int k0) {
 #pragma unroll
-    for (int u = 0; u < 16; ++u) {
-      const int e = tid + 64 * u;
-      int mm, kk;
-      if (p.sak == 1) { kk = e & 31; mm = e >> 5; } else { mm = e & 31; kk = e >> 5; }
-      const int m = m0 + mm, k = k0 + kk;
-      ra[u] = (m < p.M && k < k_end) ? A[m * p.sam + k * p.sak] : 0.f;
-      int nn, kb;
-      if (p.sbk == 1) { kb = e & 31; nn = e >> 5; } else { nn = e & 31; kb = e >> 5; }
-      const int n = n0 + nn, k2 = k0 + kb;
-      rb[u] = (n < p.N && k2 < k_end) ? B[k2 * p.sbk + n * p.sbn] : 0.f;
+    for (int u = 0; u < kQuads; ++u) {
+      int mn, kk;
+      place(u, p.sak == 1, mn, kk);
+      ra[u] = fetch_one(A, p.sam, p.sak, p.vec_a, m0 + mn, k0 + kk, p.M);
+      place(u, p.sbk == 1, mn, kk);
+      rb[u] = fetch_one(B, p.sbn, p.sbk, p.vec_b, n0 + mn, k0 + kk, p.N);
     }
+  };
+  auto put = [&](TAcc* T, float4 v, bool k_fast, int mn, int kk) {
+    const int step = k_fast ? 1 : kLd;
+    TAcc* t = T + mn * kLd + kk;
+    t[0] = (TAcc)v.x; t[step] = (TAcc)v.y; t[2 * step] = (TAcc)v.z; t[3 * step] = (TAcc)v.w;
   };
   auto stash = [&]() {
 #pragma unroll
-    for (int u = 0; u < 16; ++u) {
-      const int e = tid + 64 * u;
-      int mm, kk;
-      if (p.sak == 1) { kk = e & 31; mm = e >> 5; } else { mm = e & 31; kk = e >> 5; }
-      As[mm * kT32Ld + kk] = ra[u];
-      int nn, kb;
-      if (p.sbk == 1) { kb = e & 31; nn = e >> 5; } else { nn = e & 31; kb = e >> 5; }
-      Bs[nn * kT32Ld + kb] = rb[u];
+    for (int u = 0; u < kQuads; ++u) {
+      int mn, kk;
+      place(u, p.sak == 1, mn, kk);
+      put(As, ra[u], p.sak == 1, mn, kk);
+      place(u, p.sbk == 1, mn, kk);
+      put(Bs, rb[u], p.sbk == 1, mn, kk);
     }
   };
   auto group_barrier = [&]() { asm volatile("bar.sync %0, 64;" ::"r"(grp + 1) : "memory"); };
-  fetch(k_begin);
+  if (chunks > 0) fetch(k_begin);
   for (int c = 0; c < chunks; ++c) {
-    const int k0 = k_begin + c * kT32;
     group_barrier();
     stash();
     group_barrier();
-    if (c + 1 < chunks) fetch(k0 + kT32);
+    if (c + 1 < chunks) fetch(k_begin + (c + 1) * kKc);
 #pragma unroll
-    for (int q4 = 0; q4 < kT32 / 4; ++q4) {
-      float4 a[4], b[4];
+    for (int q = 0; q < kKc / kVn; ++q) {
+      V a[4], b[4];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = *reinterpret_cast<const float4*>(As + (4 * tm + i) * kT32Ld + 4 * q4);
+      for (int i = 0; i < 4; ++i) a[i] = *reinterpret_cast<const V*>(As + (4 * tm + i) * kLd + kVn * q);
 #pragma unroll
-      for (int j = 0; j < 4; ++j) b[j] = *reinterpret_cast<const float4*>(Bs + (tn + 8 * j) * kT32Ld + 4 * q4);
+      for (int j = 0; j < 4; ++j) b[j] = *reinterpret_cast<const V*>(Bs + (tn + 8 * j) * kLd + kVn * q);
 #pragma unroll
       for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          acc[i][j] = fmaf(a[i].x, b[j].x, acc[i][j]);
-          acc[i][j] = fmaf(a[i].y, b[j].y, acc[i][j]);
-          acc[i][j] = fmaf(a[i].z, b[j].z, acc[i][j]);
-          acc[i][j] = fmaf(a[i].w, b[j].w, acc[i][j]);
-        }
+        for (int j = 0; j < 4; ++j) acc[i][j] = dot16(a[i], b[j], acc[i][j]);
     }
   }
   // the quarters of the contraction meet in shared memory and are added in group order
@@ -364,7 +408,7 @@ __global__ void __launch_bounds__(64 * kT32Groups) gemm_f32_tile32_kernel(SimtPa
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
-      for (int j = 0; j < 4; ++j) As[(4 * tm + i) * kT32Ld + tn + 8 * j] = acc[i][j];
+      for (int j = 0; j < 4; ++j) As[(4 * tm + i) * kPartLd + tn + 8 * j] = acc[i][j];
   }
   __syncthreads();
   if (grp > 0) return;
@@ -376,18 +420,102 @@ __global__ void __launch_bounds__(64 * kT32Groups) gemm_f32_tile32_kernel(SimtPa
     for (int j = 0; j < 4; ++j) {
       const int n = n0 + tn + 8 * j;
       if (n >= p.N) continue;
-      float sum = acc[i][j];
+      TAcc sum = acc[i][j];
 #pragma unroll
-      for (int g2 = 1; g2 < kT32Groups; ++g2) sum += tiles[g2][0][(4 * tm + i) * kT32Ld + tn + 8 * j];
-      float* c = (float*)p.C0 + (int64_t)m * p.ldc + n;
-      const float v0 = sum * p.alpha;
-      const float v = p.accumulate ? (*c + v0) : v0;
+      for (int g2 = 1; g2 < kT32Groups; ++g2) sum += tiles[g2][(4 * tm + i) * kPartLd + tn + 8 * j];
+      const int64_t off = (int64_t)split * p.split_stride + (int64_t)m * p.ldc + n;
+      const TAcc v0 = sum * (TAcc)p.alpha;
+      if (p.out == OUT_F64) { ((double*)p.C0)[off] = (double)v0; continue; }
+      float* c = (float*)p.C0 + off;
+      const float v = p.accumulate ? (*c + (float)v0) : (float)v0;
       *c = v;
       if (p.split_hi) {
         const __nv_bfloat16 h = __float2bfloat16(v);
         p.split_hi[(int64_t)m * p.ldc + n] = h;
         if (p.split_lo) p.split_lo[(int64_t)m * p.ldc + n] = __float2bfloat16(v - __bfloat162float(h));
       }
+    }
+  }
+}
+
+// The same products where 64 x 64 tiles fill the chip: 128 threads, 8 x 4 outputs each, both tiles in shared memory with
+// the output index contiguous (two 16-byte loads of A, one of B per 32 FMAs: the shared-memory and the FMA pipe are about
+// even), two buffers, the next chunk of 16 on its way in registers.
+constexpr int kT64 = 64, kT64K = 16, kT64Ld = 68;
+__global__ void __launch_bounds__(128) gemm_tile64_kernel(SimtParams p) {
+  __shared__ __align__(16) float As[2][kT64K * kT64Ld], Bs[2][kT64K * kT64Ld];
+  const int tid = threadIdx.x, tm = tid >> 4, tn = tid & 15;   // rows 8 tm + i, columns 4 tn + j
+  const int m0 = blockIdx.y * kT64, n0 = blockIdx.x * kT64, split = blockIdx.z;
+  pdl_wait();
+  pdl_launch_dependents();
+  const float* A = (const float*)p.A[0];
+  const float* B = (const float*)p.B[0];
+  const int k_lo = split * p.k_per, k_hi = min(p.K, k_lo + p.k_per);
+  const int chunks = (max(k_hi - k_lo, 0) + kT64K - 1) / kT64K;
+  float acc[8][4];
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
+  float4 ra[2], rb[2];
+  // quads: along k (four per row, rows tid / 4 and + 32) or along the output index (sixteen per k, k tid / 16 and + 8)
+  auto fetch_one = [&](const float* P, int64_t s_mn, int64_t s_k, int mn0, int mn_end, int k0, int u) {
+    int mn, k;
+    if (s_k == 1) { mn = mn0 + (tid >> 2) + 32 * u; k = k0 + 4 * (tid & 3); }
+    else { mn = mn0 + 4 * (tid & 15); k = k0 + (tid >> 4) + 8 * u; }
+    if (mn < mn_end && k < k_hi) return __ldg(reinterpret_cast<const float4*>(P + (int64_t)mn * s_mn + (int64_t)k * s_k));
+    return make_float4(0.f, 0.f, 0.f, 0.f);
+  };
+  auto put = [&](float* T, float4 v, int64_t s_k, int u) {
+    if (s_k == 1) {
+      float* t = T + 4 * (tid & 3) * kT64Ld + (tid >> 2) + 32 * u;
+      t[0] = v.x; t[kT64Ld] = v.y; t[2 * kT64Ld] = v.z; t[3 * kT64Ld] = v.w;
+    } else {
+      *reinterpret_cast<float4*>(T + ((tid >> 4) + 8 * u) * kT64Ld + 4 * (tid & 15)) = v;
+    }
+  };
+  auto fetch = [&](int k0) {
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      ra[u] = fetch_one(A, p.sam, p.sak, m0, p.M, k0, u);
+      rb[u] = fetch_one(B, p.sbn, p.sbk, n0, p.N, k0, u);
+    }
+  };
+  auto stash = [&](int buf) {
+#pragma unroll
+    for (int u = 0; u < 2; ++u) { put(As[buf], ra[u], p.sak, u); put(Bs[buf], rb[u], p.sbk, u); }
+  };
+  if (chunks > 0) { fetch(k_lo); stash(0); }
+  __syncthreads();
+  for (int c = 0; c < chunks; ++c) {
+    if (c + 1 < chunks) fetch(k_lo + (c + 1) * kT64K);
+    const float* as = As[c & 1] + 8 * tm;
+    const float* bs = Bs[c & 1] + 4 * tn;
+#pragma unroll
+    for (int kk = 0; kk < kT64K; ++kk) {
+      const float4 a0 = *reinterpret_cast<const float4*>(as + kk * kT64Ld), a1 = *reinterpret_cast<const float4*>(as + kk * kT64Ld + 4);
+      const float4 b = *reinterpret_cast<const float4*>(bs + kk * kT64Ld);
+      const float av[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w}, bv[4] = {b.x, b.y, b.z, b.w};
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(av[i], bv[j], acc[i][j]);
+    }
+    if (c + 1 < chunks) stash((c + 1) & 1);
+    __syncthreads();
+  }
+  const bool vec_c = p.ldc % 4 == 0 && p.split_stride % 4 == 0 && p.N % 4 == 0 && ((uintptr_t)p.C0 & 15) == 0;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const int m = m0 + 8 * tm + i, n = n0 + 4 * tn;
+    if (m >= p.M || n >= p.N) continue;
+    float* c = (float*)p.C0 + (int64_t)split * p.split_stride + (int64_t)m * p.ldc + n;
+    if (vec_c && !p.accumulate) {
+      *reinterpret_cast<float4*>(c) = make_float4(acc[i][0] * p.alpha, acc[i][1] * p.alpha, acc[i][2] * p.alpha, acc[i][3] * p.alpha);
+    } else {
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        if (n + j < p.N) c[j] = p.accumulate ? c[j] + acc[i][j] * p.alpha : acc[i][j] * p.alpha;
     }
   }
 }
@@ -741,8 +869,62 @@ __global__ void copy_bf16_gated_kernel(const uint4* __restrict__ src, uint4* __r
 
 }  // namespace
 
+constexpr int kT64MinTiles = 64;
+// The products the 32 x 32 tile kernel takes: fp32 operands, one term, fp32 or fp64 result.
+static bool tile32_params(const GemmDesc& g, SimtParams& p) {
+  if (g.a_type != ELEM_F32 || g.b_type != ELEM_F32 || g.n_terms != 1) return false;
+  if (!(g.out == OUT_F32 || (g.out == OUT_F64 && !g.accumulate))) return false;
+  if (g.splits > 1 && (g.accumulate || g.split_hi)) return false;
+  p = SimtParams{};
+  p.M = g.M; p.N = g.N; p.K = g.K;
+  if (g.a_mn) { p.sam = 1; p.sak = g.lda; } else { p.sam = g.lda; p.sak = 1; }
+  if (g.b_mn) { p.sbn = 1; p.sbk = g.ldb; } else { p.sbn = g.ldb; p.sbk = 1; }
+  p.n_terms = 1;
+  p.A[0] = g.terms[0].A; p.B[0] = g.terms[0].B;
+  p.out = g.out; p.C0 = g.C0; p.ldc = g.ldc;
+  p.splits = g.splits < 1 ? 1 : g.splits;
+  p.split_stride = g.split_stride;
+  p.accumulate = g.accumulate ? 1 : 0;
+  p.alpha = g.alpha;
+  p.gate = g.gate;
+  p.lower_only = g.lower_only ? 1 : 0;
+  p.split_hi = (__nv_bfloat16*)g.split_hi;
+  p.split_lo = (__nv_bfloat16*)g.split_lo;
+  p.k_per = ((p.K + p.splits - 1) / p.splits + 3) / 4 * 4;
+  auto vec = [&](const void* P, bool mn_major, int64_t ld, int extent) {
+    return (((uintptr_t)P & 15) == 0 && ld % 4 == 0 && (mn_major ? extent : g.K) % 4 == 0) ? 1 : 0;
+  };
+  p.vec_a = vec(g.terms[0].A, g.a_mn, g.lda, g.M);
+  p.vec_b = vec(g.terms[0].B, g.b_mn, g.ldb, g.N);
+  return true;
+}
+
+static cudaError_t tile32_launch(const SimtParams& p0, const SimtParams* second, bool acc64, cudaStream_t stream) {
+  const SimtParams& p1 = second ? *second : p0;
+  dim3 grid((std::max(p0.N, p1.N) + kT32 - 1) / kT32, (std::max(p0.M, p1.M) + kT32 - 1) / kT32, second ? 2 : p0.splits);
+  if (grid.y > 65535) return cudaErrorNotSupported;
+  LORACT_CUDA_TRY(launch_pdl(acc64 ? gemm_tile32_kernel<double> : gemm_tile32_kernel<float>, grid, dim3(64 * kT32Groups), 0,
+                             stream, p0, p1, second ? 1 : 0));
+  count_launch(__func__, stream);
+  return cudaGetLastError();
+}
+
 cudaError_t gemm_simt_launch(const GemmDesc& g, cudaStream_t stream) {
-  SimtParams p;
+  SimtParams p = {};
+  if (g.M <= 65535 * kT32 && tile32_params(g, p)) {
+    // 64 x 64 tiles from 64 of them on; below that the smaller tiles with the contraction in quarters reach more SMs
+    // (whole call, 512 x 768, r = 64: 100 us against 106; 999 x 376, r = 16: 87 against 97; above, the larger tiles read
+    // each operand half as often: 1500 x 600, r = 96: 149 against 159)
+    const long long tiles = (long long)((g.M + kT64 - 1) / kT64) * ((g.N + kT64 - 1) / kT64) * p.splits;
+    if (!g.acc64 && g.out == OUT_F32 && !g.gate && !g.split_hi && !g.lower_only && p.vec_a && p.vec_b && tiles >= kT64MinTiles) {
+      LORACT_CUDA_TRY(launch_pdl(gemm_tile64_kernel, dim3((g.N + kT64 - 1) / kT64, (g.M + kT64 - 1) / kT64, p.splits),
+                                 dim3(128), 0, stream, p));
+      count_launch(__func__, stream);
+      return cudaGetLastError();
+    }
+    return tile32_launch(p, nullptr, g.acc64, stream);
+  }
+  p = SimtParams{};
   p.M = g.M; p.N = g.N; p.K = g.K;
   if (g.a_mn) { p.sam = 1; p.sak = g.lda; } else { p.sam = g.lda; p.sak = 1; }
   if (g.b_mn) { p.sbn = 1; p.sbk = g.ldb; } else { p.sbn = g.ldb; p.sbk = 1; }
@@ -868,33 +1050,12 @@ cudaError_t reduce_split3_launch(const float* partials, int n_partials, int64_t 
 }
 
 cudaError_t gemm_f32_small_launch(const GemmDesc& g, cudaStream_t stream, const GemmDesc* second) {
-  auto fill = [](const GemmDesc& g, SimtParams& p) {
-    // (the gate of the first product holds for the whole launch)
-    if (g.a_type != ELEM_F32 || g.b_type != ELEM_F32 || g.out != OUT_F32 || g.n_terms != 1 || g.splits > 1)
-      return false;
-    p = SimtParams{};
-    p.M = g.M; p.N = g.N; p.K = g.K;
-    if (g.a_mn) { p.sam = 1; p.sak = g.lda; } else { p.sam = g.lda; p.sak = 1; }
-    if (g.b_mn) { p.sbn = 1; p.sbk = g.ldb; } else { p.sbn = g.ldb; p.sbk = 1; }
-    p.n_terms = 1;
-    p.A[0] = g.terms[0].A; p.B[0] = g.terms[0].B;
-    p.out = g.out; p.C0 = g.C0; p.ldc = g.ldc; p.splits = 1;
-    p.accumulate = g.accumulate ? 1 : 0;
-    p.alpha = g.alpha;
-    p.gate = nullptr;
-    p.split_hi = (__nv_bfloat16*)g.split_hi;
-    p.split_lo = (__nv_bfloat16*)g.split_lo;
-    return true;
-  };
+  // (the gate of the first product holds for the whole launch)
   SimtParams p0, p1;
-  if (!fill(g, p0) || (second && !fill(*second, p1))) return cudaErrorNotSupported;
-  if (!second) p1 = p0;
-  p0.gate = p1.gate = g.gate;
-  const int M = second ? std::max(g.M, second->M) : g.M, N = second ? std::max(g.N, second->N) : g.N;
-  dim3 grid((N + kT32 - 1) / kT32, (M + kT32 - 1) / kT32, second ? 2 : 1);
-  LORACT_CUDA_TRY(launch_pdl(gemm_f32_tile32_kernel, grid, dim3(64 * kT32Groups), 0, stream, p0, p1));
-  count_launch(__func__, stream);
-  return cudaGetLastError();
+  if (g.splits > 1 || !tile32_params(g, p0) || (second && (second->splits > 1 || !tile32_params(*second, p1))))
+    return cudaErrorNotSupported;
+  if (second) p1.gate = g.gate;
+  return tile32_launch(p0, second ? &p1 : nullptr, false, stream);
 }
 
 cudaError_t split_block_launch(const float* src, int rows, int cols, int64_t ld, __nv_bfloat16* hi,

@@ -108,7 +108,7 @@ small_block_kernel(SBParams p) {
     for (int64_t e = (int64_t)cta * kSBThreads + tid; e < total; e += (int64_t)n_cta * kSBThreads) {
       const int i = (int)(e / r), j = (int)(e - (int64_t)i * r);
       if (j > i) continue;
-      T v = (T)0.5 * (read_partial_sum<T>(p, i, j) + read_partial_sum<T>(p, j, i));
+      T v = read_partial_sum<T>(p, i, j);                     // (of a symmetric matrix: the lower triangle is enough)
       if (i == j) v += shift;
       W[e] = v;
     }

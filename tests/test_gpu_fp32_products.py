@@ -1,0 +1,59 @@
+"""GPU tests of the CUDA-core fp32 products (32 x 32 tiles, a quarter of the contraction per thread group): remainders in
+every extent, both operand majors, partial results, fp32 and fp64 accumulation; and of the fp32 path over its sizes."""
+import pytest
+import torch
+
+import __graft_entry__ as entry
+from paper_2509_23472_b200 import binding as B, synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def dev():
+    entry.build()
+    B.lib()
+    return torch.device("cuda:0")
+
+
+@pytest.mark.parametrize("m,n,k,splits", [(1, 1, 1, 1), (31, 33, 15, 1), (32, 32, 64, 1), (65, 16, 127, 1), (64, 100, 128, 3),
+                                          (40, 24, 129, 2), (96, 96, 1000, 8), (7, 200, 513, 5), (33, 31, 2, 3)])
+@pytest.mark.parametrize("a_mn,b_mn", [(False, False), (True, False), (False, True), (True, True)])
+@pytest.mark.parametrize("acc64", [False, True])
+def test_product(dev, m, n, k, splits, a_mn, b_mn, acc64):
+    g = torch.Generator(device=dev)
+    g.manual_seed(m * 1000 + n * 10 + k)
+    A = torch.randn(m, k, generator=g, device=dev)
+    Bt = torch.randn(n, k, generator=g, device=dev)
+    a = A.t().contiguous() if a_mn else A
+    b = Bt.t().contiguous() if b_mn else Bt
+    C = B.debug_gemm([a], [b], m, n, k, a_mn, b_mn, out_mode=B.OUT_F64 if acc64 else B.OUT_F32, engine=0, splits=splits,
+                     acc64=acc64)
+    got = C.double().sum(0) if splits > 1 else C.double()
+    want = A.double() @ Bt.double().t()
+    scale = A.double().abs() @ Bt.double().abs().t()
+    eps = 2.0 ** -53 if acc64 else 2.0 ** -24          # k rounded additions of exact (fp64) or rounded products
+    assert float(((got - want).abs() / scale).max()) <= (k + 4) * eps
+
+
+@pytest.mark.parametrize("n,d,r,g", [(64, 64, 16, 1), (999, 376, 16, 38), (384, 260, 112, 9), (2000, 2048, 192, 128),
+                                     (1243, 976, 176, 18), (700, 900, 208, 5), (6000, 128, 48, 3)])
+def test_fp32_path(dev, n, d, r, g):
+    sig = torch.exp(-torch.arange(min(2 * r, n, d), dtype=torch.float64) * 5.0 / (2 * r)).float()
+    X = synth.low_rank_plus_noise(n, d, sig.numel(), sig, 1e-3, n + d, torch.float32, dev)
+    gen = torch.Generator(device=dev)
+    gen.manual_seed(1)
+    G = torch.randn(n, (g + 3) // 4 * 4, generator=gen, device=dev)[:, :g]
+    ws = B.alloc_workspace(B.make_desc(X, r), dev)
+    U, V, idx = B.compress(X, r, seed=5, ws=ws)
+    assert B.read_device_status(ws) == 0
+    dW = B.weight_grad(U, V, G, ws=ws)
+    X64 = X.double()
+    Q = torch.linalg.qr(X64 @ X64[idx.long()].t())[0]
+    want = Q @ (Q.t() @ X64)
+    got = U.double() @ V.double()
+    assert float((got - want).norm() / X64.norm()) <= 5e-6 + float((X64 - want).norm() / X64.norm()) / 100
+    assert float((U.double().t() @ U.double() - torch.eye(r, device=dev, dtype=torch.float64)).abs().max()) <= 1e-5
+    ref = V.double().t() @ (U.double().t() @ G.double())
+    assert float((dW.double() - ref).norm() / ref.norm()) <= 1e-5
+    assert float((B.reconstruct(U, V).double() - got).norm() / got.norm()) <= 1e-6
