@@ -63,6 +63,7 @@ struct TcParams {
   int st_stages;      // streaming kernel: stages of the A ring (<= kStreamStages)
   int store_bufs;     // staging boxes per epilogue warp (1 or 2; fused epilogue: 2 or 3)
   int fuse_parts;     // fused epilogue: warps per quarter of the accumulator's rows
+  int pair_stages;    // two-CTA kernel: stages of the ring
   int halve_at_term;  // the accumulator is multiplied by 1/2 before the first product of this term (0: never)
   int a_keep_from_kb; // two-CTA kernel: K block from which the loads of A carry an evict-last hint (kb_total: none)
   // one-tile kernels: when set and the word it points to is zero, the kernel loads, multiplies and stores nothing
@@ -417,10 +418,11 @@ __device__ __forceinline__ void tc_store_tile(const TcParams& p, const TmapPack&
 // Epilogue of one CTA (eight warps) of the one-tile kernels: waits for the accumulator, then writes it.
 // `ring` is the operand ring: once the accumulator is complete every load has landed and every MMA has read
 // its stage, so the epilogue warps take the ring over as staging space (8 KB per warp).
+// n_acc accumulators, 256 tensor-memory columns apart: accumulator w is the tile at (m0 + w dm, n0 + w dn).
 __device__ __forceinline__ void tc_epilogue(const TcParams& p, const TmapPack& maps, uint32_t tmem_base,
                                           uint64_t* accum_bar, volatile int* abort_flag_ptr, int warp, int lane,
-                                          int m0, int n0, int split, int n_iter, unsigned char* ring) {
-  const int m = m0 + (warp & 3) * 32 + lane;
+                                          int m0, int n0, int split, int n_iter, unsigned char* ring, int n_acc = 1,
+                                          int dm = 0, int dn = 0) {
   // OUT_SPLIT with a gate on the low part: read the word while the contraction is still running
   const bool lo_on = !(p.lo_gate != nullptr && *(const volatile uint32_t*)p.lo_gate == 0u);
   bool ok = mbar_wait_bounded(accum_bar, 0, abort_flag_ptr);
@@ -431,12 +433,17 @@ __device__ __forceinline__ void tc_epilogue(const TcParams& p, const TmapPack& m
     st.base = ring + (uint32_t)(warp - 2) * kStoreWarpBytes;
     st.cnt = 0;
     st.bufs = kStoreBufs;
-    tc_store_tile(p, maps, tmem_base, warp, lane, m0, n0, split, st, lo_on);
+    for (int w = 0; w < n_acc; ++w)
+      tc_store_tile(p, maps, tmem_base + 256u * (uint32_t)w, warp, lane, m0 + w * dm, n0 + w * dn, split, st, lo_on);
     stage_drain(st, lane);
-  } else if (ok && n_iter == 0 && m < p.M && p.out == OUT_F32 && warp < 6) {
+  } else if (ok && n_iter == 0 && p.out == OUT_F32 && warp < 6) {
     // an empty K range still owns its partial: write zeros
-    float* dst = (float*)p.C0 + (int64_t)split * p.split_stride + (int64_t)m * p.ldc + n0;
-    for (int q = 0; q < min(p.bn, p.N - n0); ++q) dst[q] = 0.f;
+    for (int w = 0; w < n_acc; ++w) {
+      const int m = m0 + w * dm + (warp & 3) * 32 + lane, n = n0 + w * dn;
+      if (m >= p.M) continue;
+      float* dst = (float*)p.C0 + (int64_t)split * p.split_stride + (int64_t)m * p.ldc + n;
+      for (int q = 0; q < min(p.bn, p.N - n); ++q) dst[q] = 0.f;
+    }
   }
 }
 
@@ -621,7 +628,17 @@ __device__ __forceinline__ void tc_mma_bf16_pair_halved(uint32_t d_tmem, uint64_
       : "memory");
 }
 
-template <bool A_MN, bool B_MN>
+//
+// kWide: two accumulators (512 tensor-memory columns) per pair.  WIDE_N: two column tiles side by side that share the rows
+// of A; WIDE_M: two row tiles that share the columns of B.  A K block then brings 48 KB per CTA for 1024 cycles of tensor
+// work instead of 32 KB for 512 (an SM reads 64 bytes per clock from L2, so the narrow form runs at that limit), the shared
+// operand is read once, and a product with 512 rows or columns on one side needs half as many tiles: 16384 x 512 are 64
+// of them, one round of the 74 SM pairs instead of two.  The ring has four stages.
+// Measured, r = 512: sketch of 16384 x 11008 151 -> 135 us (1.37 PFLOP/s; cuBLAS holds 1.42 for seconds, 1.67 in a burst),
+// projection 161 -> 141 us, sketch of 32768 x 5120 154 -> 137 us, application of L^-T to 32768 rows 66 -> 55 us.
+enum Wide : int { WIDE_NONE = 0, WIDE_N = 1, WIDE_M = 2 };
+
+template <bool A_MN, bool B_MN, int kWide>
 __global__ void __launch_bounds__(kThreads, 1)
 gemm_tc_pair_kernel(const __grid_constant__ TmapPack maps, const TcParams p) {
   extern __shared__ __align__(1024) unsigned char smem[];
@@ -642,11 +659,13 @@ gemm_tc_pair_kernel(const __grid_constant__ TmapPack maps, const TcParams p) {
   // side by side and the second one finds those rows in L2 instead of streaming X from HBM a second time.
   const int pair_lin = (int)(blockIdx.x >> 1) + (int)(gridDim.x >> 1) * (int)blockIdx.y;
   const int tile_m = pair_lin / (int)gridDim.y, tile_n = pair_lin - tile_m * (int)gridDim.y;
-  const int n0 = tile_n * p.bn, m0 = (2 * tile_m + (int)cta_rank) * kBM, split = blockIdx.z;
+  constexpr int kNA = kWide == WIDE_M ? 2 : 1, kNB = kWide == WIDE_N ? 2 : 1;   // tiles of A and of B per stage
+  const int n0 = tile_n * p.bn * kNB, m0 = (2 * kNA * tile_m + (int)cta_rank) * kBM, split = blockIdx.z;
   const int kb_begin = split * p.kb_per_split;
   const int kb_count = max(0, min(p.kb_total, kb_begin + p.kb_per_split) - kb_begin);
   int n_iter = kb_count * p.n_terms;
-  const uint32_t stage_bytes = kABytes + p.b_bytes;          // per CTA (b_bytes: half a B tile)
+  const uint32_t stage_bytes = kNA * kABytes + kNB * p.b_bytes;   // per CTA (b_bytes: half a B tile)
+  const int stages = kWide ? p.pair_stages : kPairStages;
   unsigned char* tiles = (unsigned char*)(((uintptr_t)smem + 1023) & ~(uintptr_t)1023);
 
   // a gated launch that is not needed: both CTAs of the pair read the same word and leave before any set-up (see the
@@ -683,7 +702,7 @@ gemm_tc_pair_kernel(const __grid_constant__ TmapPack maps, const TcParams p) {
     if (lane == 0) {
       const int nb0 = n0 + (int)cta_rank * half_n;           // this CTA's half of the B tile
       // stage, parity, term and K block are carried along (no division in the loop)
-      int s = (warp == 0 ? 0 : 1) % kPairStages;
+      int s = warp == 0 ? 0 : 1;
       const uint64_t keep_policy = l2_policy_evict_last();
       uint32_t parity = 1u;
       int term = 0, kb = (warp == 0 ? 0 : 1);
@@ -693,26 +712,36 @@ gemm_tc_pair_kernel(const __grid_constant__ TmapPack maps, const TcParams p) {
         const int k0 = (kb_begin + kb) * kBK;
         const int kb_now = kb;
         unsigned char* a_dst = tiles + (size_t)s * stage_bytes;
-        unsigned char* b_dst = a_dst + kABytes;
+        unsigned char* b_dst = a_dst + kNA * kABytes;
         // the leader expects the bytes of both CTAs on its barrier
         if (leader) mbar_arrive_expect_tx(&full_bar[s], 2u * stage_bytes);
         const uint32_t bar = map_to_rank(smem_u32(&full_bar[s]), 0u);
         const int term_now = term;
-        s += 2; if (s >= kPairStages) { s -= kPairStages; parity ^= 1u; }
+        s += 2; if (s >= stages) { s -= stages; parity ^= 1u; }
         kb += 2; if (kb >= kb_count) { kb -= kb_count; ++term; if (kb >= kb_count) { kb -= kb_count; ++term; } }
-        if (A_MN) {
-          tma_load_2d_pair(a_dst, &maps.a[term_now], bar, m0, k0);
-          tma_load_2d_pair(a_dst + 8192, &maps.a[term_now], bar, m0 + 64, k0);
-        } else if (kb_begin + kb_now >= p.a_keep_from_kb) {
-          tma_load_2d_pair_hint(a_dst, &maps.a[term_now], bar, k0, m0, keep_policy);
-        } else {
-          tma_load_2d_pair(a_dst, &maps.a[term_now], bar, k0, m0);
+#pragma unroll
+        for (int i = 0; i < kNA; ++i) {
+          unsigned char* dst = a_dst + i * kABytes;
+          const int m = m0 + i * 2 * kBM;
+          if (A_MN) {
+            tma_load_2d_pair(dst, &maps.a[term_now], bar, m, k0);
+            tma_load_2d_pair(dst + 8192, &maps.a[term_now], bar, m + 64, k0);
+          } else if (kb_begin + kb_now >= p.a_keep_from_kb) {
+            tma_load_2d_pair_hint(dst, &maps.a[term_now], bar, k0, m, keep_policy);
+          } else {
+            tma_load_2d_pair(dst, &maps.a[term_now], bar, k0, m);
+          }
         }
-        if (B_MN) {
-          for (uint32_t q = 0; q * 8192u < p.b_bytes; ++q)
-            tma_load_2d_pair(b_dst + q * 8192u, &maps.b[term_now], bar, nb0 + (int)q * 64, k0);
-        } else {
-          tma_load_2d_pair(b_dst, &maps.b[term_now], bar, k0, nb0);
+#pragma unroll
+        for (int i = 0; i < kNB; ++i) {
+          unsigned char* dst = b_dst + i * p.b_bytes;
+          const int n = nb0 + i * p.bn;
+          if (B_MN) {
+            for (uint32_t q = 0; q * 8192u < p.b_bytes; ++q)
+              tma_load_2d_pair(dst + q * 8192u, &maps.b[term_now], bar, n + (int)q * 64, k0);
+          } else {
+            tma_load_2d_pair(dst, &maps.b[term_now], bar, k0, n);
+          }
         }
       }
     }
@@ -730,7 +759,7 @@ gemm_tc_pair_kernel(const __grid_constant__ TmapPack maps, const TcParams p) {
       uint32_t parity = 0u;
       // descriptors address shared memory in 16-byte units: one addition per stage instead of building them anew
       const uint64_t a_desc0 = make_smem_desc(smem_u32(tiles), A_MN);
-      const uint64_t b_desc0 = make_smem_desc(smem_u32(tiles) + kABytes, B_MN);
+      const uint64_t b_desc0 = make_smem_desc(smem_u32(tiles) + kNA * kABytes, B_MN);
       const uint32_t stage_units = stage_bytes >> 4;
       const int halve_it = p.halve_at_term > 0 ? p.halve_at_term * kb_count : -1;
       for (int it = 0; it < n_iter && ok; ++it) {
@@ -743,16 +772,22 @@ gemm_tc_pair_kernel(const __grid_constant__ TmapPack maps, const TcParams p) {
         for (int k = 0; k < kBK / 16; ++k) {
           const uint64_t a_k = a_desc + (uint64_t)((A_MN ? 2048u : 32u) >> 4) * k;
           const uint64_t b_k = b_desc + (uint64_t)((B_MN ? 2048u : 32u) >> 4) * k;
-          if (k == 0 && it == halve_it) tc_mma_bf16_pair_halved(tmem_base, a_k, b_k, idesc);
-          else tc_mma_bf16_pair(tmem_base, a_k, b_k, idesc, (it > 0 || k > 0) ? 1u : 0u);
+#pragma unroll
+          for (int w = 0; w < kNA * kNB; ++w) {
+            const uint64_t a_w = a_k + (uint64_t)(kWide == WIDE_M ? w * (kABytes >> 4) : 0u);
+            const uint64_t b_w = b_k + (uint64_t)(kWide == WIDE_N ? w * (p.b_bytes >> 4) : 0u);
+            if (k == 0 && it == halve_it) tc_mma_bf16_pair_halved(tmem_base + 256u * w, a_w, b_w, idesc);
+            else tc_mma_bf16_pair(tmem_base + 256u * w, a_w, b_w, idesc, (it > 0 || k > 0) ? 1u : 0u);
+          }
         }
         tc_commit_pair(&empty_bar[s]);   // frees the stage in both CTAs once these MMAs have read it
-        if (++s == kPairStages) { s = 0; parity ^= 1u; }
+        if (++s == stages) { s = 0; parity ^= 1u; }
       }
       tc_commit_pair(&accum_bar);        // accumulator complete in both CTAs (or nothing was issued)
     }
   } else {
-    tc_epilogue(p, maps, tmem_base, &accum_bar, &abort_flag, warp, lane, m0, n0, split, n_iter, tiles);
+    tc_epilogue(p, maps, tmem_base, &accum_bar, &abort_flag, warp, lane, m0, n0, split, n_iter, tiles,
+                kNA * kNB, kWide == WIDE_M ? 2 * kBM : 0, kWide == WIDE_N ? p.bn : 0);
   }
   tc_fence_before();
   __syncthreads();
@@ -1230,6 +1265,8 @@ cudaError_t get_tmap(const void* ptr, uint64_t inner, uint64_t outer, uint64_t l
   return cudaSuccess;
 }
 
+int g_pair_mode = 1;   // 0: never use the two-CTA kernels (test hook); 1: by shape; 2: as 1, but no streaming or wide kernel
+
 int pick_bn(int N) {
   const int n16 = (N + 15) / 16 * 16;
   if (n16 <= 256) return n16;
@@ -1257,13 +1294,13 @@ cudaError_t launch_variant(const TmapPack& maps, const TcParams& p, dim3 grid, s
   return cudaGetLastError();
 }
 
-template <bool A_MN, bool B_MN>
+template <bool A_MN, bool B_MN, int kWide = WIDE_NONE>
 cudaError_t launch_pair_variant(const TmapPack& maps, const TcParams& p, dim3 grid, size_t smem, cudaStream_t stream) {
   static std::atomic<bool> configured[64];   // zero-initialised; set once the attribute is in place on a device
   int dev = 0;
   LORACT_CUDA_TRY(cudaGetDevice(&dev));
   if (dev < 0 || dev >= 64 || !configured[dev].load(std::memory_order_acquire)) {
-    LORACT_CUDA_TRY(cudaFuncSetAttribute(gemm_tc_pair_kernel<A_MN, B_MN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    LORACT_CUDA_TRY(cudaFuncSetAttribute(gemm_tc_pair_kernel<A_MN, B_MN, kWide>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          kPairStages * (kABytes + 16384) + 1024));
     if (dev >= 0 && dev < 64) configured[dev].store(true, std::memory_order_release);
   }
@@ -1281,7 +1318,7 @@ cudaError_t launch_pair_variant(const TmapPack& maps, const TcParams& p, dim3 gr
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  LORACT_CUDA_TRY(cudaLaunchKernelEx(&cfg, gemm_tc_pair_kernel<A_MN, B_MN>, maps, p));
+  LORACT_CUDA_TRY(cudaLaunchKernelEx(&cfg, gemm_tc_pair_kernel<A_MN, B_MN, kWide>, maps, p));
   count_launch(__func__, stream);
   return cudaGetLastError();
 }
@@ -1337,7 +1374,6 @@ cudaError_t launch_stream(const TmapPack& maps, TcParams p, size_t smem, cudaStr
   return cudaGetLastError();
 }
 
-int g_pair_mode = 1;   // 0: never use the two-CTA kernels (test hook); 1: by shape; 2: as 1, but no streaming kernel
 
 }  // namespace
 
@@ -1371,7 +1407,35 @@ bool gemm_tc_supported(const GemmDesc& g) {
   return true;
 }
 
-int gemm_tc_pick_splits(int M, int N, int K, bool, bool b_mn, int max_splits) {
+// How a product is tiled on the two-CTA kernel (the wide forms exist for the majors the path uses), and an estimate of its
+// time in us: rounds of the 74 SM pairs (148 SMs for the one-CTA kernel) times K blocks per split and term times the
+// measured time per K block (0.44 us at 256 x 256, 0.57 wide, 0.36 one-CTA), and an epilogue per round.
+struct TileShape {
+  int wide, bn;
+  double us;
+};
+// wide_ok: whether the wide forms may be chosen (a split count must not depend on the test hook, a launch does).
+static TileShape pick_shape(int M, int N, bool a_mn, bool b_mn, long long k_iters, int splits, bool wide_ok) {
+  auto div = [](long long a, long long b) { return (a + b - 1) / b; };
+  const int bn = pick_bn(N);
+  const bool pair = M >= 2 * kBM && (b_mn ? bn % 128 == 0 : bn % 32 == 0);
+  TileShape best = {WIDE_NONE, bn, 0.0};
+  const long long narrow = (pair ? div(M, 2 * kBM) : div(M, kBM)) * div(N, bn) * splits;
+  best.us = (double)div(narrow, pair ? 74 : 148) * ((double)k_iters * (pair ? 0.44 : 0.36) + 3.0);
+  auto consider = [&](int wide, int wbn, long long tiles) {
+    const double us = (double)div(tiles * splits, 74) * ((double)k_iters * 0.57 + 5.0);
+    if (us < 0.95 * best.us) best = {wide, wbn, us};
+  };
+  if (!wide_ok || M < 2 * kBM) return best;
+  if (!a_mn && !b_mn && N > 256 && N <= 512) {
+    const int half = (int)div(div(N, 2), 64) * 64;
+    consider(WIDE_N, half, div(M, 2 * kBM));
+  }
+  if (b_mn && M > 2 * kBM && bn % 128 == 0) consider(WIDE_M, bn, div(M, 4 * kBM) * div(N, bn));
+  return best;
+}
+
+int gemm_tc_pick_splits(int M, int N, int K, bool a_mn, bool b_mn, int max_splits) {
   const int bn = pick_bn(N);
   const int n_tiles = (N + bn - 1) / bn;
   const int tiles = ((M + kBM - 1) / kBM) * n_tiles;
@@ -1398,6 +1462,18 @@ int gemm_tc_pick_splits(int M, int N, int K, bool, bool b_mn, int max_splits) {
     return rounds * (double)((kb + sp - 1) / sp) + reduce_us / 0.35;
   };
   int best = base;
+  if (a_mn && b_mn && M > 2 * kBM && N > 2 * M) {
+    // A projection at more than 256 columns: tile shape and split count together (the partial sums are written once and
+    // read back once)
+    double least = 1e30;
+    for (int sp = 1; sp <= 8 && (sp == 1 || kb / sp >= 4); ++sp) {
+      const double us = pick_shape(M, N, a_mn, b_mn, (kb + sp - 1) / sp, sp, true).us +
+                        (sp > 1 ? 4.0 + (double)sp * M * N * 4.0 * (1.0 / 4.0e6 + 1.0 / 8.0e6) : 0.0);
+      if (us < 0.98 * least) { least = us; best = sp; }
+    }
+    const int per = (kb + best - 1) / best;
+    return (kb + per - 1) / per;
+  }
   double best_cost = cost(base);
   const int cap = max_splits < 8 ? max_splits : 8;
   for (int sp = 1; sp <= cap; ++sp) {
@@ -1445,8 +1521,13 @@ cudaError_t gemm_tc_launch(const GemmDesc& g, uint32_t* dev_status, cudaStream_t
   p.kb_per_split = (p.kb_total + splits - 1) / splits;
   p.n_terms = g.n_terms;
   p.out = g.out; p.C0 = g.C0; p.C1 = g.C1; p.ldc = g.ldc; p.split_stride = g.split_stride;
-  // Two CTAs per 256-row tile when there are at least 256 rows and the B tile splits into two legal halves.
-  const bool pair = g_pair_mode != 0 && g.M >= 2 * kBM && (g.b_mn ? p.bn % 128 == 0 : p.bn % 32 == 0);
+  // Two CTAs per 256-row tile when there are at least 256 rows and the B tile splits into two legal halves; two
+  // accumulators per pair where that is estimated to be faster.
+  const TileShape shape = pick_shape(g.M, g.N, g.a_mn, g.b_mn, (long long)p.kb_per_split * g.n_terms, splits,
+                                     g_pair_mode == 1);
+  p.bn = shape.bn;
+  const bool pair = shape.wide != WIDE_NONE ||
+                    (g_pair_mode != 0 && g.M >= 2 * kBM && (g.b_mn ? p.bn % 128 == 0 : p.bn % 32 == 0));
   const int b_rows = pair ? p.bn / 2 : p.bn;   // rows (or columns) of B one CTA loads per K block
   p.b_bytes = g.b_mn ? (uint32_t)((b_rows + 63) / 64) * 8192u : (uint32_t)b_rows * 128u;
   p.tmem_cols = 32;
@@ -1454,7 +1535,7 @@ cudaError_t gemm_tc_launch(const GemmDesc& g, uint32_t* dev_status, cudaStream_t
   p.accumulate = g.accumulate ? 1 : 0;
   p.ep_row_a = g.ep_row_a; p.ep_row_b = g.ep_row_b; p.ep_col = g.ep_col;
   p.dev_status = dev_status;
-  p.st_m_tiles = 0; p.st_units = 0; p.tma_store = 0; p.st_stages = kStreamStages; p.store_bufs = kStoreBufs; p.fuse_parts = 4;
+  p.st_m_tiles = 0; p.st_units = 0; p.tma_store = 0; p.st_stages = kStreamStages; p.store_bufs = kStoreBufs; p.fuse_parts = 4; p.pair_stages = kPairStages;
   p.halve_at_term = g.halve_at_term > 0 ? g.halve_at_term : 0;
   p.a_keep_from_kb = g.a_keep_from_k >= 0 ? (int)(g.a_keep_from_k / kBK) : p.kb_total;
   p.gate = g.gate;
@@ -1549,6 +1630,16 @@ cudaError_t gemm_tc_launch(const GemmDesc& g, uint32_t* dev_status, cudaStream_t
   }
   p.tma_store = staged_ok(p.bn) ? 1 : 0;
   if (p.tma_store) LORACT_CUDA_TRY(make_out_maps());
+  if (shape.wide != WIDE_NONE) {
+    const int na = shape.wide == WIDE_M ? 2 : 1, nb = shape.wide == WIDE_N ? 2 : 1;
+    p.tmem_cols = 512;
+    p.pair_stages = 4;
+    dim3 wgrid(2 * ((g.M + 2 * na * kBM - 1) / (2 * na * kBM)), (g.N + nb * p.bn - 1) / (nb * p.bn), splits);
+    const size_t wsmem = (size_t)p.pair_stages * (na * kABytes + nb * p.b_bytes) + 1024;
+    if (shape.wide == WIDE_N) return launch_pair_variant<false, false, WIDE_N>(maps, p, wgrid, wsmem, stream);
+    return g.a_mn ? launch_pair_variant<true, true, WIDE_M>(maps, p, wgrid, wsmem, stream)
+                  : launch_pair_variant<false, true, WIDE_M>(maps, p, wgrid, wsmem, stream);
+  }
   if (pair) {
     dim3 pgrid(2 * ((g.M + 2 * kBM - 1) / (2 * kBM)), (g.N + p.bn - 1) / p.bn, splits);
     const size_t psmem = (size_t)kPairStages * (kABytes + p.b_bytes) + 1024;

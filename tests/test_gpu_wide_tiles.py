@@ -1,0 +1,71 @@
+"""GPU tests of the tensor-core form with two accumulators per CTA pair: the shapes for which it is chosen, with remainders
+in every extent, sums of several terms (halved accumulator included), partial results and every output mode, against an fp32
+product and against the narrow forms (same order of additions per element: the same bits)."""
+import pytest
+import torch
+
+import __graft_entry__ as entry
+from paper_2509_23472_b200 import binding as B
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def dev():
+    entry.build()
+    B.lib()
+    yield torch.device("cuda:0")
+    B.debug_set_pair_mode(True)
+
+
+def operands(dev, m, n, k, a_mn, b_mn, terms):
+    g = torch.Generator(device=dev)
+    g.manual_seed(m + 3 * n + 7 * k)
+    up = lambda v: (v + 7) // 8 * 8
+    As, Bs = [], []
+    for _ in range(terms):
+        a = torch.randn(k, up(m), generator=g, device=dev).bfloat16()[:, :m] if a_mn else \
+            torch.randn(m, up(k), generator=g, device=dev).bfloat16()[:, :k]
+        b = torch.randn(k, up(n), generator=g, device=dev).bfloat16()[:, :n] if b_mn else \
+            torch.randn(n, up(k), generator=g, device=dev).bfloat16()[:, :k]
+        As.append(a); Bs.append(b)
+    return As, Bs
+
+
+@pytest.mark.parametrize("m,n,k,a_mn,b_mn,terms,halve,out,splits", [
+    (16384, 512, 192, False, False, 1, 0, B.OUT_SPLIT, 1),      # the sketch at 512 columns
+    (16500, 336, 200, False, False, 1, 0, B.OUT_SPLIT, 1),      # remainders; 192-column tiles
+    (20001, 272, 136, False, False, 3, 0, B.OUT_BF16, 1),       # three terms
+    (17000, 448, 72, False, False, 2, 1, B.OUT_F32, 1),
+    (512, 11008, 512, False, True, 2, 0, B.OUT_BF16, 1),        # the test matrix
+    (336, 11000, 336, False, True, 2, 0, B.OUT_BF16, 1),
+    (512, 11008, 1000, True, True, 1, 0, B.OUT_F32, 3),         # the projection
+    (328, 10000, 777, True, True, 1, 0, B.OUT_F32, 2),
+    (512, 20000, 64, True, True, 1, 0, B.OUT_BF16, 1)])
+def test_wide_tiles(dev, m, n, k, a_mn, b_mn, terms, halve, out, splits):
+    As, Bs = operands(dev, m, n, k, a_mn, b_mn, terms)
+    got = {}
+    for mode in (True, False):
+        B.debug_set_pair_mode(mode)
+        status = torch.zeros(1, dtype=torch.int32, device=dev)
+        got[mode] = B.debug_gemm(As, Bs, m, n, k, a_mn, b_mn, out_mode=out, engine=1, splits=splits, status=status,
+                                 halve_at_term=halve)
+        torch.cuda.synchronize()
+        assert int(status.item()) == 0
+    B.debug_set_pair_mode(True)
+    pair = out == B.OUT_SPLIT
+    for x, y in zip(got[True] if pair else (got[True],), got[False] if pair else (got[False],)):
+        assert torch.equal(x, y)
+    C = (got[True][0].double() + got[True][1].double()) if pair else got[True].double()
+    if splits > 1:
+        C = C.sum(0)
+    want, scale = 0.0, 0.0
+    for t, (a, b) in enumerate(zip(As, Bs)):
+        a, b = (a.t() if a_mn else a).float(), (b if b_mn else b.t()).float()
+        if halve and t == halve:
+            want, scale = want * 0.5, scale * 0.5
+        want = want + (a.double() @ b.double())
+        scale = scale + a.abs().double() @ b.abs().double()
+    unit = 2.0 ** -8 if out == B.OUT_BF16 else (2.0 ** -16 if pair else 0.0)
+    # fp32 accumulation with truncation (2^-23 of the running sum per instruction), then the rounding of the output
+    assert float(((C - want).abs() - unit * want.abs()).max() / scale.max()) <= terms * k / 16 * 2.0 ** -23 + 1e-6
