@@ -156,12 +156,8 @@ void carve_basis(Carver& c, const Plan& p, BasisWs* w) {
   if (p.bf16) {
     w->Lh = (__nv_bfloat16*)c.take(l * l * 2);
     w->Ll = (__nv_bfloat16*)c.take(l * l * 2);
-    // r <= 256 needs none (shared-memory kernel); above that the block scheme keeps W, X and, per level, two
-    // (width - 256) x 256 temporaries here
-    const size_t lvl1 = l > 256 ? l - 256 : 0, lvl2 = l > 512 ? l - 512 : 0;
-    size_t tmp = 2 * 256 * (lvl1 + lvl2);
-    if (tmp < 2 * 256 * 256) tmp = 2 * 256 * 256;
-    w->sb_scratch = c.take((2 * l * l + tmp) * sizeof(float));
+    // the summed Gram matrix; above 512 columns the fp64 working set of the general kernel
+    w->sb_scratch = c.take(l <= 512 ? l * l * sizeof(float) : (l * l + (l + 31) / 32 * 1024) * sizeof(double));
     const size_t gs = (size_t)(p.splits_gs > p.splits_w ? p.splits_gs : p.splits_w);
     w->gram_partials = (float*)c.take(gs * l * l * 4);
     w->Yh = (__nv_bfloat16*)c.take(n * l * 2);
@@ -239,9 +235,9 @@ cudaError_t factor(int l, bool bf16, int n_partials, float shift, const BasisWs&
       // before it writes them, and no other CTA touches them (the scratch area is the factorisation's own)
       LORACT_CUDA_TRY(reduce_sym_launch(w.gram_partials, n_partials, a.partial_stride, l, w.gram_partials, stream, gate));
       a.n_partials = 1;
-    } else if (l <= 256 && n_partials >= kReduceFirst && !sum_in_kernel) {
-      // The factorisation runs on eight SMs; summing many partials there is a read of several MB through
-      // eight SMs' worth of bandwidth.  All SMs sum them first (same order of additions, so the same bits).
+    } else if (l <= 512 && n_partials >= (l <= 256 ? kReduceFirst : 2) && !sum_in_kernel) {
+      // The factorisation runs on up to sixteen SMs; summing many partials there is a read of several MB through
+      // their share of the bandwidth.  All SMs sum them first (same order of additions, so the same bits).
       float* W = (float*)w.sb_scratch;
       LORACT_CUDA_TRY(reduce_partials_launch(w.gram_partials, n_partials, a.partial_stride, (int64_t)l * l, W, nullptr,
                                              stream));
@@ -380,6 +376,7 @@ cudaError_t range_basis(const void* X, int64_t ldx, const Plan& p, const void* O
     if (Cl) { g.out = OUT_SPLIT; g.C0 = Ch; g.C1 = Cl; } else { g.out = OUT_BF16; g.C0 = Ch; }
     g.gate = gt;
     g.lo_gate = lo_gt;
+    g.whole_rows = Ch == Yh;
     return run_gemm(g, status, stream);
   };
   trace_label("Gram 1");
@@ -387,21 +384,15 @@ cudaError_t range_basis(const void* X, int64_t ldx, const Plan& p, const void* O
   const int kb_total = (n + 63) / 64, n_split = w.splits_gram < 1 ? 1 : w.splits_gram;
   const float chain_blocks = (float)((kb_total + n_split - 1) / n_split);
   const float threshold = can_gate ? g_round_gate.load() / chain_blocks : -1.f;
-  // up to 256 columns the factorisation kernel forms the estimate itself while it writes L^-1 out
-  const bool gate_in_factor = l <= 256 && l % 8 == 0;
   trace_label("small block 2");
   // (widths above 512 take the general fp64 kernel, which knows the shift relative to the mean diagonal only)
   LORACT_CUDA_TRY(factor(l, true, w.splits_gram, l <= 512 ? 0.f : kShiftFirstMean, w, status, stream, true,
-                         l <= 512 ? kShiftFirstDiag : 0.f, nullptr, gate_in_factor ? gate_words : nullptr, threshold));
-  if (!gate_in_factor) {
-    trace_label("round gate");
-    LORACT_CUDA_TRY(round_gate_launch(w.gram_partials, w.Lh, l, threshold, status, gate_words, stream));
-  }
+                         l <= 512 ? kShiftFirstDiag : 0.f, nullptr, can_gate ? gate_words : nullptr, threshold));
   trace_label("apply L^-T 1");
   // the remainder of Q1 is only read by the second round: not written when the decision (taken before this kernel
   // starts) is that one round is enough
   LORACT_CUDA_TRY(apply(w.Yh, w.Yl, U, w.Ql, nullptr, gate));
-  if (gate_in_factor) {
+  if (can_gate) {
     // Round 2 is the rare path, and each of its launches costs the common path a few microseconds even when it
     // leaves at once.  So here the Gram matrix is the plain three-term sum (no halving, no symmetrising pass) and the
     // factorisation kernel adds the partial sums itself: three launches instead of four.  Q1 is orthonormal to a few
@@ -426,13 +417,9 @@ cudaError_t range_basis(const void* X, int64_t ldx, const Plan& p, const void* O
   }
   trace_label("apply L^-T 2");
   // In place when one CTA (pair) owns whole rows of the product: it has read its rows of U and of the remainder
-  // completely before its epilogue stores them.  With several column tiles per row block another CTA may still be
-  // reading the rows, so the result goes to the workspace and is copied.
-  GemmDesc probe;
-  probe.M = n; probe.N = l; probe.K = l; probe.lda = l; probe.ldb = l; probe.ldc = l; probe.n_terms = 3;
-  probe.terms[0] = {U, w.Lh}; probe.terms[1] = {U, w.Ll}; probe.terms[2] = {w.Ql, w.Lh};
-  probe.out = OUT_BF16; probe.C0 = U;
-  if (l <= 256 && gemm_tc_supported(probe)) {
+  // completely before its epilogue stores them.  Otherwise (fewer than 256 rows, more than 512 columns) another CTA may still
+  // be reading the rows, so the result goes to the workspace and is copied.
+  if (gemm_tc_can_own_rows(n, l)) {
     LORACT_CUDA_TRY(apply(U, w.Ql, U, nullptr, gate));
   } else {
     LORACT_CUDA_TRY(apply(U, w.Ql, w.Qh, nullptr, gate));

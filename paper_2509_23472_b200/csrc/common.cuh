@@ -114,10 +114,10 @@ struct GemmDesc {
   const uint32_t* gate = nullptr;
   // Tensor-core path: the launch stores zero into the status word before any of its waits can set a bit in it (the
   // first kernel of a call clears the word itself instead of a memset in front of it).
-  // fp32 32 x 32 tile kernel (gemm_f32_small_launch): optional bf16 hi / lo copies of the result (leading dimension ldc)
-  void* split_hi = nullptr;
-  void* split_lo = nullptr;
   bool clear_status = false;
+  // Tensor-core path, both operands K-major, N <= 512: one CTA pair must own whole rows of the product (it has read its rows
+  // of A before it stores them, so C may be A); see gemm_tc_can_own_rows.
+  bool whole_rows = false;
   // Tensor-core path, OUT_SPLIT: a device word written by an earlier kernel; when it is zero only C0 (the leading bf16
   // part) is written and C1 keeps its old contents.
   const uint32_t* lo_gate = nullptr;
@@ -130,6 +130,8 @@ cudaError_t gemm_tc_launch(const GemmDesc& g, uint32_t* dev_status, cudaStream_t
 int gemm_tc_pick_splits(int M, int N, int K, bool a_mn, bool b_mn, int max_splits = 32);
 // Splits over K of a product with many rows (M x N, both operands K-major) whose tiles do not fill the chip.
 int gemm_tc_pick_tall_splits(int M, int N, int K);
+// Whether a launch with whole_rows set can give one CTA (pair) whole rows of an M x N product.
+bool gemm_tc_can_own_rows(int M, int N);
 void gemm_tc_set_pair_mode(int on);   // test hook: 0 keeps every contraction on the one-CTA kernel
 // Test hooks for the give-up path of the bounded waits: a kernel that waits (with the engine's / the cluster
 // kernel's own wait) on a barrier nothing completes, for at most limit_ns, then sets LORACT_DEV_WAIT_EXPIRED.
@@ -138,10 +140,6 @@ cudaError_t small_block_cluster_wait_probe_launch(uint32_t* dev_status, uint64_t
 
 // Plain CUDA-core kernel for any shape and type (fp32 path, small or odd shapes).
 cudaError_t gemm_simt_launch(const GemmDesc& g, cudaStream_t stream);
-// fp32 x fp32 -> fp32 for matrices of a few hundred rows and columns (32 x 32 tiles, one per CTA).
-// `second`: an independent product carried by the same launch (both may read what earlier launches wrote;
-// neither may read the other's output).
-cudaError_t gemm_f32_small_launch(const GemmDesc& g, cudaStream_t stream, const GemmDesc* second = nullptr);
 
 // ---------------------------------------------------------------- sampler and gather
 // idx_copy (optional) receives the same indices; clear_status: the kernel sets the status word instead of OR-ing
@@ -176,13 +174,13 @@ struct SmallBlockArgs {
   bool use_f64 = false;  // compute type
   void* scratch = nullptr;
   float shift_rel = 0.f;
-  // shared-memory cluster kernel and the block scheme built on it: each diagonal entry is also multiplied by
+  // shared-memory cluster kernel: each diagonal entry is also multiplied by
   // (1 + shift_diag_rel), a shift relative to the entry itself (the scale-invariant form, which leaves a
   // matrix whose diagonal spans several orders of magnitude as well conditioned as its scaled form)
   float shift_diag_rel = 0.f;
   // device word written by an earlier kernel of the stream; zero: the launch does nothing.  nullptr: unconditional.
   const uint32_t* gate = nullptr;
-  // shared-memory cluster kernel only (r <= 256): three words that receive what round_gate_launch would write for
+  // shared-memory cluster kernel only: three words that receive what round_gate_launch would write for
   // this matrix and its inverse factor, computed inside the factorisation (no extra launch)
   uint32_t* gate_out = nullptr;
   float gate_threshold = 0.f;
@@ -191,33 +189,17 @@ struct SmallBlockArgs {
   __nv_bfloat16* linv_hi = nullptr;
   __nv_bfloat16* linv_lo = nullptr;
   uint32_t* dev_status = nullptr;
-  // row strides (elements) of the partial matrices and of the outputs; 0 means r.  The matrix may be a
-  // diagonal sub-block of a larger one (the r > 256 path factors a 512 x 512 matrix through its 256 x 256 blocks)
+  // row strides (elements) of the partial matrices and of the outputs; 0 means r
   int64_t in_ld = 0, out_ld = 0;
-  // Where the scale of the shift and of the pivot floor comes from: by default the mean of the matrix's own
-  // diagonal.  A Schur complement that is handed in as "the matrix" can be all rounding noise, so the two-level
-  // path points this at the diagonal of the block it was taken from (scale_n entries, stride scale_ld + 1).
-  const float* scale_diag = nullptr;
-  int scale_n = 0;
-  int64_t scale_ld = 0;
 };
 cudaError_t small_block_launch(const SmallBlockArgs& a, cudaStream_t stream);
-// The same computation for r <= 256 in fp32 from fp32 partials, or r <= 192 in fp64 from fp64 partials, entirely in the
-// shared memory of a cluster of up to eight CTAs (no scratch).  small_block_launch uses it whenever it applies.
+// The same computation for r <= 512 in fp32 from fp32 partials, or r <= 192 in fp64 from fp64 partials, entirely in the
+// shared memory of a cluster of up to sixteen CTAs (no scratch).  small_block_launch uses it whenever it applies.
 bool small_block_cluster_supported(const SmallBlockArgs& a);
 cudaError_t small_block_cluster_launch(const SmallBlockArgs& a, cudaStream_t stream);
 
 // ---------------------------------------------------------------- elementwise helpers
 // out = sum_s partials[s] (fixed order), written as fp32 and/or bf16.
-// X21 of a 2 x 2 block lower-triangular inverse as bf16 hi/lo (and optionally fp32), plus zeros in the block
-// above the diagonal: src (rows x cols fp32, leading dimension ld) -> hi/lo at the same place.
-cudaError_t split_block_launch(const float* src, int rows, int cols, int64_t ld, __nv_bfloat16* hi,
-                               __nv_bfloat16* lo, cudaStream_t stream, const uint32_t* gate = nullptr);
-// Zero fill of up to three ranges (16-byte aligned, sizes multiples of 16; a null range has size 0), one launch.
-// Optionally the same launch also forms sum_dst[i] = sum over n_src partials of sum_src[q * src_stride + i], i < count.
-cudaError_t zero3_gated_launch(void* a, size_t a_bytes, void* b, size_t b_bytes, void* c, size_t c_bytes,
-                               const uint32_t* gate, cudaStream_t stream, const float* sum_src = nullptr,
-                               int n_src = 0, int64_t src_stride = 0, int64_t count = 0, float* sum_dst = nullptr);
 cudaError_t reduce_partials_launch(const float* partials, int n_partials, int64_t stride,
                                    int64_t count, float* out_f32, __nv_bfloat16* out_bf16,
                                    cudaStream_t stream, const uint32_t* gate = nullptr);

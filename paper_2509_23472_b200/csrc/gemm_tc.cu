@@ -1415,7 +1415,8 @@ struct TileShape {
   double us;
 };
 // wide_ok: whether the wide forms may be chosen (a split count must not depend on the test hook, a launch does).
-static TileShape pick_shape(int M, int N, bool a_mn, bool b_mn, long long k_iters, int splits, bool wide_ok) {
+static TileShape pick_shape(int M, int N, bool a_mn, bool b_mn, long long k_iters, int splits, bool wide_ok,
+                            bool whole_rows = false) {
   auto div = [](long long a, long long b) { return (a + b - 1) / b; };
   const int bn = pick_bn(N);
   const bool pair = M >= 2 * kBM && (b_mn ? bn % 128 == 0 : bn % 32 == 0);
@@ -1429,11 +1430,14 @@ static TileShape pick_shape(int M, int N, bool a_mn, bool b_mn, long long k_iter
   if (!wide_ok || M < 2 * kBM) return best;
   if (!a_mn && !b_mn && N > 256 && N <= 512) {
     const int half = (int)div(div(N, 2), 64) * 64;
+    if (whole_rows) return {WIDE_N, half, 0.0};
     consider(WIDE_N, half, div(M, 2 * kBM));
   }
   if (b_mn && M > 2 * kBM && bn % 128 == 0) consider(WIDE_M, bn, div(M, 4 * kBM) * div(N, bn));
   return best;
 }
+
+bool gemm_tc_can_own_rows(int M, int N) { return N <= 256 || (N <= 512 && M >= 2 * kBM && g_pair_mode == 1); }
 
 int gemm_tc_pick_splits(int M, int N, int K, bool a_mn, bool b_mn, int max_splits) {
   const int bn = pick_bn(N);
@@ -1524,7 +1528,7 @@ cudaError_t gemm_tc_launch(const GemmDesc& g, uint32_t* dev_status, cudaStream_t
   // Two CTAs per 256-row tile when there are at least 256 rows and the B tile splits into two legal halves; two
   // accumulators per pair where that is estimated to be faster.
   const TileShape shape = pick_shape(g.M, g.N, g.a_mn, g.b_mn, (long long)p.kb_per_split * g.n_terms, splits,
-                                     g_pair_mode == 1);
+                                     g_pair_mode == 1, g.whole_rows);
   p.bn = shape.bn;
   const bool pair = shape.wide != WIDE_NONE ||
                     (g_pair_mode != 0 && g.M >= 2 * kBM && (g.b_mn ? p.bn % 128 == 0 : p.bn % 32 == 0));

@@ -33,10 +33,6 @@ struct SimtParams {
   int k_per;          // fp32 tile kernels: contraction elements per split
   int lower_only;     // 32 x 32 tile kernel: tiles above the diagonal are not formed
   int halve_at_term;  // the sum so far is multiplied by 1/2 before this term (0: never)
-  const uint32_t* gate;  // 32 x 32 tile kernel: optional device word, zero means the launch does nothing
-  // 32 x 32 tile kernel: optional bf16 hi / lo copies of the result, same leading dimension as C0
-  __nv_bfloat16* split_hi;
-  __nv_bfloat16* split_lo;
 };
 
 constexpr int kTile = 64;   // output tile 64 x 64, 256 threads, 4 x 4 outputs per thread
@@ -276,13 +272,12 @@ __global__ void reduce_split3_kernel(const float* __restrict__ partials, int n_p
   }
 }
 
-// fp32 x fp32 products on CUDA cores: the whole fp32 path, and the r x r blocks of the two-level small-block scheme.
+// fp32 x fp32 products on CUDA cores: the whole fp32 path.
 // C = alpha * A B (+ C), accumulated in fp32, or in fp64 (Gram matrices).  Everything here is small, so what bounds it is
 // latency and the number of SMs at work: 32 x 32 output tiles, four groups of 64 threads per tile, each group on a quarter
 // of the contraction (4 x 4 outputs per thread, operands read from shared memory along the contraction index with 16-byte
 // loads; the four partial tiles are added in group order), the K loop double-buffered through registers.  fp64: operands
-// are converted once, on their way into shared memory.  grid.z: splits over K (partial results), or, with `has_second`, one
-// of two independent products that the two-level scheme has at one point of its chain.
+// are converted once, on their way into shared memory.  grid.z: splits over K (partial results).
 // (Measured against 64 x 64 tiles with a conversion per use and no dependent launch, whole calls with the same
 // factorisation: 512 x 768, r = 64: 152 -> 100 us; 2000 x 2000, r = 192: 510 -> 324 us.)
 template <typename TAcc> struct Tile32;
@@ -299,23 +294,21 @@ __device__ __forceinline__ double dot16(double2 a, double2 b, double c) { return
 constexpr int kT32 = 32;
 constexpr int kT32Groups = 4;   // thread groups of 64 that share one output tile, each on a quarter of the contraction
 template <typename TAcc>
-__global__ void __launch_bounds__(64 * kT32Groups) gemm_tile32_kernel(SimtParams p0, SimtParams p1, int has_second) {
+__global__ void __launch_bounds__(64 * kT32Groups) gemm_tile32_kernel(SimtParams p) {
   constexpr int kKc = Tile32<TAcc>::kKc, kLd = Tile32<TAcc>::kLd, kPartLd = Tile32<TAcc>::kPartLd;
   typedef typename Vec16<TAcc>::type V;
   constexpr int kVn = Vec16<TAcc>::kN;
   constexpr int kPer = kT32 * kKc / 64;                // elements of either tile a thread stages per K chunk
   // per group: As [m][k] and Bs [n][k]; after the K loop the same memory carries the partial tiles of groups 1..3
   __shared__ __align__(16) TAcc tiles[kT32Groups][2 * kT32 * kLd];
-  const SimtParams& p = has_second && blockIdx.z ? p1 : p0;
-  const int split = has_second ? 0 : (int)blockIdx.z;
+  const int split = (int)blockIdx.z;
   const int grp = threadIdx.x >> 6, tid = threadIdx.x & 63;
   TAcc* As = tiles[grp];
   TAcc* Bs = tiles[grp] + kT32 * kLd;
   const int m0 = blockIdx.y * kT32, n0 = blockIdx.x * kT32;
   pdl_wait();
   pdl_launch_dependents();
-  if (p.gate != nullptr && *(const volatile uint32_t*)p.gate == 0u) return;
-  if (m0 >= p.M || n0 >= p.N || (p.lower_only && n0 > m0)) return;
+  if (p.lower_only && n0 > m0) return;
   const int tm = tid >> 3, tn = tid & 7;               // outputs (4 tm + i, tn + 8 j)
   const float* A = (const float*)p.A[0];
   const float* B = (const float*)p.B[0];
@@ -429,11 +422,6 @@ __global__ void __launch_bounds__(64 * kT32Groups) gemm_tile32_kernel(SimtParams
       float* c = (float*)p.C0 + off;
       const float v = p.accumulate ? (*c + (float)v0) : (float)v0;
       *c = v;
-      if (p.split_hi) {
-        const __nv_bfloat16 h = __float2bfloat16(v);
-        p.split_hi[(int64_t)m * p.ldc + n] = h;
-        if (p.split_lo) p.split_lo[(int64_t)m * p.ldc + n] = __float2bfloat16(v - __bfloat162float(h));
-      }
     }
   }
 }
@@ -517,21 +505,6 @@ __global__ void __launch_bounds__(128) gemm_tile64_kernel(SimtParams p) {
       for (int j = 0; j < 4; ++j)
         if (n + j < p.N) c[j] = p.accumulate ? c[j] + acc[i][j] * p.alpha : acc[i][j] * p.alpha;
     }
-  }
-}
-
-// hi/lo split of a block of an fp32 matrix, in place of the same block of two bf16 matrices.
-__global__ void split_block_kernel(const float* __restrict__ src, int rows, int cols, int64_t ld,
-                                   __nv_bfloat16* __restrict__ hi, __nv_bfloat16* __restrict__ lo,
-                                   const uint32_t* gate) {
-  if (gate != nullptr && *(const volatile uint32_t*)gate == 0u) return;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < (int64_t)rows * cols;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t row = i / cols, col = i - row * cols;
-    const float v = src[row * ld + col];
-    const __nv_bfloat16 h = __float2bfloat16(v);
-    hi[row * ld + col] = h;
-    if (lo) lo[row * ld + col] = __float2bfloat16(v - __bfloat162float(h));
   }
 }
 
@@ -837,27 +810,6 @@ __global__ void __launch_bounds__(1024) round_gate_kernel(const float* __restric
   }
 }
 
-// Zero fill of up to three 16-byte aligned ranges (counts in 16-byte units) and, in the same launch, an optional
-// fixed-order sum of partial matrices (dst[i] = sum_q src[q * stride + i], i < count; count 0: none).  Skipped when
-// *gate == 0.
-__global__ void zero3_gated_kernel(uint4* a, int64_t na, uint4* b, int64_t nb, uint4* c, int64_t nc,
-                                   const float* __restrict__ src, int n_src, int64_t src_stride, int64_t count,
-                                   float* __restrict__ dst, const uint32_t* gate) {
-  pdl_wait();
-  pdl_launch_dependents();
-  if (gate != nullptr && *(const volatile uint32_t*)gate == 0u) return;
-  const uint4 z = make_uint4(0u, 0u, 0u, 0u);
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x, t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  for (int64_t i = t0; i < count; i += stride) {
-    float sum = 0.f;
-    for (int q = 0; q < n_src; ++q) sum += src[(int64_t)q * src_stride + i];
-    dst[i] = sum;
-  }
-  for (int64_t i = t0; i < na; i += stride) a[i] = z;
-  for (int64_t i = t0; i < nb; i += stride) b[i] = z;
-  for (int64_t i = t0; i < nc; i += stride) c[i] = z;
-}
-
 __global__ void copy_bf16_gated_kernel(const uint4* __restrict__ src, uint4* __restrict__ dst, int64_t n16,
                                        const uint32_t* gate) {
   pdl_wait();
@@ -874,7 +826,7 @@ constexpr int kT64MinTiles = 64;
 static bool tile32_params(const GemmDesc& g, SimtParams& p) {
   if (g.a_type != ELEM_F32 || g.b_type != ELEM_F32 || g.n_terms != 1) return false;
   if (!(g.out == OUT_F32 || (g.out == OUT_F64 && !g.accumulate))) return false;
-  if (g.splits > 1 && (g.accumulate || g.split_hi)) return false;
+  if (g.splits > 1 && g.accumulate) return false;
   p = SimtParams{};
   p.M = g.M; p.N = g.N; p.K = g.K;
   if (g.a_mn) { p.sam = 1; p.sak = g.lda; } else { p.sam = g.lda; p.sak = 1; }
@@ -886,10 +838,7 @@ static bool tile32_params(const GemmDesc& g, SimtParams& p) {
   p.split_stride = g.split_stride;
   p.accumulate = g.accumulate ? 1 : 0;
   p.alpha = g.alpha;
-  p.gate = g.gate;
   p.lower_only = g.lower_only ? 1 : 0;
-  p.split_hi = (__nv_bfloat16*)g.split_hi;
-  p.split_lo = (__nv_bfloat16*)g.split_lo;
   p.k_per = ((p.K + p.splits - 1) / p.splits + 3) / 4 * 4;
   auto vec = [&](const void* P, bool mn_major, int64_t ld, int extent) {
     return (((uintptr_t)P & 15) == 0 && ld % 4 == 0 && (mn_major ? extent : g.K) % 4 == 0) ? 1 : 0;
@@ -899,12 +848,10 @@ static bool tile32_params(const GemmDesc& g, SimtParams& p) {
   return true;
 }
 
-static cudaError_t tile32_launch(const SimtParams& p0, const SimtParams* second, bool acc64, cudaStream_t stream) {
-  const SimtParams& p1 = second ? *second : p0;
-  dim3 grid((std::max(p0.N, p1.N) + kT32 - 1) / kT32, (std::max(p0.M, p1.M) + kT32 - 1) / kT32, second ? 2 : p0.splits);
-  if (grid.y > 65535) return cudaErrorNotSupported;
+static cudaError_t tile32_launch(const SimtParams& p, bool acc64, cudaStream_t stream) {
+  dim3 grid((p.N + kT32 - 1) / kT32, (p.M + kT32 - 1) / kT32, p.splits);
   LORACT_CUDA_TRY(launch_pdl(acc64 ? gemm_tile32_kernel<double> : gemm_tile32_kernel<float>, grid, dim3(64 * kT32Groups), 0,
-                             stream, p0, p1, second ? 1 : 0));
+                             stream, p));
   count_launch(__func__, stream);
   return cudaGetLastError();
 }
@@ -916,13 +863,13 @@ cudaError_t gemm_simt_launch(const GemmDesc& g, cudaStream_t stream) {
     // (whole call, 512 x 768, r = 64: 100 us against 106; 999 x 376, r = 16: 87 against 97; above, the larger tiles read
     // each operand half as often: 1500 x 600, r = 96: 149 against 159)
     const long long tiles = (long long)((g.M + kT64 - 1) / kT64) * ((g.N + kT64 - 1) / kT64) * p.splits;
-    if (!g.acc64 && g.out == OUT_F32 && !g.gate && !g.split_hi && !g.lower_only && p.vec_a && p.vec_b && tiles >= kT64MinTiles) {
+    if (!g.acc64 && g.out == OUT_F32 && !g.lower_only && p.vec_a && p.vec_b && tiles >= kT64MinTiles) {
       LORACT_CUDA_TRY(launch_pdl(gemm_tile64_kernel, dim3((g.N + kT64 - 1) / kT64, (g.M + kT64 - 1) / kT64, p.splits),
                                  dim3(128), 0, stream, p));
       count_launch(__func__, stream);
       return cudaGetLastError();
     }
-    return tile32_launch(p, nullptr, g.acc64, stream);
+    return tile32_launch(p, g.acc64, stream);
   }
   p = SimtParams{};
   p.M = g.M; p.N = g.N; p.K = g.K;
@@ -1013,17 +960,6 @@ cudaError_t round_gate_launch(const float* W, const __nv_bfloat16* linv_hi, int 
   return cudaGetLastError();
 }
 
-cudaError_t zero3_gated_launch(void* a, size_t a_bytes, void* b, size_t b_bytes, void* c, size_t c_bytes,
-                               const uint32_t* gate, cudaStream_t stream, const float* sum_src, int n_src,
-                               int64_t src_stride, int64_t count, float* sum_dst) {
-  if (((uintptr_t)a | (uintptr_t)b | (uintptr_t)c | a_bytes | b_bytes | c_bytes) & 15) return cudaErrorInvalidValue;
-  LORACT_CUDA_TRY(launch_pdl(zero3_gated_kernel, dim3(148), dim3(512), 0, stream, (uint4*)a, (int64_t)(a_bytes / 16),
-                             (uint4*)b, (int64_t)(b_bytes / 16), (uint4*)c, (int64_t)(c_bytes / 16), sum_src, n_src,
-                             src_stride, sum_src ? count : (int64_t)0, sum_dst, gate));
-  count_launch(__func__, stream);
-  return cudaGetLastError();
-}
-
 cudaError_t copy_bf16_gated_launch(const __nv_bfloat16* src, __nv_bfloat16* dst, int64_t count, const uint32_t* gate,
                                    cudaStream_t stream) {
   if (count % 8 || ((uintptr_t)src & 15) || ((uintptr_t)dst & 15) || !gate) return cudaErrorInvalidValue;
@@ -1045,24 +981,6 @@ cudaError_t reduce_split3_launch(const float* partials, int n_partials, int64_t 
   if (grid < 1) grid = 1;
   LORACT_CUDA_TRY(launch_pdl(reduce_split3_kernel, dim3(grid), dim3(256), 0, stream, partials, n_partials, stride, rows,
                              cols, ld_in, ld_out, hi, mid, lo));
-  count_launch(__func__, stream);
-  return cudaGetLastError();
-}
-
-cudaError_t gemm_f32_small_launch(const GemmDesc& g, cudaStream_t stream, const GemmDesc* second) {
-  // (the gate of the first product holds for the whole launch)
-  SimtParams p0, p1;
-  if (g.splits > 1 || !tile32_params(g, p0) || (second && (second->splits > 1 || !tile32_params(*second, p1))))
-    return cudaErrorNotSupported;
-  if (second) p1.gate = g.gate;
-  return tile32_launch(p0, second ? &p1 : nullptr, false, stream);
-}
-
-cudaError_t split_block_launch(const float* src, int rows, int cols, int64_t ld, __nv_bfloat16* hi,
-                               __nv_bfloat16* lo, cudaStream_t stream, const uint32_t* gate) {
-  int grid = (int)(((int64_t)rows * cols + 255) / 256);
-  if (grid > 148 * 4) grid = 148 * 4;
-  split_block_kernel<<<grid, 256, 0, stream>>>(src, rows, cols, ld, hi, lo, gate);
   count_launch(__func__, stream);
   return cudaGetLastError();
 }

@@ -274,98 +274,9 @@ cudaError_t launch_typed(const SBParams& p, cudaStream_t stream) {
 
 }  // namespace
 
-// r > 256 in fp32: the matrix as 2 x 2 blocks, W = [W11 . ; W21 W22], the leading block 256 wide.
-//   L11 = chol(W11), X11 = L11^-1            (shared-memory cluster kernel)
-//   L21 = W21 X11^T,  S = W22 - L21 L21^T    (fp32 CUDA-core products)
-//   L22 = chol(S), X22 = L22^-1              (the same again if S is wider than 256, else the cluster kernel)
-//   X21 = -X22 (L21 X11)                     (fp32 CUDA-core products)
-// W (n x n, leading dimension ld) is overwritten by the Schur complements; X (fp32) and the bf16 pair receive the
-// inverse factor at the same place and leading dimension.  T: 2 * 256 * (n - 256) floats for this level's two
-// temporaries, followed by what the levels below need.  The shift and the pivot floor of every level come from
-// the diagonal of the whole matrix's leading block (`scale`): a Schur complement may be nothing but rounding noise.
-struct TwoLevelCtx {
-  float shift_rel;
-  float shift_diag_rel;
-  const uint32_t* gate;
-  uint32_t* dev_status;
-  int64_t ld;
-  const float* scale_diag;
-  int scale_n;
-  cudaStream_t stream;
-};
-
-cudaError_t factor_blocks(const TwoLevelCtx& c, float* W, float* X, __nv_bfloat16* hi, __nv_bfloat16* lo, int n,
-                          float* T, bool top) {
-  const int64_t ld = c.ld;
-  if (n <= 256) {
-    SmallBlockArgs s;
-    s.r = n; s.partials = W; s.partial_type = ELEM_F32; s.n_partials = 1; s.partial_stride = 0;
-    s.use_f64 = false; s.shift_rel = c.shift_rel; s.shift_diag_rel = c.shift_diag_rel; s.in_ld = ld; s.out_ld = ld;
-    s.linv_f32 = X; s.linv_hi = hi; s.linv_lo = lo; s.dev_status = c.dev_status; s.gate = c.gate;
-    if (!top) { s.scale_diag = c.scale_diag; s.scale_n = c.scale_n; s.scale_ld = ld; }
-    return small_block_cluster_launch(s, c.stream);
-  }
-  const int r1 = 256, r2 = n - r1;
-  float* T1 = T;
-  float* T2 = T1 + (size_t)r2 * r1;
-  float* Tnext = T2 + (size_t)r2 * r1;
-  LORACT_CUDA_TRY(factor_blocks(c, W, X, hi, lo, r1, Tnext, top));
-  auto product = [&](int M, int N, int K, const float* A, int64_t lda, const float* B, int64_t ldb, bool b_mn,
-                     float* C, int64_t ldc, float alpha, bool accumulate) {
-    GemmDesc g;
-    g.M = M; g.N = N; g.K = K; g.lda = lda; g.ldb = ldb; g.b_mn = b_mn;
-    g.a_type = g.b_type = ELEM_F32;
-    g.terms[0] = {A, B};
-    g.out = OUT_F32; g.C0 = C; g.ldc = ldc; g.alpha = alpha; g.accumulate = accumulate;
-    g.gate = c.gate;
-    return g;
-  };
-  const float* W21 = W + (size_t)r1 * ld;
-  float* W22 = W + (size_t)r1 * ld + r1;
-  float* X22 = X + (size_t)r1 * ld + r1;
-  float* X21 = X + (size_t)r1 * ld;
-  // L21 = W21 X11^T : C[m][n] = sum_k W21[m][k] X11[n][k]
-  LORACT_CUDA_TRY(gemm_f32_small_launch(product(r2, r1, r1, W21, ld, X, ld, false, T1, r1, 1.f, false), c.stream));
-  // One launch, two products that both read L21: S = W22 - L21 L21^T (in place) and
-  // T2 = L21 X11, T2[m][n] = sum_k L21[m][k] X11[k][n], which the last product below needs.
-  {
-    const GemmDesc schur = product(r2, r2, r1, T1, r1, T1, r1, false, W22, ld, -1.f, true);
-    const GemmDesc l21x11 = product(r2, r1, r1, T1, r1, X, ld, true, T2, r1, 1.f, false);
-    LORACT_CUDA_TRY(gemm_f32_small_launch(schur, c.stream, &l21x11));
-  }
-  LORACT_CUDA_TRY(factor_blocks(c, W22, X22, hi + (size_t)r1 * ld + r1, lo ? lo + (size_t)r1 * ld + r1 : nullptr, r2,
-                                Tnext, false));
-  // X21 = -X22 T2 : X21[m][n] = -sum_k X22[m][k] T2[k][n], written as fp32 and as the bf16 pair in the same launch
-  GemmDesc last = product(r2, r1, r2, X22, ld, T2, r1, true, X21, ld, -1.f, false);
-  last.split_hi = hi + (size_t)r1 * ld;
-  last.split_lo = lo ? lo + (size_t)r1 * ld : nullptr;
-  return gemm_f32_small_launch(last, c.stream);
-}
-
-// scratch: W (r x r) + X (r x r) + the temporaries of every level, fp32.
-cudaError_t small_block_two_level(const SmallBlockArgs& a, cudaStream_t stream) {
-  const int r = a.r;
-  float* W = (float*)a.scratch;
-  float* X = a.linv_f32 ? a.linv_f32 : W + (size_t)r * r;
-  float* T = W + 2 * (size_t)r * r;
-  // one launch: W = sum of the partials, and zeros where the blocks above the diagonal are never written below (X is
-  // read as a whole by the products of the next level up)
-  LORACT_CUDA_TRY(zero3_gated_launch(X, (size_t)r * r * 4, a.linv_hi, (size_t)r * r * 2, a.linv_lo,
-                                     a.linv_lo ? (size_t)r * r * 2 : 0, a.gate, stream, (const float*)a.partials,
-                                     a.n_partials, a.partial_stride, (int64_t)r * r, W));
-  TwoLevelCtx c;
-  c.shift_rel = a.shift_rel; c.shift_diag_rel = a.shift_diag_rel; c.gate = a.gate; c.dev_status = a.dev_status; c.ld = r; c.scale_diag = W; c.scale_n = 256;
-  c.stream = stream;
-  return factor_blocks(c, W, X, a.linv_hi, a.linv_lo, r, T, true);
-}
-
 cudaError_t small_block_launch(const SmallBlockArgs& a, cudaStream_t stream) {
   if (small_block_cluster_supported(a)) return small_block_cluster_launch(a, stream);
   if (a.gate_out) return cudaErrorNotSupported;   // only the shared-memory kernel forms the estimate
-  if (!a.use_f64 && a.partial_type == ELEM_F32 && a.r > 256 && a.r <= 512 && a.r % 8 == 0 && !a.linv_full &&
-      a.linv_hi && a.in_ld == 0 && a.out_ld == 0 && (((uintptr_t)a.partials & 15) == 0) &&
-      (a.partial_stride % 4 == 0))
-    return small_block_two_level(a, stream);
   if (a.gate) return cudaErrorNotSupported;   // the general kernel is unconditional
   SBParams p;
   p.r = a.r;
@@ -380,9 +291,8 @@ cudaError_t small_block_launch(const SmallBlockArgs& a, cudaStream_t stream) {
   p.linv_hi = a.linv_hi;
   p.linv_lo = a.linv_lo;
   p.dev_status = a.dev_status;
-  // Widths above 512 (the comparator with extra test vectors at rank 512) would need a third level of fp32 Schur
-  // complements, whose rounding noise reaches the smallest pivots (measured: clamped pivots at 520 columns,
-  // non-finite factors at 32768 rows): they take the general kernel in fp64 instead.
+  // Widths above 512 (the comparator with extra test vectors at rank 512) take this kernel in fp64: their un-preconditioned
+  // sketch left clamped pivots at 520 columns and non-finite factors at 32768 rows in fp32.
   return (a.use_f64 || a.r > 512) ? launch_typed<double>(p, stream) : launch_typed<float>(p, stream);
 }
 

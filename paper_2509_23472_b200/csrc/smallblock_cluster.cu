@@ -1,6 +1,6 @@
 // Small-block factorisation: Cholesky factor of an r x r Gram matrix and the inverse of that factor (the serial part of
 // the orthonormalisation, the QR step of Algorithm 1 done through Gram matrices), as one thread-block-cluster kernel
-// whose working set never leaves shared memory.  fp32 up to r = 256, fp64 up to r = 192.
+// whose working set never leaves shared memory.  fp32 up to r = 512, fp64 up to r = 192.
 //
 // What bounds it is the chain of r pivots: nothing else is large (11 MFLOP at r = 256).  So the matrix is cut into
 // 32 x 32 blocks, block ROW i and block COLUMN i of the inverse belong to CTA i of the cluster, and everything flows
@@ -15,7 +15,8 @@
 //     factored, and later the block column of the inverse, whose transpose solves the same system.  No inverse of a
 //     diagonal block is formed.
 //   * bulk warps (eight, two to a block): the updates nobody waits for, and the output.
-//   * the sender copies finished groups and blocks to the CTAs that need them (bulk distributed-shared-memory copies).
+//   * sender warps (one, above eight blocks three taking turns) copy finished groups and blocks to the CTAs that need them (bulk
+//     distributed-shared-memory copies; one round of wait, proxy fence and up to fifteen copies takes longer than a group).
 // A block is stored as eight groups of [32 rows][4 columns]: a group is one contiguous copy, a lane's row and a
 // broadcast row are one 16-byte load each, without bank conflicts.  Loops over groups are rolled.  The hand-offs of the
 // pivot warp are named barriers (31 cycles against 110 for an mbarrier), all others are mbarriers that complete once.
@@ -26,6 +27,8 @@
 //
 // Measured (one Gram matrix, back to back, against a form with one chain CTA, workers that sent blocks back to it and an
 // inverse of every diagonal block): fp32 r = 32 / 64 / 128 / 256: 7.1 / 8.5 / 13.8 / 28.8 us (7.4 / 11.8 / 20.0 / 40.4).
+// r = 336 / 512, against two factorisations of up to 256 columns joined by fp32 products: 42 / 74 us (69 / 91, and six
+// helper launches fewer).  Above eight blocks the early steps are bound by the bulk updates and by what an SM can send.
 // fp64, against a kernel that kept the matrix in global memory: r = 64 / 96 / 192: 13.0 / 17.7 / 33.7 us (75.8 / 120.9 /
 // 282).  Cycles per group of four columns: 398 in the pivot warp alone, about 475 with its companions at work; the step
 // from one diagonal block to the next adds about 1000.
@@ -42,24 +45,23 @@ namespace loract {
 namespace {
 
 constexpr int kB = 32;                   // block edge
-constexpr int kMaxBlk = 8;               // block rows, and CTAs of the cluster
-constexpr int kWarps = 18;
-constexpr int kCThreads = kWarps * 32;
+constexpr int kMaxWarps = 20;            // two senders fewer up to eight blocks
+__host__ __device__ constexpr int warps_of(bool big) { return big ? kMaxWarps : kMaxWarps - 2; }
 constexpr int kPan = 8;                  // groups of four columns in a block
-constexpr int kMaxOff = kMaxBlk * (kMaxBlk - 1) / 2;
 constexpr uint64_t kClusterWaitNs = 50000000ull;  // 50 ms
 // Warp -> role (plus the index inside the role).  The scheduler a warp shares is its number mod 4: the pivot warp's
-// companions are the sender and three bulk warps, which are idle while it works.
+// companions are senders and bulk warps, which are idle or waiting while it works.
 enum Role : int { R_PIVOT = 0, R_FOLLOW = 1, R_SOLVE = 5, R_BULK = 9, R_SEND = 17 };
 constexpr int kBulkWarps = 8;
-__constant__ unsigned char kRoleOf[kWarps] = {R_PIVOT, R_FOLLOW + 0, R_FOLLOW + 1, R_FOLLOW + 2, R_SEND, R_SOLVE + 0,
+__constant__ unsigned char kRoleOf[kMaxWarps] = {R_PIVOT, R_FOLLOW + 0, R_FOLLOW + 1, R_FOLLOW + 2, R_SEND + 0, R_SOLVE + 0,
                                               R_FOLLOW + 3, R_SOLVE + 2, R_BULK + 0, R_SOLVE + 3, R_SOLVE + 1, R_BULK + 6,
-                                              R_BULK + 1, R_BULK + 3, R_BULK + 5, R_BULK + 7, R_BULK + 2, R_BULK + 4};
+                                              R_BULK + 1, R_BULK + 3, R_BULK + 5, R_BULK + 7, R_BULK + 2, R_BULK + 4,
+                                              R_SEND + 1, R_SEND + 2};
 
 constexpr int kGrp = kB * 4;             // elements of a group of four columns
 constexpr int kBlk = kB * kB;            // elements of a block
 template <typename T> struct Cfg;
-template <> struct Cfg<float> { static constexpr int kMaxR = 256; };
+template <> struct Cfg<float> { static constexpr int kMaxR = 256; };    // (kept whole; see kBig)
 template <> struct Cfg<double> { static constexpr int kMaxR = 192; };
 
 struct SCParams {
@@ -80,9 +82,6 @@ struct SCParams {
   __nv_bfloat16* linv_lo;
   uint32_t* dev_status;
   int64_t in_ld, out_ld;   // row strides of the partial matrices and of the outputs
-  const float* scale_diag; // optional: another matrix whose diagonal sets the scale of shift and floor (fp32)
-  int scale_n;
-  int64_t scale_ld;
 };
 
 __device__ __forceinline__ int off_slot(int i, int k) { return i * (i - 1) / 2 + k; }   // block (i, k), i > k
@@ -362,18 +361,28 @@ __device__ __forceinline__ void load_quad(const double* src, V4<double>& s) {
   s.v[0] += a.x; s.v[1] += a.y; s.v[2] += b.x; s.v[3] += b.y;
 }
 
-// Shared memory of every CTA (the same layout in all of them, so a local address maps to any peer), in elements of T:
-// off-diagonal blocks (own row: A, then L; other rows: L as it arrives), the blocks of the own column of the inverse
-// (transposed), and the published diagonal blocks.  The own diagonal block borrows a slot of the inverse that is not in
-// use yet (the last one, first written after the block has been factored) or never used by this CTA.
+// Shared memory of every CTA (the same layout in all of them, so a local address maps to any peer), in elements of T.
+// Up to eight blocks: off-diagonal blocks (own row: A, then L; other rows: L as it arrives), the blocks of the own column of
+// the inverse (transposed), and the published diagonal blocks.  The own diagonal block borrows a slot of the inverse that is
+// not in use yet (the last one, first written after the block has been factored) or never used by this CTA.
+// kBig, nine to sixteen blocks (a cluster of sixteen CTAs): what a CTA holds for good is its own row up to the diagonal
+// and its own column of the inverse from there on, sixteen slots together, and the diagonal block.  Received blocks are
+// needed during one step only: two sets of fifteen, used in turn, and a ring of six published diagonal blocks.  A set may
+// be overwritten once every warp of every CTA that reads it has said so (free_bar, two steps back).
 __host__ __device__ constexpr int x_slots(int nblk) { return nblk < 3 ? 3 : nblk; }
-template <typename T>
+constexpr int kBigBlk = 16, kBigPans = 6;
+constexpr int kReaders = 16;             // warps of a CTA that read received blocks or panels: follow-up, solver, bulk
+template <typename T, bool kBig>
 __host__ __device__ constexpr size_t smem_elems(int nblk) {
-  return (size_t)kBlk * (nblk * (nblk - 1) / 2 + x_slots(nblk)) + (size_t)nblk * kPan * kPanElems;
+  return kBig ? (size_t)kBlk * (kBigBlk + 1 + 2 * (kBigBlk - 1)) + (size_t)kBigPans * kPan * kPanElems
+              : (size_t)kBlk * (nblk * (nblk - 1) / 2 + x_slots(nblk)) + (size_t)nblk * kPan * kPanElems;
 }
 
-template <typename T>
-__global__ void __launch_bounds__(kCThreads, 1) small_block_cluster_kernel(SCParams p) {
+template <typename T, bool kBig>
+__global__ void __launch_bounds__(32 * warps_of(kBig), 1) small_block_cluster_kernel(SCParams p) {
+  constexpr int kWarps = warps_of(kBig), kCThreads = 32 * kWarps, kSendWarps = kBig ? 3 : 1;
+  constexpr int kMaxBlk = kBig ? kBigBlk : 8;              // block rows, and CTAs of the cluster
+  constexpr int kMaxOff = kMaxBlk * (kMaxBlk - 1) / 2;
   constexpr uint32_t kBlkBytes = (uint32_t)(kBlk * sizeof(T)), kGrpBytes = (uint32_t)(kGrp * sizeof(T));
   constexpr uint32_t kPanBytes = (uint32_t)(kPanElems * sizeof(T));
   extern __shared__ __align__(16) unsigned char sc_smem[];
@@ -383,6 +392,7 @@ __global__ void __launch_bounds__(kCThreads, 1) small_block_cluster_kernel(SCPar
   __shared__ __align__(8) uint64_t sol_bar[kMaxBlk][kPan];   // group g of L(own, k), k < own, or X(k, own) is solved
   __shared__ __align__(8) uint64_t rdy_bar[kMaxBlk];         // the block to solve at step k has every update
   __shared__ __align__(8) uint64_t bulk_bar[kMaxBlk];        // block j has every update but that of step j - 1
+  __shared__ __align__(8) uint64_t free_bar[kBig ? kMaxBlk : 1];   // every peer is done with what step k received
   __shared__ T s_red[kWarps];
   __shared__ T s_shift, s_floor;
   __shared__ int s_gave_up;
@@ -397,13 +407,18 @@ __global__ void __launch_bounds__(kCThreads, 1) small_block_cluster_kernel(SCPar
   const int noff = nblk * (nblk - 1) / 2;
   const bool active = me < nblk;
   T* off = reinterpret_cast<T*>(sc_smem);
-  T* xt = off + (size_t)noff * kBlk;                     // block (k, own) of the inverse at slot k
-  T* pans = xt + (size_t)x_slots(nblk) * kBlk;
-  T* own = xt + (size_t)(me + 2 <= nblk - 1 ? nblk - 1 : (me >= 1 ? 0 : 2)) * kBlk;
-  auto slot = [&](int i, int k) { return off + (size_t)off_slot(i, k) * kBlk; };
-  auto panel = [&](int k) { return pans + (size_t)k * kPan * kPanElems; };
+  T* xt = off + (size_t)noff * kBlk;                     // (small) block (k, own) of the inverse at slot k
+  T* pans = kBig ? off + (size_t)kBlk * (kBigBlk + 1 + 2 * (kBigBlk - 1)) : xt + (size_t)x_slots(nblk) * kBlk;
+  T* own = kBig ? off + (size_t)kBigBlk * kBlk : xt + (size_t)(me + 2 <= nblk - 1 ? nblk - 1 : (me >= 1 ? 0 : 2)) * kBlk;
+  // L(i, k) of another CTA's row (and, as an address in a peer, where this CTA's own L(me, k) is sent)
+  auto slot = [&](int i, int k) {
+    return kBig ? off + (size_t)(kBigBlk + 1 + (k & 1) * (kBigBlk - 1) + i - 1) * kBlk : off + (size_t)off_slot(i, k) * kBlk;
+  };
+  auto panel = [&](int k) { return pans + (size_t)(kBig ? k % kBigPans : k) * kPan * kPanElems; };
   // the block this CTA solves at step k, and where an update of block j (row: j < me, diagonal: j = me) goes
-  auto solved = [&](int k) { return k < me ? slot(me, k) : xt + (size_t)k * kBlk; };
+  auto solved = [&](int k) {
+    return kBig ? off + (size_t)k * kBlk : (k < me ? off + (size_t)off_slot(me, k) * kBlk : xt + (size_t)k * kBlk);
+  };
   auto target = [&](int j) { return j == me ? own : solved(j); };
 
   // A gated launch that is not needed leaves before any set-up: the same word in every CTA of the cluster, written at
@@ -419,18 +434,19 @@ __global__ void __launch_bounds__(kCThreads, 1) small_block_cluster_kernel(SCPar
     bar_init(&next_bar[k][q], 1);
     bar_init(&sol_bar[k][q], 4);
     if (q == 0) { bar_init(&rdy_bar[k], 4); bar_init(&bulk_bar[k], 2); }
+    if (kBig && q == 1) bar_init(&free_bar[k], (uint32_t)(kReaders * (nblk - 1)));
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     if (active && k < nblk && k != me) bar_expect(&pan_bar[k][q], kPanBytes);
     if (active && k + 1 < nblk && k + 1 != me) bar_expect(&next_bar[k][q], kGrpBytes);
-  } else if (tid >= 64 && tid < 64 + kMaxOff) {
-    const int b = tid - 64;
+  } else if (tid >= kMaxBlk * kPan && tid < kMaxBlk * kPan + kMaxOff) {
+    const int b = tid - kMaxBlk * kPan;
     int i = 1;
     while (off_slot(i + 1, 0) <= b) ++i;
     const int k = b - off_slot(i, 0);
     bar_init(&off_bar[b], 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     if (active && i < nblk && i != me && i >= k + 2 && (me <= k || me > i)) bar_expect(&off_bar[b], kBlkBytes);
-  } else if (tid == 64 + kMaxOff) {
+  } else if (tid == kMaxBlk * kPan + kMaxOff) {
     s_gave_up = 0;
   }
   __syncthreads();
@@ -444,19 +460,14 @@ __global__ void __launch_bounds__(kCThreads, 1) small_block_cluster_kernel(SCPar
   {
     const T* parts = (const T*)p.partials;
     T t = (T)0;
-    const int n_scale = p.scale_diag ? p.scale_n : r;
-    if (p.scale_diag) {
-      for (int i = tid; i < n_scale; i += kCThreads) t += (T)__ldg(p.scale_diag + (int64_t)i * (p.scale_ld + 1));
-    } else {
-      for (int i = tid; i < r; i += kCThreads) {
-        T d = (T)0;
-        for (int q = 0; q < p.n_partials; ++q)
-          d += __ldg(parts + (int64_t)q * p.partial_stride + (int64_t)i * p.in_ld + i);
-        t += d;
-      }
+    for (int i = tid; i < r; i += kCThreads) {
+      T d = (T)0;
+      for (int q = 0; q < p.n_partials; ++q)
+        d += __ldg(parts + (int64_t)q * p.partial_stride + (int64_t)i * p.in_ld + i);
+      t += d;
     }
     constexpr int kQuads = kB * kB / 4;
-    constexpr int kPerThread = ((Cfg<T>::kMaxR / kB) * kQuads + kCThreads - 1) / kCThreads;
+    constexpr int kPerThread = ((kBig ? kBigBlk : Cfg<T>::kMaxR / kB) * kQuads + kCThreads - 1) / kCThreads;
     V4<T> acc[kPerThread];
     const int n_quads = active ? (me + 1) * kQuads : 0;
 #pragma unroll
@@ -477,7 +488,7 @@ __global__ void __launch_bounds__(kCThreads, 1) small_block_cluster_kernel(SCPar
     if (tid == 0) {
       T tr = (T)0;
       for (int q = 0; q < kWarps; ++q) tr += s_red[q];
-      T mean_diag = tr / (T)n_scale;
+      T mean_diag = tr / (T)r;
       if (!(mean_diag == mean_diag) || mean_diag > (T)3.0e38 || mean_diag < (T)0) {
         if (p.dev_status && me == 0) atomicOr(p.dev_status, LORACT_DEV_NONFINITE);
         mean_diag = (T)1;
@@ -511,22 +522,33 @@ __global__ void __launch_bounds__(kCThreads, 1) small_block_cluster_kernel(SCPar
   volatile int* gave_up = &s_gave_up;
   const T floor_ = s_floor;
   const int role = kRoleOf[warp];
-  const bool peer = lane < nblk && lane != me;
-  // Lane c copies something this CTA has finished to CTA c, if `to_me` says so.  Whoever wrote it arrived on a barrier
+  // the CTA this lane signals and copies to: the next one of the chain first
+  const int to = lane < nblk ? (me + 1 + lane) % nblk : 0;
+  const bool peer = lane + 1 < nblk;
+  // Each lane copies something this CTA has finished to its CTA `to`, if `wanted` there.  Whoever wrote it arrived on a barrier
   // this warp has waited for (or is this warp); the proxy fence makes those stores visible to the copy.
-  auto send = [&](const T* what, uint32_t bytes, uint64_t* bar, bool to_me) {
+  auto send = [&](const T* what, const T* where, uint32_t bytes, uint64_t* bar, bool wanted) {
     fence_async_proxy();
     __syncwarp();
-    if (to_me) {
-      const uint32_t src = smem_addr(what);
-      bulk_to_peer(map_to_cta(src, lane), src, bytes, map_to_cta(smem_addr(bar), lane));
-    }
+    if (wanted) bulk_to_peer(map_to_cta(smem_addr(where), to), smem_addr(what), bytes, map_to_cta(smem_addr(bar), to));
   };
+  // kBig: this warp has read all it will of what step k brought here.  Relaxed: the values have been used, nothing this
+  // warp wrote has to become visible with the arrival.
+  auto done_with = [&](int k) {
+    if (!kBig || k + 2 >= nblk) return;
+    __syncwarp();
+    if (peer)
+      asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];"
+                   ::"r"(map_to_cta(smem_addr(&free_bar[k]), to)) : "memory");
+  };
+  // kBig: before the first copy of step k leaves: its set of slots was last used two steps ago
+  auto may_send = [&](int k) { if (kBig && k >= 2) bar_wait(&free_bar[k - 2], gave_up); };
   if (!active) {
     // a CTA without a block row (the cluster size is a power of two)
   } else if (role == R_PIVOT) {
     const bool clamped = factor_diagonal<T>(own, panel(me), pan_bar[me], floor_, lane);
-    send(panel(me) + (kPan - 1) * kPanElems, kPanBytes, &pan_bar[me][kPan - 1], peer);
+    if (kBig && me >= kBigPans) bar_wait(&free_bar[me - kBigPans], gave_up);   // the ring slot is free in every peer
+    send(panel(me) + (kPan - 1) * kPanElems, panel(me) + (kPan - 1) * kPanElems, kPanBytes, &pan_bar[me][kPan - 1], peer);
     if (clamped && lane == 0 && p.dev_status) atomicOr(p.dev_status, LORACT_DEV_PIVOT_CLAMPED);
   } else if (role < R_SOLVE) {
     // ---- follow-up warps: lane = row, columns 8 w .. 8 w + 7
@@ -553,6 +575,7 @@ __global__ void __launch_bounds__(kCThreads, 1) small_block_cluster_kernel(SCPar
           if (j != me) bar_wait(&next_bar[k][q], gave_up);
           take_off_group<T>(acc, A + q * kGrp, Bm + q * kGrp, w, lane);
         }
+        done_with(k);
       }
       if (j != me) {
 #pragma unroll
@@ -597,10 +620,10 @@ __global__ void __launch_bounds__(kCThreads, 1) small_block_cluster_kernel(SCPar
       }
       solve_half<T, 0>(acc, blk, panel(k), pan_bar[k], sol_bar[k], k >= me, row, lane, gave_up);
       solve_half<T, 1>(acc, blk, panel(k), pan_bar[k], sol_bar[k], k >= me, row, lane, gave_up);
+      done_with(k);
     }
   } else if (role < R_SEND) {
-    // ---- bulk warps: the updates of step k to blocks beyond k + 1 (block j always by the same pair of warps), and the
-    // output
+    // ---- bulk warps: the updates of step k to blocks beyond k + 1, and the output
     const int m = role - R_BULK;
     const int col = me * kB + lane;
     float wdiag = 0.f, est = 0.f;
@@ -625,11 +648,12 @@ __global__ void __launch_bounds__(kCThreads, 1) small_block_cluster_kernel(SCPar
       bar_wait(&sol_bar[k][kPan - 1], gave_up);
       const int j_end = k < me ? me + 1 : nblk;
       for (int j = k + 2; j < j_end; ++j) {
-        if ((j & 3) != (m >> 1)) continue;
+        if ((j & 3) != (m >> 1)) continue;                     // the same pair of warps for a block in every step
         if (j != me) bar_wait(&off_bar[off_slot(j, k)], gave_up);
         take_off_half<T>(target(j), blk, j == me ? blk : slot(j, k), k == me, m & 1, lane);
         if (j == k + 2) warp_arrive(&bulk_bar[j], lane);
       }
+      done_with(k);
       if (k < me) continue;
       // rows 32 k + 4 m .. + 3 of the result: element (32 k + 4 m + u, col) = X[group m][lane][u]
       const V4<T> v4 = ld4(blk + m * kGrp + lane * 4);
@@ -657,22 +681,26 @@ __global__ void __launch_bounds__(kCThreads, 1) small_block_cluster_kernel(SCPar
                      : "memory");
     }
   } else {
-    // ---- the sender
-    for (int k = 0; k + 1 < me; ++k) {
+    // ---- senders
+    const int w = role - R_SEND;
+    for (int k = w; k + 1 < me; k += kSendWarps) {
       bar_wait(&sol_bar[k][kPan - 1], gave_up);
-      send(slot(me, k), kBlkBytes, &off_bar[off_slot(me, k)], peer && (lane <= k || lane > me));
+      may_send(k);
+      send(solved(k), slot(me, k), kBlkBytes, &off_bar[off_slot(me, k)], peer && (to <= k || to > me));
     }
     if (me > 0) {
 #pragma unroll 1
-      for (int q = 0; q < kPan; ++q) {
+      for (int q = w; q < kPan; q += kSendWarps) {
         bar_wait(&sol_bar[me - 1][q], gave_up);
-        send(slot(me, me - 1) + q * kGrp, kGrpBytes, &next_bar[me - 1][q], peer);
+        may_send(me - 1);
+        send(solved(me - 1) + q * kGrp, slot(me, me - 1) + q * kGrp, kGrpBytes, &next_bar[me - 1][q], peer);
       }
     }
+    // (every peer is done with what the ring slot of this panel held: a later step has been waited for above)
 #pragma unroll 1
-    for (int q = 0; q + 1 < kPan; ++q) {   // (the pivot warp sends the last one itself)
+    for (int q = w; q + 1 < kPan; q += kSendWarps) {   // (the pivot warp sends the last one itself)
       bar_wait(&pan_bar[me][q], gave_up);
-      send(panel(me) + q * kPanElems, kPanBytes, &pan_bar[me][q], peer);
+      send(panel(me) + q * kPanElems, panel(me) + q * kPanElems, kPanBytes, &pan_bar[me][q], peer);
     }
   }
   __syncthreads();
@@ -716,7 +744,7 @@ __global__ void __cluster_dims__(2, 1, 1) cluster_wait_probe_kernel(uint32_t* de
   cluster_wait();
 }
 
-template <typename T>
+template <typename T, bool kBig>
 cudaError_t launch_cluster(const SCParams& p, cudaStream_t stream) {
   const int nblk = (p.r + kB - 1) / kB;
   int ctas = 1;                           // cluster sizes are powers of two
@@ -725,14 +753,17 @@ cudaError_t launch_cluster(const SCParams& p, cudaStream_t stream) {
   int dev = 0;
   LORACT_CUDA_TRY(cudaGetDevice(&dev));
   if (dev < 0 || dev >= 64 || !configured[dev].load(std::memory_order_acquire)) {
-    LORACT_CUDA_TRY(cudaFuncSetAttribute(small_block_cluster_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)(smem_elems<T>(Cfg<T>::kMaxR / kB) * sizeof(T))));
+    LORACT_CUDA_TRY(cudaFuncSetAttribute(small_block_cluster_kernel<T, kBig>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)(smem_elems<T, kBig>(Cfg<T>::kMaxR / kB) * sizeof(T))));
+    if (kBig)   // a cluster of sixteen CTAs
+      LORACT_CUDA_TRY(cudaFuncSetAttribute(small_block_cluster_kernel<T, kBig>,
+                                           cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
     if (dev >= 0 && dev < 64) configured[dev].store(true, std::memory_order_release);
   }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(ctas, 1, 1);
-  cfg.blockDim = dim3(kCThreads, 1, 1);
-  cfg.dynamicSmemBytes = smem_elems<T>(nblk) * sizeof(T);
+  cfg.blockDim = dim3(32 * warps_of(kBig), 1, 1);
+  cfg.dynamicSmemBytes = smem_elems<T, kBig>(nblk) * sizeof(T);
   cfg.stream = stream;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -743,7 +774,7 @@ cudaError_t launch_cluster(const SCParams& p, cudaStream_t stream) {
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  LORACT_CUDA_TRY(cudaLaunchKernelEx(&cfg, small_block_cluster_kernel<T>, p));
+  LORACT_CUDA_TRY(cudaLaunchKernelEx(&cfg, small_block_cluster_kernel<T, kBig>, p));
   count_launch(__func__, stream);
   return cudaGetLastError();
 }
@@ -758,8 +789,8 @@ cudaError_t small_block_cluster_wait_probe_launch(uint32_t* dev_status, uint64_t
 
 bool small_block_cluster_supported(const SmallBlockArgs& a) {
   if (a.linv_full != nullptr || ((uintptr_t)a.partials & 15) || a.partial_stride % 4 || a.in_ld % 4 || a.r % 4) return false;
-  if (a.use_f64) return a.partial_type == ELEM_F64 && a.r <= Cfg<double>::kMaxR && a.scale_diag == nullptr;
-  return a.partial_type == ELEM_F32 && a.r <= Cfg<float>::kMaxR;
+  if (a.use_f64) return a.partial_type == ELEM_F64 && a.r <= Cfg<double>::kMaxR;
+  return a.partial_type == ELEM_F32 && a.r <= kBigBlk * kB;
 }
 
 cudaError_t small_block_cluster_launch(const SmallBlockArgs& a, cudaStream_t stream) {
@@ -779,10 +810,8 @@ cudaError_t small_block_cluster_launch(const SmallBlockArgs& a, cudaStream_t str
   p.linv_hi = a.linv_hi;
   p.linv_lo = a.linv_lo;
   p.dev_status = a.dev_status;
-  p.scale_diag = a.scale_diag;
-  p.scale_n = a.scale_n;
-  p.scale_ld = a.scale_ld;
-  return a.use_f64 ? launch_cluster<double>(p, stream) : launch_cluster<float>(p, stream);
+  if (a.use_f64) return launch_cluster<double, false>(p, stream);
+  return a.r <= Cfg<float>::kMaxR ? launch_cluster<float, false>(p, stream) : launch_cluster<float, true>(p, stream);
 }
 
 }  // namespace loract

@@ -20,7 +20,9 @@ def dev():
 
 
 @pytest.mark.parametrize("f64,r,n_partials", [(False, 24, 1), (False, 40, 2), (False, 104, 1), (False, 136, 3),
-                                              (False, 232, 1), (False, 248, 2), (True, 16, 1), (True, 24, 3), (True, 40, 1),
+                                              (False, 232, 1), (False, 248, 2), (False, 264, 1),
+                                              (False, 288, 3), (False, 296, 1), (False, 360, 2), (False, 424, 1),
+                                              (False, 480, 1), (False, 488, 4), (False, 504, 1), (False, 512, 2), (True, 16, 1), (True, 24, 3), (True, 40, 1),
                                               (True, 64, 2), (True, 96, 8), (True, 136, 1), (True, 160, 4), (True, 184, 1),
                                               (True, 192, 2), (True, 200, 1)])
 def test_inverse_factor_at_tile_edges(dev, f64, r, n_partials):
@@ -46,10 +48,9 @@ def test_inverse_factor_at_tile_edges(dev, f64, r, n_partials):
     assert np.abs(pair - X).max() <= 2.0 ** -15 * np.abs(X).max()
 
 
-@pytest.mark.parametrize("f64", [False, True])
-@pytest.mark.parametrize("at", [0, 3, 4, 17, 31, 32, 50, 95])
-def test_clamped_pivot_drops_its_column_only(dev, f64, at):
-    r = 96
+@pytest.mark.parametrize("f64,r,at", [(f64, 96, at) for f64 in (False, True) for at in (0, 3, 4, 17, 31, 32, 50, 95)] +
+                         [(False, 320, 0), (False, 512, 100), (False, 512, 511)])
+def test_clamped_pivot_drops_its_column_only(dev, f64, r, at):
     W = spd(r, 1e2, seed=at)
     W[at, :] = 0.0
     W[:, at] = 0.0                                     # a pivot of exactly zero, coupled to nothing
