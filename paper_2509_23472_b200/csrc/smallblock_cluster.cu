@@ -18,7 +18,8 @@
 //   * sender warps (one, above eight blocks three taking turns) copy finished groups and blocks to the CTAs that need them (bulk
 //     distributed-shared-memory copies; one round of wait, proxy fence and up to fifteen copies takes longer than a group).
 // A block is stored as eight groups of [32 rows][4 columns]: a group is one contiguous copy, a lane's row and a
-// broadcast row are one 16-byte load each, without bank conflicts.  Loops over groups are rolled.  The hand-offs of the
+// broadcast row are one 16-byte load each, without bank conflicts.  Loops are rolled: the kernel runs cold in every call, and
+// fetching its code is part of its time (90 KB instead of 50 cost 2 to 4 us a launch).  The hand-offs of the
 // pivot warp are named barriers (31 cycles against 110 for an mbarrier), all others are mbarriers that complete once.
 //
 // Shared-memory rates that fixed the shapes (measured on B200, cycles of the SM's pipe per warp instruction): a 16-byte
@@ -128,6 +129,7 @@ __device__ __forceinline__ uint64_t timer_ns() {
 __device__ __forceinline__ bool bar_wait(uint64_t* bar, volatile int* gave_up, uint64_t limit_ns = kClusterWaitNs) {
   if (bar_try(bar)) return true;
   uint64_t t0 = 0;
+#pragma unroll 1
   for (uint32_t spin = 1;; ++spin) {
     if (bar_try(bar)) return true;
     if ((spin & 255u) == 0u) {
@@ -460,8 +462,10 @@ __global__ void __launch_bounds__(32 * warps_of(kBig), 1) small_block_cluster_ke
   {
     const T* parts = (const T*)p.partials;
     T t = (T)0;
+#pragma unroll 1
     for (int i = tid; i < r; i += kCThreads) {
       T d = (T)0;
+#pragma unroll 4
       for (int q = 0; q < p.n_partials; ++q)
         d += __ldg(parts + (int64_t)q * p.partial_stride + (int64_t)i * p.in_ld + i);
       t += d;
@@ -478,6 +482,7 @@ __global__ void __launch_bounds__(32 * warps_of(kBig), 1) small_block_cluster_ke
       const int row = me * kB + ((e & (kQuads - 1)) >> 3), col = (e / kQuads) * kB + 4 * (e & 7);
       if (row < r && col < r) {
         const T* src = parts + (int64_t)row * p.in_ld + col;
+#pragma unroll 4
         for (int q = 0; q < p.n_partials; ++q) load_quad(src + (int64_t)q * p.partial_stride, acc[u]);
       }
     }
@@ -487,6 +492,7 @@ __global__ void __launch_bounds__(32 * warps_of(kBig), 1) small_block_cluster_ke
     __syncthreads();
     if (tid == 0) {
       T tr = (T)0;
+#pragma unroll 1
       for (int q = 0; q < kWarps; ++q) tr += s_red[q];
       T mean_diag = tr / (T)r;
       if (!(mean_diag == mean_diag) || mean_diag > (T)3.0e38 || mean_diag < (T)0) {
@@ -553,6 +559,7 @@ __global__ void __launch_bounds__(32 * warps_of(kBig), 1) small_block_cluster_ke
   } else if (role < R_SOLVE) {
     // ---- follow-up warps: lane = row, columns 8 w .. 8 w + 7
     const int w = role - R_FOLLOW;
+#pragma unroll 1
     for (int k = -1; k + 1 < nblk; ++k) {
       // step k: the block that step k + 1 works on takes L(own, k) or X(k, own) off, group by group
       const int j = k + 1;
@@ -605,6 +612,7 @@ __global__ void __launch_bounds__(32 * warps_of(kBig), 1) small_block_cluster_ke
   } else if (role < R_BULK) {
     // ---- solver warps: eight rows each
     const int row = 8 * (role - R_SOLVE) + (lane & 7), cg = lane >> 3;
+#pragma unroll 1
     for (int k = 0; k < nblk; ++k) {
       T* blk = solved(k);
       V4<T> acc[2];
@@ -631,11 +639,13 @@ __global__ void __launch_bounds__(32 * warps_of(kBig), 1) small_block_cluster_ke
       // for the estimate: the diagonal entry of this lane's column, as factored
       const T* parts = (const T*)p.partials;
       T d = (T)0;
+#pragma unroll 4
       for (int q = 0; q < p.n_partials; ++q)
         d += __ldg(parts + (int64_t)q * p.partial_stride + (int64_t)col * p.in_ld + col);
       wdiag = (float)(d + d * (T)p.shift_diag_rel + s_shift);
     }
     // zeros above the diagonal block
+#pragma unroll 1
     for (int row = m; row < me * kB; row += kBulkWarps) {
       if (col >= r) continue;
       const int64_t o = (int64_t)row * p.out_ld + col;
@@ -643,10 +653,12 @@ __global__ void __launch_bounds__(32 * warps_of(kBig), 1) small_block_cluster_ke
       if (p.linv_hi) p.linv_hi[o] = __float2bfloat16(0.f);
       if (p.linv_lo) p.linv_lo[o] = __float2bfloat16(0.f);
     }
+#pragma unroll 1
     for (int k = 0; k < nblk; ++k) {
       const T* blk = solved(k);
       bar_wait(&sol_bar[k][kPan - 1], gave_up);
       const int j_end = k < me ? me + 1 : nblk;
+#pragma unroll 1
       for (int j = k + 2; j < j_end; ++j) {
         if ((j & 3) != (m >> 1)) continue;                     // the same pair of warps for a block in every step
         if (j != me) bar_wait(&off_bar[off_slot(j, k)], gave_up);
@@ -683,6 +695,7 @@ __global__ void __launch_bounds__(32 * warps_of(kBig), 1) small_block_cluster_ke
   } else {
     // ---- senders
     const int w = role - R_SEND;
+#pragma unroll 1
     for (int k = w; k + 1 < me; k += kSendWarps) {
       bar_wait(&sol_bar[k][kPan - 1], gave_up);
       may_send(k);
@@ -711,6 +724,7 @@ __global__ void __launch_bounds__(32 * warps_of(kBig), 1) small_block_cluster_ke
   if (p.gate_out && me == 0 && tid == 0) {
     // after the cluster barrier: every share has arrived, every status bit of this call is set
     float est = 0.f;
+#pragma unroll 1
     for (int c = 0; c < kBulkWarps * nblk; ++c) est += s_est[c];
     const uint32_t st = p.dev_status ? atomicOr(p.dev_status, 0u) : 0u;
     const bool again = !(est <= p.gate_threshold) || st != 0u;
