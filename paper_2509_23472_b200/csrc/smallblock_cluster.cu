@@ -15,7 +15,7 @@
 //     factored, and later the block column of the inverse, whose transpose solves the same system.  No inverse of a
 //     diagonal block is formed.
 //   * bulk warps (eight, two to a block): the updates nobody waits for, and the output.
-//   * sender warps (one, above eight blocks three taking turns) copy finished groups and blocks to the CTAs that need them (bulk
+//   * sender warps (three taking turns, one in fp64) copy finished groups and blocks to the CTAs that need them (bulk
 //     distributed-shared-memory copies; one round of wait, proxy fence and up to fifteen copies takes longer than a group).
 // A block is stored as eight groups of [32 rows][4 columns]: a group is one contiguous copy, a lane's row and a
 // broadcast row are one 16-byte load each, without bank conflicts.  Loops are rolled: the kernel runs cold in every call, and
@@ -27,10 +27,10 @@
 // a warp barrier take 30 cycles, a bulk copy to another CTA 280 (512 bytes) to 480 (4.6 KB) or 730 with seven receivers.
 //
 // Measured (one Gram matrix, back to back, against a form with one chain CTA, workers that sent blocks back to it and an
-// inverse of every diagonal block): fp32 r = 32 / 64 / 128 / 256: 7.1 / 8.5 / 13.8 / 28.8 us (7.4 / 11.8 / 20.0 / 40.4).
-// r = 336 / 512, against two factorisations of up to 256 columns joined by fp32 products: 42 / 74 us (69 / 91, and six
+// inverse of every diagonal block): fp32 r = 32 / 64 / 128 / 256: 6.9 / 9.0 / 14.1 / 27.9 us (7.4 / 11.8 / 20.0 / 40.4).
+// r = 336 / 512, against two factorisations of up to 256 columns joined by fp32 products: 42 / 71 us (69 / 91, and six
 // helper launches fewer).  Above eight blocks the early steps are bound by the bulk updates and by what an SM can send.
-// fp64, against a kernel that kept the matrix in global memory: r = 64 / 96 / 192: 13.0 / 17.7 / 33.7 us (75.8 / 120.9 /
+// fp64, against a kernel that kept the matrix in global memory: r = 64 / 96 / 192: 13.4 / 18.0 / 31.9 us (75.8 / 120.9 /
 // 282).  Cycles per group of four columns: 398 in the pivot warp alone, about 475 with its companions at work; the step
 // from one diagonal block to the next adds about 1000.
 //
@@ -46,8 +46,12 @@ namespace loract {
 namespace {
 
 constexpr int kB = 32;                   // block edge
-constexpr int kMaxWarps = 20;            // two senders fewer up to eight blocks
-__host__ __device__ constexpr int warps_of(bool big) { return big ? kMaxWarps : kMaxWarps - 2; }
+constexpr int kMaxWarps = 20;
+// fp32: three senders.  An SM issues a copy of one group every 56 cycles, so that a sender which waits, fences and copies to
+// seven peers falls behind the groups (one sender: r = 224 / 256 25.5 / 29.8 us instead of 24.4 / 28.8).  fp64, at most
+// six blocks and a slower chain: one (three: 0.2 to 0.6 us more).
+template <typename T> __host__ __device__ constexpr int senders_of() { return sizeof(T) == 8 ? 1 : 3; }
+template <typename T> __host__ __device__ constexpr int warps_of() { return kMaxWarps - 3 + senders_of<T>(); }
 constexpr int kPan = 8;                  // groups of four columns in a block
 constexpr uint64_t kClusterWaitNs = 50000000ull;  // 50 ms
 // Warp -> role (plus the index inside the role).  The scheduler a warp shares is its number mod 4: the pivot warp's
@@ -322,36 +326,43 @@ __device__ __forceinline__ void take_off_group(V4<T> (&acc)[2], const T* A, cons
 #pragma unroll
     for (int j = 0; j < 4; ++j) acc[h].v[j] = sub4(acc[h].v[j], a, ld4(Bg + (8 * w + 4 * h + j) * 4));
 }
-// C (or zero) -= A B^T for rows 16 half .. 16 half + 15 of a block, 4 x 4 outputs per lane: rows tm + 4 i (one address per
-// quarter warp), columns tn + 8 j (32 consecutive rows of B).
+// C (or zero) -= A B^T for columns 16 half .. 16 half + 15 of a block, 4 x 4 outputs per lane: rows row0 + 8 i, columns
+// col0 + 4 j.  With eight warps at it the shared-memory pipe is the bound: per group four loads of A at four cycles, four of
+// B at two (two addresses per quarter warp), and C in single elements without conflicts (a warp access covers eight rows of a
+// group); one warp alone waits for its loads, hence the unrolled loop (fp32 by eight: the code costs small launches 2 us).
+// Against rows 16 half .., with conflicts on C, unrolled by two: 2340 -> 2200 cycles for eight halves with eight warps, 1350
+// -> 1100 with one; r = 256 / 512 28.8 / 74 -> 27.9 / 71 us.  A whole block per warp (a third fewer loads) or two halves at a
+// time (a quarter fewer) leave too few warps at work: r = 512 75 and 73 us.
 template <typename T>
 __device__ __forceinline__ void take_off_half(T* C, const T* A, const T* Bm, bool from_zero, int half, int lane) {
-  const int row0 = 16 * half + (lane >> 3), col0 = lane & 7;
+  const int row0 = (lane & 3) + 4 * (lane >> 4), col0 = (lane >> 2) & 3;
+  C += 4 * half * kGrp + row0 * 4 + col0;
+  A += row0 * 4;
+  Bm += (16 * half + col0) * 4;
   T acc[4][4];
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int j = 0; j < 4; ++j)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = (T)0;
-#pragma unroll 2
+    for (int i = 0; i < 4; ++i) acc[i][j] = from_zero ? (T)0 : C[j * kGrp + 32 * i];
+  constexpr int kUnroll = sizeof(T) == 8 ? 8 : 4;
+#pragma unroll kUnroll
   for (int q = 0; q < kPan; ++q) {
-    V4<T> b[4];
+    V4<T> a[4], b[4];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) b[j] = ld4(Bm + q * kGrp + (col0 + 8 * j) * 4);
+    for (int j = 0; j < 4; ++j) b[j] = ld4(Bm + q * kGrp + 16 * j);
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const V4<T> a = ld4(A + q * kGrp + (row0 + 4 * i) * 4);
+    for (int i = 0; i < 4; ++i) a[i] = ld4(A + q * kGrp + 32 * i);
 #pragma unroll
-      for (int j = 0; j < 4; ++j) acc[i][j] = sub4(acc[i][j], a, b[j]);
-    }
+    for (int u = 0; u < 4; ++u)
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = fma(-a[i].v[u], b[j].v[u], acc[i][j]);
   }
 #pragma unroll
   for (int j = 0; j < 4; ++j)
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int col = col0 + 8 * j;
-      T* c = C + (col >> 2) * kGrp + (row0 + 4 * i) * 4 + (col & 3);
-      *c = from_zero ? acc[i][j] : *c + acc[i][j];
-    }
+    for (int i = 0; i < 4; ++i) C[j * kGrp + 32 * i] = acc[i][j];
 }
 
 __device__ __forceinline__ void load_quad(const float* src, V4<float>& s) {
@@ -381,8 +392,8 @@ __host__ __device__ constexpr size_t smem_elems(int nblk) {
 }
 
 template <typename T, bool kBig>
-__global__ void __launch_bounds__(32 * warps_of(kBig), 1) small_block_cluster_kernel(SCParams p) {
-  constexpr int kWarps = warps_of(kBig), kCThreads = 32 * kWarps, kSendWarps = kBig ? 3 : 1;
+__global__ void __launch_bounds__(32 * warps_of<T>(), 1) small_block_cluster_kernel(SCParams p) {
+  constexpr int kWarps = warps_of<T>(), kCThreads = 32 * kWarps, kSendWarps = senders_of<T>();
   constexpr int kMaxBlk = kBig ? kBigBlk : 8;              // block rows, and CTAs of the cluster
   constexpr int kMaxOff = kMaxBlk * (kMaxBlk - 1) / 2;
   constexpr uint32_t kBlkBytes = (uint32_t)(kBlk * sizeof(T)), kGrpBytes = (uint32_t)(kGrp * sizeof(T));
@@ -776,7 +787,7 @@ cudaError_t launch_cluster(const SCParams& p, cudaStream_t stream) {
   }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(ctas, 1, 1);
-  cfg.blockDim = dim3(32 * warps_of(kBig), 1, 1);
+  cfg.blockDim = dim3(32 * warps_of<T>(), 1, 1);
   cfg.dynamicSmemBytes = smem_elems<T, kBig>(nblk) * sizeof(T);
   cfg.stream = stream;
   cudaLaunchAttribute attr[2];
