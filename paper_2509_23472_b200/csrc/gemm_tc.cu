@@ -60,6 +60,7 @@ struct TcParams {
   int tma_store;      // 1: the epilogue stages 32-row boxes in shared memory and writes them with TMA stores
   int st_m_tiles;     // streaming kernel: 256-row tiles along M
   int st_units;       // streaming kernel: tiles in all (column tile major, then M)
+  int st_keep_a;      // streaming kernel: ask for A to stay in L2
   int st_stages;      // streaming kernel: stages of the A ring (<= kStreamStages)
   int store_bufs;     // staging boxes per epilogue warp (1 or 2; fused epilogue: 2 or 3)
   int fuse_parts;     // fused epilogue: warps per quarter of the accumulator's rows
@@ -598,6 +599,11 @@ __device__ __forceinline__ void tma_load_2d_pair_hint(void* smem_dst, const CUte
       ::"r"(smem_u32(smem_dst)), "l"((uint64_t)map), "r"(bar_cluster_addr), "r"(x), "r"(y), "l"(policy)
       : "memory");
 }
+__device__ __forceinline__ uint64_t l2_policy_evict_normal() {
+  uint64_t pol;
+  asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(pol));
+  return pol;
+}
 __device__ __forceinline__ uint64_t l2_policy_evict_last() {
   uint64_t pol;
   asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(pol));
@@ -822,6 +828,10 @@ gemm_tc_pair_kernel(const __grid_constant__ TmapPack maps, const TcParams p) {
 // acc_full[j] (each CTA, by commit): buffer j holds a finished tile; acc_empty[j] (leader, one arrival
 // per CTA, sent by the first epilogue warp once all eight have arrived on the CTA's own epi_done[j]): buffer j has been read in both CTAs.  No load uses cluster multicast.
 constexpr int kStreamStages = 6;
+// Every column tile reads A again, while the output (and the matrix it is combined with) passes through L2 once: loads of A
+// ask to stay.  16384 x 11008, K = 512 (A 17 MB): reconstruction 162 -> 152 us, SiLU backward 215 -> 205; 49152 x 3072 (A
+// 50 MB) 174 -> 170 and 207 -> 203.  At 67 MB, more than half of L2, it makes no difference: not asked for there.
+constexpr long long kStreamKeepBytes = 60ll << 20;
 constexpr int kStreamSmemMax = 226 * 1024;                 // dynamic shared memory the streaming kernel may ask for
 
 // An arrival on a barrier of the peer CTA.  Relaxed: it announces that tensor-memory reads have completed
@@ -865,20 +875,30 @@ __device__ __forceinline__ bool mbar_wait_cluster_bounded(uint64_t* bar, uint32_
 // boxes ahead by each epilogue warp for itself; the result overwrites E in the box and leaves by TMA from there.
 // The epilogue is bound by the instructions it issues and their latency: up to sixteen warps, four per quarter of the
 // accumulator's rows.  Measured, SiLU / GELU backward: 16384 x 11008, K = 512: 686 / 670 us with direct loads, 252 / 376
-// with the boxes and eight warps, 227 / 251 with twelve and the derivatives written out; 16384 x 4096, K = 256: 258 / 251,
-// 96 / 141, 67 / 80 (floor 43).
+// with the boxes and eight warps, 227 / 251 with twelve and the derivatives written out, 207 / 234 now; 16384 x 4096,
+// K = 256: 258 / 251, 96 / 141, 67 / 80, 60 / 73 (floor 43).  Of the 207, 187 are left without the derivatives, 152 without
+// E as well: SiLU's two special-function instructions an element (16 lanes a cycle) and the shared-memory pipe, which the
+// operands, E and the result share.  An L2 prefetch of E or plain stores of the result cost more than they save.
 enum EpKind : int { EP_NONE = 0, EP_RMS = 1, EP_SILU = 2, EP_GELU = 3 };
 constexpr int kFuseMaxBufs = 3;
 constexpr int kFuseMaxWarps = 16;
 constexpr uint32_t kFuseBoxBytes = 2048;                   // 32 rows x 64 bytes
 
 // Boxes of 32 columns that one epilogue warp goes through: every fuse_parts-th box of its row group, running on from unit to
-// unit (so that a number of warps that does not divide the boxes of a tile is balanced over several tiles).
+// unit (so that a number of warps that does not divide the boxes of a tile is balanced over several tiles).  Row and
+// column are carried along: divisions, about three a box, were a tenth of the kernel (SiLU, 16384 x 4096, K = 256: 66 ->
+// 60 us).
 struct FuseCursor {
-  int u, c0;
+  int u, mt, c0;         // unit, its row tile, column inside the tile
+  int row, n0;           // first row of the box, first column of the tile
   __device__ __forceinline__ void advance(const TcParams& p) {
     c0 += 32 * p.fuse_parts;
-    while (c0 >= p.bn) { c0 -= p.bn; ++u; }
+    while (c0 >= p.bn) {
+      c0 -= p.bn;
+      ++u;
+      row += 2 * kBM;
+      if (++mt == p.st_m_tiles) { mt = 0; row -= p.st_m_tiles * 2 * kBM; n0 += p.bn; }
+    }
   }
 };
 
@@ -898,11 +918,10 @@ __device__ __forceinline__ void fused_epilogue(const TcParams& p, const TmapPack
   const uint32_t bufs = (uint32_t)p.store_bufs;
   const int threads = 128 * p.fuse_parts;    // of all epilogue warps
   const __nv_bfloat16* gamma = (const __nv_bfloat16*)p.ep_col;
-  auto row_of = [&](int u) { return ((u % p.st_m_tiles) * 2 + cta_rank) * kBM + quad * 32; };
-  auto col_of = [&](const FuseCursor& k) { return (k.u / p.st_m_tiles) * p.bn + k.c0; };
   // boxes outside the output are neither loaded nor stored
-  auto live = [&](const FuseCursor& k) { return row_of(k.u) < p.M && col_of(k) < p.N; };
-  FuseCursor ld{u_begin, 32 * part}, k = ld;
+  auto live = [&](const FuseCursor& k) { return k.row < p.M && k.n0 + k.c0 < p.N; };
+  const int nt_begin = u_begin / p.st_m_tiles, mt_begin = u_begin - nt_begin * p.st_m_tiles;
+  FuseCursor ld{u_begin, mt_begin, 32 * part, (2 * mt_begin + cta_rank) * kBM + quad * 32, nt_begin * p.bn}, k = ld;
   uint32_t n_ld = 0, n_use = 0;              // live boxes requested / used so far
   uint32_t ld_slot = 0, use_slot = 0, use_phase = 0;
   auto request = [&]() {                      // the next live box, if any
@@ -910,20 +929,20 @@ __device__ __forceinline__ void fused_epilogue(const TcParams& p, const TmapPack
     if (ld.u >= u_end) return;
     if (lane == 0) {
       mbar_arrive_expect_tx(&e_full[ld_slot], kFuseBoxBytes);
-      tma_load_2d(boxes + ld_slot * kFuseBoxBytes, &maps.c[1], &e_full[ld_slot], col_of(ld), row_of(ld.u));
+      tma_load_2d(boxes + ld_slot * kFuseBoxBytes, &maps.c[1], &e_full[ld_slot], ld.n0 + ld.c0, ld.row);
     }
     ++n_ld;
     if (++ld_slot == bufs) ld_slot = 0;
     ld.advance(p);
   };
   for (uint32_t b = 0; b + 1 < bufs; ++b) request();
-  int cur_nt = -1;
   bool ok = true;
-  for (int u = u_begin, ui = 0; u < u_end; ++u, ++ui) {
+  int mt = mt_begin, nt = nt_begin;
+  for (int u = u_begin, ui = 0; u < u_end; ++u, ++ui, ++mt) {
     const int j = ui & 1;
-    const int nt = u / p.st_m_tiles;
-    const int row0 = row_of(u), m = row0 + lane;
-    if (kEp == EP_RMS && nt != cur_nt) {
+    if (mt == p.st_m_tiles) { mt = 0; ++nt; }
+    const int row0 = (2 * mt + cta_rank) * kBM + quad * 32, m = row0 + lane;
+    if (kEp == EP_RMS && (ui == 0 || mt == 0)) {
       // 1 / gamma of this column tile, for all epilogue warps (which all come through here, even once a wait has expired)
       asm volatile("bar.sync 1, %0;" ::"r"(threads) : "memory");
       for (int c = (warp - 2) * 32 + lane; c < p.bn; c += threads) {
@@ -931,7 +950,6 @@ __device__ __forceinline__ void fused_epilogue(const TcParams& p, const TmapPack
         col_inv[c] = n < p.N ? 1.f / __bfloat162float(gamma[n]) : 0.f;
       }
       asm volatile("bar.sync 1, %0;" ::"r"(threads) : "memory");
-      cur_nt = nt;
     }
     if (!ok) continue;
     float ra = 0.f, rb = 0.f;
@@ -950,7 +968,7 @@ __device__ __forceinline__ void fused_epilogue(const TcParams& p, const TmapPack
       ok = __all_sync(0xffffffffu, ok);
       tc_wait_ld();
       if (!ok) break;
-      const int n = col_of(k);
+      const int n = k.n0 + k.c0;
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         if (q == 2) {
@@ -1068,6 +1086,7 @@ gemm_tc_stream_kernel(const __grid_constant__ TmapPack maps, const TcParams p) {
   if (warp == 0) {
     if (lane == 0) {
       const uint32_t bar_b = map_to_rank(smem_u32(&b_full), 0u);
+      const uint64_t a_policy = p.st_keep_a ? l2_policy_evict_last() : l2_policy_evict_normal();
       int nb = 0, cur_nt = -1;
       int s = 0;                 // ring stage and its phase, carried along (no division in the loop)
       uint32_t ph = 0u;
@@ -1092,7 +1111,8 @@ gemm_tc_stream_kernel(const __grid_constant__ TmapPack maps, const TcParams p) {
           ok = mbar_wait_bounded(&a_empty[s], ph ^ 1u, &abort_flag);
           if (!ok) break;
           if (leader) mbar_arrive_expect_tx(&a_full[s], 2u * kABytes);
-          tma_load_2d_pair(ring + (size_t)s * kABytes, &maps.a[0], map_to_rank(smem_u32(&a_full[s]), 0u), kb * kBK, m0);
+          tma_load_2d_pair_hint(ring + (size_t)s * kABytes, &maps.a[0], map_to_rank(smem_u32(&a_full[s]), 0u), kb * kBK, m0,
+                                a_policy);
           if (++s == p.st_stages) { s = 0; ph ^= 1u; }
         }
       }
@@ -1539,7 +1559,7 @@ cudaError_t gemm_tc_launch(const GemmDesc& g, uint32_t* dev_status, cudaStream_t
   p.accumulate = g.accumulate ? 1 : 0;
   p.ep_row_a = g.ep_row_a; p.ep_row_b = g.ep_row_b; p.ep_col = g.ep_col;
   p.dev_status = dev_status;
-  p.st_m_tiles = 0; p.st_units = 0; p.tma_store = 0; p.st_stages = kStreamStages; p.store_bufs = kStoreBufs; p.fuse_parts = 4; p.pair_stages = kPairStages;
+  p.st_m_tiles = 0; p.st_units = 0; p.st_keep_a = (long long)g.M * g.K * 2 <= kStreamKeepBytes; p.tma_store = 0; p.st_stages = kStreamStages; p.store_bufs = kStoreBufs; p.fuse_parts = 4; p.pair_stages = kPairStages;
   p.halve_at_term = g.halve_at_term > 0 ? g.halve_at_term : 0;
   p.a_keep_from_kb = g.a_keep_from_k >= 0 ? (int)(g.a_keep_from_k / kBK) : p.kb_total;
   p.gate = g.gate;
