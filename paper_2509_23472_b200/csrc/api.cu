@@ -452,7 +452,6 @@ cudaError_t project(const void* U, const void* X, int64_t ldx, const Plan& p, vo
 // ------------------------------------------------------------------ compress
 struct CompressWs {
   uint32_t* status;
-  int32_t* idx;
   void* S;      // sampled rows, l x d
   void* Omega;  // preconditioned test matrix, l x d
   void* A;      // normalised input of the pre-norm entry (only when it is not returned)
@@ -465,7 +464,6 @@ size_t carve_compress(void* ws, const loract_desc_t* desc, bool with_A, Compress
   Carver c(ws);
   CompressWs w;
   w.status = (uint32_t*)c.take(256);
-  w.idx = (int32_t*)c.take((size_t)desc->rank * 4);
   const size_t es = (size_t)elem_bytes(desc);
   w.S = c.take((size_t)desc->rank * desc->d * es);
   w.Omega = c.take((size_t)desc->rank * desc->d * es);
@@ -480,13 +478,10 @@ cudaError_t compress_core(const loract_desc_t* desc, const void* X, int64_t ldx,
                           int32_t* idx_out, const CompressWs& w, const Plan& plan, cudaStream_t stream) {
   const bool bf16 = plan.bf16;
   const int r = desc->rank;
-  // the sampling step: sample rows, gather them.  The sampler is the first kernel of the call: it clears the status word
-  // and writes the caller's copy of the indices itself.
-  trace_label("sample");
-  LORACT_CUDA_TRY(sample_indices_launch(desc->seed, desc->call_id, (uint32_t)desc->n_tokens, r, w.idx,
-                                        w.status, stream, idx_out, true));
-  trace_label("gather");
-  LORACT_CUDA_TRY(gather_rows_launch(X, ldx, w.idx, r, desc->d, elem_bytes(desc), w.S, stream));
+  // the sampling step: sample rows, gather them
+  trace_label("sample and gather");
+  LORACT_CUDA_TRY(sample_gather_launch(desc->seed, desc->call_id, (uint32_t)desc->n_tokens, r, idx_out, w.status, X, ldx,
+                                       desc->d, elem_bytes(desc), 0, desc->n_tokens, w.S, stream));
   // From the sketch to the orthonormal basis.  The test matrix (the sampled rows A_k at first, Q^T X in the power
   // iterations of the loop
   // 3 to 6) is preconditioned before every product with X: with T T^T = L L^T, Omega = L^{-1} T has the row
@@ -532,7 +527,6 @@ size_t carve_wgrad(void* ws, const loract_desc_t* desc, int g, WgradWs* out) {
 // the sketch, the once-orthonormalised sketch, L^-1) stays in the shard's workspace.
 struct JointWs {
   uint32_t* status;
-  int32_t* idx;
   void* Omega;
   BasisWs b;
 };
@@ -542,7 +536,6 @@ size_t carve_joint(void* ws, const loract_desc_t* desc, JointWs* out, Plan* plan
   Carver c(ws);
   JointWs w;
   w.status = (uint32_t*)c.take(256);
-  w.idx = (int32_t*)c.take((size_t)desc->rank * 4);
   w.Omega = c.take((size_t)desc->rank * desc->d * 2);
   carve_basis(c, *plan, &w.b);
   if (out) *out = w;
@@ -841,13 +834,9 @@ loract_status_t loract_joint_sample_rows(const loract_desc_t* desc, int64_t n_gl
   Plan plan;
   if (ws_bytes < carve_joint(ws, desc, &w, &plan)) return LORACT_ERR_WORKSPACE_TOO_SMALL;
   cudaStream_t st = (cudaStream_t)stream;
-  trace_label("joint: sample");
-  cudaError_t e = sample_indices_launch(desc->seed, desc->call_id, (uint32_t)n_global, desc->rank, w.idx, w.status, st,
-                                        idx_out, true);
-  trace_label("joint: gather own rows");
-  if (e == cudaSuccess)
-    e = gather_rows_window_launch(X_local, desc->ldx, w.idx, desc->rank, desc->d, 2, row0, desc->n_tokens, S, st);
-  return from_cuda(e);
+  trace_label("joint: sample and gather own rows");
+  return from_cuda(sample_gather_launch(desc->seed, desc->call_id, (uint32_t)n_global, desc->rank, idx_out, w.status,
+                                        X_local, desc->ldx, desc->d, 2, row0, desc->n_tokens, S, st));
 }
 
 loract_status_t loract_joint_sketch(const loract_desc_t* desc, const void* X_local, const void* S_sum, float* W_partial,

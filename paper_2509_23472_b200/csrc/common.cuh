@@ -142,18 +142,14 @@ cudaError_t small_block_cluster_wait_probe_launch(uint32_t* dev_status, uint64_t
 cudaError_t gemm_simt_launch(const GemmDesc& g, cudaStream_t stream);
 
 // ---------------------------------------------------------------- sampler and gather
-// idx_copy (optional) receives the same indices; clear_status: the kernel sets the status word instead of OR-ing
-// into it (for the first kernel of a call).
-cudaError_t sample_indices_launch(uint64_t seed, uint64_t call_id, uint32_t n_rows, int rank,
-                                  int32_t* idx_dev, uint32_t* dev_status, cudaStream_t stream,
-                                  int32_t* idx_copy = nullptr, bool clear_status = false);
-// dst (rank x d, stride d) = src[idx, :] (stride ld); 16-byte loads.  elem_bytes 2 or 4.
-cudaError_t gather_rows_launch(const void* src, int64_t ld, const int32_t* idx, int rank, int64_t d,
-                               int elem_bytes, void* dst, cudaStream_t stream);
-// The same for one shard of a token-sharded matrix (src = rows [row0, row0 + n_local) of the whole matrix, idx in
-// whole-matrix row numbers): rows that live on another shard are written as zeros.
-cudaError_t gather_rows_window_launch(const void* src, int64_t ld, const int32_t* idx, int rank, int64_t d,
-                                      int elem_bytes, int64_t row0, int64_t n_local, void* dst, cudaStream_t stream);
+cudaError_t sample_indices_launch(uint64_t seed, uint64_t call_id, uint32_t n_rows, int rank, int32_t* idx_dev,
+                                  uint32_t* dev_status, cudaStream_t stream);
+// The first kernel of a call: draws the indices (to idx_out if not null), sets the status word, and gathers
+// dst (rank x d, stride d) = rows idx of the whole matrix, of which src (stride ld) holds [row0, row0 + n_local); rows that
+// live elsewhere are written as zeros.  16-byte loads, elem_bytes 2 or 4.
+cudaError_t sample_gather_launch(uint64_t seed, uint64_t call_id, uint32_t n_rows, int rank, int32_t* idx_out,
+                                 uint32_t* dev_status, const void* src, int64_t ld, int64_t d, int elem_bytes, int64_t row0,
+                                 int64_t n_local, void* dst, cudaStream_t stream);
 // Gaussian test matrix for the RSVD comparator: dst (l x d bf16, row-major) with
 // dst[c][j] = z(j * l + c), z the Philox + Box-Muller stream (counter word 1 = 1).
 cudaError_t gaussian_rows_launch(uint64_t seed, uint64_t call_id, int l, int64_t d,
