@@ -708,6 +708,9 @@ loract_status_t loract_weight_grad(const loract_desc_t* desc, const void* U, con
   if (gemm_tc_supported(t)) t.clear_status = true;
   else e = cudaMemsetAsync(status, 0, 4, st);
   if (e == cudaSuccess) e = run_gemm(t, status, st);
+  // a small T: summed and multiplied by one kernel
+  if (e == cudaSuccess && small_dw_supported(r, g, w.splits))
+    return from_cuda(small_dw_launch(V, el, desc->d, r, g, w.partials, w.splits, dW, accumulate != 0, st));
   if (e == cudaSuccess && el == ELEM_BF16) {
     // dW = V^T T on the tensor cores: T (fp32) is carried as a bf16 triple, so that the three products
     // together are as accurate as one fp32 product

@@ -223,6 +223,11 @@ cudaError_t copy_bf16_gated_launch(const __nv_bfloat16* src, __nv_bfloat16* dst,
 cudaError_t reduce_split3_launch(const float* partials, int n_partials, int64_t stride, int rows, int cols,
                                  int64_t ld_in, int64_t ld_out, __nv_bfloat16* hi, __nv_bfloat16* mid,
                                  __nv_bfloat16* lo, cudaStream_t stream);
+// dW (d x g, fp32) = V^T T (+ dW), V r x d, T (r x g) the sum of n_partials matrices stored one behind the other: where
+// small_dw_supported says so.
+bool small_dw_supported(int r, int g, int n_partials);
+cudaError_t small_dw_launch(const void* V, int elem_type, int64_t d, int r, int g, const float* partials, int n_partials,
+                            float* dW, int accumulate, cudaStream_t stream);
 // Section 3.3 backward, row coefficients: inner_i = (1 / d) sum_k U[i][k] P[i][k] (P = grad_A V^T, fp32, n x r, the sum of n_partials
 // matrices stored one behind the other),
 // row_a[i] = rstd[i], row_b[i] = rstd[i] * inner_i.  One warp per row.

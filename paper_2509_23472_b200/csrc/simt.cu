@@ -1,6 +1,7 @@
 // CUDA-core kernels: the generic contraction used by the fp32 path and for shapes the tensor-core
 // engine does not take, the fixed-order reduction of split-K partials, and the pre-norm forward.
 #include <algorithm>
+#include <atomic>
 
 #include "common.cuh"
 
@@ -270,6 +271,112 @@ __global__ void reduce_split3_kernel(const float* __restrict__ partials, int n_p
     const int64_t o = row * ld_out + col;
     hi[o] = h; mid[o] = m; lo[o] = __float2bfloat16(r2);
   }
+}
+
+// dW = V^T T for a small T = U^T G, given as partial sums: the whole second half of a weight gradient in one kernel.  A CTA
+// owns 128 bytes of every row of V (64 columns in bf16, 32 in fp32; copied to shared memory ahead of the wait for the
+// previous kernel, which does not write V) and all g columns of dW; it adds up T for itself in a fixed order.  A warp takes
+// four columns of dW, or a part of the contraction where there are fewer than eight such groups.
+// Everything is latency here: a launch less than a reduction and a tensor-core product, whose set-up alone takes as long.
+// Two launches against three, us: bf16 n x d = 4096 x 5120, r = 64, g = 16 10.4 -> 7.9; 384 x 8000, r = 16, g = 8 9.8 -> 6.3;
+// fp32 512 x 768, r = 64, g = 16 14.4 -> 12.1.  The line: every CTA reads all partial sums and multiplies on CUDA cores, so
+// T is at most 1536 elements (96 x 32: 9.7 -> 10.0 in bf16, 18.5 -> 20.5 in fp32; 128 x 64 is 11.2 -> 15.3) in at most 24576
+// (64 x 24 in 16 parts breaks even, 64 x 48 is 12.1 -> 13.6), g a multiple of four (single elements: 18.8 -> 26.6 at g = 19).
+template <typename TV> __device__ __forceinline__ void unpack4(uint32_t w, float (&v)[4 / sizeof(TV)]);
+template <> __device__ __forceinline__ void unpack4<float>(uint32_t w, float (&v)[1]) { v[0] = __uint_as_float(w); }
+template <> __device__ __forceinline__ void unpack4<__nv_bfloat16>(uint32_t w, float (&v)[2]) {
+  v[0] = __uint_as_float(w << 16);
+  v[1] = __uint_as_float(w & 0xffff0000u);
+}
+constexpr int kSmallDwThreads = 256;
+constexpr int kSmallDwFloats = 1536;             // of T
+constexpr int kSmallDwPartialFloats = 24576;    // of its partial sums
+// parts of the contraction for nq groups of four columns
+__host__ __device__ constexpr int small_dw_parts(int nq) { return nq == 1 ? 8 : nq == 2 ? 4 : nq <= 4 ? 2 : 1; }
+template <typename TV>
+__host__ __device__ constexpr size_t small_dw_smem(int r, int g) {
+  return (size_t)r * 128 + (size_t)r * g * 4 + (size_t)small_dw_parts(g / 4) * (128 / sizeof(TV)) * (g | 1) * 4;
+}
+constexpr int kSmallDwSmemMax = 80 * 1024;       // r <= 384 (g >= 4), at most 25 KB of sums (g = 96)
+
+template <typename TV>
+__global__ void __launch_bounds__(kSmallDwThreads) small_dw_kernel(const TV* __restrict__ V, int64_t d, int r, int g,
+                                                                   const float* __restrict__ partials, int n_partials,
+                                                                   float* __restrict__ dW, int accumulate) {
+  constexpr int kPerLane = 4 / sizeof(TV), kCols = 32 * kPerLane;
+  extern __shared__ __align__(16) unsigned char smem[];
+  unsigned char* vt = smem;                                              // [r][128 bytes]
+  float* T = reinterpret_cast<float*>(smem + (size_t)r * 128);           // [r][g]
+  float* red = T + (size_t)r * g;                                        // [part][column of V][g | 1]
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int64_t c0 = (int64_t)blockIdx.x * kCols;
+  for (int i = tid; i < r * 8; i += kSmallDwThreads) {
+    const int64_t col = c0 + (i & 7) * (16 / (int)sizeof(TV));
+    const bool in = col < d;                                             // (d is a multiple of a 16-byte chunk)
+    const TV* src = V + (in ? (int64_t)(i >> 3) * d + col : 0);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;"
+                 ::"r"((uint32_t)__cvta_generic_to_shared(vt + (size_t)i * 16)), "l"(src), "r"(in ? 16 : 0)
+                 : "memory");
+  }
+  pdl_wait();
+  pdl_launch_dependents();
+  const int n4 = r * g / 4;                                              // (r is a multiple of 16)
+  for (int e = tid; e < n4; e += kSmallDwThreads) {
+    const float4* src = reinterpret_cast<const float4*>(partials) + e;
+    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 8
+    for (int q = 0; q < n_partials; ++q) {
+      const float4 v = src[(int64_t)q * n4];
+      s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
+    }
+    reinterpret_cast<float4*>(T)[e] = s;
+  }
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  __syncthreads();
+  const int nq = g / 4, parts = small_dw_parts(nq), part = nq > 4 ? 0 : warp / nq;
+  const int k_per = r / parts;
+  for (int q = nq > 4 ? warp : warp - part * nq; q < nq && part < parts; q += 8) {
+    float acc[kPerLane][4] = {};
+#pragma unroll 8
+    for (int k = part * k_per; k < (part + 1) * k_per; ++k) {
+      float v[kPerLane];
+      unpack4<TV>(*reinterpret_cast<const uint32_t*>(vt + (size_t)k * 128 + lane * 4), v);
+      const float4 t4 = *reinterpret_cast<const float4*>(T + (size_t)k * g + 4 * q);
+      const float t[4] = {t4.x, t4.y, t4.z, t4.w};
+#pragma unroll
+      for (int c = 0; c < kPerLane; ++c)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[c][j] = fmaf(v[c], t[j], acc[c][j]);
+    }
+#pragma unroll
+    for (int c = 0; c < kPerLane; ++c)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) red[(size_t)(part * kCols + lane * kPerLane + c) * (g | 1) + 4 * q + j] = acc[c][j];
+  }
+  __syncthreads();
+  float* out = dW + c0 * g;
+  const int n_out = (int)min((int64_t)kCols, d - c0) * g;
+  for (int e = tid; e < n_out; e += kSmallDwThreads) {
+    const int col = e / g, j = e - col * g;
+    float s = accumulate ? out[e] : 0.f;
+    for (int p = 0; p < parts; ++p) s += red[(size_t)(p * kCols + col) * (g | 1) + j];
+    out[e] = s;
+  }
+}
+
+template <typename TV>
+cudaError_t launch_small_dw(const TV* V, int64_t d, int r, int g, const float* partials, int n_partials, float* dW,
+                            int accumulate, cudaStream_t stream) {
+  static std::atomic<bool> configured[64];
+  int dev = 0;
+  LORACT_CUDA_TRY(cudaGetDevice(&dev));
+  if (dev < 0 || dev >= 64 || !configured[dev].load(std::memory_order_acquire)) {
+    LORACT_CUDA_TRY(cudaFuncSetAttribute(small_dw_kernel<TV>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmallDwSmemMax));
+    if (dev >= 0 && dev < 64) configured[dev].store(true, std::memory_order_release);
+  }
+  constexpr int kCols = 128 / sizeof(TV);
+  return launch_pdl(small_dw_kernel<TV>, dim3((unsigned)((d + kCols - 1) / kCols)), dim3(kSmallDwThreads),
+                    small_dw_smem<TV>(r, g), stream, V, d, r, g, partials, n_partials, dW, accumulate);
 }
 
 // fp32 x fp32 products on CUDA cores: the whole fp32 path.
@@ -981,6 +1088,19 @@ cudaError_t reduce_split3_launch(const float* partials, int n_partials, int64_t 
   if (grid < 1) grid = 1;
   LORACT_CUDA_TRY(launch_pdl(reduce_split3_kernel, dim3(grid), dim3(256), 0, stream, partials, n_partials, stride, rows,
                              cols, ld_in, ld_out, hi, mid, lo));
+  count_launch(__func__, stream);
+  return cudaGetLastError();
+}
+
+bool small_dw_supported(int r, int g, int n_partials) {
+  return r % 16 == 0 && g % 4 == 0 && r * g <= kSmallDwFloats && (int64_t)n_partials * r * g <= kSmallDwPartialFloats;
+}
+
+cudaError_t small_dw_launch(const void* V, int elem_type, int64_t d, int r, int g, const float* partials, int n_partials,
+                            float* dW, int accumulate, cudaStream_t stream) {
+  LORACT_CUDA_TRY(elem_type == ELEM_BF16
+                      ? launch_small_dw((const __nv_bfloat16*)V, d, r, g, partials, n_partials, dW, accumulate, stream)
+                      : launch_small_dw((const float*)V, d, r, g, partials, n_partials, dW, accumulate, stream));
   count_launch(__func__, stream);
   return cudaGetLastError();
 }
