@@ -54,7 +54,7 @@ loract_status_t loract_debug_project(const loract_desc_t* desc, const void* U, c
 void loract_debug_set_pair_mode(int32_t on);
 
 /* The orthonormalisation of the bf16 path runs its second Gram round only when the first round's Gram matrix W
- * was not conditioned well enough for one: a one-CTA kernel forms est = trace((D W D)^-1), D = diag(W)^(-1/2),
+ * was not conditioned well enough for one: the factorisation kernel forms est = trace((D W D)^-1), D = diag(W)^(-1/2),
  * from the inverse factor and compares est times the number of 64-row blocks per accumulation chain of the Gram
  * product with a threshold (widths up to 512; above that both rounds always run).
  * This sets the threshold, process-wide: a negative value forces both rounds, +infinity allows one round whenever
@@ -62,7 +62,7 @@ void loract_debug_set_pair_mode(int32_t on);
  * holds, as 32-bit words 4, 5, 6: whether the second round ran (0 / 1), est (float bits), the number of rounds. */
 void loract_debug_set_round_gate(float threshold);
 
-/* The deciding kernel alone.  W: r x r fp32 (device, leading dimension r), linv_hi: r x r bf16 lower triangular
+/* The same decision in a kernel of its own, from a finished factor.  W: r x r fp32 (device, leading dimension r), linv_hi: r x r bf16 lower triangular
  * (device), r a multiple of 8 up to 640; status_word: device uint32 or NULL.  words (device, 3 x uint32) receives
  * { est > threshold or est not finite or *status_word != 0,  est = sum_ij linv_ij^2 W_jj as float bits,
  *   1 or 2 = the number of rounds }. */

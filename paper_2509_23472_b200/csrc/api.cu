@@ -343,8 +343,8 @@ cudaError_t range_basis(const void* X, int64_t ldx, const Plan& p, const void* O
     return cudaSuccess;
   }
   // bf16 inputs.  Round 1 always runs and writes the leading bf16 part of Q1 = Y L^-T straight into U (the rounded Q1
-  // is the result when one round is enough), the remainder into the workspace.  A one-CTA kernel then decides from the
-  // factor whether the Gram matrix was conditioned well enough for one round (gate word: 0 = done).  The kernels of
+  // is the result when one round is enough), the remainder into the workspace.  The factorisation decides while it writes
+  // the factor out whether the Gram matrix was conditioned well enough for one round (gate word: 0 = done).  The kernels of
   // round 2 are launched in any case and leave at once when the gate word is zero: no host synchronisation.
   uint32_t* gate_words = status + kGateWord;
   const bool can_gate = l <= 512 && l % 8 == 0;   // widths above 512 (general fp64 kernel) always run both rounds
