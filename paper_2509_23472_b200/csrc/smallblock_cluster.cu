@@ -14,7 +14,7 @@
 //   * solver warps (four, eight rows each): L(i, k) = A(i, k) L(k, k)^-T by forward substitution while block k is being
 //     factored, and later the block column of the inverse, whose transpose solves the same system.  No inverse of a
 //     diagonal block is formed.
-//   * bulk warps (eight, two to a block): the updates nobody waits for, and the output.
+//   * bulk warps (six or eight, two to a block): the updates nobody waits for, and the output.
 //   * sender warps (three taking turns, one in fp64) copy finished groups and blocks to the CTAs that need them (bulk
 //     distributed-shared-memory copies; one round of wait, proxy fence and up to fifteen copies takes longer than a group).
 // A block is stored as eight groups of [32 rows][4 columns]: a group is one contiguous copy, a lane's row and a
@@ -28,9 +28,9 @@
 //
 // Measured (one Gram matrix, back to back, against a form with one chain CTA, workers that sent blocks back to it and an
 // inverse of every diagonal block): fp32 r = 32 / 64 / 128 / 256: 6.9 / 9.0 / 14.1 / 27.9 us (7.4 / 11.8 / 20.0 / 40.4).
-// r = 336 / 512, against two factorisations of up to 256 columns joined by fp32 products: 42 / 71 us (69 / 91, and six
+// r = 336 / 512, against two factorisations of up to 256 columns joined by fp32 products: 42 / 70 us (69 / 91, and six
 // helper launches fewer).  Above eight blocks the early steps are bound by the bulk updates and by what an SM can send.
-// fp64, against a kernel that kept the matrix in global memory: r = 64 / 96 / 192: 13.4 / 18.0 / 31.9 us (75.8 / 120.9 /
+// fp64, against a kernel that kept the matrix in global memory: r = 64 / 96 / 192: 12.9 / 17.2 / 30.4 us (75.8 / 120.9 /
 // 282).  Cycles per group of four columns: 398 in the pivot warp alone, about 475 with its companions at work; the step
 // from one diagonal block to the next adds about 1000.
 //
@@ -46,22 +46,27 @@ namespace loract {
 namespace {
 
 constexpr int kB = 32;                   // block edge
-constexpr int kMaxWarps = 20;
 // fp32: three senders.  An SM issues a copy of one group every 56 cycles, so that a sender which waits, fences and copies to
 // seven peers falls behind the groups (one sender: r = 224 / 256 25.5 / 29.8 us instead of 24.4 / 28.8).  fp64, at most
 // six blocks and a slower chain: one (three: 0.2 to 0.6 us more).
 template <typename T> __host__ __device__ constexpr int senders_of() { return sizeof(T) == 8 ? 1 : 3; }
-template <typename T> __host__ __device__ constexpr int warps_of() { return kMaxWarps - 3 + senders_of<T>(); }
+// Six bulk warps; eight above eight block rows, where theirs is the work that lags (six: r = 400 / 512 54 / 74 us instead of
+// 52 / 70.6; ten or twelve get in the way of the chain, 75).  Below, the registers and the issue slots of two fewer are worth
+// more: r = 256 28.1 -> 27.7 us, fp64 r = 64 / 192 13.4 / 32 -> 12.9 / 30.4.
+template <bool kBig> __host__ __device__ constexpr int bulk_of() { return kBig ? 8 : 6; }
+template <typename T, bool kBig> __host__ __device__ constexpr int warps_of() { return 9 + bulk_of<kBig>() + senders_of<T>(); }
 constexpr int kPan = 8;                  // groups of four columns in a block
 constexpr uint64_t kClusterWaitNs = 50000000ull;  // 50 ms
 // Warp -> role (plus the index inside the role).  The scheduler a warp shares is its number mod 4: the pivot warp's
 // companions are senders and bulk warps, which are idle or waiting while it works.
 enum Role : int { R_PIVOT = 0, R_FOLLOW = 1, R_SOLVE = 5, R_BULK = 9, R_SEND = 17 };
-constexpr int kBulkWarps = 8;
-__constant__ unsigned char kRoleOf[kMaxWarps] = {R_PIVOT, R_FOLLOW + 0, R_FOLLOW + 1, R_FOLLOW + 2, R_SEND + 0, R_SOLVE + 0,
+__constant__ unsigned char kRoleBig[20] = {R_PIVOT, R_FOLLOW + 0, R_FOLLOW + 1, R_FOLLOW + 2, R_SEND + 0, R_SOLVE + 0,
                                               R_FOLLOW + 3, R_SOLVE + 2, R_BULK + 0, R_SOLVE + 3, R_SOLVE + 1, R_BULK + 6,
                                               R_BULK + 1, R_BULK + 3, R_BULK + 5, R_BULK + 7, R_BULK + 2, R_BULK + 4,
                                               R_SEND + 1, R_SEND + 2};
+__constant__ unsigned char kRoleSmall[18] = {R_PIVOT, R_FOLLOW + 0, R_FOLLOW + 1, R_FOLLOW + 2, R_SEND + 0, R_SOLVE + 0,
+                                             R_FOLLOW + 3, R_SOLVE + 2, R_BULK + 0, R_SOLVE + 3, R_SOLVE + 1, R_BULK + 1,
+                                             R_BULK + 2, R_BULK + 3, R_BULK + 5, R_BULK + 4, R_SEND + 1, R_SEND + 2};
 
 constexpr int kGrp = kB * 4;             // elements of a group of four columns
 constexpr int kBlk = kB * kB;            // elements of a block
@@ -329,11 +334,12 @@ __device__ __forceinline__ void take_off_group(V4<T> (&acc)[2], const T* A, cons
 // C (or zero) -= A B^T for columns 16 half .. 16 half + 15 of a block, 4 x 4 outputs per lane: rows row0 + 8 i, columns
 // col0 + 4 j.  With eight warps at it the shared-memory pipe is the bound: per group four loads of A at four cycles, four of
 // B at two (two addresses per quarter warp), and C in single elements without conflicts (a warp access covers eight rows of a
-// group); one warp alone waits for its loads, hence the unrolled loop (fp32 by eight: the code costs small launches 2 us).
+// group); one warp alone waits for its loads, hence the unrolled loop (by eight in the kernels for
+// many blocks and for fp64; in the small fp32 kernel the code of that costs 2 us a launch).
 // Against rows 16 half .., with conflicts on C, unrolled by two: 2340 -> 2200 cycles for eight halves with eight warps, 1350
 // -> 1100 with one; r = 256 / 512 28.8 / 74 -> 27.9 / 71 us.  A whole block per warp (a third fewer loads) or two halves at a
 // time (a quarter fewer) leave too few warps at work: r = 512 75 and 73 us.
-template <typename T>
+template <typename T, int kUnroll>
 __device__ __forceinline__ void take_off_half(T* C, const T* A, const T* Bm, bool from_zero, int half, int lane) {
   const int row0 = (lane & 3) + 4 * (lane >> 4), col0 = (lane >> 2) & 3;
   C += 4 * half * kGrp + row0 * 4 + col0;
@@ -344,7 +350,6 @@ __device__ __forceinline__ void take_off_half(T* C, const T* A, const T* Bm, boo
   for (int j = 0; j < 4; ++j)
 #pragma unroll
     for (int i = 0; i < 4; ++i) acc[i][j] = from_zero ? (T)0 : C[j * kGrp + 32 * i];
-  constexpr int kUnroll = sizeof(T) == 8 ? 8 : 4;
 #pragma unroll kUnroll
   for (int q = 0; q < kPan; ++q) {
     V4<T> a[4], b[4];
@@ -392,8 +397,9 @@ __host__ __device__ constexpr size_t smem_elems(int nblk) {
 }
 
 template <typename T, bool kBig>
-__global__ void __launch_bounds__(32 * warps_of<T>(), 1) small_block_cluster_kernel(SCParams p) {
-  constexpr int kWarps = warps_of<T>(), kCThreads = 32 * kWarps, kSendWarps = senders_of<T>();
+__global__ void __launch_bounds__(32 * warps_of<T, kBig>(), 1) small_block_cluster_kernel(SCParams p) {
+  constexpr int kWarps = warps_of<T, kBig>(), kCThreads = 32 * kWarps, kSendWarps = senders_of<T>();
+  constexpr int kBulkWarps = bulk_of<kBig>();
   constexpr int kMaxBlk = kBig ? kBigBlk : 8;              // block rows, and CTAs of the cluster
   constexpr int kMaxOff = kMaxBlk * (kMaxBlk - 1) / 2;
   constexpr uint32_t kBlkBytes = (uint32_t)(kBlk * sizeof(T)), kGrpBytes = (uint32_t)(kGrp * sizeof(T));
@@ -538,7 +544,7 @@ __global__ void __launch_bounds__(32 * warps_of<T>(), 1) small_block_cluster_ker
 
   volatile int* gave_up = &s_gave_up;
   const T floor_ = s_floor;
-  const int role = kRoleOf[warp];
+  const int role = kBig ? kRoleBig[warp] : kRoleSmall[warp];
   // the CTA this lane signals and copies to: the next one of the chain first
   const int to = lane < nblk ? (me + 1 + lane) % nblk : 0;
   const bool peer = lane + 1 < nblk;
@@ -671,28 +677,32 @@ __global__ void __launch_bounds__(32 * warps_of<T>(), 1) small_block_cluster_ker
       const int j_end = k < me ? me + 1 : nblk;
 #pragma unroll 1
       for (int j = k + 2; j < j_end; ++j) {
-        if ((j & 3) != (m >> 1)) continue;                     // the same pair of warps for a block in every step
+        if (j % (kBulkWarps / 2) != (m >> 1)) continue;        // the same pair of warps for a block in every step
         if (j != me) bar_wait(&off_bar[off_slot(j, k)], gave_up);
-        take_off_half<T>(target(j), blk, j == me ? blk : slot(j, k), k == me, m & 1, lane);
+        take_off_half<T, (kBig || sizeof(T) == 8) ? 8 : 4>(target(j), blk, j == me ? blk : slot(j, k), k == me, m & 1, lane);
         if (j == k + 2) warp_arrive(&bulk_bar[j], lane);
       }
       done_with(k);
       if (k < me) continue;
-      // rows 32 k + 4 m .. + 3 of the result: element (32 k + 4 m + u, col) = X[group m][lane][u]
-      const V4<T> v4 = ld4(blk + m * kGrp + lane * 4);
-      const int row = k * kB + 4 * m;
+#pragma unroll 1
+      for (int q = m; q < kPan; q += kBulkWarps) {
+        // rows 32 k + 4 q .. + 3 of the result: element (32 k + 4 q + u, col) = X[group q][lane][u]
+        const V4<T> v4 = ld4(blk + q * kGrp + lane * 4);
+        const int row = k * kB + 4 * q;
 #pragma unroll
-      for (int a = 0; a < 4; ++a) {
-        if (row + a >= r || col >= r) continue;
-        const float v = (float)v4.v[a];
-        est = fmaf(v * v, wdiag, est);
-        const int64_t o = (int64_t)(row + a) * p.out_ld + col;
-        if (p.linv_f32) p.linv_f32[o] = v;
-        if (p.linv_hi) {
-          const __nv_bfloat16 hi = __float2bfloat16(v);
-          p.linv_hi[o] = hi;
-          if (p.linv_lo) p.linv_lo[o] = __float2bfloat16(v - __bfloat162float(hi));
+        for (int a = 0; a < 4; ++a) {
+          if (row + a >= r || col >= r) continue;
+          const float v = (float)v4.v[a];
+          est = fmaf(v * v, wdiag, est);
+          const int64_t o = (int64_t)(row + a) * p.out_ld + col;
+          if (p.linv_f32) p.linv_f32[o] = v;
+          if (p.linv_hi) {
+            const __nv_bfloat16 hi = __float2bfloat16(v);
+            p.linv_hi[o] = hi;
+            if (p.linv_lo) p.linv_lo[o] = __float2bfloat16(v - __bfloat162float(hi));
+          }
         }
+        if (kBulkWarps >= kPan) break;
       }
     }
     if (p.gate_out) {
@@ -787,7 +797,7 @@ cudaError_t launch_cluster(const SCParams& p, cudaStream_t stream) {
   }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(ctas, 1, 1);
-  cfg.blockDim = dim3(32 * warps_of<T>(), 1, 1);
+  cfg.blockDim = dim3(32 * warps_of<T, kBig>(), 1, 1);
   cfg.dynamicSmemBytes = smem_elems<T, kBig>(nblk) * sizeof(T);
   cfg.stream = stream;
   cudaLaunchAttribute attr[2];
