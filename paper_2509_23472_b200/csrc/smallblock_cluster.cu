@@ -27,8 +27,8 @@
 // a warp barrier take 30 cycles, a bulk copy to another CTA 280 (512 bytes) to 480 (4.6 KB) or 730 with seven receivers.
 //
 // Measured (one Gram matrix, back to back, against a form with one chain CTA, workers that sent blocks back to it and an
-// inverse of every diagonal block): fp32 r = 32 / 64 / 128 / 256: 6.9 / 9.0 / 14.1 / 27.9 us (7.4 / 11.8 / 20.0 / 40.4).
-// r = 336 / 512, against two factorisations of up to 256 columns joined by fp32 products: 42 / 70 us (69 / 91, and six
+// inverse of every diagonal block): fp32 r = 32 / 64 / 128 / 256: 6.9 / 9.0 / 14.0 / 27.2 us (7.4 / 11.8 / 20.0 / 40.4).
+// r = 336 / 512, against two factorisations of up to 256 columns joined by fp32 products: 41 / 69 us (69 / 91, and six
 // helper launches fewer).  Above eight blocks the early steps are bound by the bulk updates and by what an SM can send.
 // fp64, against a kernel that kept the matrix in global memory: r = 64 / 96 / 192: 12.9 / 17.2 / 30.4 us (75.8 / 120.9 /
 // 282).  Cycles per group of four columns: 398 in the pivot warp alone, about 475 with its companions at work; the step
@@ -304,6 +304,15 @@ __device__ __forceinline__ void solve_half(V4<T> (&acc)[2], T* blk, const T* pan
     bar_wait(pan_bars + p, gave_up);
     const V4<T> rr = ld4(pan + kGrp + (inverse ? 4 : 0));
     const V4<T> r1 = ld4(low + 4), r2 = ld4(low + 8), r3 = ld4(low + 12);
+    // fp32: the rows that the group is taken off with are fetched before x is known (r = 336 / 512 42.1 / 70.1 -> 41.5 / 69.1
+    // us); fp64 has no registers for them
+    V4<T> b[2][4];
+    if (sizeof(T) == 4) {
+#pragma unroll
+      for (int h = H; h < 2; ++h)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) b[h][j] = ld4(pan + (4 * (cg + 4 * h) + j) * 4);
+    }
     const V4<T>& t = acc[H];
     V4<T> x;
     x.v[0] = t.v[0] * rr.v[0];
@@ -317,19 +326,40 @@ __device__ __forceinline__ void solve_half(V4<T> (&acc)[2], T* blk, const T* pan
 #pragma unroll
     for (int h = H; h < 2; ++h)
 #pragma unroll
-      for (int j = 0; j < 4; ++j) acc[h].v[j] = sub4(acc[h].v[j], x, ld4(pan + (4 * (cg + 4 * h) + j) * 4));
+      for (int j = 0; j < 4; ++j)
+        acc[h].v[j] = sub4(acc[h].v[j], x, sizeof(T) == 4 ? b[h][j] : ld4(pan + (4 * (cg + 4 * h) + j) * 4));
   }
 }
 
 // ------------------------------------------------------------------ block updates
-// acc (this lane's row, columns 8 w .. 8 w + 7) -= (row of group A) . (rows of group B)
+// A follow-up warp w holds columns 8 w .. 8 w + 7 of a block, a lane two quads acc[h] of them: in fp32 rows lane % 16 and
+// lane % 16 + 16 of group 2 w + lane / 16 (six loads a group; with one row and both groups, as in fp64, nine, and r = 256
+// takes 27.5 instead of 27.0 us; fp64 is 2 % faster with one row).
 template <typename T>
-__device__ __forceinline__ void take_off_group(V4<T> (&acc)[2], const T* A, const T* Bg, int w, int lane) {
-  const V4<T> a = ld4(A + lane * 4);
+struct FollowLane {
+  static constexpr bool kTwoRows = sizeof(T) == 4;
+  int w, lane;
+  __device__ __forceinline__ int group(int h) const { return kTwoRows ? 2 * w + (lane >> 4) : 2 * w + h; }
+  __device__ __forceinline__ int at(int h) const { return group(h) * kGrp + (kTwoRows ? (lane & 15) + 16 * h : lane) * 4; }
+};
+// acc -= (rows of group A) . (rows of group B)
+template <typename T>
+__device__ __forceinline__ void take_off_group(V4<T> (&acc)[2], const T* A, const T* Bg, const FollowLane<T>& f) {
+  if (FollowLane<T>::kTwoRows) {
+    const V4<T> a0 = ld4(A + (f.lane & 15) * 4), a1 = ld4(A + (f.lane & 15) * 4 + 64);
 #pragma unroll
-  for (int h = 0; h < 2; ++h)
+    for (int j = 0; j < 4; ++j) {
+      const V4<T> b = ld4(Bg + (4 * f.group(0) + j) * 4);
+      acc[0].v[j] = sub4(acc[0].v[j], a0, b);
+      acc[1].v[j] = sub4(acc[1].v[j], a1, b);
+    }
+  } else {
+    const V4<T> a = ld4(A + f.lane * 4);
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[h].v[j] = sub4(acc[h].v[j], a, ld4(Bg + (8 * w + 4 * h + j) * 4));
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) acc[h].v[j] = sub4(acc[h].v[j], a, ld4(Bg + (4 * f.group(h) + j) * 4));
+  }
 }
 // C (or zero) -= A B^T for columns 16 half .. 16 half + 15 of a block, 4 x 4 outputs per lane: rows row0 + 8 i, columns
 // col0 + 4 j.  With eight warps at it the shared-memory pipe is the bound: per group four loads of A at four cycles, four of
@@ -574,8 +604,9 @@ __global__ void __launch_bounds__(32 * warps_of<T, kBig>(), 1) small_block_clust
     send(panel(me) + (kPan - 1) * kPanElems, panel(me) + (kPan - 1) * kPanElems, kPanBytes, &pan_bar[me][kPan - 1], peer);
     if (clamped && lane == 0 && p.dev_status) atomicOr(p.dev_status, LORACT_DEV_PIVOT_CLAMPED);
   } else if (role < R_SOLVE) {
-    // ---- follow-up warps: lane = row, columns 8 w .. 8 w + 7
+    // ---- follow-up warps
     const int w = role - R_FOLLOW;
+    const FollowLane<T> f{w, lane};
 #pragma unroll 1
     for (int k = -1; k + 1 < nblk; ++k) {
       // step k: the block that step k + 1 works on takes L(own, k) or X(k, own) off, group by group
@@ -588,7 +619,7 @@ __global__ void __launch_bounds__(32 * warps_of<T, kBig>(), 1) small_block_clust
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         acc[h] = {{(T)0, (T)0, (T)0, (T)0}};
-        if (!fresh) acc[h] = ld4(tgt + (2 * w + h) * kGrp + lane * 4);
+        if (!fresh) acc[h] = ld4(tgt + f.at(h));
       }
       if (k >= 0) {
         const T* A = solved(k);
@@ -597,13 +628,13 @@ __global__ void __launch_bounds__(32 * warps_of<T, kBig>(), 1) small_block_clust
         for (int q = 0; q < kPan; ++q) {
           bar_wait(&sol_bar[k][q], gave_up);
           if (j != me) bar_wait(&next_bar[k][q], gave_up);
-          take_off_group<T>(acc, A + q * kGrp, Bm + q * kGrp, w, lane);
+          take_off_group<T>(acc, A + q * kGrp, Bm + q * kGrp, f);
         }
         done_with(k);
       }
       if (j != me) {
 #pragma unroll
-        for (int h = 0; h < 2; ++h) st4(tgt + (2 * w + h) * kGrp + lane * 4, acc[h]);
+        for (int h = 0; h < 2; ++h) st4(tgt + f.at(h), acc[h]);
         warp_arrive(&rdy_bar[j], lane);
         continue;
       }
@@ -611,17 +642,20 @@ __global__ void __launch_bounds__(32 * warps_of<T, kBig>(), 1) small_block_clust
       // it has been taken off
       if (w == 0) {
 #pragma unroll
-        for (int h = 0; h < 2; ++h) { st4(own + h * kGrp + lane * 4, acc[h]); named_arrive(id_staged(h), 64); }
+        for (int h = 0; h < 2; ++h) st4(own + f.at(h), acc[h]);
+        named_arrive(id_staged(0), 64);
+        named_arrive(id_staged(1), 64);
       }
       const T* pan = panel(me);
 #pragma unroll 1
       for (int g = 0; g < 2 * w; ++g) {
         named_sync(id_published(g), readers_of(g));
-        take_off_group<T>(acc, pan, pan, w, lane);
+        take_off_group<T>(acc, pan, pan, f);
         pan += kPanElems;
         if (g + 2 >= 2 * w) {
-          const int h = g + 2 - 2 * w;
-          st4(own + (g + 2) * kGrp + lane * 4, h ? acc[1] : acc[0]);
+#pragma unroll
+          for (int h = 0; h < 2; ++h)
+            if (f.group(h) == g + 2) st4(own + f.at(h), acc[h]);
           named_arrive(id_staged(g + 2), 64);
         }
       }
