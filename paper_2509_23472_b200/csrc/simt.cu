@@ -691,13 +691,14 @@ __global__ void __launch_bounds__(256) norm_forward_kernel(const T* __restrict__
   }
 }
 
-// The same unit with 16-byte accesses.  A row is shared by kWarps warps of a block: thread t of the row takes the chunks
-// t, t + 32 kWarps, ... (8 bf16 or 4 fp32 values each), so every load and store instruction of a warp covers 512 contiguous
-// bytes, and keeps them in registers, packed as loaded: X is read from memory exactly once and the statistics (mean, then
-// the centred second moment, as in the kernel above) are taken from the registers.  What bounds it is bytes in flight: few
-// chunks per thread keep the registers low and many rows resident.  (Measured with one warp per row and up to sixteen
-// chunks per lane: 16384 x 4096 bf16, LayerNorm 73 us, RMS 58; x 11008: 257 and 187.  Now 60, 49, 155, 124 (floor
-// 41 and 110).)
+// The same unit with 16-byte accesses.  A warp owns a row: lane l takes the chunks l, l + 32, ... (8 bf16 or 4 fp32 values
+// each), so every load and store instruction of the warp covers 512 contiguous bytes.  Up to sixteen chunks a lane stay in
+// registers, packed as loaded, and X is read from memory once; longer rows are read again in each pass, mostly from L2.
+// The order of the sums is part of the result: the last bit of 1 / rms decides how entries of A that lie on a rounding
+// boundary are stored, and the trailing directions of a large rank move with them (entries of U by up to a tenth of their
+// size), so a row is always added up in this order, whatever its length.  Sharing a row between warps, with another order,
+// took 103 us instead of 112 for an RMS unit of 8192 x 4096 at rank 16 (305 instead of 365 for 16384 x 11008) and was given
+// up for that; in the same order, the warps taking turns, 110 and 461.
 
 template <typename T>
 struct NormChunk;
@@ -733,7 +734,7 @@ struct NormChunk<float> {
   }
 };
 
-template <typename T, int kWarps, int kKeep>
+template <typename T, int kKeep>   // kKeep: chunks a lane keeps in registers; 0: none
 __global__ void __launch_bounds__(256) norm_forward_vec_kernel(const T* __restrict__ X, int64_t n, int64_t d,
                                                                int64_t ldx, const T* __restrict__ gamma,
                                                                const T* __restrict__ beta, float eps, int kind,
@@ -742,56 +743,52 @@ __global__ void __launch_bounds__(256) norm_forward_vec_kernel(const T* __restri
                                                                float* __restrict__ mean_out) {
   using C = NormChunk<T>;
   constexpr int kV = C::kVals;
-  __shared__ float s_part[2][8];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int sub = warp % kWarps, t = sub * 32 + lane;        // position inside the row
-  const int64_t row = (int64_t)blockIdx.x * (8 / kWarps) + warp / kWarps;
+  const int lane = threadIdx.x & 31;
+  const int64_t row = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
   pdl_wait();
   pdl_launch_dependents();
-  const int n_chunks = row < n ? (int)(d / kV) : 0;          // (a row past the end takes part in the barriers only)
+  if (row >= n) return;
+  const int n_chunks = (int)(d / kV);
   const uint4* x = reinterpret_cast<const uint4*>(X + row * ldx);
-  uint4 keep[kKeep];
+  uint4 keep[kKeep ? kKeep : 1];
 #pragma unroll
   for (int i = 0; i < kKeep; ++i) {
-    const int c = t + 32 * kWarps * i;
+    const int c = lane + 32 * i;
     keep[i] = c < n_chunks ? __ldg(x + c) : make_uint4(0u, 0u, 0u, 0u);
   }
-  // sum over the row, in the same order for every thread
-  auto row_sum = [&](float v, float* part) {
+  auto chunk = [&](int i, int c) -> uint4 { return kKeep ? keep[i] : __ldg(x + c); };
+  const int per_lane = kKeep ? kKeep : (n_chunks + 31) / 32;
+  auto row_sum = [](float v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if (kWarps == 1) return v;
-    if (lane == 0) part[warp] = v;
-    __syncthreads();
-    v = 0.f;
-#pragma unroll
-    for (int q = 0; q < kWarps; ++q) v += part[warp - sub + q];
     return v;
   };
   float mean = 0.f;
   if (kind == LORACT_NORM_LAYER) {
     float s = 0.f;
 #pragma unroll
-    for (int i = 0; i < kKeep; ++i) {
+    for (int i = 0; i < per_lane; ++i) {
+      const int c = lane + 32 * i;
+      if (c >= n_chunks) break;
       float v[kV];
-      C::unpack(keep[i], v);
+      C::unpack(chunk(i, c), v);
 #pragma unroll
-      for (int q = 0; q < kV; ++q) s += v[q];                // (chunks past the row are zeros)
+      for (int q = 0; q < kV; ++q) s += v[q];
     }
-    mean = row_sum(s, s_part[0]) / (float)d;
+    mean = row_sum(s) / (float)d;
   }
   float ss = 0.f;
 #pragma unroll
-  for (int i = 0; i < kKeep; ++i) {
-    if (t + 32 * kWarps * i >= n_chunks) continue;
+  for (int i = 0; i < per_lane; ++i) {
+    const int c = lane + 32 * i;
+    if (c >= n_chunks) break;
     float v[kV];
-    C::unpack(keep[i], v);
+    C::unpack(chunk(i, c), v);
 #pragma unroll
     for (int q = 0; q < kV; ++q) { const float u = v[q] - mean; ss += u * u; }
   }
-  const float rstd = rsqrtf(row_sum(ss, s_part[1]) / (float)d + eps);
-  if (row >= n) return;
-  if (t == 0) {
+  const float rstd = rsqrtf(row_sum(ss) / (float)d + eps);
+  if (lane == 0) {
     rstd_out[row] = rstd;
     if (mean_out) mean_out[row] = mean;
   }
@@ -799,11 +796,11 @@ __global__ void __launch_bounds__(256) norm_forward_vec_kernel(const T* __restri
   const uint4* bt = reinterpret_cast<const uint4*>(beta);
   uint4* a = reinterpret_cast<uint4*>(A + row * lda);
 #pragma unroll
-  for (int i = 0; i < kKeep; ++i) {
-    const int c = t + 32 * kWarps * i;
-    if (c >= n_chunks) continue;
+  for (int i = 0; i < per_lane; ++i) {
+    const int c = lane + 32 * i;
+    if (c >= n_chunks) break;
     float v[kV], g[kV], b[kV];
-    C::unpack(keep[i], v);
+    C::unpack(chunk(i, c), v);
     C::unpack(__ldg(gm + c), g);
     if (beta) C::unpack(__ldg(bt + c), b);
 #pragma unroll
@@ -815,13 +812,11 @@ __global__ void __launch_bounds__(256) norm_forward_vec_kernel(const T* __restri
   }
 }
 
-template <typename T, int kWarps, int kKeep>
+template <typename T, int kKeep>
 cudaError_t launch_norm_vec(const void* X, int64_t n, int64_t d, int64_t ldx, const void* gamma, const void* beta, float eps,
                             int kind, void* A, int64_t lda, float* rstd, float* mean, cudaStream_t stream) {
-  const int rows = 8 / kWarps;
-  LORACT_CUDA_TRY(launch_pdl(norm_forward_vec_kernel<T, kWarps, kKeep>, dim3((unsigned)((n + rows - 1) / rows)), dim3(256), 0,
-                             stream, (const T*)X, n, d, ldx, (const T*)gamma, (const T*)beta, eps, kind, (T*)A, lda, rstd,
-                             mean));
+  LORACT_CUDA_TRY(launch_pdl(norm_forward_vec_kernel<T, kKeep>, dim3((unsigned)((n + 7) / 8)), dim3(256), 0, stream,
+                             (const T*)X, n, d, ldx, (const T*)gamma, (const T*)beta, eps, kind, (T*)A, lda, rstd, mean));
   return cudaGetLastError();
 }
 
@@ -833,15 +828,13 @@ cudaError_t launch_norm(const void* X, int64_t n, int64_t d, int64_t ldx, const 
   const bool vec = d % kV == 0 && ldx % kV == 0 && lda % kV == 0 && (((uintptr_t)X | (uintptr_t)A |
                    (uintptr_t)gamma | (uintptr_t)beta) & 15) == 0;
   const int64_t chunks = d / kV;
-#define LORACT_NORM(W, K) return launch_norm_vec<T, W, K>(X, n, d, ldx, gamma, beta, eps, kind, A, lda, rstd, mean, stream)
-  // at most four chunks per thread up to 1024 chunks (d = 8192 in bf16), eight beyond; longer rows take the plain kernel
+#define LORACT_NORM(K) return launch_norm_vec<T, K>(X, n, d, ldx, gamma, beta, eps, kind, A, lda, rstd, mean, stream)
   if (vec) {
-    if (chunks <= 64) LORACT_NORM(1, 2);
-    if (chunks <= 128) LORACT_NORM(1, 4);
-    if (chunks <= 256) LORACT_NORM(2, 4);
-    if (chunks <= 512) LORACT_NORM(4, 4);
-    if (chunks <= 1024) LORACT_NORM(8, 4);
-    if (chunks <= 2048) LORACT_NORM(8, 8);
+    if (chunks <= 64) LORACT_NORM(2);
+    if (chunks <= 128) LORACT_NORM(4);
+    if (chunks <= 256) LORACT_NORM(8);
+    if (chunks <= 512) LORACT_NORM(16);
+    LORACT_NORM(0);
   }
 #undef LORACT_NORM
   const int warps = 8;

@@ -1,5 +1,5 @@
-"""GPU tests of the pre-norm forward at the widths where its launch shape changes (how many warps share a row and how many
-16-byte chunks a thread keeps), with row counts that do not fill a block and a row stride wider than the row."""
+"""GPU tests of the pre-norm forward at the widths where its form changes (how many 16-byte chunks a lane keeps in
+registers, and none), with row counts that do not fill a block and a row stride wider than the row."""
 import pytest
 import torch
 
