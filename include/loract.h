@@ -21,7 +21,9 @@
  *     in a 32-bit word at the start of `ws`; read it with loract_read_device_status.  After a clamped pivot
  *     or a non-finite input the outputs are still fully written (finite where the input was).  After an
  *     expired wait (LORACT_DEV_WAIT_EXPIRED) the kernel that gave up has skipped its stores: the outputs
- *     are unspecified and must not be used.
+ *     are unspecified and must not be used.  loract_reconstruct and loract_activation_backward take no `ws` and
+ *     have no such word: the library cannot report an expired wait there (two seconds without progress on the
+ *     device), and a caller that has to rule one out checks the result itself.
  *   - `ws` is scratch of at least loract_workspace_bytes(desc) bytes, 256-byte aligned, private to one
  *     in-flight call.  The same (seed, call_id, n_tokens, rank) always selects the same rows.
  */
@@ -145,7 +147,7 @@ loract_status_t loract_prenorm_backward(const loract_desc_t* desc, const void* U
  * grad_Z: device, n_tokens x d, row stride ldx.  grad_X: device, n_tokens x d, row stride ldx, written.  A~ is
  * never stored: its tiles exist only in tensor memory, inside the kernel that writes grad_X (grad_Z is read
  * once, grad_X written once, the factors read once).  bf16 only (LORACT_ERR_UNSUPPORTED for fp32).  Needs no
- * workspace. */
+ * workspace, and so has no device status word (see the conventions at the top). */
 loract_status_t loract_activation_backward(const loract_desc_t* desc, const void* U, const void* V,
                                            const void* grad_Z, int32_t kind, void* grad_X, void* stream);
 

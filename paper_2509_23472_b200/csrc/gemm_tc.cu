@@ -70,6 +70,7 @@ struct TcParams {
   int fuse_parts;     // fused epilogue: warps per quarter of the accumulator's rows
   int stages;         // one-tile kernels: stages of the ring
   int lower;          // wide forms: the operand with two tiles is lower triangular (see GemmDesc::lower)
+  int a_rows;         // rows of an A tile that one load brings: 64 (one-CTA kernel, up to 64 rows in all), otherwise kBM
   int panels;         // MN-major operands whose map has three dimensions (one load for all panels): bit 0 A, bit 1 B
   int early;          // operands that may be loaded before griddepcontrol.wait: bit 0 A, bit 1 B (streaming kernel: all)
   int halve_at_term;  // the accumulator is multiplied by 1/2 before the first product of this term (0: never)
@@ -508,7 +509,7 @@ gemm_tc_kernel(const __grid_constant__ TmapPack maps, const TcParams p) {
   int n_iter = kb_count * (kShareA ? 1 : p.n_terms);
   const uint32_t stage_bytes = kABytes + (uint32_t)b_tiles * p.b_bytes;
   // up to 64 rows the second half of the A tile is not loaded: its accumulator rows are never read
-  const uint32_t tx_bytes = stage_bytes - (p.M <= 64 ? kABytes / 2 : 0u);
+  const uint32_t tx_bytes = stage_bytes - (uint32_t)(kBM - p.a_rows) * (kBK * 2);
   // dynamic shared memory is declared 1024-aligned; round up anyway (swizzle atoms need it)
   unsigned char* tiles = (unsigned char*)(((uintptr_t)smem + 1023) & ~(uintptr_t)1023);
 
@@ -541,7 +542,7 @@ gemm_tc_kernel(const __grid_constant__ TmapPack maps, const TcParams p) {
       tma_load_panels(dst, &maps.a[term], &full_bar[s], k0, m0 >> 6);
     } else if (A_MN) {
       tma_load_2d(dst, &maps.a[term], &full_bar[s], m0, k0);
-      if (p.M > 64) tma_load_2d(dst + 8192, &maps.a[term], &full_bar[s], m0 + 64, k0);
+      if (p.a_rows > 64) tma_load_2d(dst + 8192, &maps.a[term], &full_bar[s], m0 + 64, k0);
     } else {
       tma_load_2d(dst, &maps.a[term], &full_bar[s], k0, m0);
     }
@@ -1726,6 +1727,7 @@ cudaError_t launch_variant(const TmapPack& maps, const TcParams& p, dim3 grid, s
 
 template <bool A_MN, bool B_MN, int kWide = WIDE_NONE>
 cudaError_t launch_pair_variant(const TmapPack& maps, const TcParams& p, dim3 grid, size_t smem, cudaStream_t stream) {
+  if (p.a_rows != kBM) return cudaErrorInvalidValue;   // the kernel waits for whole tiles of A
   static std::atomic<bool> configured[64];   // zero-initialised; set once the attribute is in place on a device
   int dev = 0;
   LORACT_CUDA_TRY(cudaGetDevice(&dev));
@@ -1756,6 +1758,7 @@ cudaError_t launch_pair_variant(const TmapPack& maps, const TcParams& p, dim3 gr
 // Pairs the streaming kernel is launched with: as many as can be resident at once (one CTA per SM).
 template <int kEp>
 cudaError_t launch_stream(const TmapPack& maps, TcParams p, size_t smem, cudaStream_t stream) {
+  if (p.a_rows != kBM) return cudaErrorInvalidValue;   // the kernel waits for whole tiles of A
   static std::atomic<bool> configured[64];   // zero-initialised; set once the attribute is in place on a device
   static std::atomic<int> max_pairs[64];
   int dev = 0;
@@ -2058,13 +2061,16 @@ cudaError_t gemm_tc_launch(const GemmDesc& g, uint32_t* dev_status, cudaStream_t
   };
 
   TmapPack maps;
+  // The fused epilogues run on the persistent kernel however few rows there are, and that one, like the other two-CTA forms (from
+  // 256 rows), expects whole tiles of A.
+  const bool fused = g.out == OUT_RMS_BWD || g.out == OUT_ACT_BWD;
+  p.a_rows = g.M <= 64 && !fused ? 64 : kBM;
   // MN-major operands whose extent and tiles are whole panels of 64: one load for all panels of a tile
-  const int a_rows = g.M <= 64 ? 64 : kBM;   // (one-CTA kernel: rows of an A tile that are loaded)
   p.panels = (g.a_mn && g.M % 64 == 0 ? 1 : 0) | (g.b_mn && g.N % 64 == 0 && b_rows % 64 == 0 ? 2 : 0);
   for (int t = 0; t < g.n_terms; ++t) {
-    if (p.panels & 1) LORACT_CUDA_TRY(get_tmap(g.terms[t].A, g.M, g.K, g.lda, 64, 64, &maps.a[t], 2, (uint32_t)a_rows / 64));
+    if (p.panels & 1) LORACT_CUDA_TRY(get_tmap(g.terms[t].A, g.M, g.K, g.lda, 64, 64, &maps.a[t], 2, (uint32_t)p.a_rows / 64));
     else if (g.a_mn) LORACT_CUDA_TRY(get_tmap(g.terms[t].A, g.M, g.K, g.lda, 64, 64, &maps.a[t]));
-    else LORACT_CUDA_TRY(get_tmap(g.terms[t].A, g.K, g.M, g.lda, 64, (uint32_t)a_rows, &maps.a[t]));
+    else LORACT_CUDA_TRY(get_tmap(g.terms[t].A, g.K, g.M, g.lda, 64, (uint32_t)p.a_rows, &maps.a[t]));
     if (p.panels & 2) LORACT_CUDA_TRY(get_tmap(g.terms[t].B, g.N, g.K, g.ldb, 64, 64, &maps.b[t], 2, (uint32_t)b_rows / 64));
     else if (g.b_mn) LORACT_CUDA_TRY(get_tmap(g.terms[t].B, g.N, g.K, g.ldb, 64, 64, &maps.b[t]));
     else LORACT_CUDA_TRY(get_tmap(g.terms[t].B, g.K, g.N, g.ldb, 64, (uint32_t)b_rows, &maps.b[t]));
@@ -2093,7 +2099,7 @@ cudaError_t gemm_tc_launch(const GemmDesc& g, uint32_t* dev_status, cudaStream_t
 
   // The fused epilogues (pre-norm and activation backward) exist in the persistent kernel only, which takes any number
   // of tiles: 256 columns wide where that gives every SM pair a tile, 128 otherwise.
-  if (g.out == OUT_RMS_BWD || g.out == OUT_ACT_BWD) {
+  if (fused) {
     TcParams sp = p;
     sp.early = g.out == OUT_RMS_BWD && g.a_early && g.b_early ? 1 : 0;
     sp.st_m_tiles = (g.M + 2 * kBM - 1) / (2 * kBM);

@@ -79,3 +79,24 @@ def test_nothing_is_written_past_the_row(dev):
     torch.cuda.synchronize()
     assert bool((gX[:, d:] == 3.0).all())
     assert torch.equal(gX[:, :d], B.activation_backward(U, V, gZ, B.ACT_SILU))
+
+
+# up to 64 rows the one-CTA kernel loads half tiles of A; the kernel of the fused epilogues takes whole ones at every size
+@pytest.mark.parametrize("n", [16, 40, 63, 64, 65])
+@pytest.mark.parametrize("d,r", [(136, 16), (1000, 16)])
+def test_few_rows(dev, n, d, r):
+    U, V, gZ, g = draw(dev, n, d, r, 5 * n + d)
+    a = U.double() @ V.double()
+    s = torch.sigmoid(a)
+    check(B.activation_backward(U, V, gZ, B.ACT_SILU), gZ.double() * s * (1 + a * (1 - s)), 1.0)
+    gelu = 0.5 * (1 + torch.erf(a / 2 ** 0.5)) + a * torch.exp(-a * a / 2) / (2 * torch.pi) ** 0.5
+    check(B.activation_backward(U, V, gZ, B.ACT_GELU), gZ.double() * gelu, 1.0)
+    gamma = (1.0 + 0.2 * torch.randn(d, generator=g, device=dev)).bfloat16()
+    rstd = torch.rand(n, generator=g, device=dev) + 0.5
+    ws = B.alloc_workspace(B.make_desc(gZ, r), dev)
+    got = B.prenorm_backward(U, V, gamma, rstd, gZ, ws=ws)
+    assert B.read_device_status(ws) == 0
+    gm, ga = gamma.double(), gZ.double()
+    inner = (ga * a).mean(dim=1, keepdim=True)
+    check(got, rstd.double()[:, None] * (ga * gm - a / gm * inner),
+          float((ga * gm).square().mean().sqrt() + (a / gm * inner).square().mean().sqrt()))
