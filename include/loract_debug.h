@@ -59,6 +59,12 @@ void loract_debug_set_pair_mode(int32_t on);
 int32_t loract_debug_wide_form(int32_t M, int32_t N, int32_t K, int32_t a_mn, int32_t b_mn, int32_t n_terms,
                                int32_t splits);
 
+/* The number of ranges into which the contraction of a product is split (host only): at most `max_splits`, and as many as fill
+ * the chip up to `free_sums`, the number of partial sums that cost nothing to add up.  A range is ceil(K blocks of 64 / ranges)
+ * blocks long, and none is empty. */
+int32_t loract_debug_planned_splits(int32_t M, int32_t N, int32_t K, int32_t a_mn, int32_t b_mn, int32_t max_splits,
+                                    int32_t free_sums);
+
 /* W (l x l fp32) = (Yh + Yl)^T (Yh + Yl) of a tall bf16 pair (n x l) as the orthonormalisation forms it above 256 columns
  * (256 < l <= 512, l % 8 == 0).  partials: loract_debug_gram_bytes(n, l) bytes, 256-byte aligned; 0: l is not taken. */
 size_t loract_debug_gram_bytes(int64_t n, int32_t l);

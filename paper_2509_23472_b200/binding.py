@@ -361,7 +361,8 @@ DEBUG_EXPORTS = ("loract_debug_gemm", "loract_debug_small_block", "loract_debug_
                  "loract_debug_last_cuda_error", "loract_debug_trace_begin", "loract_debug_trace_end",
                  "loract_debug_wait_expiry", "loract_debug_project", "loract_debug_gemm_halved",
                  "loract_debug_reduce_sym", "loract_debug_set_round_gate", "loract_debug_round_gate",
-                 "loract_debug_set_big_clusters", "loract_debug_wide_form", "loract_debug_gram_bytes", "loract_debug_gram")
+                 "loract_debug_set_big_clusters", "loract_debug_wide_form", "loract_debug_gram_bytes", "loract_debug_gram",
+                 "loract_debug_planned_splits")
 
 
 def _debug_lib():
@@ -458,6 +459,14 @@ def debug_wide_form(M: int, N: int, K: int, a_mn: bool, b_mn: bool, terms: int =
     l.loract_debug_wide_form.restype = ctypes.c_int32
     l.loract_debug_wide_form.argtypes = [ctypes.c_int32] * 7
     return int(l.loract_debug_wide_form(M, N, K, int(a_mn), int(b_mn), terms, splits))
+
+
+def debug_planned_splits(M: int, N: int, K: int, a_mn: bool, b_mn: bool, max_splits: int = 32, free_sums: int = 1) -> int:
+    """Test hook: the number of ranges into which the contraction of a product is split.  Host only."""
+    l = _debug_lib()
+    l.loract_debug_planned_splits.restype = ctypes.c_int32
+    l.loract_debug_planned_splits.argtypes = [ctypes.c_int32] * 7
+    return int(l.loract_debug_planned_splits(M, N, K, int(a_mn), int(b_mn), max_splits, free_sums))
 
 
 def debug_gram(Yh: torch.Tensor, Yl: torch.Tensor, status: Optional[torch.Tensor] = None) -> torch.Tensor:

@@ -1903,7 +1903,13 @@ int gemm_tc_pick_splits(int M, int N, int K, bool a_mn, bool b_mn, int max_split
   const bool pair = M >= 2 * kBM && (b_mn ? bn % 128 == 0 : bn % 32 == 0);   // by shape (not by the test hook)
   const long long units = pair ? (long long)((M + 2 * kBM - 1) / (2 * kBM)) * n_tiles : tiles;
   const int slots = pair ? 74 : 148;
-  if (base > 1 && base <= free_sums) return base;
+  // no empty split: with ceil(kb / sp) K blocks each, fewer splits may already cover the contraction (197 blocks
+  // in 32 splits of 7 leave three splits with nothing to do but write zeros)
+  auto without_empty = [&](int sp) {
+    const int per = (kb + sp - 1) / sp;
+    return (kb + per - 1) / per;
+  };
+  if (base > 1 && base <= free_sums) return without_empty(base);
   auto cost = [&](int sp) {
     const double rounds = (double)((units * sp + slots - 1) / slots);
     // the partial sums are read back once by the reduction (about 4 TB/s) behind one more launch
@@ -1920,8 +1926,7 @@ int gemm_tc_pick_splits(int M, int N, int K, bool a_mn, bool b_mn, int max_split
                         (sp > 1 ? 4.0 + (double)sp * M * N * 4.0 * (1.0 / 4.0e6 + 1.0 / 8.0e6) : 0.0);
       if (us < 0.98 * least) { least = us; best = sp; }
     }
-    const int per = (kb + best - 1) / best;
-    return (kb + per - 1) / per;
+    return without_empty(best);
   }
   double best_cost = cost(base);
   const int cap = max_splits < 8 ? max_splits : 8;
@@ -1930,11 +1935,7 @@ int gemm_tc_pick_splits(int M, int N, int K, bool a_mn, bool b_mn, int max_split
     const double c = cost(sp);
     if (c < best_cost && c < 0.85 * cost(base)) { best = sp; best_cost = c; }
   }
-  // no empty split: with ceil(kb / best) K blocks each, fewer splits may already cover the contraction (197 blocks
-  // in 32 splits of 7 leave three splits with nothing to do but write zeros)
-  const int per = (kb + best - 1) / best;
-  best = (kb + per - 1) / per;
-  return best < 1 ? 1 : best;
+  return without_empty(best);
 }
 
 // A product with many rows streams one operand (X) once, and its tiles take about 0.36 us per 64-wide K block whatever

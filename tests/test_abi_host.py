@@ -90,6 +90,15 @@ def test_bad_arguments_return_codes_and_launch_nothing(lib):
     assert B.status_string(4) == "workspace too small"
 
 
+@pytest.mark.parametrize("free_sums,max_splits", [(1, 32), (7, 32), (1, 64)])
+@pytest.mark.parametrize("m,n,mn_major", [(16, 16, False), (96, 96, False), (128, 128, False), (256, 256, False), (336, 336, True),
+                                          (64, 16, True), (256, 96, True), (512, 4096, True)])
+def test_no_range_of_a_contraction_is_empty(lib, m, n, mn_major, free_sums, max_splits):
+    for blocks in range(1, 513):
+        s = B.debug_planned_splits(m, n, 64 * blocks, mn_major, mn_major, max_splits, free_sums)
+        assert 1 <= s <= max_splits and (s - 1) * -(-blocks // s) < blocks, (blocks, s)
+
+
 def test_binding_refuses_cpu_tensors(lib):
     import torch
     with pytest.raises(RuntimeError):
