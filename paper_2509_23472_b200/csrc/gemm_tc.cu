@@ -2052,7 +2052,7 @@ cudaError_t gemm_tc_launch(const GemmDesc& g, uint32_t* dev_status, cudaStream_t
   p.lo_gate = g.lo_gate;
   p.lower = g.lower ? 1 : 0;
   p.early = g.gate ? 0 : (g.a_early ? 1 : 0) | (g.b_early ? 2 : 0);
-  // A ring of at least four stages; the epilogue takes it over as staging space, four boxes per warp where it holds them (a
+  // A ring of at least four stages (three where a stage holds the B tiles of several terms); the epilogue takes it over as staging space, four boxes per warp where it holds them (a
   // pair of outputs fills two at a time: 16384 x 4096, r = 256, a step of 190.4 -> 189.8 us).
   auto take_ring = [&](uint32_t stage_bytes) -> size_t {
     const int fit = std::min(kMaxStages, (int)(kRingBytes / stage_bytes));
@@ -2179,9 +2179,14 @@ cudaError_t gemm_tc_launch(const GemmDesc& g, uint32_t* dev_status, cudaStream_t
     return launch_pair_variant<false, false>(maps, p, pgrid, psmem, stream);
   }
   dim3 grid((g.N + p.bn - 1) / p.bn, (g.M + kBM - 1) / kBM, splits);
-  // Terms with one A (V^T (Th + Tm + Tl), the second product of a weight gradient) load it once, where the B tiles of all of
-  // them leave room for three stages.
-  bool one_a = g.a_mn && g.b_mn && g.n_terms > 1 && p.halve_at_term == 0 &&
+  // Terms with one A (V^T (Th + Tm + Tl), the second product of a weight gradient) load it once where its tile takes two loads (M
+  // not in whole panels) and there are four K blocks or more, and the B tiles of all terms leave room for three stages.  Measured,
+  // whole weight gradients in us, shared / not: d = 1000, g = 23: r = 128 12.4 / 11.9, r = 256 13.4 / 14.0, r = 512 15.5 / 18.7;
+  // g = 96: 10.9 / 10.8, 11.9 / 12.8, 14.6 / 17.2.  With A in panels the wait for the larger stage costs more than the loads
+  // it saves (d = 1024, g = 96: 10.9 / 10.3, 11.8 / 11.5, 14.3 / 14.2; d = 4096, r = 128: 11.0 / 10.4), but for narrow
+  // tiles of B over eight K blocks (r = 512, g = 16: d = 1024 11.3 / 11.6, d = 11008 14.9 / 15.7; g = 23: 23.7 / 24.3).
+  const bool one_a_pays = p.panels & 1 ? p.kb_total >= 8 && p.bn <= 32 : p.kb_total >= 4;
+  bool one_a = g.a_mn && g.b_mn && g.n_terms > 1 && p.halve_at_term == 0 && one_a_pays &&
                kABytes + (uint32_t)g.n_terms * p.b_bytes <= kRingBytes / 3;
   for (int t = 1; t < g.n_terms; ++t) one_a = one_a && g.terms[t].A == g.terms[0].A;
   const size_t smem = take_ring(kABytes + (one_a ? (uint32_t)g.n_terms : 1u) * p.b_bytes);

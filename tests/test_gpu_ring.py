@@ -33,6 +33,23 @@ def test_panels_and_stages(dev, m, n, k, a_mn, b_mn):
     assert float((C - a @ b).abs().max() / (a.abs() @ b.abs()).max()) <= (k / 16 + 1) * 2.0 ** -23 + 1e-6
 
 
+@pytest.mark.parametrize("m", [72, 136, 1000, 1024])   # (1024: whole panels, one term after the other)
+@pytest.mark.parametrize("n", [16, 24, 48, 96, 112])
+@pytest.mark.parametrize("k", [200, 256, 336, 512, 1600])
+def test_terms_that_share_their_first_operand(dev, m, n, k):
+    g = torch.Generator(device=dev)
+    g.manual_seed(m + 3 * n + 7 * k)
+    a = torch.randn(k, m, generator=g, device=dev).bfloat16()
+    b = [torch.randn(k, n, generator=g, device=dev).bfloat16() for _ in range(3)]   # of one size: each term counts in full
+    status = torch.zeros(1, dtype=torch.int32, device=dev)
+    C = B.debug_gemm([a, a, a], b, m, n, k, True, True, out_mode=B.OUT_F32, engine=1, status=status).double()
+    assert int(status.item()) == 0
+    want = a.t().double() @ (b[0].double() + b[1].double() + b[2].double())
+    size = a.t().double().abs() @ (b[0].double().abs() + b[1].double().abs() + b[2].double().abs())
+    # fp32 accumulation with truncation: 2^-23 of the running sum per instruction of sixteen products
+    assert float((C - want).abs().max() / size.max()) <= (3 * k / 16 + 3) * 2.0 ** -23
+
+
 @pytest.mark.parametrize("n,d,r,t", [(1024, 768, 64, 0), (5003, 1000, 336, 0), (4096, 2048, 128, 1), (16384, 1024, 256, 0)])
 def test_inputs_written_right_before_the_call(dev, n, d, r, t):
     """X, V and grad_A are written by a kernel of the same stream right in front of the call, over other values: the results
