@@ -37,6 +37,33 @@ def test_gram_above_256_columns(dev, n, l):
     assert float(err) <= (16 + n / 64 / 22 + 32) * 2.0 ** -23
 
 
+@pytest.mark.parametrize("n,l", [(264, 264), (600, 336), (5003, 336), (4095, 448), (16384, 512), (40001, 504)])
+def test_every_product_of_the_gram_matrix_counts(dev, n, l):
+    g = torch.Generator(device=dev)
+    g.manual_seed(n + 2 * l)
+    # two independent matrices of one size: each of the four products, the halved sum and the mirrored tile are of order one
+    A, Bm = (torch.randn(n, l, generator=g, device=dev).bfloat16() for _ in range(2))
+    W = B.debug_gram(A, Bm).double()
+    Yd = A.double() + Bm.double()
+    size = (A.double().abs() + Bm.double().abs())
+    err = ((W - Yd.t() @ Yd).abs() / (size.t() @ size)).max()
+    assert float(err) <= (16 + n / 64 / 22 + 32) * 2.0 ** -23
+
+
+@pytest.mark.parametrize("n,l", [(4096, 272), (16384, 320), (32768, 512)])
+def test_diagonal_of_the_gram_matrix_has_no_bias(dev, n, l):
+    g = torch.Generator(device=dev)
+    g.manual_seed(n + 3 * l)
+    Y = torch.randn(n, l, generator=g, device=dev)
+    Yh = Y.bfloat16()
+    Yl = (Y - Yh.float()).bfloat16()
+    want = (Yh.double() + Yl.double()).square().sum(0)
+    bias = ((B.debug_gram(Yh, Yl).diagonal().double() - want) / want).mean()
+    # twelve instructions of a block truncate a running sum that grows from nothing: at most half of 12 * 2^-23 = 7.2e-7 of it.
+    # Without the product of the low parts it would be 2.8e-6, with chains of thirty blocks 4e-6
+    assert abs(float(bias)) <= 8e-7
+
+
 @pytest.mark.parametrize("n,d,r", [(4096, 768, 272), (16384, 768, 512), (9000, 640, 448), (700, 11008, 512)])
 def test_steps_with_a_triangular_factor_in_two_tiles(dev, n, d, r):
     """Shapes at which the application of L^-T (many rows) or the test matrix (many columns) takes two tiles per CTA pair."""
