@@ -508,7 +508,8 @@ gemm_tc_kernel(const __grid_constant__ TmapPack maps, const TcParams p) {
   const int b_tiles = kShareA ? p.n_terms : 1;
   int n_iter = kb_count * (kShareA ? 1 : p.n_terms);
   const uint32_t stage_bytes = kABytes + (uint32_t)b_tiles * p.b_bytes;
-  // up to 64 rows the second half of the A tile is not loaded: its accumulator rows are never read
+  // up to 64 rows the second half of the A tile is not loaded: its accumulator rows are never read.  (Whole steps, half / whole
+  // tiles: 4096 x 5120, r = 64 80.9 / 81.3 us, 8192 x 4096, r = 48 87.6 / 88.4, 16384 x 2048, r = 16 79.5 / 80.4.)
   const uint32_t tx_bytes = stage_bytes - (uint32_t)(kBM - p.a_rows) * (kBK * 2);
   // dynamic shared memory is declared 1024-aligned; round up anyway (swizzle atoms need it)
   unsigned char* tiles = (unsigned char*)(((uintptr_t)smem + 1023) & ~(uintptr_t)1023);
@@ -1701,7 +1702,11 @@ int g_pair_mode = 1;   // 0: never use the two-CTA kernels (test hook); 1: by sh
 
 // Tile width.  Up to 256 columns one tile of whole 16s; above, the multiple of 64 with the least padding, the widest of these:
 // a tile of whole 64s leaves through staged stores (whole lines), and is one that a CTA pair can share.  (By padding alone, 336
-// columns were two tiles of 176: direct stores and one CTA a tile, 9 thousand cycles for an epilogue instead of 4.)
+// columns were two tiles of 176: direct stores and one CTA a tile, 9 thousand cycles for an epilogue instead of 4.)  It is the
+// better rule where it pads most, too (steps in us, this rule / least padding in 16s): 4096 x 1024, r = 272 143 / 154, r = 288
+// 144 / 159, r = 304 153 / 162; 16384 x 4096, r = 288 238 / 242, r = 304 250.0 / 249.6; 8192 rows, r = 128: 520 columns 88 / 95,
+// 776 88 / 91, 1160 95 / 105, 1920 102 / 116.  (Tiles of whole 32s: the same as this rule within 1 us, but 147 to 162 at r = 272
+// to 304 and 4096 rows.)
 int pick_bn(int N) {
   if (N <= 256) return (N + 15) / 16 * 16;
   int best = 256;

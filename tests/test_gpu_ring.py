@@ -33,6 +33,26 @@ def test_panels_and_stages(dev, m, n, k, a_mn, b_mn):
     assert float((C - a @ b).abs().max() / (a.abs() @ b.abs()).max()) <= (k / 16 + 1) * 2.0 ** -23 + 1e-6
 
 
+# up to 64 rows half a tile of A is loaded; the accumulator's other rows come from what the stage held
+@pytest.mark.parametrize("m", [8, 40, 56, 64, 72])
+@pytest.mark.parametrize("k", [72, 640, 1600])
+@pytest.mark.parametrize("a_mn,b_mn", [(False, False), (True, True)])
+def test_products_of_few_rows(dev, m, k, a_mn, b_mn):
+    g = torch.Generator(device=dev)
+    g.manual_seed(m + k)
+    n = 152
+    a = torch.randn(*((k, m) if a_mn else (m, k)), generator=g, device=dev).bfloat16()
+    b = torch.randn(*((k, n) if b_mn else (n, k)), generator=g, device=dev).bfloat16()
+    ad, bd = (a.t() if a_mn else a).double(), (b if b_mn else b.t()).double()
+    for splits in (1, 3):
+        status = torch.zeros(1, dtype=torch.int32, device=dev)
+        C = B.debug_gemm([a], [b], m, n, k, a_mn, b_mn, out_mode=B.OUT_F32, engine=1, splits=splits, status=status).double()
+        assert int(status.item()) == 0
+        C = C.sum(0) if splits > 1 else C
+        # fp32 accumulation with truncation: 2^-23 of the running sum per instruction of sixteen products
+        assert float((C - ad @ bd).abs().max() / (ad.abs() @ bd.abs()).max()) <= (k / 16 + 4) * 2.0 ** -23
+
+
 @pytest.mark.parametrize("m", [72, 136, 1000, 1024])   # (1024: whole panels, one term after the other)
 @pytest.mark.parametrize("n", [16, 24, 48, 96, 112])
 @pytest.mark.parametrize("k", [200, 256, 336, 512, 1600])
