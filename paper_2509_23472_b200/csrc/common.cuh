@@ -124,7 +124,8 @@ struct GemmDesc {
   bool a_early = false, b_early = false;
   // Tensor-core path: the K-major factor (B where both are K-major, A otherwise) is lower triangular, element (i, k) zero for
   // k > i, and its zeros may be left out: the forms with two accumulators skip the first one's K blocks beyond its rows.
-  // (512 columns, a quarter of the work: application of L^-T to 32768 rows 43 -> 36 us, test matrix of 512 x 11008 16.7 -> 14.5.)
+  // (512 columns, a quarter of the work; traced, with an event behind every kernel: application of L^-T to 32768 / 16384 rows 55.3 ->
+  // 49.2 / 30.8 -> 26.7 us, test matrix of 512 x 11008 22.4 -> 20.4.)
   bool lower = false;
   // Tensor-core path, both operands K-major, N <= 512: one CTA pair must own whole rows of the product (it has read its rows
   // of A before it stores them, so C may be A); see gemm_tc_can_own_rows.

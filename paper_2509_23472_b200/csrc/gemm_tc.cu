@@ -271,7 +271,7 @@ __device__ __forceinline__ float act_derivative(float a) {
 // instructions.  Instead each epilogue warp puts its 32 rows x 128 bytes into shared memory in the layout of a
 // 128-byte-swizzled TMA box (conflict free: the 16-byte chunk c of row i goes to chunk c ^ (i & 7)) and one
 // lane sends the box with a TMA store, which writes whole lines and clips at the edges of the output.  Each
-// warp cycles through kStoreBufs boxes of its own, so no barrier between warps is needed.  Two warps share each
+// warp cycles through one, two or four boxes of its own, so no barrier between warps is needed.  Two warps share each
 // quarter of the accumulator rows (a warp may only read the tensor-memory lanes 32 * (warp % 4) .. + 31); they
 // take alternate column groups.
 constexpr int kStoreBufs = 2;
@@ -458,7 +458,7 @@ __device__ __forceinline__ void tc_store_tile(const TcParams& p, const TmapPack&
 
 // Epilogue of one CTA (eight warps) of the one-tile kernels: waits for the accumulator, then writes it.
 // `ring` is the operand ring: once the accumulator is complete every load has landed and every MMA has read
-// its stage, so the epilogue warps take the ring over as staging space (8 KB per warp).
+// its stage, so the epilogue warps take the ring over as staging space (two or four boxes of 4 KB per warp).
 // n_acc accumulators, 256 tensor-memory columns apart: accumulator w is the tile at (m0 + w dm, n0 + w dn).
 __device__ __forceinline__ void tc_epilogue(const TcParams& p, const TmapPack& maps, uint32_t tmem_base,
                                           uint64_t* accum_bar, volatile int* abort_flag_ptr, int warp, int lane,
@@ -1390,7 +1390,8 @@ gemm_tc_stream_kernel(const __grid_constant__ TmapPack maps, const TcParams p) {
 //     rounding.  A chain of the tensor cores is 64 rows long whatever n is.  The reading costs nothing: 128 columns a thread and K block
 //     take the eight warps 500 cycles, the products 1536 or 2048.
 // The tiles below the diagonal get more ranges than the others, as their K blocks take longer.  Partial sums are whole tiles,
-// 256 x 256 in fp32, unit after unit.  Measured with the sum over them: 32768 x 512 53 -> 38 us, 16384 x 512 37 -> 26 us.
+// 256 x 256 in fp32, unit after unit.  Measured with the sum over them (traced, an event behind either kernel): 32768 x 512 59 ->
+// 47 us, 16384 x 512 45 -> 35 us.
 constexpr int kGramStages = 3;
 constexpr int kGramTile = 2 * kBM;
 struct GramParams {
