@@ -2190,8 +2190,9 @@ cudaError_t gemm_tc_launch(const GemmDesc& g, uint32_t* dev_status, cudaStream_t
   // whole weight gradients in us, shared / not: d = 1000, g = 23: r = 128 12.4 / 11.9, r = 256 13.4 / 14.0, r = 512 15.5 / 18.7;
   // g = 96: 10.9 / 10.8, 11.9 / 12.8, 14.6 / 17.2.  With A in panels the wait for the larger stage costs more than the loads
   // it saves (d = 1024, g = 96: 10.9 / 10.3, 11.8 / 11.5, 14.3 / 14.2; d = 4096, r = 128: 11.0 / 10.4), but for narrow
-  // tiles of B over eight K blocks (r = 512, g = 16: d = 1024 11.3 / 11.6, d = 11008 14.9 / 15.7; g = 23: 23.7 / 24.3).
-  const bool one_a_pays = p.panels & 1 ? p.kb_total >= 8 && p.bn <= 32 : p.kb_total >= 4;
+  // tiles of B over many K blocks: 16 columns from six on (r = 336: d = 1024 10.5 / 10.6, d = 11008 13.7 / 14.2; r = 512 11.3 /
+  // 11.6, 14.9 / 15.7; r = 256 not: 9.6 / 9.5, 12.9 / 12.4), 32 from eight on (d = 11008, g = 23: r = 512 23.7 / 24.3, r = 336 21.4 / 20.2).
+  const bool one_a_pays = p.kb_total >= 4 + (p.panels & 1 ? p.bn / 8 : 0);
   bool one_a = g.a_mn && g.b_mn && g.n_terms > 1 && p.halve_at_term == 0 && one_a_pays &&
                kABytes + (uint32_t)g.n_terms * p.b_bytes <= kRingBytes / 3;
   for (int t = 1; t < g.n_terms; ++t) one_a = one_a && g.terms[t].A == g.terms[0].A;
