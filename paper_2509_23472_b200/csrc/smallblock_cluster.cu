@@ -431,14 +431,6 @@ __device__ __forceinline__ void take_off_half(T* C, const T* A, const T* Bm, boo
       C[j * kGrp + 32 * i] = kBlockSums<T> && !from_zero ? C[j * kGrp + 32 * i] + acc[i][j] : acc[i][j];
 }
 
-__device__ __forceinline__ V4<float> ld4_global(const float* src) {
-  const float4 v = __ldg(reinterpret_cast<const float4*>(src));
-  return {{v.x, v.y, v.z, v.w}};
-}
-__device__ __forceinline__ V4<double> ld4_global(const double* src) {
-  const double2 a = __ldg(reinterpret_cast<const double2*>(src)), b = __ldg(reinterpret_cast<const double2*>(src) + 1);
-  return {{a.x, a.y, b.x, b.y}};
-}
 __device__ __forceinline__ void load_quad(const float* src, V4<float>& s) {
   const float4 v = __ldg(reinterpret_cast<const float4*>(src));
   s.v[0] += v.x; s.v[1] += v.y; s.v[2] += v.z; s.v[3] += v.w;
@@ -547,26 +539,34 @@ __global__ void __launch_bounds__(32 * warps_of<T, kBig>(), 1) small_block_clust
   pdl_wait();
   pdl_launch_dependents();
 
-  // ---- load: this CTA's block row, summed over the partials; the trace of W (same order of additions in every CTA)
-  // gives the diagonal shift and the pivot floor.  Up to eight blocks one matrix, the usual case, is fetched without a loop over the
-  // partials, at whose end every load is waited for in turn (with it a CTA with eight block rows started 5000 cycles after the
-  // first, and its solver lagged behind the chain from there on), and every warp adds up the trace for itself: r = 128 / 256
-  // 14.1 / 26.9 -> 13.5 / 25.2 us, fp64 r = 64 / 128 13.0 / 21.6 -> 12.2 / 20.9.  Above, where it is not the late rows that lag, the
-  // same costs 2 us (r = 512 67.9 -> 70.4).
+  // ---- load: this CTA's block row, summed over the partials, raw into its place.  One matrix, the usual case, is copied with
+  // cp.async: every copy is in flight before anything waits.  (Through registers, a CTA with sixteen block rows waited for seven loads in
+  // turn and started 4.3 us after the first; now 1.6.  Steps: fp32 512 x 768, r = 64 103.2 -> 100.9 us, 5003 x 1000, r = 336 174.4 -> 170.8, 16384 x 11008,
+  // r = 512 527 -> 521.6, 4096 x 5120, r = 64 80.6 -> 79.9.)  Meanwhile the trace of W (the same order of additions in every CTA
+  // and warp) gives the diagonal shift and the pivot floor.  The thread that wrote a quad of the diagonal adds the shift to it.
   {
     const T* parts = (const T*)p.partials;
     constexpr int kQuads = kB * kB / 4;
-    constexpr int kPerThread = ((kBig ? kBigBlk : Cfg<T>::kMaxR / kB) * kQuads + kCThreads - 1) / kCThreads;
-    V4<T> acc[kPerThread];
     const int n_quads = active ? (me + 1) * kQuads : 0;
-    const bool one = !kBig && p.n_partials == 1;
-    if (one) {
+    auto quad_at = [&](int e) { return target(e / kQuads) + (e & 7) * kGrp + ((e & (kQuads - 1)) >> 3) * 4; };
+#pragma unroll 1
+    for (int e = tid; e < n_quads; e += kCThreads) {
+      const int row = me * kB + ((e & (kQuads - 1)) >> 3), col = (e / kQuads) * kB + 4 * (e & 7);
+      const bool in = row < r && col < r;
+      const T* src = parts + (in ? (int64_t)row * p.in_ld + col : 0);
+      T* dst = quad_at(e);
+      if (p.n_partials == 1) {
 #pragma unroll
-      for (int u = 0; u < kPerThread; ++u) {
-        acc[u] = {{(T)0, (T)0, (T)0, (T)0}};
-        const int e = tid + u * kCThreads;
-        const int row = me * kB + ((e & (kQuads - 1)) >> 3), col = (e / kQuads) * kB + 4 * (e & 7);
-        if (e < n_quads && row < r && col < r) acc[u] = ld4_global(parts + (int64_t)row * p.in_ld + col);
+        for (int h = 0; h < (int)sizeof(T) / 4; ++h)
+          asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;"
+                       ::"r"(smem_addr(dst) + 16 * h), "l"((const unsigned char*)src + 16 * h), "r"(in ? 16 : 0) : "memory");
+      } else {
+        V4<T> acc = {{(T)0, (T)0, (T)0, (T)0}};
+        if (in) {
+#pragma unroll 4
+          for (int q = 0; q < p.n_partials; ++q) load_quad(src + (int64_t)q * p.partial_stride, acc);
+        }
+        st4(dst, acc);
       }
     }
     T t = (T)0;
@@ -578,68 +578,32 @@ __global__ void __launch_bounds__(32 * warps_of<T, kBig>(), 1) small_block_clust
         d += __ldg(parts + (int64_t)q * p.partial_stride + (int64_t)i * p.in_ld + i);
       t += d;
     }
-    if (!one) {
-#pragma unroll
-      for (int u = 0; u < kPerThread; ++u) {
-        acc[u] = {{(T)0, (T)0, (T)0, (T)0}};
-        const int e = tid + u * kCThreads;
-        if (e >= n_quads) continue;
-        const int row = me * kB + ((e & (kQuads - 1)) >> 3), col = (e / kQuads) * kB + 4 * (e & 7);
-        if (row < r && col < r) {
-          const T* src = parts + (int64_t)row * p.in_ld + col;
-#pragma unroll 4
-          for (int q = 0; q < p.n_partials; ++q) load_quad(src + (int64_t)q * p.partial_stride, acc[u]);
-        }
-      }
-    }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
     if (lane == 0) s_red[warp] = t;
     __syncthreads();
-    auto shift_and_floor = [&](T tr, T& shift_out) {
-      T mean_diag = tr / (T)r;
-      if (!(mean_diag == mean_diag) || mean_diag > (T)3.0e38 || mean_diag < (T)0) {
-        if (p.dev_status && me == 0 && tid == 0) atomicOr(p.dev_status, LORACT_DEV_NONFINITE);
-        mean_diag = (T)1;
-      }
-      if (mean_diag == (T)0) mean_diag = (T)1;
-      shift_out = (T)p.shift_rel * mean_diag;
-      if (tid == 0) {
-        s_shift = shift_out;
-        s_floor = mean_diag * (sizeof(T) == 8 ? (T)1e-15 : (T)1e-7);
-      }
-    };
-    T shift;
-    if (kBig) {
-      if (tid == 0) {
-        T tr = (T)0;
-#pragma unroll 1
-        for (int q = 0; q < kWarps; ++q) tr += s_red[q];
-        shift_and_floor(tr, shift);
-      }
-      __syncthreads();
-      shift = s_shift;
-    } else {
-      t = lane < kWarps ? s_red[lane] : (T)0;
+    t = lane < kWarps ? s_red[lane] : (T)0;
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-      shift_and_floor(t, shift);
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    T mean_diag = t / (T)r;
+    if (!(mean_diag == mean_diag) || mean_diag > (T)3.0e38 || mean_diag < (T)0) {
+      if (p.dev_status && me == 0 && tid == 0) atomicOr(p.dev_status, LORACT_DEV_NONFINITE);
+      mean_diag = (T)1;
     }
-#pragma unroll
-    for (int u = 0; u < kPerThread; ++u) {
-      const int e = tid + u * kCThreads;
-      if (e >= n_quads) continue;
-      const int bj = e / kQuads, a = (e & (kQuads - 1)) >> 3, q4 = e & 7;
-      T* dst = target(bj) + q4 * kGrp + a * 4;
-      if (bj == me) {
-        const int dcol = a - 4 * q4;  // position of the diagonal element inside this quad, if any
-        const bool in_range = (me * kB + a) < r;            // padding rows of a ragged last block: identity
-        const T mul = in_range ? (T)p.shift_diag_rel : (T)0, add = in_range ? shift : (T)1;
-#pragma unroll
-        for (int h = 0; h < 4; ++h)
-          if (dcol == h) acc[u].v[h] += acc[u].v[h] * mul + add;
-      }
-      st4(dst, acc[u]);
+    if (mean_diag == (T)0) mean_diag = (T)1;
+    const T shift = (T)p.shift_rel * mean_diag;
+    if (tid == 0) {
+      s_shift = shift;
+      s_floor = mean_diag * (sizeof(T) == 8 ? (T)1e-15 : (T)1e-7);
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    // this thread's quad of the diagonal block, if any (a block has fewer quads than the CTA threads)
+    const int a0 = me * kQuads, e = a0 + (tid + kCThreads - a0 % kCThreads) % kCThreads;
+    const int a = (e & (kQuads - 1)) >> 3, dcol = a - 4 * (e & 7);
+    if (active && e < a0 + kQuads && dcol >= 0 && dcol < 4) {
+      const bool in_range = me * kB + a < r;              // padding rows of a ragged last block: identity
+      T* at = quad_at(e) + dcol;
+      *at = in_range ? *at + (*at * (T)p.shift_diag_rel + shift) : (T)1;
     }
   }
   __syncthreads();
