@@ -110,13 +110,16 @@ __device__ __forceinline__ void bar_expect(uint64_t* bar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar)), "r"(bytes)
                : "memory");
 }
-__device__ __forceinline__ void bar_arrive_local(uint64_t* bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(bar)) : "memory");
-}
-// All lanes have written; one arrival announces it.
+// All lanes have written; one arrival announces it.  Predicated, like the stores of single lanes on the chain: a branch around
+// them costs more than they do.
 __device__ __forceinline__ void warp_arrive(uint64_t* bar, int lane) {
   __syncwarp();
-  if (lane == 0) bar_arrive_local(bar);
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.eq.s32 p, %1, 0;\n\t"
+      "@p mbarrier.arrive.shared::cta.b64 _, [%0];\n\t}"
+      ::"r"(smem_addr(bar)), "r"(lane)
+      : "memory");
 }
 // kFromPeers: what warps of other CTAs did before they arrived has to be ordered as well (acquire at cluster scope).
 template <bool kFromPeers>
@@ -210,6 +213,24 @@ __device__ __forceinline__ void st4(double* p, const V4<double>& x) {
   *reinterpret_cast<double2*>(p) = make_double2(x.v[0], x.v[1]);
   *reinterpret_cast<double2*>(p + 2) = make_double2(x.v[2], x.v[3]);
 }
+// The same for the lanes with `on` set, without a branch.
+__device__ __forceinline__ void st4_if(bool on, float* p, const V4<float>& x) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ne.s32 p, %5, 0;\n\t"
+      "@p st.shared.v4.f32 [%0], {%1, %2, %3, %4};\n\t}"
+      ::"r"(smem_addr(p)), "f"(x.v[0]), "f"(x.v[1]), "f"(x.v[2]), "f"(x.v[3]), "r"((int)on)
+      : "memory");
+}
+__device__ __forceinline__ void st4_if(bool on, double* p, const V4<double>& x) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ne.s32 p, %5, 0;\n\t"
+      "@p st.shared.v2.f64 [%0], {%1, %2};\n\t"
+      "@p st.shared.v2.f64 [%0 + 16], {%3, %4};\n\t}"
+      ::"r"(smem_addr(p)), "d"(x.v[0]), "d"(x.v[1]), "d"(x.v[2]), "d"(x.v[3]), "r"((int)on)
+      : "memory");
+}
 // acc - a . b over four elements
 template <typename T>
 __device__ __forceinline__ T sub4(T acc, const V4<T>& a, const V4<T>& b) {
@@ -296,11 +317,11 @@ __device__ __forceinline__ bool factor_diagonal(const T* staged, T* panels, uint
     pivot(3, f3);
     x.v[3] = w3 * rz.v[3];
     st4(pan + lane * 4, x);
-    if (lane == 0) st4(pan + kGrp, rz);
-    if (lane == 1) st4(pan + kGrp + 4, rd);
+    st4(pan + kGrp, rz);                   // (the same values in every lane)
+    st4(pan + kGrp + 4, rd);
     __syncwarp();
     if (p < kPan - 2) named_arrive(id_published(p), readers_of(p));
-    if (lane == 0) bar_arrive_local(bars + p);
+    warp_arrive(bars + p, lane);
     staged += kGrp;
     pan += kPanElems;
   }
@@ -349,7 +370,7 @@ __device__ __forceinline__ void solve_half(const V4<T> (&was)[2], V4<T> (&acc)[2
     x.v[1] = fma(-x.v[0], r1.v[0], t.v[1]) * rr.v[1];
     x.v[2] = fma(-x.v[1], r2.v[1], fma(-x.v[0], r2.v[0], t.v[2])) * rr.v[2];
     x.v[3] = fma(-x.v[2], r3.v[2], fma(-x.v[1], r3.v[1], fma(-x.v[0], r3.v[0], t.v[3]))) * rr.v[3];
-    if (cg == q) st4(blk + p * kGrp + row * 4, x);
+    st4_if(cg == q, blk + p * kGrp + row * 4, x);
     warp_arrive(sol_bars + p, lane);
 #pragma unroll
     for (int u = 0; u < 4; ++u) x.v[u] = __shfl_sync(0xffffffffu, x.v[u], (q << 3) | (lane & 7));
