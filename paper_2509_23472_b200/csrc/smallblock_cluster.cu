@@ -172,6 +172,8 @@ __device__ __forceinline__ void bar_drain(uint64_t* bar) {
   while (!bar_try<false>(bar) && timer_ns() - t0 <= kClusterWaitNs) {}
 }
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+// Execution only: does not wait for this thread's stores (the output) to reach L2, which takes 0.6 us.
+__device__ __forceinline__ void cluster_arrive_relaxed() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 // Named barriers between the pivot warp and the follow-up warps, each used once: group g of the diagonal block has been
 // handed over (64 threads), group g has been published (the pivot warp and every follow-up warp that needs it).
@@ -494,6 +496,7 @@ __global__ void __launch_bounds__(32 * warps_of<T, kBig>(), 1) small_block_clust
   __shared__ __align__(8) uint64_t rdy_bar[kMaxBlk];         // the block to solve at step k has every update
   __shared__ __align__(8) uint64_t bulk_bar[kMaxBlk];        // block j has every update but that of step j - 1
   __shared__ __align__(8) uint64_t free_bar[kBig ? kMaxBlk : 1];   // every peer is done with what step k received
+  __shared__ __align__(8) uint64_t est_bar;                  // CTA 0: every share of the estimate is here
   __shared__ uint32_t s_done[kBig ? kMaxBlk : 1];            // warps of this CTA that are done with what step k received
   __shared__ T s_red[kWarps];
   __shared__ T s_shift, s_floor;
@@ -553,9 +556,12 @@ __global__ void __launch_bounds__(32 * warps_of<T, kBig>(), 1) small_block_clust
     if (block_comes(i, b - off_slot(i, 0))) bar_expect(&off_bar[b], kBlkBytes);
   } else if (tid == kMaxBlk * kPan + kMaxOff) {
     s_gave_up = 0;
+    bar_init(&est_bar, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    if (!kBig && p.gate_out && me == 0) bar_expect(&est_bar, (uint32_t)(kBulkWarps * nblk * sizeof(float)));
   }
   __syncthreads();
-  cluster_arrive();                       // waited for below: nobody sends before every CTA's barriers exist
+  cluster_arrive();                       // waited for under the load: nobody sends before every CTA's barriers exist
   // everything above overlaps the tail of the previous kernel; global memory only from here on
   pdl_wait();
   pdl_launch_dependents();
@@ -590,6 +596,11 @@ __global__ void __launch_bounds__(32 * warps_of<T, kBig>(), 1) small_block_clust
         st4(dst, acc);
       }
     }
+    // (0.4 us however long ago the others arrived: under the copies; kBig: 0.5 us slower so)
+    if (!kBig) {
+      __syncwarp();
+      cluster_wait();
+    }
     T t = (T)0;
 #pragma unroll 1
     for (int i = tid; i < r; i += kCThreads) {
@@ -608,7 +619,7 @@ __global__ void __launch_bounds__(32 * warps_of<T, kBig>(), 1) small_block_clust
     for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
     T mean_diag = t / (T)r;
     if (!(mean_diag == mean_diag) || mean_diag > (T)3.0e38 || mean_diag < (T)0) {
-      if (p.dev_status && me == 0 && tid == 0) atomicOr(p.dev_status, LORACT_DEV_NONFINITE);
+      if (p.dev_status && me == 0 && tid == 0) { atomicOr(p.dev_status, LORACT_DEV_NONFINITE); __threadfence(); }
       mean_diag = (T)1;
     }
     if (mean_diag == (T)0) mean_diag = (T)1;
@@ -628,7 +639,7 @@ __global__ void __launch_bounds__(32 * warps_of<T, kBig>(), 1) small_block_clust
     }
   }
   __syncthreads();
-  cluster_wait();
+  if (kBig) cluster_wait();
 
   volatile int* gave_up = &s_gave_up;
   const T floor_ = s_floor;
@@ -666,7 +677,7 @@ __global__ void __launch_bounds__(32 * warps_of<T, kBig>(), 1) small_block_clust
     const bool clamped = factor_diagonal<T>(own, panel(me), pan_bar[me], floor_, lane);
     if (kBig && me >= kBigPans) bar_wait<true>(&free_bar[me - kBigPans], gave_up);   // the ring slot is free in every peer
     send(panel(me) + (kPan - 1) * kPanElems, panel(me) + (kPan - 1) * kPanElems, kPanBytes, &pan_bar[me][kPan - 1], peer);
-    if (clamped && lane == 0 && p.dev_status) atomicOr(p.dev_status, LORACT_DEV_PIVOT_CLAMPED);
+    if (clamped && lane == 0 && p.dev_status) { atomicOr(p.dev_status, LORACT_DEV_PIVOT_CLAMPED); __threadfence(); }
   } else if (role < R_SOLVE) {
     // ---- follow-up warps
     const int w = role - R_FOLLOW;
@@ -781,8 +792,8 @@ __global__ void __launch_bounds__(32 * warps_of<T, kBig>(), 1) small_block_clust
 #pragma unroll 1
     for (int k = 0; k < nblk; ++k) {
       const T* blk = solved(k);
-      bar_wait(&sol_bar[k][kPan - 1], gave_up);
       const int j_end = k < me ? me + 1 : nblk;
+      if (kBig || k + 2 < j_end) bar_wait(&sol_bar[k][kPan - 1], gave_up);
 #pragma unroll 1
       for (int j = k + 2; j < j_end; ++j) {
         if (j % (kBulkWarps / 2) != (m >> 1)) continue;        // the same pair of warps for a block in every step
@@ -794,6 +805,9 @@ __global__ void __launch_bounds__(32 * warps_of<T, kBig>(), 1) small_block_clust
       if (k < me) continue;
 #pragma unroll 1
       for (int q = m; q < kPan; q += kBulkWarps) {
+        // without updates in front, as in the last step, group by group (kBig: a warp waits for the whole block in any case, as
+        // the repeated look at a barrier costs 1 us at r = 512)
+        if (!kBig) bar_wait(&sol_bar[k][q], gave_up);
         // rows 32 k + 4 q .. + 3 of the result: element (32 k + 4 q + u, col) = X[group q][lane][u]
         const V4<T> v4 = ld4(blk + q * kGrp + lane * 4);
         const int row = k * kB + 4 * q;
@@ -817,8 +831,13 @@ __global__ void __launch_bounds__(32 * warps_of<T, kBig>(), 1) small_block_clust
       // this warp's share of the estimate, summed in a fixed order and handed to CTA 0
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) est += __shfl_xor_sync(0xffffffffu, est, o);
-      if (lane == 0)
+      if (kBig && lane == 0)
         asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(map_to_cta(smem_addr(&s_est[kBulkWarps * me + m]), 0)), "f"(est)
+                     : "memory");
+      if (!kBig && lane == 0)
+        asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];"
+                     ::"r"(map_to_cta(smem_addr(&s_est[kBulkWarps * me + m]), 0)), "r"(__float_as_uint(est)),
+                       "r"(map_to_cta(smem_addr(&est_bar), 0))
                      : "memory");
     }
   } else {
@@ -847,7 +866,7 @@ __global__ void __launch_bounds__(32 * warps_of<T, kBig>(), 1) small_block_clust
   }
   __syncthreads();
   if (s_gave_up) {
-    if (tid == 0 && p.dev_status) atomicOr(p.dev_status, LORACT_DEV_WAIT_EXPIRED);
+    if (tid == 0 && p.dev_status) { atomicOr(p.dev_status, LORACT_DEV_WAIT_EXPIRED); __threadfence(); }
     // what nobody waited for to the end must land before the shared memory goes away
     if (tid < kMaxBlk * kPan) {
       const int k = tid / kPan, q = tid % kPan;
@@ -859,11 +878,15 @@ __global__ void __launch_bounds__(32 * warps_of<T, kBig>(), 1) small_block_clust
     }
     __syncthreads();
   }
-  // no CTA leaves while another may still write into its shared memory or read its own through a copy
-  cluster_arrive();
+  // No CTA leaves while another may still write into its shared memory or read its own through a copy.  kBig: the arrivals on
+  // other CTAs' free_bar must have been performed as well, hence the releasing form there; elsewhere everything that is written into
+  // another CTA is waited for there.
+  if (kBig) cluster_arrive(); else cluster_arrive_relaxed();
   cluster_wait();
   if (p.gate_out && me == 0 && warp == 0) {
-    // after the cluster barrier: every share has arrived, every status bit of this call is set
+    // after the cluster barrier every status bit of this call is set (who sets one fences); the shares of the estimate are here (kBig)
+    // or counted
+    if (!kBig && !bar_wait<true>(&est_bar, gave_up)) bar_drain(&est_bar);
     const uint32_t st = p.dev_status ? *(const volatile uint32_t*)p.dev_status : 0u;
     float est = 0.f;
 #pragma unroll 1
