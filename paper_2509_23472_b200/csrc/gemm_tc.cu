@@ -32,6 +32,7 @@ constexpr int kBK = 64;          // bf16 elements = one 128-byte swizzle row
 constexpr int kMaxStages = 12;
 constexpr uint32_t kRingBytes = 208 * 1024;
 constexpr int kThreads = 320;    // warp 0: TMA, warp 1: MMA + tensor memory, warps 2..9: epilogue
+constexpr int kProducers = 4;    // one-CTA kernel: warps that fill the ring (two in the two-CTA kernel)
 constexpr int kEpiWarps = 8;     // two per quarter of the tensor-memory lanes: they take alternate column groups
 constexpr uint32_t kABytes = kBM * kBK * 2;
 constexpr uint64_t kWaitLimitNs = 2000000000ull;  // 2 s
@@ -502,6 +503,10 @@ gemm_tc_kernel(const __grid_constant__ TmapPack maps, const TcParams p) {
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int stages = p.stages;
+  // No more producers than stages: a producer that waits for a stage then knows that the use before the last one of it is over (its own
+  // previous wait was for a later K block), and cannot take the parity of that use for the one it waits for.
+  const int producers = stages < kProducers ? 2 : kProducers;
+  const int producer = warp == 0 ? 0 : (warp >= 2 && warp <= producers ? warp - 1 : -1);
   const int n0 = blockIdx.x * p.bn, m0 = blockIdx.y * kBM, split = blockIdx.z;
   const int kb_begin = split * p.kb_per_split;
   const int kb_count = max(0, min(p.kb_total, kb_begin + p.kb_per_split) - kb_begin);
@@ -561,19 +566,21 @@ gemm_tc_kernel(const __grid_constant__ TmapPack maps, const TcParams p) {
       }
     }
   };
-  // K block and term of the next iteration of a producer: warps 0 and 2 (which becomes an epilogue warp) take turns.
-  // One producer alone, with up to six loads and a barrier to wait for per K block, takes 440 to 900 cycles for it.
+  // K block and term of the next iteration of a producer: warps 0 and 2 to 4 (which become epilogue warps) take turns (0 and 2
+  // where the ring has three stages).  One producer alone, with up to six loads and a barrier to wait for per K block, takes 440 to 900 cycles for it.  (Four instead of
+  // two: steps of 12608 x 768, r = 96 95.6 -> 94.1 us, 8192 x 5120, r = 128 with a power
+  // iteration 207.7 -> 207.3, 4096 x 5120, r = 64 78.5 -> 78.3.)
   auto next_block = [&](int& term, int& kb) {
-    kb += 2;
+    kb += producers;
     while (kb >= kb_count) { kb -= kb_count; ++term; }
   };
   // The ring is filled with what does not depend on the previous kernel (see GemmDesc::a_early).
   const int n_pre = p.early ? min(stages, n_iter) : 0;
-  if (n_pre > 0 && (warp == 0 || warp == 2)) {
+  if (n_pre > 0 && producer >= 0) {
     if (elect_one()) {
-      int term = 0, kb = warp == 0 ? -2 : -1;
+      int term = 0, kb = producer - producers;
       next_block(term, kb);
-      for (int it = warp == 0 ? 0 : 1; it < n_pre; it += 2) {
+      for (int it = producer; it < n_pre; it += producers) {
         mbar_arrive_expect_tx(&full_bar[it], tx_bytes);
         if (p.early & 1) load_a(it, term, (kb_begin + kb) * kBK);
         if (p.early & 2) load_b(it, term, (kb_begin + kb) * kBK);
@@ -589,13 +596,13 @@ gemm_tc_kernel(const __grid_constant__ TmapPack maps, const TcParams p) {
   if (p.clear_status && p.dev_status && threadIdx.x == 0 && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0)
     *(volatile uint32_t*)p.dev_status = 0u;
 
-  if ((warp == 0 || warp == 2) && n_iter > 0) {
+  if (producer >= 0 && n_iter > 0) {
     if (elect_one()) {
       // stage, parity, term and K block are carried along (no division in the loop)
-      int s = warp == 0 ? 0 : 1, term = 0, kb = warp == 0 ? -2 : -1;
+      int s = producer, term = 0, kb = producer - producers;
       next_block(term, kb);
       uint32_t parity = 1u;
-      for (int it = warp == 0 ? 0 : 1; it < n_iter; it += 2) {
+      for (int it = producer; it < n_iter; it += producers) {
         const int k0 = (kb_begin + kb) * kBK;
         const bool pre = it < n_pre;
         if (!pre) {
@@ -604,7 +611,7 @@ gemm_tc_kernel(const __grid_constant__ TmapPack maps, const TcParams p) {
         }
         if (!(pre && (p.early & 1))) load_a(s, term, k0);
         if (!(pre && (p.early & 2))) load_b(s, term, k0);
-        s += 2; if (s >= stages) { s -= stages; parity ^= 1u; }
+        s += producers; if (s >= stages) { s -= stages; parity ^= 1u; }
         next_block(term, kb);
       }
     }
