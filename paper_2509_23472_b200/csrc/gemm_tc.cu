@@ -32,7 +32,7 @@ constexpr int kBK = 64;          // bf16 elements = one 128-byte swizzle row
 constexpr int kMaxStages = 12;
 constexpr uint32_t kRingBytes = 208 * 1024;
 constexpr int kThreads = 320;    // warp 0: TMA, warp 1: MMA + tensor memory, warps 2..9: epilogue
-constexpr int kProducers = 4;    // one-CTA kernel: warps that fill the ring (two in the two-CTA kernel)
+constexpr int kProducers = 4;    // warps that fill the ring, at most
 constexpr int kEpiWarps = 8;     // two per quarter of the tensor-memory lanes: they take alternate column groups
 constexpr uint32_t kABytes = kBM * kBK * 2;
 constexpr uint64_t kWaitLimitNs = 2000000000ull;  // 2 s
@@ -781,7 +781,9 @@ gemm_tc_pair_kernel(const __grid_constant__ TmapPack maps, const TcParams p) {
   const int kb_count = max(0, min(p.kb_total, kb_begin + p.kb_per_split) - kb_begin);
   int n_iter = kb_count * p.n_terms;
   const uint32_t stage_bytes = kNA * kABytes + kNB * p.b_bytes;   // per CTA (b_bytes: half a B tile)
-  const int stages = p.stages;
+  const int stages = p.stages;                               // (four or more)
+  const int producers = kWide == WIDE_NONE && p.bn <= 128 ? kProducers : 2;
+  const int producer = warp == 0 ? 0 : (warp >= 2 && warp <= producers ? warp - 1 : -1);
   unsigned char* tiles = (unsigned char*)(((uintptr_t)smem + 1023) & ~(uintptr_t)1023);
 
   // a gated launch that is not needed: both CTAs of the pair read the same word and leave before any set-up (see the
@@ -857,18 +859,20 @@ gemm_tc_pair_kernel(const __grid_constant__ TmapPack maps, const TcParams p) {
       }
     }
   };
-  // K block and term of the next iteration of a producer (two producers take turns)
+  // K block and term of the next iteration of a producer.  Two producers take turns (warps 0 and 2), or four (0, 2, 3 and 4) where
+  // the tile of B is narrow and a K block short: up to 128 columns (steps of 4096 x 5120, r = 64 76.5 -> 75.7 us, 8192 x 5120, r = 128 with
+  // a power iteration 205.8 -> 204.5, 12608 x 768, r = 96 92.7 -> 92.0; above, 5003 x 1000, r = 336 171.2 -> 171.9).
   auto next_block = [&](int& term, int& kb) {
-    kb += 2;
+    kb += producers;
     while (kb >= kb_count) { kb -= kb_count; ++term; }
   };
   // The ring is filled with what does not depend on the previous kernel (see GemmDesc::a_early).
   const int n_pre = p.early ? min(stages, n_iter) : 0;
-  if (n_pre > 0 && (warp == 0 || warp == 2)) {
+  if (n_pre > 0 && producer >= 0) {
     if (elect_one()) {
-      int term = 0, kb = warp == 0 ? -2 : -1;
+      int term = 0, kb = producer - producers;
       next_block(term, kb);
-      for (int it = warp == 0 ? 0 : 1; it < n_pre; it += 2) {
+      for (int it = producer; it < n_pre; it += producers) {
         if (leader) mbar_arrive_expect_tx(&full_bar[it], 2u * tx_bytes(kb));
         if (p.early & 1) load_a(it, term, kb);
         if (p.early & 2) load_b(it, term, kb);
@@ -883,14 +887,14 @@ gemm_tc_pair_kernel(const __grid_constant__ TmapPack maps, const TcParams p) {
   if (p.clear_status && p.dev_status && threadIdx.x == 0 && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0)
     *(volatile uint32_t*)p.dev_status = 0u;
 
-  if ((warp == 0 || warp == 2) && n_iter > 0) {
+  if (producer >= 0 && n_iter > 0) {
     if (elect_one()) {
       // stage, parity, term and K block are carried along (no division in the loop)
-      int s = warp == 0 ? 0 : 1;
+      int s = producer;
       uint32_t parity = 1u;
-      int term = 0, kb = warp == 0 ? -2 : -1;
+      int term = 0, kb = producer - producers;
       next_block(term, kb);
-      for (int it = warp == 0 ? 0 : 1; it < n_iter; it += 2) {
+      for (int it = producer; it < n_iter; it += producers) {
         const bool pre = it < n_pre;
         if (!pre) {
           if (!mbar_wait_bounded(&empty_bar[s], parity, &abort_flag)) break;
@@ -899,7 +903,7 @@ gemm_tc_pair_kernel(const __grid_constant__ TmapPack maps, const TcParams p) {
         }
         if (!(pre && (p.early & 1))) load_a(s, term, kb);
         if (!(pre && (p.early & 2))) load_b(s, term, kb);
-        s += 2; if (s >= stages) { s -= stages; parity ^= 1u; }
+        s += producers; if (s >= stages) { s -= stages; parity ^= 1u; }
         next_block(term, kb);
       }
     }
