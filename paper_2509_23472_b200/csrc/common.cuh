@@ -120,7 +120,8 @@ struct GemmDesc {
   // Tensor-core path: every A (every B) of the terms was written ahead of the previous kernel of the stream, i.e. at least two
   // launches back.  A grid only starts once its predecessor has passed its own griddepcontrol.wait, which is once everything
   // ahead of the predecessor is complete and visible; so such an operand may be loaded before this grid's own wait, under
-  // the predecessor's work.  OUT_RMS_BWD: both flags together speak for A, B and ep_E.
+  // the predecessor's work.  (Behind a row of gated launches: written ahead of the kernel before the last one that is not gated.)
+  // OUT_RMS_BWD: both flags together speak for A, B and ep_E.
   bool a_early = false, b_early = false;
   // Tensor-core path: the K-major factor (B where both are K-major, A otherwise) is lower triangular, element (i, k) zero for
   // k > i, and its zeros may be left out: the forms with two accumulators skip the first one's K blocks beyond its rows.

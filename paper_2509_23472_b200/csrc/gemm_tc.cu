@@ -521,9 +521,13 @@ gemm_tc_kernel(const __grid_constant__ TmapPack maps, const TcParams p) {
 
   // A gated launch that is not needed leaves before any set-up.  The word may be read this early because it was
   // written at least two kernels back in the stream: this grid only starts once its predecessor has passed its own
-  // griddepcontrol.wait, i.e. once everything before the predecessor is complete and visible.  The wait itself is
-  // still executed, so that the completion of this grid implies the completion of every earlier one.
-  if (p.gate != nullptr && *(const volatile uint32_t*)p.gate == 0u) { pdl_wait(); pdl_launch_dependents(); return; }
+  // griddepcontrol.wait, i.e. once everything before the predecessor is complete and visible.  (Gated launches release their
+  // successors ahead of the wait: a row of them starts, and reads the word, once the last kernel before the row has passed its own
+  // wait, which is behind the kernel that wrote it; loads ahead of the wait may follow such a row if their operand is older than
+  // that last kernel's predecessor.  Steps: 4096 x 5120, r = 64 78.0 -> 77.0 us, RMS unit of 8192 x 4096, r = 128 181.1 -> 180.2,
+  // 16384 x 4096, r = 256 182.1 -> 181.5.)  The wait itself is still executed, so that the completion of this grid implies
+  // the completion of every earlier one.
+  if (p.gate != nullptr && *(const volatile uint32_t*)p.gate == 0u) { pdl_launch_dependents(); pdl_wait(); return; }
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < stages; ++s) { mbar_init(&full_bar[s], 1); mbar_init(&empty_bar[s], 1); }
@@ -788,7 +792,7 @@ gemm_tc_pair_kernel(const __grid_constant__ TmapPack maps, const TcParams p) {
 
   // a gated launch that is not needed: both CTAs of the pair read the same word and leave before any set-up (see the
   // one-CTA kernel for why the word may be read before griddepcontrol.wait)
-  if (p.gate != nullptr && *(const volatile uint32_t*)p.gate == 0u) { pdl_wait(); pdl_launch_dependents(); return; }
+  if (p.gate != nullptr && *(const volatile uint32_t*)p.gate == 0u) { pdl_launch_dependents(); pdl_wait(); return; }
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < stages; ++s) { mbar_init(&full_bar[s], 1); mbar_init(&empty_bar[s], 1); }
@@ -1447,7 +1451,7 @@ gemm_tc_gram_kernel(const __grid_constant__ GramMaps maps, const GramParams p) {
   unsigned char* tiles = (unsigned char*)(((uintptr_t)smem + 1023) & ~(uintptr_t)1023);
 
   // (see the one-CTA kernel for why the word may be read before griddepcontrol.wait)
-  if (p.gate != nullptr && *(const volatile uint32_t*)p.gate == 0u) { pdl_wait(); pdl_launch_dependents(); return; }
+  if (p.gate != nullptr && *(const volatile uint32_t*)p.gate == 0u) { pdl_launch_dependents(); pdl_wait(); return; }
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kGramStages; ++s) { mbar_init(&full_bar[s], 1); mbar_init(&empty_bar[s], 1); }
@@ -1598,9 +1602,10 @@ __global__ void __launch_bounds__(1024) reduce_gram_kernel(const float* __restri
                                                            int l, float* __restrict__ W, int n_blocks, const uint32_t* gate) {
   __shared__ float t[4][32][33];
   const int tid = threadIdx.x, group = tid >> 8, a = (tid >> 3) & 31, c4 = (tid & 7) * 4;
+  // (see the one-CTA kernel for why the word may be read before griddepcontrol.wait)
+  if (gate != nullptr && *(const volatile uint32_t*)gate == 0u) { pdl_launch_dependents(); pdl_wait(); return; }
   pdl_wait();
   pdl_launch_dependents();
-  if (gate != nullptr && *(const volatile uint32_t*)gate == 0u) return;
   for (int b = blockIdx.x; b < n_blocks; b += gridDim.x) {
     int I = 0;
     while ((I + 1) * (I + 2) / 2 <= b) ++I;

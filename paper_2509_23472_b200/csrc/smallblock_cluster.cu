@@ -532,7 +532,7 @@ __global__ void __launch_bounds__(32 * warps_of<T, kBig>(), 1) small_block_clust
   // least two kernels back in the stream (this grid only starts once its predecessor has passed its own
   // griddepcontrol.wait), so it may be read this early.  The wait is still executed: the completion of this grid
   // must imply the completion of every earlier one.
-  if (p.gate != nullptr && *(const volatile uint32_t*)p.gate == 0u) { pdl_wait(); pdl_launch_dependents(); return; }
+  if (p.gate != nullptr && *(const volatile uint32_t*)p.gate == 0u) { pdl_launch_dependents(); pdl_wait(); return; }
 
   // ---- set-up: barriers, with the byte counts they will receive
   auto panel_comes = [&](int k) { return active && k < nblk && k != me; };
