@@ -1898,8 +1898,21 @@ static int k_blocks_per_split(const GemmDesc& g) {
   return (kb + splits - 1) / splits;
 }
 static TileShape launch_shape(const GemmDesc& g) {
-  return pick_shape(g.M, g.N, g.a_mn, g.b_mn, (long long)k_blocks_per_split(g) * g.n_terms, g.splits < 1 ? 1 : g.splits,
-                    g_pair_mode == 1, g.whole_rows);
+  TileShape s = pick_shape(g.M, g.N, g.a_mn, g.b_mn, (long long)k_blocks_per_split(g) * g.n_terms, g.splits < 1 ? 1 : g.splits,
+                           g_pair_mode == 1, g.whole_rows);
+  // Few rows and many columns, not split (the test matrix L^-1 T, r x d): with tiles of 256 columns most SMs are idle, and what the
+  // others load per K block and store at the end is the product's time.  The narrowest of 64 (one CTA a tile) and 128 columns whose
+  // tiles still run in one round.  Steps, 256 columns /
+  // this: 8192 x 5120, r = 128 with a power iteration 202.8 / 198.9 us, RMS unit of 8192 x 4096, r = 128 180.3 / 178.0, 12608 x 768,
+  // r = 96 92.4 / 90.9, 16384 x 4096, r = 256 181.4 / 180.3, 5003 x 1000, r = 336 171.5 / 170.4, 4096 x 5120, r = 64 75.4 / 74.4 (128 columns
+  // at least: 200.8, 179.0, 91.3, 180.4, 170.3, 74.6).
+  if (s.wide == WIDE_NONE && g.b_mn && g.N > 256 && g.splits <= 1) {
+    const bool pair = g_pair_mode != 0 && g.M >= 2 * kBM;
+    const long long m_tiles = (g.M + (pair ? 2 * kBM : kBM) - 1) / (pair ? 2 * kBM : kBM);
+    for (int bn = pair ? 128 : 64; bn <= 128 && bn < s.bn; bn *= 2)
+      if (m_tiles * ((g.N + bn - 1) / bn) <= (pair ? 74 : 148)) { s.bn = bn; break; }
+  }
+  return s;
 }
 int gemm_tc_wide_form(const GemmDesc& g) { return launch_shape(g).wide; }
 

@@ -1,0 +1,35 @@
+"""GPU test of products with few rows and many columns (the test matrix L^-1 T), whose tiles are as narrow as one round of the
+SMs allows: row counts on either side of the one-CTA and two-CTA kernels, column counts on either side of where 64, 128 and
+256 columns take over, ragged ends.  Reference: the product in float64."""
+import pytest
+import torch
+
+import __graft_entry__ as entry
+from paper_2509_23472_b200 import binding as B
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def dev():
+    entry.build()
+    B.lib()
+    return torch.device("cuda:0")
+
+
+@pytest.mark.parametrize("m,n", [(16, 264), (64, 1000), (64, 9472), (64, 9480), (96, 776), (128, 11008), (136, 4736), (136, 4744),
+                                 (248, 5120), (256, 264), (256, 9472), (256, 9480), (336, 1000), (336, 4744), (512, 11008)])
+def test_tiles_of_few_rows(dev, m, n):
+    g = torch.Generator(device=dev)
+    g.manual_seed(m + n)
+    L = torch.randn(m, m, generator=g, device=dev).tril()
+    hi = L.bfloat16()
+    lo = (L - hi.float()).bfloat16()
+    T = torch.randn(m, n, generator=g, device=dev).bfloat16()
+    status = torch.zeros(1, dtype=torch.int32, device=dev)
+    want = (hi.double() + lo.double()) @ T.double()
+    got = B.debug_gemm([hi, lo], [T, T], m, n, m, False, True, out_mode=B.OUT_BF16, engine=1, status=status).double()
+    assert int(status.item()) == 0
+    # one rounding to bf16 (2^-9 of the value); the sum over m products in fp32 is far below 1e-3 of the row's size
+    assert float(((got - want).abs() - 2.0 ** -8 * want.abs()).max()) <= 1e-3 * m ** 0.5
+    assert float((got - want).norm() / want.norm()) <= 2.5e-3
