@@ -26,13 +26,13 @@
 // load takes two cycles when each quarter of the warp reads one address, four otherwise; a store and a load of it behind
 // a warp barrier take 30 cycles, a bulk copy to another CTA 280 (512 bytes) to 480 (4.6 KB) or 730 with seven receivers.
 //
-// Measured (one Gram matrix, back to back, against a form with one chain CTA, workers that sent blocks back to it and an
-// inverse of every diagonal block): fp32 r = 32 / 64 / 128 / 256: 6.9 / 9.0 / 14.1 / 26.9 us (7.4 / 11.8 / 20.0 / 40.4).
-// r = 336 / 512, against two factorisations of up to 256 columns joined by fp32 products: 41 / 69 us (86 / 116 with its
-// six helper launches).  Above eight blocks the early steps are bound by the bulk updates and by what an SM can send.
-// fp64, against a kernel that kept the matrix in global memory: r = 64 / 96 / 192: 12.9 / 17.2 / 30.4 us (75.8 / 120.9 /
-// 282).  Cycles per group of four columns: 398 in the pivot warp alone, about 475 with its companions at work; the step
-// from one diagonal block to the next adds about 1000.
+// Measured (one Gram matrix, back to back): fp32 r = 32 / 64 / 128 / 256: 4.4 / 7.0 / 11.6 / 24.3 us, r = 336 / 512 40.1 / 67.9,
+// fp64 r = 64 / 128 / 192 10.2 / 18.1 / 27.2.  Before the load by cp.async, the predicated stores and arrivals and the shorter tail:
+// 6.5 / 8.8 / 13.6 / 25.6, 41.0 / 68.3 and 12.3 / 20.9 / 29.9; a form with one chain CTA, workers that sent blocks back to it and
+// an inverse of every diagonal block: 7.4 / 11.8 / 20.0 / 40.4 and, two of them joined by fp32 products, 86 / 116.
+// Cycles per group of four columns: about 400 (pivots 120 of them); the step from one diagonal block to the next adds about 460.
+// From the sixth block on the rows behind the chain lag and a block takes 6000 cycles instead of 3700; above eight blocks the early
+// steps are bound by the bulk updates and by what an SM can send (up to 16000 cycles a block).
 //
 // Every wait on another CTA is bounded by a wall-clock limit; on expiry the CTA records LORACT_DEV_WAIT_EXPIRED, stops
 // waiting and runs to its end (results are then invalid but every access stays in bounds), where it waits once more, with
