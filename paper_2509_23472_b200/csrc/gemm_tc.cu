@@ -1912,15 +1912,18 @@ static TileShape launch_shape(const GemmDesc& g) {
     for (int bn = pair ? 128 : 64; bn <= 128 && bn < s.bn; bn *= 2)
       if (m_tiles * ((g.N + bn - 1) / bn) <= (pair ? 74 : 148)) { s.bn = bn; break; }
   }
-  // Small results in partial sums (Gram matrices up to 256 columns, T = U^T G): the same with the widths that divide the columns, from
+  // Small results in partial sums (Gram matrices, T = U^T G): the same with the widths that divide the columns, from
   // 32 (a staged box of fp32; 64 where B is MN-major, 128 where a pair shares it).  Steps, one tile / this: 8192 x 5120, r = 128
   // with a power iteration 198.6 / 195.9 us, 16384 x 4096, r = 256 179.7 / 177.7, RMS unit of 8192 x 4096, r = 128 177.5 / 176.3,
-  // 12608 x 768, r = 96 91.4 / 90.5, 4096 x 5120, r = 64 73.6 / 73.3.
-  if (s.wide == WIDE_NONE && g.N <= 256 && g.M <= 256 && g.out == OUT_F32 && !g.whole_rows && g.splits > 1) {
+  // 12608 x 768, r = 96 91.4 / 90.5, 4096 x 5120, r = 64 73.6 / 73.3.  Above 256 columns (the sampled rows', K-major: there the widths
+  // that pad no more than the tile they replace) 5003 x 1000, r = 336 165.9 / 164.9, 2048 x 1024, r = 288 133.4 / 132.0, r = 512 the same.
+  const int largest = g.a_mn || g.b_mn ? 256 : 512;
+  if (s.wide == WIDE_NONE && g.N <= largest && g.M <= largest && g.out == OUT_F32 && !g.whole_rows && g.splits > 1) {
     const bool pair = g_pair_mode != 0 && g.M >= 2 * kBM && (g.b_mn ? s.bn % 128 == 0 : s.bn % 32 == 0);
     const long long units = (long long)((g.M + (pair ? 2 * kBM : kBM) - 1) / (pair ? 2 * kBM : kBM)) * g.splits;
     for (int bn = g.b_mn ? (pair ? 128 : 64) : 32; bn < s.bn; bn *= 2)
-      if (g.N % bn == 0 && units * (g.N / bn) <= (pair ? 74 : 148)) { s.bn = bn; break; }
+      if ((g.N + bn - 1) / bn * bn <= (g.N > 256 ? (g.N + s.bn - 1) / s.bn * s.bn : g.N) &&
+          units * ((g.N + bn - 1) / bn) <= (pair ? 74 : 148)) { s.bn = bn; break; }
   }
   return s;
 }

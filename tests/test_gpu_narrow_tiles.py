@@ -38,7 +38,8 @@ def test_tiles_of_few_rows(dev, m, n):
 
 @pytest.mark.parametrize("mn_major", [False, True])
 @pytest.mark.parametrize("l,splits", [(16, 3), (48, 2), (64, 148), (64, 74), (96, 40), (128, 37), (128, 38), (128, 75), (160, 20),
-                                      (192, 12), (256, 9), (256, 18), (256, 37), (256, 38)])
+                                      (192, 12), (256, 9), (256, 18), (256, 37), (256, 38), (272, 4), (336, 4), (336, 7), (400, 6), (512, 4),
+                                      (512, 9), (512, 10)])
 def test_partial_sums_of_small_results(dev, l, splits, mn_major):
     g = torch.Generator(device=dev)
     g.manual_seed(l + splits)
