@@ -94,6 +94,13 @@ loract_status_t loract_debug_round_gate(int32_t r, const float* W, float shift_d
                                         void* linv_hi, void* linv_lo, uint32_t* status_word, uint32_t* words,
                                         void* stream);
 
+/* The same decision with the last of its waits running out: the factorisation (up to 256 columns) waits for four bytes of the
+ * shares of est more than its warps send.  After the kernel's own limit (50 ms, and as long again for what may still be on
+ * its way) it ORs LORACT_DEV_WAIT_EXPIRED into *status_word (may be NULL) and asks for the second round whatever the threshold:
+ * words = { 1, NaN, 2 }.  The factor is complete and the context stays usable. */
+loract_status_t loract_debug_round_gate_expiry(int32_t r, const float* W, float threshold, void* scratch, void* linv_hi,
+                                               void* linv_lo, uint32_t* status_word, uint32_t* words, void* stream);
+
 /* Stage trace.  Between trace_begin and trace_end every kernel the library launches on `stream` is followed by
  * a CUDA event; trace_end synchronises the stream and writes, per kernel in launch order, a label (64 bytes
  * each, zero-terminated: the step of the path and the kernel's launch function) and the time from the

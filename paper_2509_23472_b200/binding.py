@@ -515,6 +515,22 @@ def debug_round_gate(W: torch.Tensor, threshold: float, status: Optional[torch.T
     return int(w[0]), float(w[1:2].view(torch.float32).item()), int(w[2])
 
 
+def debug_round_gate_expiry(W: torch.Tensor, threshold: float, status: Optional[torch.Tensor] = None):
+    """Test hook: the same decision where the wait for the shares of the estimate runs out."""
+    l = _debug_lib()
+    vp = ctypes.c_void_p
+    l.loract_debug_round_gate_expiry.restype = ctypes.c_int
+    l.loract_debug_round_gate_expiry.argtypes = [ctypes.c_int32, vp, ctypes.c_float, vp, vp, vp, vp, vp, vp]
+    r, dev = W.shape[0], W.device
+    scratch = torch.empty(r * r + 1024 * ((r + 31) // 32), dtype=torch.float64, device=dev)
+    Lh, Ll = (torch.empty(r, r, dtype=torch.bfloat16, device=dev) for _ in range(2))
+    words = torch.zeros(3, dtype=torch.int32, device=dev)
+    _check(l.loract_debug_round_gate_expiry(r, _ptr(W), threshold, _ptr(scratch), _ptr(Lh), _ptr(Ll), _ptr(status),
+                                            _ptr(words), _stream(dev)), "loract_debug_round_gate_expiry")
+    w = words.cpu()
+    return int(w[0]), float(w[1:2].view(torch.float32).item()), int(w[2])
+
+
 def round_gate_words(ws: torch.Tensor):
     """(second round ran, estimate trace((D W D)^-1), rounds) of the last orthonormalisation run on workspace `ws`."""
     w = ws[16:28].cpu()

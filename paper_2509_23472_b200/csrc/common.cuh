@@ -210,6 +210,8 @@ struct SmallBlockArgs {
   // bits); gate_out[2] = rounds that will run (1 or 2).  Fixed summation order.
   uint32_t* gate_out = nullptr;
   float gate_threshold = 0.f;
+  // test hook, up to 256 columns: so many bytes of the shares of the estimate are waited for and never sent
+  uint32_t absent_share_bytes = 0;
   void* linv_full = nullptr;  // fp64, r x r
   float* linv_f32 = nullptr;  // fp32 copy, r x r
   __nv_bfloat16* linv_hi = nullptr;

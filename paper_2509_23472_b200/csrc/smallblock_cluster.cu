@@ -88,6 +88,7 @@ struct SCParams {
   // est = sum_ij Linv_ij^2 W_jj (W_jj the diagonal as factored): trace of the inverse of the diagonally scaled matrix
   uint32_t* gate_out;
   float gate_threshold;
+  uint32_t absent_share_bytes;   // test hook: bytes of the shares that CTA 0 waits for and nobody sends
   float* linv_f32;
   __nv_bfloat16* linv_hi;
   __nv_bfloat16* linv_lo;
@@ -558,7 +559,7 @@ __global__ void __launch_bounds__(32 * warps_of<T, kBig>(), 1) small_block_clust
     s_gave_up = 0;
     bar_init(&est_bar, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    if (!kBig && p.gate_out && me == 0) bar_expect(&est_bar, (uint32_t)(kBulkWarps * nblk * sizeof(float)));
+    if (!kBig && p.gate_out && me == 0) bar_expect(&est_bar, (uint32_t)(kBulkWarps * nblk * sizeof(float)) + p.absent_share_bytes);
   }
   __syncthreads();
   cluster_arrive();                       // waited for under the load: nobody sends before every CTA's barriers exist
@@ -885,14 +886,20 @@ __global__ void __launch_bounds__(32 * warps_of<T, kBig>(), 1) small_block_clust
   cluster_wait();
   if (p.gate_out && me == 0 && warp == 0) {
     // after the cluster barrier every status bit of this call is set (who sets one fences); the shares of the estimate are here (kBig)
-    // or counted
-    if (!kBig && !bar_wait<true>(&est_bar, gave_up)) bar_drain(&est_bar);
+    // or counted.  Where that count does not complete, the wait is reported here (the block above is past) and the second round runs.
+    const bool here = kBig || __all_sync(0xffffffffu, bar_wait<true>(&est_bar, gave_up));
+    if (!here) {
+      bar_drain(&est_bar);
+      __syncwarp();
+      if (lane == 0 && p.dev_status) atomicOr(p.dev_status, LORACT_DEV_WAIT_EXPIRED);
+    }
     const uint32_t st = p.dev_status ? *(const volatile uint32_t*)p.dev_status : 0u;
     float est = 0.f;
 #pragma unroll 1
     for (int c = lane; c < kBulkWarps * nblk; c += 32) est += s_est[c];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) est += __shfl_xor_sync(0xffffffffu, est, o);
+    if (!here) est = __uint_as_float(0x7fc00000u);          // (not a number: what is in s_est is not the sum)
     const bool again = !(est <= p.gate_threshold) || st != 0u;
     if (lane == 0) {
       p.gate_out[0] = again ? 1u : 0u;
@@ -1030,6 +1037,7 @@ cudaError_t small_block_cluster_launch(const SmallBlockArgs& a, cudaStream_t str
   p.gate = a.gate;
   p.gate_out = a.gate_out;
   p.gate_threshold = a.gate_threshold;
+  p.absent_share_bytes = a.absent_share_bytes;
   p.linv_f32 = a.linv_f32;
   p.linv_hi = a.linv_hi;
   p.linv_lo = a.linv_lo;

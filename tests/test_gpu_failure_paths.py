@@ -2,6 +2,8 @@
 
 (a) A bounded device-side wait that runs out: a tiny kernel waits, with the library's own wait helpers, on a
     barrier that nothing completes; after a millisecond it gives up, records LORACT_DEV_WAIT_EXPIRED and returns.
+    The factorisation's wait for the shares of its estimate runs out likewise (it waits for bytes that are never sent): it
+    records the same bit and asks for the second orthonormalisation round.
 (b) A non-finite input: the factorisation notices it (the trace of a Gram matrix is not finite), records
     LORACT_DEV_NONFINITE and runs to its end; the next call on clean data is clean.
 """
@@ -43,6 +45,24 @@ def test_a_bounded_wait_runs_out_and_reports_it(dev, which):
     U, V, _ = B.compress(X, 64, seed=w.seed, ws=ws)
     assert B.read_device_status(ws) == 0
     assert bool(torch.isfinite(U.float()).all())
+
+
+@pytest.mark.parametrize("r", [16, 40, 64, 256])            # one, two and eight CTAs
+def test_an_estimate_that_does_not_arrive_asks_for_the_second_round(dev, r):
+    g = torch.Generator().manual_seed(r)
+    Y = torch.randn(4 * r, r, generator=g)
+    W = (Y.t() @ Y).to(dev)
+    status = torch.zeros(1, dtype=torch.int32, device=dev)
+    assert B.debug_round_gate(W, float("inf"), status)[::2] == (0, 1)
+    t0 = time.perf_counter()
+    again, est, rounds = B.debug_round_gate_expiry(W, float("inf"), status)
+    assert time.perf_counter() - t0 < 1.0                    # two limits of 50 ms
+    assert int(status.item()) & 0xFFFFFFFF == B.DEV_WAIT_EXPIRED
+    assert (again, rounds) == (1, 2) and est != est
+    assert B.debug_round_gate_expiry(W, float("inf"), None)[0] == 1    # without a word to report it in, too
+    status.zero_()
+    assert B.debug_round_gate(W, float("inf"), status)[::2] == (0, 1)
+    assert int(status.item()) == 0
 
 
 def test_status_word_mapping_is_a_pure_host_function(dev):
