@@ -362,7 +362,7 @@ DEBUG_EXPORTS = ("loract_debug_gemm", "loract_debug_small_block", "loract_debug_
                  "loract_debug_wait_expiry", "loract_debug_project", "loract_debug_gemm_halved",
                  "loract_debug_reduce_sym", "loract_debug_set_round_gate", "loract_debug_round_gate",
                  "loract_debug_set_big_clusters", "loract_debug_wide_form", "loract_debug_gram_bytes", "loract_debug_gram",
-                 "loract_debug_planned_splits")
+                 "loract_debug_planned_splits", "loract_debug_round_gate_expiry")
 
 
 def _debug_lib():
