@@ -59,6 +59,10 @@ void loract_debug_set_pair_mode(int32_t on);
 int32_t loract_debug_wide_form(int32_t M, int32_t N, int32_t K, int32_t a_mn, int32_t b_mn, int32_t n_terms,
                                int32_t splits);
 
+/* The columns of a tile that loract_debug_gemm takes for a product (not of the persistent kernel's tiles).  Host only. */
+int32_t loract_debug_tile_width(int32_t M, int32_t N, int32_t K, int32_t a_mn, int32_t b_mn, int32_t n_terms, int32_t out_mode,
+                                int32_t splits);
+
 /* The number of ranges into which the contraction of a product is split (host only): at most `max_splits`, and as many as fill
  * the chip up to `free_sums`, the number of partial sums that cost nothing to add up.  A range is ceil(K blocks of 64 / ranges)
  * blocks long, and none is empty. */

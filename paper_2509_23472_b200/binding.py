@@ -362,7 +362,7 @@ DEBUG_EXPORTS = ("loract_debug_gemm", "loract_debug_small_block", "loract_debug_
                  "loract_debug_wait_expiry", "loract_debug_project", "loract_debug_gemm_halved",
                  "loract_debug_reduce_sym", "loract_debug_set_round_gate", "loract_debug_round_gate",
                  "loract_debug_set_big_clusters", "loract_debug_wide_form", "loract_debug_gram_bytes", "loract_debug_gram",
-                 "loract_debug_planned_splits", "loract_debug_round_gate_expiry")
+                 "loract_debug_planned_splits", "loract_debug_round_gate_expiry", "loract_debug_tile_width")
 
 
 def _debug_lib():
@@ -459,6 +459,15 @@ def debug_wide_form(M: int, N: int, K: int, a_mn: bool, b_mn: bool, terms: int =
     l.loract_debug_wide_form.restype = ctypes.c_int32
     l.loract_debug_wide_form.argtypes = [ctypes.c_int32] * 7
     return int(l.loract_debug_wide_form(M, N, K, int(a_mn), int(b_mn), terms, splits))
+
+
+def debug_tile_width(M: int, N: int, K: int, a_mn: bool, b_mn: bool, terms: int = 1, out_mode: int = OUT_F32,
+                     splits: int = 1) -> int:
+    """Test hook: the columns of a tile that a product takes (not of the persistent kernel's).  Host only."""
+    l = _debug_lib()
+    l.loract_debug_tile_width.restype = ctypes.c_int32
+    l.loract_debug_tile_width.argtypes = [ctypes.c_int32] * 8
+    return int(l.loract_debug_tile_width(M, N, K, int(a_mn), int(b_mn), terms, out_mode, splits))
 
 
 def debug_planned_splits(M: int, N: int, K: int, a_mn: bool, b_mn: bool, max_splits: int = 32, free_sums: int = 1) -> int:

@@ -149,6 +149,7 @@ int gemm_tc_wide_form(const GemmDesc& g);
 // Whether a launch with whole_rows set can give one CTA (pair) whole rows of an M x N product.
 bool gemm_tc_can_own_rows(int M, int N);
 void gemm_tc_set_pair_mode(int on);   // test hook: 0 keeps every contraction on the one-CTA kernel
+int gemm_tc_tile_width(const GemmDesc& g);      // test hook: columns of a tile (not of the persistent kernel's)
 // Test hooks for the give-up path of the bounded waits: a kernel that waits (with the engine's / the cluster
 // kernel's own wait) on a barrier nothing completes, for at most limit_ns, then sets LORACT_DEV_WAIT_EXPIRED.
 cudaError_t gemm_tc_wait_probe_launch(uint32_t* dev_status, uint64_t limit_ns, cudaStream_t stream);

@@ -1931,6 +1931,7 @@ int gemm_tc_wide_form(const GemmDesc& g) { return launch_shape(g).wide; }
 
 bool gemm_tc_can_own_rows(int M, int N) { return N <= 256 || (N <= 512 && M >= 2 * kBM && g_pair_mode == 1); }
 
+int gemm_tc_tile_width(const GemmDesc& g) { return launch_shape(g).bn; }
 int gemm_tc_pick_splits(int M, int N, int K, bool a_mn, bool b_mn, int max_splits, int free_sums) {
   const int bn = pick_bn(N);
   const int n_tiles = (N + bn - 1) / bn;
