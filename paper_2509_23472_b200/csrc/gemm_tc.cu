@@ -1900,17 +1900,24 @@ static int k_blocks_per_split(const GemmDesc& g) {
 static TileShape launch_shape(const GemmDesc& g) {
   TileShape s = pick_shape(g.M, g.N, g.a_mn, g.b_mn, (long long)k_blocks_per_split(g) * g.n_terms, g.splits < 1 ? 1 : g.splits,
                            g_pair_mode == 1, g.whole_rows);
-  // Few rows and many columns, not split (the test matrix L^-1 T, r x d): with tiles of 256 columns most SMs are idle, and what the
-  // others load per K block and store at the end is the product's time.  The narrowest of 64 (one CTA a tile) and 128 columns whose
-  // tiles still run in one round.  Steps, 256 columns /
-  // this: 8192 x 5120, r = 128 with a power iteration 202.8 / 198.9 us, RMS unit of 8192 x 4096, r = 128 180.3 / 178.0, 12608 x 768,
-  // r = 96 92.4 / 90.9, 16384 x 4096, r = 256 181.4 / 180.3, 5003 x 1000, r = 336 171.5 / 170.4, 4096 x 5120, r = 64 75.4 / 74.4 (128 columns
-  // at least: 200.8, 179.0, 91.3, 180.4, 170.3, 74.6).
+  // Few rows and many columns, not split (the test matrix L^-1 T, an unsplit U^T X, Reconstruct of few tiles): with tiles of 256 columns
+  // most SMs are idle, and what the others load per K block and store at the end is the product's time.  The narrowest of 64 (one CTA a
+  // tile) and 128 columns whose tiles still run in one round.  Steps (256 columns / this): 4096 x 5120, r = 64 70.9 / 70.7 us, 12608 x
+  // 768, r = 96 88.7 / 87.2, 999 x 4096, r = 256 118.2 / 114.0, 8192 x 5120, r = 128 with a power iteration 196.1 / 194.1,
+  // 5003 x 1000, r = 336 169.2 / 167.3.  Reconstruct of 64 to 4096 rows, r = 64 to 512, 146 sizes: 0.84 of the time in the geometric
+  // mean, 1.03 at worst (256 x 9472, r = 64); U^T X of 64 to 2048 rows, 149 sizes: 0.72 and 0.91.
+  // Rows of A of less than 128 bytes (rank 16 to 48): every tile reads the same short rows, and from 64 tiles of 64 columns side by side
+  // on 128 are better, from 80 of those on 256.  U^T X of 512 rows, r = 16, 64 / 128 / 256 columns: d = 4096 5.0 / - / 6.0 us, d = 5120
+  // 6.4 / 4.6 / 6.0, d = 9472 7.3 / 5.9 / 6.1; L^-1 T, r = 16: d = 5120 4.0 / 3.2 / 3.7, d = 11008 - / 4.2 / 3.9.
+  // The split counts are picked for the tiles of pick_bn all the same: the K ranges, and with them the bits of a result, stay put.
   if (s.wide == WIDE_NONE && g.b_mn && g.N > 256 && g.splits <= 1) {
     const bool pair = g_pair_mode != 0 && g.M >= 2 * kBM;
+    const bool short_rows = !pair && (g.a_mn ? g.M : g.K) < 64;
     const long long m_tiles = (g.M + (pair ? 2 * kBM : kBM) - 1) / (pair ? 2 * kBM : kBM);
-    for (int bn = pair ? 128 : 64; bn <= 128 && bn < s.bn; bn *= 2)
-      if (m_tiles * ((g.N + bn - 1) / bn) <= (pair ? 74 : 148)) { s.bn = bn; break; }
+    for (int bn = pair ? 128 : 64; bn <= 128 && bn < s.bn; bn *= 2) {
+      const int n_tiles = (g.N + bn - 1) / bn;
+      if (m_tiles * n_tiles <= (pair ? 74 : 148) && (!short_rows || n_tiles <= (bn == 64 ? 64 : 80))) { s.bn = bn; break; }
+    }
   }
   // Small results in partial sums (Gram matrices, T = U^T G): the same with the widths that divide the columns, from
   // 32 (a staged box of fp32; 64 where B is MN-major, 128 where a pair shares it).  Steps, one tile / this: 8192 x 5120, r = 128

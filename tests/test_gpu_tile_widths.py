@@ -27,6 +27,18 @@ def test_width_of_few_rows(built, m, n, width):
     assert B.debug_tile_width(m, n, m, False, True, 2, B.OUT_BF16) == width
 
 
+# Rows of A of less than 128 bytes (rank 16, 32 or 48: A = U or L^-1), one CTA a tile: up to 64 tiles of 64 columns side by
+# side, up to 80 of 128.
+@pytest.mark.parametrize("m,n,k,mn_major,terms,width", [
+    (16, 4096, 512, True, 1, 64), (16, 4104, 512, True, 1, 128), (48, 5120, 192, True, 1, 128), (16, 10240, 448, True, 1, 128),
+    (16, 10248, 448, True, 1, 192), (32, 11008, 64, True, 1, 256), (64, 9472, 448, True, 1, 64),
+    (96, 4096, 16, False, 1, 64), (96, 5120, 16, False, 1, 128), (200, 4096, 32, False, 1, 64), (200, 4104, 32, False, 1, 128),
+    (200, 9472, 48, False, 1, 128), (128, 11008, 48, False, 1, 256), (128, 9472, 64, False, 1, 64), (255, 5120, 16, False, 1, 128),
+    (256, 9472, 16, False, 1, 128), (16, 4096, 16, False, 2, 64), (16, 9472, 16, False, 2, 128), (32, 11008, 32, False, 2, 256)])
+def test_width_where_rows_of_a_are_short(built, m, n, k, mn_major, terms, width):
+    assert B.debug_tile_width(m, n, k, mn_major, True, terms, B.OUT_BF16) == width
+
+
 # One term and the other operand orders and results that reach the same rule: Reconstruct (A K-major) and U^T X (both MN-major, bf16 or
 # fp32); a pair of bf16 results.  (No product that the rule reaches adds to what is there.)
 @pytest.mark.gpu
@@ -37,7 +49,8 @@ def test_width_of_few_rows(built, m, n, width):
     (100, 1000, 72, False, B.OUT_SPLIT, 64), (100, 1000, 72, False, B.OUT_F32, 64),
     (64, 4096, 200, True, B.OUT_BF16, 64), (96, 9472, 448, True, B.OUT_F32, 64), (96, 9480, 448, True, B.OUT_F32, 128),
     (240, 1000, 500, True, B.OUT_F32, 64), (256, 768, 511, True, B.OUT_BF16, 128), (496, 3000, 510, True, B.OUT_F32, 128),
-    (16, 1360, 500, True, B.OUT_BF16, 64)])
+    (16, 1360, 500, True, B.OUT_BF16, 64), (16, 5120, 500, True, B.OUT_BF16, 128), (48, 9472, 192, True, B.OUT_F32, 128),
+    (96, 5120, 16, False, B.OUT_BF16, 128)])
 def test_other_products_of_few_tiles(dev, m, n, k, mn_major, out, width):
     assert B.debug_tile_width(m, n, k, mn_major, True, 1, out) == width
     g = torch.Generator(device=dev)
