@@ -109,19 +109,24 @@ struct GemmDesc {
   // (result = (t_0 + ... + t_{h-1}) / 2 + t_h + ...); 0 or negative: plain sum.  With the pair {A^T A, A^T B} and
   // h = 1 the result D gives D + D^T = A^T A + A^T B + B^T A: a symmetric three-term sum for two terms' work.
   int halve_at_term = 0;
-  // Tensor-core path: a device word written by a kernel at least TWO launches earlier in the same stream (the gated
-  // kernel reads it before its griddepcontrol.wait); when it is zero the launch does nothing (no loads, no products,
-  // C untouched).  nullptr: unconditional.
+  // What a kernel may read ahead of its own griddepcontrol.wait (here: the gate word and early operands).  A launch without a gate, or
+  // with one that is not zero, releases its dependents behind its wait; a gated launch that leaves releases them first and waits
+  // then.  So a grid starts once the last kernel of the stream that was not such a launch, K, has passed its wait, and that is once
+  // everything ahead of K is complete and visible.  Whatever was written AHEAD OF K may be read early; what K itself wrote may not, even
+  // where gated launches stand between K and the reader.  Two launches back is enough only if the launch in between has no gate.
+  // (sample_indices_kernel releases first, too; a call whose products load early has a kernel of its own in between.)  Every kernel
+  // waits before it ends, so the completion of one implies that of all earlier ones.
+  //
+  // Tensor-core path: a device word, written ahead of the last kernel without a gate in front of the row of gated launches that read
+  // it; when it is zero the launch does nothing (no loads, no products, C untouched).  nullptr: unconditional.
   const uint32_t* gate = nullptr;
   // Tensor-core path: the launch stores zero into the status word before any of its waits can set a bit in it (the
   // first kernel of a call clears the word itself instead of a memset in front of it).
   bool clear_status = false;
   uint32_t* clear_word = nullptr;   // SIMT path: the same, the word to clear
-  // Tensor-core path: every A (every B) of the terms was written ahead of the previous kernel of the stream, i.e. at least two
-  // launches back.  A grid only starts once its predecessor has passed its own griddepcontrol.wait, which is once everything
-  // ahead of the predecessor is complete and visible; so such an operand may be loaded before this grid's own wait, under
-  // the predecessor's work.  (Behind a row of gated launches: written ahead of the kernel before the last one that is not gated.)
-  // OUT_RMS_BWD: both flags together speak for A, B and ep_E.
+  // Tensor-core path: every A (every B) of the terms was written ahead of the previous kernel of the stream (behind a row of gated
+  // launches: ahead of the last kernel in front of the row), so it may be loaded before this grid's own wait, under the
+  // predecessor's work (see the rule at `gate`).  Not for a launch with a gate.  OUT_RMS_BWD: both flags together speak for A, B and ep_E.
   bool a_early = false, b_early = false;
   // Tensor-core path: the K-major factor (B where both are K-major, A otherwise) is lower triangular, element (i, k) zero for
   // k > i, and its zeros may be left out: the forms with two accumulators skip the first one's K blocks beyond its rows.
@@ -200,7 +205,7 @@ struct SmallBlockArgs {
   // each diagonal entry is also multiplied by (1 + shift_diag_rel), a shift relative to the entry itself (the scale-invariant form, which leaves a
   // matrix whose diagonal spans several orders of magnitude as well conditioned as its scaled form)
   float shift_diag_rel = 0.f;
-  // device word written by an earlier kernel of the stream; zero: the launch does nothing.  nullptr: unconditional.
+  // device word (written as GemmDesc::gate says); zero: the launch does nothing.  nullptr: unconditional.
   const uint32_t* gate = nullptr;
   // optional, three words: the decision after the first orthonormalisation round whether a second one is needed, W being the
   // Gram matrix that is factored.  With D = diag(W)^(-1/2) the kernel forms

@@ -1,9 +1,9 @@
 // Tensor-core engine for the dense contractions of the path (the sketch and the projection of Algorithm 1, the Gram
 // matrices of the orthonormalisation, the application of the triangular factors, Reconstruct).
 //
-// One kernel, written for sm_100a: TMA (cp.async.bulk.tensor, 128-byte swizzle, no multicast) fills a
-// 4-stage shared-memory ring, one thread issues tcgen05.mma (kind::f16, bf16 operands, M = 128,
-// N <= 256, K = 16 per instruction) into an fp32 accumulator in tensor memory, four warps read the
+// Written for sm_100a: up to four threads fill a shared-memory ring of three to twelve stages by TMA (cp.async.bulk.tensor,
+// 128-byte swizzle, no multicast), one thread issues tcgen05.mma (kind::f16, bf16 operands, M = 128,
+// N <= 256, K = 16 per instruction) into an fp32 accumulator in tensor memory, eight warps read the
 // accumulator back with tcgen05.ld and write the result.  Operands may be K-major or MN-major, which
 // covers X Omega^T (K/K), U^T X and Y^T Y (MN/MN) and U V (K/MN) without transposing anything in memory.
 // A contraction can be the sum of up to three products over the same shapes (split-precision terms),
@@ -31,7 +31,7 @@ constexpr int kBK = 64;          // bf16 elements = one 128-byte swizzle row
 // flight.
 constexpr int kMaxStages = 12;
 constexpr uint32_t kRingBytes = 208 * 1024;
-constexpr int kThreads = 320;    // warp 0: TMA, warp 1: MMA + tensor memory, warps 2..9: epilogue
+constexpr int kThreads = 320;    // warps 0, 2, 3, 4: TMA (kProducers), warp 1: MMA + tensor memory, warps 2..9: epilogue
 constexpr int kProducers = 4;    // warps that fill the ring, at most
 constexpr int kEpiWarps = 8;     // two per quarter of the tensor-memory lanes: they take alternate column groups
 constexpr uint32_t kABytes = kBM * kBK * 2;
@@ -519,14 +519,10 @@ gemm_tc_kernel(const __grid_constant__ TmapPack maps, const TcParams p) {
   // dynamic shared memory is declared 1024-aligned; round up anyway (swizzle atoms need it)
   unsigned char* tiles = (unsigned char*)(((uintptr_t)smem + 1023) & ~(uintptr_t)1023);
 
-  // A gated launch that is not needed leaves before any set-up.  The word may be read this early because it was
-  // written at least two kernels back in the stream: this grid only starts once its predecessor has passed its own
-  // griddepcontrol.wait, i.e. once everything before the predecessor is complete and visible.  (Gated launches release their
-  // successors ahead of the wait: a row of them starts, and reads the word, once the last kernel before the row has passed its own
-  // wait, which is behind the kernel that wrote it; loads ahead of the wait may follow such a row if their operand is older than
-  // that last kernel's predecessor.  Steps: 4096 x 5120, r = 64 78.0 -> 77.0 us, RMS unit of 8192 x 4096, r = 128 181.1 -> 180.2,
-  // 16384 x 4096, r = 256 182.1 -> 181.5.)  The wait itself is still executed, so that the completion of this grid implies
-  // the completion of every earlier one.
+  // A gated launch that is not needed leaves before any set-up, and releases its successor first of all (the rule at GemmDesc::gate
+  // says why the word may be read this early and why the wait is still executed).  Steps, released behind the wait / ahead of it:
+  // 999 x 4096, r = 256 117.5 / 114.0 us, 4096 x 5120, r = 64 71.1 / 70.7, 16384 x 4096, r = 256 178.0 / 177.5, 2048 x 1024, r = 288 133.3 /
+  // 132.7; 8192 x 5120, r = 128 with a power iteration 193.9 / 194.1.
   if (p.gate != nullptr && *(const volatile uint32_t*)p.gate == 0u) { pdl_launch_dependents(); pdl_wait(); return; }
 
   if (threadIdx.x == 0) {
@@ -571,9 +567,9 @@ gemm_tc_kernel(const __grid_constant__ TmapPack maps, const TcParams p) {
     }
   };
   // K block and term of the next iteration of a producer: warps 0 and 2 to 4 (which become epilogue warps) take turns (0 and 2
-  // where the ring has three stages).  One producer alone, with up to six loads and a barrier to wait for per K block, takes 440 to 900 cycles for it.  (Four instead of
-  // two: steps of 12608 x 768, r = 96 95.6 -> 94.1 us, 8192 x 5120, r = 128 with a power
-  // iteration 207.7 -> 207.3, 4096 x 5120, r = 64 78.5 -> 78.3.)
+  // where the ring has three stages).  One producer alone, with up to six loads and a barrier to wait for per K block, takes 440 to
+  // 900 cycles for it.  Steps, two producers / four: 12608 x 768, r = 96 88.5 / 87.2 us, 8192 x 5120, r = 128 with a power iteration
+  // 194.8 / 194.1, 2048 x 1024, r = 288 133.3 / 132.7, 16384 x 4096, r = 256 178.0 / 177.5; 5003 x 1000, r = 336 166.7 / 167.3.
   auto next_block = [&](int& term, int& kb) {
     kb += producers;
     while (kb >= kb_count) { kb -= kb_count; ++term; }
@@ -790,8 +786,7 @@ gemm_tc_pair_kernel(const __grid_constant__ TmapPack maps, const TcParams p) {
   const int producer = warp == 0 ? 0 : (warp >= 2 && warp <= producers ? warp - 1 : -1);
   unsigned char* tiles = (unsigned char*)(((uintptr_t)smem + 1023) & ~(uintptr_t)1023);
 
-  // a gated launch that is not needed: both CTAs of the pair read the same word and leave before any set-up (see the
-  // one-CTA kernel for why the word may be read before griddepcontrol.wait)
+  // a gated launch that is not needed: both CTAs of the pair read the same word and leave before any set-up (see the one-CTA kernel)
   if (p.gate != nullptr && *(const volatile uint32_t*)p.gate == 0u) { pdl_launch_dependents(); pdl_wait(); return; }
 
   if (threadIdx.x == 0) {
@@ -864,8 +859,9 @@ gemm_tc_pair_kernel(const __grid_constant__ TmapPack maps, const TcParams p) {
     }
   };
   // K block and term of the next iteration of a producer.  Two producers take turns (warps 0 and 2), or four (0, 2, 3 and 4) where
-  // the tile of B is narrow and a K block short: up to 128 columns (steps of 4096 x 5120, r = 64 76.5 -> 75.7 us, 8192 x 5120, r = 128 with
-  // a power iteration 205.8 -> 204.5, 12608 x 768, r = 96 92.7 -> 92.0; above, 5003 x 1000, r = 336 171.2 -> 171.9).
+  // the tile of B is narrow and a K block short: up to 128 columns.  Steps, two / four: 4096 x 5120, r = 64 71.7 / 70.7 us, 8192 x 5120,
+  // r = 128 with a power iteration 195.5 / 194.1, 4090 x 1000, r = 128 83.0 / 81.9, 12608 x 768, r = 96 87.9 / 87.2.  (On wider tiles, too,
+  // 5003 x 1000, r = 336 took 0.7 more.)
   auto next_block = [&](int& term, int& kb) {
     kb += producers;
     while (kb >= kb_count) { kb -= kb_count; ++term; }
@@ -1450,7 +1446,7 @@ gemm_tc_gram_kernel(const __grid_constant__ GramMaps maps, const GramParams p) {
   const uint32_t stage_bytes = 4 * kABytes, tx_bytes = diag ? 2 * kABytes : 4 * kABytes;
   unsigned char* tiles = (unsigned char*)(((uintptr_t)smem + 1023) & ~(uintptr_t)1023);
 
-  // (see the one-CTA kernel for why the word may be read before griddepcontrol.wait)
+  // (see the one-CTA kernel)
   if (p.gate != nullptr && *(const volatile uint32_t*)p.gate == 0u) { pdl_launch_dependents(); pdl_wait(); return; }
 
   if (threadIdx.x == 0) {
@@ -1602,7 +1598,7 @@ __global__ void __launch_bounds__(1024) reduce_gram_kernel(const float* __restri
                                                            int l, float* __restrict__ W, int n_blocks, const uint32_t* gate) {
   __shared__ float t[4][32][33];
   const int tid = threadIdx.x, group = tid >> 8, a = (tid >> 3) & 31, c4 = (tid & 7) * 4;
-  // (see the one-CTA kernel for why the word may be read before griddepcontrol.wait)
+  // (see the one-CTA kernel)
   if (gate != nullptr && *(const volatile uint32_t*)gate == 0u) { pdl_launch_dependents(); pdl_wait(); return; }
   pdl_wait();
   pdl_launch_dependents();
@@ -1920,10 +1916,11 @@ static TileShape launch_shape(const GemmDesc& g) {
     }
   }
   // Small results in partial sums (Gram matrices, T = U^T G): the same with the widths that divide the columns, from
-  // 32 (a staged box of fp32; 64 where B is MN-major, 128 where a pair shares it).  Steps, one tile / this: 8192 x 5120, r = 128
-  // with a power iteration 198.6 / 195.9 us, 16384 x 4096, r = 256 179.7 / 177.7, RMS unit of 8192 x 4096, r = 128 177.5 / 176.3,
-  // 12608 x 768, r = 96 91.4 / 90.5, 4096 x 5120, r = 64 73.6 / 73.3.  Above 256 columns (the sampled rows', K-major: there the widths
-  // that pad no more than the tile they replace) 5003 x 1000, r = 336 165.9 / 164.9, 2048 x 1024, r = 288 133.4 / 132.0, r = 512 the same.
+  // 32 (a staged box of fp32; 64 where B is MN-major, 128 where a pair shares it).  Steps, one tile / this: 999 x 4096, r = 256 118.0 /
+  // 114.0 us, 8192 x 5120, r = 128 with a power iteration 197.3 / 194.1, 16384 x 4096, r = 256 179.5 / 177.5, RMS unit of 8192 x 4096,
+  // r = 128 178.2 / 176.2, 4090 x 1000, r = 128 83.9 / 81.9, 12608 x 768, r = 96 88.2 / 87.2, 4096 x 5120, r = 64 the same.  Above 256
+  // columns (the sampled rows', K-major: there the widths that pad no more than the tile they replace) 2048 x 1024, r = 288 133.7 / 132.7,
+  // 5003 x 1000, r = 336 168.0 / 167.3, 4096 x 2048, r = 272 144.2 / 143.7.
   const int largest = g.a_mn || g.b_mn ? 256 : 512;
   if (s.wide == WIDE_NONE && g.N <= largest && g.M <= largest && g.out == OUT_F32 && !g.whole_rows && g.splits > 1) {
     const bool pair = g_pair_mode != 0 && g.M >= 2 * kBM && (g.b_mn ? s.bn % 128 == 0 : s.bn % 32 == 0);

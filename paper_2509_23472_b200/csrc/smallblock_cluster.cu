@@ -26,10 +26,9 @@
 // load takes two cycles when each quarter of the warp reads one address, four otherwise; a store and a load of it behind
 // a warp barrier take 30 cycles, a bulk copy to another CTA 280 (512 bytes) to 480 (4.6 KB) or 730 with seven receivers.
 //
-// Measured (one Gram matrix, back to back): fp32 r = 32 / 64 / 128 / 256: 4.4 / 7.0 / 11.6 / 24.3 us, r = 336 / 512 40.1 / 67.9,
-// fp64 r = 64 / 128 / 192 10.2 / 18.1 / 27.2.  Before the load by cp.async, the predicated stores and arrivals and the shorter tail:
-// 6.5 / 8.8 / 13.6 / 25.6, 41.0 / 68.3 and 12.3 / 20.9 / 29.9; a form with one chain CTA, workers that sent blocks back to it and
-// an inverse of every diagonal block: 7.4 / 11.8 / 20.0 / 40.4 and, two of them joined by fp32 products, 86 / 116.
+// Measured (one Gram matrix, back to back from a graph): fp32 r = 32 / 64 / 128 / 256: 4.3 / 6.8 / 11.4 / 24.1 us, r = 336 / 512 39.3 /
+// 67.0, fp64 r = 64 / 128 / 192 10.2 / 18.3 / 27.2.  The figures beside the choices below were taken in turn with these; where
+// they belong to an earlier form, they say so.
 // Cycles per group of four columns: about 400 (pivots 120 of them); the step from one diagonal block to the next adds about 460.
 // From the sixth block on the rows behind the chain lag and a block takes 6000 cycles instead of 3700; above eight blocks the early
 // steps are bound by the bulk updates and by what an SM can send (up to 16000 cycles a block).
@@ -48,12 +47,13 @@ namespace {
 
 constexpr int kB = 32;                   // block edge
 // fp32: three senders.  An SM issues a copy of one group every 56 cycles, so that a sender which waits, fences and copies to
-// seven peers falls behind the groups (one sender: r = 224 / 256 25.5 / 29.8 us instead of 24.4 / 28.8).  fp64, at most
-// six blocks and a slower chain: one (three: 0.2 to 0.6 us more).
+// seven peers falls behind the groups (one sender: r = 128 / 256 / 336 / 512 11.6 / 25.9 / 48.3 / 87.3 us instead of 11.4 / 24.1 / 39.3 /
+// 67.1; 0.1 less at r = 32 and 64).  fp64, at most six blocks and a slower chain: one (three: r = 64 / 128 / 192 10.8 / 19.2 / 28.0
+// instead of 10.3 / 18.2 / 27.2).
 template <typename T> __host__ __device__ constexpr int senders_of() { return sizeof(T) == 8 ? 1 : 3; }
-// Six bulk warps; eight above eight block rows, where theirs is the work that lags (six: r = 400 / 512 54 / 74 us instead of
-// 52 / 70.6; ten or twelve get in the way of the chain, 75).  Below, the registers and the issue slots of two fewer are worth
-// more: r = 256 28.1 -> 27.7 us, fp64 r = 64 / 192 13.4 / 32 -> 12.9 / 30.4.
+// Six bulk warps; eight above eight block rows, where theirs is the work that lags (six: r = 336 / 400 / 512 39.3 / 53.7 / 75.2 us instead
+// of 39.3 / 49.6 / 67.1).  Below, the registers and the issue slots of two fewer are worth more (eight: r = 64 / 128 / 256
+// 7.2 / 12.3 / 25.6 us instead of 6.9 / 11.4 / 24.1, fp64 r = 64 / 192 11.0 / 28.1 instead of 10.3 / 27.2).
 template <bool kBig> __host__ __device__ constexpr int bulk_of() { return kBig ? 8 : 6; }
 template <typename T, bool kBig> __host__ __device__ constexpr int warps_of() { return 9 + bulk_of<kBig>() + senders_of<T>(); }
 constexpr int kPan = 8;                  // groups of four columns in a block
@@ -335,8 +335,8 @@ __device__ __forceinline__ bool factor_diagonal(const T* staged, T* panels, uint
 // follow-up and bulk warps).  Taken off one by one, every product is rounded at the size of the block, and the error of the
 // factor grows with the square root of r: relative error of L^-1 against fp64 at condition number 1e2 / 1e4, r = 256:
 // 1.2e-6 / 4.5e-5 so, 5.0e-7 / 2.5e-5 in sums (products of 32 x 32 blocks, the form before: 4.8e-7 / 2.6e-5), r = 512: 1.7e-6 /
-// 6.3e-5, 5.3e-7 / 2.6e-5 (6.1e-7 / 4.8e-5).  It costs no time (r = 256 / 512: 26.9 / 68.5 us).  fp64 results are rounded to
-// fp32 and have no need of it.
+// 6.3e-5, 5.3e-7 / 2.6e-5 (6.1e-7 / 4.8e-5).  It costs no time (one by one, r = 256 / 336 / 512: 24.1 / 40.1 / 68.0 us
+// instead of 24.1 / 39.3 / 67.1).  fp64 results are rounded to fp32 and have no need of it.
 template <typename T> constexpr bool kBlockSums = sizeof(T) == 4;
 
 // ------------------------------------------------------------------ forward substitution (four warps, eight rows each)
@@ -355,8 +355,8 @@ __device__ __forceinline__ void solve_half(const V4<T> (&was)[2], V4<T> (&acc)[2
     bar_wait(pan_bars + p, gave_up);
     const V4<T> rr = ld4(pan + kGrp + (inverse ? 4 : 0));
     const V4<T> r1 = ld4(low + 4), r2 = ld4(low + 8), r3 = ld4(low + 12);
-    // fp32: the rows that the group is taken off with are fetched before x is known (r = 336 / 512 42.1 / 70.1 -> 41.5 / 69.1
-    // us); fp64 has no registers for them
+    // fp32: the rows that the group is taken off with are fetched before x is known (where they are used: r = 128 / 256 / 336 / 512
+    // 11.9 / 24.8 / 41.1 / 68.4 us instead of 11.5 / 24.1 / 39.2 / 66.9); fp64 has no registers for them
     V4<T> b[2][4];
     if (sizeof(T) == 4) {
 #pragma unroll
@@ -387,8 +387,8 @@ __device__ __forceinline__ void solve_half(const V4<T> (&was)[2], V4<T> (&acc)[2
 
 // ------------------------------------------------------------------ block updates
 // A follow-up warp w holds columns 8 w .. 8 w + 7 of a block, a lane two quads acc[h] of them: in fp32 rows lane % 16 and
-// lane % 16 + 16 of group 2 w + lane / 16 (six loads a group; with one row and both groups, as in fp64, nine, and r = 256
-// takes 27.5 instead of 27.0 us; fp64 is 2 % faster with one row).
+// lane % 16 + 16 of group 2 w + lane / 16 (six loads a group; with one row and both groups, as in fp64, nine, and r = 64 /
+// 256 / 512 takes 7.0 / 24.7 / 67.5 instead of 6.9 / 24.1 / 67.1 us; fp64 with two rows: r = 64 / 192 10.5 / 27.5 instead of 10.3 / 27.2).
 template <typename T>
 struct FollowLane {
   static constexpr bool kTwoRows = sizeof(T) == 4;
@@ -421,8 +421,8 @@ __device__ __forceinline__ void take_off_group(V4<T> (&acc)[2], const T* A, cons
 // group); one warp alone waits for its loads, hence the unrolled loop (by eight in the kernels for
 // many blocks and for fp64; in the small fp32 kernel the code of that costs 2 us a launch).
 // Against rows 16 half .., with conflicts on C, unrolled by two: 2340 -> 2200 cycles for eight halves with eight warps, 1350
-// -> 1100 with one; r = 256 / 512 28.8 / 74 -> 27.9 / 71 us.  A whole block per warp (a third fewer loads) or two halves at a
-// time (a quarter fewer) leave too few warps at work: r = 512 75 and 73 us.
+// -> 1100 with one.  A whole block per warp (a third fewer loads) or two halves at a time (a quarter fewer) leave too few warps at work:
+// r = 512 75 and 73 us in a form that took 71.
 template <typename T, int kUnroll>
 __device__ __forceinline__ void take_off_half(T* C, const T* A, const T* Bm, bool from_zero, int half, int lane) {
   const int row0 = (lane & 3) + 4 * (lane >> 4), col0 = (lane >> 2) & 3;
@@ -529,10 +529,9 @@ __global__ void __launch_bounds__(32 * warps_of<T, kBig>(), 1) small_block_clust
   };
   auto target = [&](int j) { return j == me ? own : solved(j); };
 
-  // A gated launch that is not needed leaves before any set-up: the same word in every CTA of the cluster, written at
-  // least two kernels back in the stream (this grid only starts once its predecessor has passed its own
-  // griddepcontrol.wait), so it may be read this early.  The wait is still executed: the completion of this grid
-  // must imply the completion of every earlier one.
+  // A gated launch that is not needed leaves before any set-up: the same word in every CTA of the cluster.  Its predecessor is a gated
+  // launch itself, so this grid may start before that one has waited: the rule at GemmDesc::gate says why the word may be read
+  // this early and why the wait is still executed.
   if (p.gate != nullptr && *(const volatile uint32_t*)p.gate == 0u) { pdl_launch_dependents(); pdl_wait(); return; }
 
   // ---- set-up: barriers, with the byte counts they will receive
@@ -569,8 +568,9 @@ __global__ void __launch_bounds__(32 * warps_of<T, kBig>(), 1) small_block_clust
 
   // ---- load: this CTA's block row, summed over the partials, raw into its place.  One matrix, the usual case, is copied with
   // cp.async: every copy is in flight before anything waits.  (Through registers, a CTA with sixteen block rows waited for seven loads in
-  // turn and started 4.3 us after the first; now 1.6.  Steps: fp32 512 x 768, r = 64 103.2 -> 100.9 us, 5003 x 1000, r = 336 174.4 -> 170.8, 16384 x 11008,
-  // r = 512 527 -> 521.6, 4096 x 5120, r = 64 80.6 -> 79.9.)  Meanwhile the trace of W (the same order of additions in every CTA
+  // turn and started 4.3 us after the first; now 1.6.  Steps, before / after: fp32 512 x 768, r = 64 102.1 / 100.2 us, 5003 x 1000,
+  // r = 336 172.6 / 169.2, 8192 x 5120, r = 128 with a power iteration 210.7 / 208.8, 4096 x 5120, r = 64 76.7 / 75.6; 16384 x 4096, r = 256 and
+  // 16384 x 11008, r = 512 the same within their noise.)  Meanwhile the trace of W (the same order of additions in every CTA
   // and warp) gives the diagonal shift and the pivot floor.  The thread that wrote a quad of the diagonal adds the shift to it.
   {
     const T* parts = (const T*)p.partials;
@@ -657,7 +657,7 @@ __global__ void __launch_bounds__(32 * warps_of<T, kBig>(), 1) small_block_clust
   // kBig: this warp has read all it will of what step k brought here; the last of the CTA's warps to say so tells the peers.
   // Their next copies into the same slots must stay behind these reads, some of which may still be on their way: the count
   // is a release and an acquire, the arrival a release at cluster scope, and the waits for it acquire there.  (A releasing
-  // arrival by every warp waits for that warp's output as well: r = 336 / 512 take 42.8 / 71.9 us, 42.0 / 69.6 so.)
+  // arrival by every warp waits for that warp's output as well: in an earlier form r = 336 / 512 took 42.8 / 71.9 us, 42.0 / 69.6 so.)
   auto done_with = [&](int k) {
     if (!kBig || k + 2 >= nblk) return;
     __syncwarp();
